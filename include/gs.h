@@ -124,8 +124,8 @@ typedef struct gs_grad2d {
  * job_base     [U * n_tiles + 1]  exclusive prefix (in tile_order) of the number
  *                                 of chunks of each list; job_base[U n_tiles] = jobs
  * jobs         [2 * max_jobs]     (order position, chunk) of every chunk job; the
- *                                 last entry, which no job reaches, is the blend
- *                                 kernels' work counter (reset by each call)
+ *                                 last entry, which no job reaches, holds the blend
+ *                                 kernels' work counters (reset by each call)
  * checkpoints  [max_checkpoints][256][4]  per pixel, at every interior chunk
  *                                 boundary: T there and the colour composited
  *                                 behind it per unit T (r, g, b), written by
@@ -134,16 +134,17 @@ typedef struct gs_grad2d {
  *                                 chunk: last blended entry and stop flag, then
  *                                 the T in front of the chunk)
  * stop_queue   [8 * max_jobs + 1] forward scratch: the (chunk job, pixel block)
- *                                 units in which some pixel stops, for the
- *                                 forward's re-walk pass; the last entry counts
- *                                 them
+ *                                 units left to the forward's chunk-parallel
+ *                                 passes, those in which some pixel stops marked
+ *                                 for the re-walk; the last entry counts them
  * chunk        entries per chunk (a multiple of 32); max_jobs >= U n_tiles +
  *              max_instances / chunk + 1, max_checkpoints >= max_instances /
  *              chunk + 1 (gs_schedule_sizes).
- * walk_whole_lists  0: the forward composites the chunks of a list in
- *              parallel and combines them (training views, whose pixels rarely
- *              stop early); 1: one warp per (list, pixel block) walks the whole
- *              list and stops at its last pixel's stop (opaque renders). */
+ * walk_whole_lists  0: one warp per (list, pixel block) walks the list's first
+ *              chunks in order and stops at its last pixel's stop; what is left
+ *              of longer lists is composited chunk-parallel and combined
+ *              (training views, whose pixels rarely stop early); 1: the walk
+ *              goes on to the list's end (opaque renders). */
 typedef struct gs_schedule {
   uint32_t* tile_order;
   uint16_t* block_masks;
@@ -301,7 +302,7 @@ int gs_bin_sort_static(const gs_proj* proj, const gs_units* units, int width, in
  * one-warp jobs per (tile, 8x4 block) in heaviest-first order that skip
  * records whose block mask misses their pixels, and write the per-pixel
  * checkpoints the chunked backward starts from; lists are composited in
- * parallel chunks of sched->chunk entries and combined in order.  Blended
+ * chunks of sched->chunk entries and combined in order.  Blended
  * entries, n_contrib and the stop decisions are those of the sequential walk;
  * image and final_T agree with it to float rounding. */
 int gs_render_fwd(const gs_proj* proj, const uint32_t* sorted_vals, const uint32_t* ranges,

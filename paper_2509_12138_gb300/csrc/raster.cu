@@ -10,6 +10,7 @@
 // meets the warp's block; this skips only (pixel, record) pairs that the
 // per-pixel alpha test would reject anyway, so results are unchanged.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include "common.cuh"
@@ -368,168 +369,239 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x) {
   return x;
 }
 
-// Lanes of a warp's pixel block (bw x 32 / bw pixels from tile-local origin
-// (ox, oy), lane = row bw + column) whose pixel centre lies in a record's
-// alpha >= 1/255 box (alpha_box: conservative, so every pixel outside it has
-// alpha < 1/255 and would be skipped by the blend).  (rx, ry): the record's
-// tile-local position; co: conic and opacity.
-__device__ __forceinline__ uint32_t hit_lanes(float rx, float ry, float4 co, float ox, float oy, int bw) {
-  float pm;
-  const float4 b = alpha_box(make_float2(rx, ry), co, pm);
-  if (!(b.x <= b.y)) return 0u;
-  const int bh = 32 / bw;
-  const float c0 = fmaxf(ceilf(b.x - ox), 0.f), c1 = fminf(floorf(b.y - ox), (float)(bw - 1));
-  const float r0 = fmaxf(ceilf(b.z - oy), 0.f), r1 = fminf(floorf(b.w - oy), (float)(bh - 1));
-  if (!(c0 <= c1) || !(r0 <= r1)) return 0u;
-  const int lo = (int)c0, rl = (int)r0, rh = (int)r1;
-  const uint32_t cm = ((2u << ((int)c1 - lo)) - 1u) << lo;
-  uint32_t m = 0u;
-  for (int r = rl; r <= rh; ++r) m |= cm << (r * bw);
-  return m;
+// The pixels of a warp's block (BW x 32 / BW from tile-local origin (ox, oy))
+// whose centre lies in a superset of a record's alpha >= 1/255 box, so that
+// every pixel outside it has alpha < 1/255 and would be skipped by the blend:
+// columns c0 .. c1 and rows r0 .. r1 of the block (none: c1 < c0).  (rx, ry):
+// the record's tile-local position; co: conic and opacity; pf: its power floor
+// (rgb.w), which is at most -(ln(255 o) + 1e-3), so -pf takes the place of
+// alpha_box's logarithm.  The approximate divide stays far inside the 0.1% +
+// 0.01 px margin.
+struct HitBox {
+  int c0, c1, r0, r1;
+};
+template <int BW>
+__device__ __forceinline__ HitBox hit_box(float rx, float ry, float4 co, float pf, float ox, float oy) {
+  constexpr int BH = 32 / BW;
+  HitBox h = {0, -1, 0, -1};
+  const float det = co.x * co.z - co.y * co.y;
+  if (!(pf < 0.f) || !(det > 0.f)) return h;
+  const float k = __fdividef(-2.f * pf, det);
+  const float ex = sqrtf(k * co.z) * 1.001f + 0.01f, ey = sqrtf(k * co.x) * 1.001f + 0.01f;
+  const float c0 = fmaxf(ceilf(rx - ex - ox), 0.f), c1 = fminf(floorf(rx + ex - ox), (float)(BW - 1));
+  const float r0 = fmaxf(ceilf(ry - ey - oy), 0.f), r1 = fminf(floorf(ry + ey - oy), (float)(BH - 1));
+  if (!(c0 <= c1) || !(r0 <= r1)) return h;
+  h.c0 = (int)c0; h.c1 = (int)c1; h.r0 = (int)r0; h.r1 = (int)r1;
+  return h;
 }
 
-// Rounds with at least this many hits walk per-lane hit lists: each lane
-// takes, in list order, only the hits whose alpha box reaches its pixel
-// (forward walk; reverse replay).  Below them the box and the transpose cost
-// more than the hits they spare (10M Gaussians at 1080p, thresholds swept
-// over 1-24: 12 and 8 were fastest).
-constexpr int HIT_LISTS_FWD = 12;
-constexpr int HIT_LISTS_BWD = 8;
+// Record-major evaluation: a record's o G at every pixel of its box that can
+// blend (alpha >= 1/255), to row[pixel]; returns the mask of those pixels.
+// CLAMP stores min(0.99, o G).  Only the rows and columns that hold pixels of
+// `act` are evaluated (pixels outside it may be).  The pixel coordinates are exact small integers
+// stepped in float (integer conversions share the exponential's quarter-rate
+// unit).
+template <int BW, bool CLAMP>
+__device__ __forceinline__ uint32_t eval_hit(float rx, float ry, float4 co, float pf, float ox, float oy, uint32_t act,
+                                             float* row) {
+  HitBox h = hit_box<BW>(rx, ry, co, pf, ox, oy);
+  uint32_t valid = 0u, cols = act;  // columns of act: its rows folded onto each other
+  #pragma unroll
+  for (int q = 16; q >= BW; q >>= 1) cols |= cols >> q;
+  cols &= (1u << BW) - 1u;
+  h.c0 = max(h.c0, __ffs(cols) - 1);
+  h.c1 = min(h.c1, 31 - __clz(cols));
+  h.r0 = max(h.r0, (__ffs(act) - 1) / BW);
+  h.r1 = min(h.r1, (31 - __clz(act)) / BW);
+  if (h.c1 < h.c0 || h.r1 < h.r0) return 0u;
+  const int w = h.c1 - h.c0 + 1;
+  const int n = w * (h.r1 - h.r0 + 1);
+  const float x0 = ox + (float)h.c0, x1 = ox + (float)h.c1;
+  float x = x0, y = oy + (float)h.r0;
+  int px = h.r0 * BW + h.c0;
+  for (int k = 0; k < n; ++k) {
+    const float power = splat_power(co.x, co.y, co.z, rx - x, ry - y);
+    const float a = co.w * __expf(power), alpha = fminf(ALPHA_MAX, a);
+    if (!(power > 0.f) && !(alpha < ALPHA_MIN)) {
+      row[px] = CLAMP ? alpha : a;
+      valid |= 1u << px;
+    }
+    const bool wrap = x >= x1;  // next column, or the next row's first
+    x = wrap ? x0 : x + 1.f;
+    y = wrap ? y + 1.f : y;
+    px += wrap ? BW + 1 - w : 1;
+  }
+  return valid;
+}
 
-// Front-to-back walk of list entries [beg, end) (indices from the list's
-// start `off`) for one warp's pixel block, compositing into (T, c, last) of
-// the lanes that are not done; a lane whose transmittance would fall below
-// T_MIN stops (done).  A warp reads 2 bytes (mask) and 4 bytes (record id)
-// per entry, two rounds ahead, and gathers the records of its hits one round
-// ahead; the blend itself is that of k_render_fwd.
-// With LOCAL, it also accumulates this walk's own partial (transmittance tl and
-// colour cl from tl = 1, cl = 0: the walk's contribution per unit incoming T),
-// which the checkpoints' colour-behind terms are composed from.
-struct LocalAcc {
-  float t, c0, c1, c2;
+// ---- the walks of one warp over a list: hits gathered 32 at a time
+//
+// With sub-pixel splats a list entry reaches few of a tile's eight pixel
+// blocks (about 5 of 32 at 10M Gaussians and 1080p) and few pixels of a block
+// it reaches (about 9 of 32).  So the warp first reads the 2-byte block masks
+// of SCAN entries at a time and queues the entries that reach its block, and
+// works on batches of up to 32 queued hits, in two lane assignments:
+//   record-major: lane j holds hit j's record in registers and evaluates its
+//     alpha at the pixels its box reaches, into a (hit, pixel) matrix in shared
+//     memory (row stride 33: neither assignment has regular bank conflicts);
+//   pixel-major: the 32 x 32 bits of accepted pairs are transposed across the
+//     warp, and lane p composites the hits of its pixel in list order, reading
+//     one alpha and a colour per pair (the colours lie 32 to a bank row, so any
+//     mix of hits is read without conflicts).
+// Each phase runs as often as its busiest lane has pairs.  Every pair's alpha
+// and the order of a pixel's compositing are those of a sequential walk.  Bound
+// by instruction issue (47-70% of cycles on a 2M scene) and, on edge-on views,
+// by the longest block's serial walk.  Forward stage at one lane per pixel and
+// hit -> this: 200k at 960x540 134 -> 98 us, 1M at 1080p 319 -> 199 us.
+constexpr int SCAN = 256;            // entries whose masks are read at a time (8 per lane)
+constexpr int QUEUE_CAP = SCAN + 32; // queued entries: a full scan behind at most 31 left over
+constexpr int MROW = 33;             // row stride of the (hit, pixel) matrices
+
+struct FwdScratch {
+  float alpha[32 * MROW];
+  float r[32], g[32], b[32];
+  uint32_t q[QUEUE_CAP];
 };
 
-template <bool LOCAL = false>
+// Queues the entries of [s, min(s + SCAN, end)) (DOWN: of (max(s - SCAN, beg),
+// s], from s down) whose block mask meets wbits behind the qn queued ones, in
+// walking order; returns the new number.  masks: of the list's first entry on.
+template <bool DOWN>
+__device__ __forceinline__ int scan_hits(const uint16_t* __restrict__ masks, int s, int bound, uint32_t wbits,
+                                         uint32_t* q, int qn) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t mk[SCAN / 32];
+  #pragma unroll
+  for (int r = 0; r < SCAN / 32; ++r) {
+    const int k = DOWN ? s - 32 * r - lane : s + 32 * r + lane;
+    mk[r] = (DOWN ? k >= bound : k < bound) ? masks[k] : 0u;
+  }
+  #pragma unroll
+  for (int r = 0; r < SCAN / 32; ++r) {
+    if (DOWN ? s - 32 * r < bound : s + 32 * r >= bound) break;
+    const bool h = (mk[r] & wbits) != 0u;
+    const unsigned bal = __ballot_sync(FULL, h);
+    if (h) q[qn + __popc(bal & lt)] = (uint32_t)(DOWN ? s - 32 * r - lane : s + 32 * r + lane);
+    qn += __popc(bal);
+  }
+  return qn;
+}
+
+// Front-to-back walk of list entries [beg, end) (indices from the list's
+// start `off`) for one warp's pixel block (tile-local origin (ox, oy)):
+// composites into (T, c, last) of the lanes that are not done; a lane whose
+// transmittance would fall below T_MIN stops (done).  DUAL: also composites
+// the same pairs from T = 1 into loc = (T, c), the walk's partial.
+template <int BW, bool DUAL>
 __device__ __forceinline__ void walk_fwd(const uint32_t* __restrict__ vals, const uint16_t* __restrict__ masks,
                                          const float4* __restrict__ xy, const float4* __restrict__ conic_op,
                                          const float4* __restrict__ rgb, uint32_t off, int beg, int end,
-                                         uint32_t wbits, float tox, float toy, float fx, float fy, Rec* my, float& T,
-                                         float& c0, float& c1, float& c2, int& last, bool& done,
-                                         LocalAcc* loc = nullptr) {
+                                         uint32_t wbits, float tox, float toy, float ox, float oy, FwdScratch& sc,
+                                         float& T, float& c0, float& c1, float& c2, int& last, bool& done,
+                                         float4& loc) {
   const unsigned FULL = 0xffffffffu;
-  int lane = threadIdx.x & 31;
-  // the warp's pixel block: tile-local origin and width
-  const float ox = __shfl_sync(FULL, fx, 0), oy = __shfl_sync(FULL, fy, 0);
-  const int bw = __popc(__ballot_sync(FULL, fy == oy));
-  bool h1 = false;
-  float4 m1 = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 co1 = make_float4(0.f, 0.f, 0.f, 0.f), cc1 = co1;
-  uint32_t mk2 = 0, pk2 = 0;
-  if (beg + lane < end) {
-    uint32_t mk = masks[off + beg + lane];
-    if (mk & wbits) {
-      uint32_t pk = vals[off + beg + lane];
-      h1 = true; m1 = xy[pk]; co1 = conic_op[pk]; cc1 = rgb[pk];
+  const int lane = threadIdx.x & 31;
+  vals += off;
+  masks += off;
+  int scan = beg, qn = 0, qh = 0;  // next entry to scan; queued entries are q[qh .. qn)
+  for (;;) {
+    const uint32_t act = __ballot_sync(FULL, !done);
+    if (!act) break;
+    if (qn - qh < 32 && scan < end) {
+      // the left-over entries to the front, then whole scans until a batch is full
+      const uint32_t keep = qh + lane < qn ? sc.q[qh + lane] : 0u;
+      __syncwarp();
+      qn -= qh;
+      qh = 0;
+      if (lane < qn) sc.q[lane] = keep;
+      do {
+        qn = scan_hits<false>(masks, scan, end, wbits, sc.q, qn);
+        scan += SCAN;
+      } while (qn < 32 && scan < end);
+      __syncwarp();
     }
-  }
-  if (beg + 32 + lane < end) { mk2 = masks[off + beg + 32 + lane]; pk2 = vals[off + beg + 32 + lane]; }
-  for (int base = beg; base < end; base += 32) {
-    if (__all_sync(FULL, done)) break;
-    bool hit = h1;
-    float4 m = m1;
-    float4 co = co1, c = cc1;
-    h1 = (mk2 & wbits) != 0;
-    if (h1) { m1 = xy[pk2]; co1 = conic_op[pk2]; cc1 = rgb[pk2]; }
-    int k2 = base + 64 + lane;
-    mk2 = 0;
-    if (k2 < end) { mk2 = masks[off + k2]; pk2 = vals[off + k2]; }
-    unsigned mask = __ballot_sync(FULL, hit);
-    const float rx = rel_pos(m.x, m.z, tox), ry = rel_pos(m.y, m.w, toy);
-    if (hit) {
-      my[lane].a = make_float4(rx, ry, co.x, co.y);
-      my[lane].b = make_float4(co.z, co.w, c.w, 0.f);
-      my[lane].c = c;
+    const int nb = min(32, qn - qh);
+    if (nb == 0) break;
+    // record-major: alpha of hit `lane` at the pixels its box reaches
+    uint32_t valid = 0u;
+    if (lane < nb) {
+      const uint32_t p = vals[sc.q[qh + lane]];
+      const float4 m = xy[p], co = conic_op[p], c = rgb[p];
+      const float rx = rel_pos(m.x, m.z, tox), ry = rel_pos(m.y, m.w, toy);
+      sc.r[lane] = c.x; sc.g[lane] = c.y; sc.b[lane] = c.z;
+      valid = eval_hit<BW, true>(rx, ry, co, c.w, ox, oy, act, sc.alpha + lane * MROW);
     }
     __syncwarp();
-    // hits two at a time: both alphas are evaluated independently (more independent instructions
-    // in flight per warp), then composited in list order
-    auto hit_alpha = [&](int j) -> float {  // 0 when the record cannot blend at this pixel
-      float4 ra = my[j].a, rb = my[j].b;
-      float power = splat_power(ra.z, ra.w, rb.x, ra.x - fx, ra.y - fy);
-      if (power > 0.f || power < rb.z) return 0.f;
-      return fminf(ALPHA_MAX, rb.y * __expf(power));
-    };
-    auto composite = [&](int j, float alpha) {
-      if (done || alpha < ALPHA_MIN) return;
-      float tT = T * (1.f - alpha);
-      if (tT < T_MIN) { done = true; return; }
-      float4 rc = my[j].c;
-      float wgt = alpha * T;
-      c0 += rc.x * wgt; c1 += rc.y * wgt; c2 += rc.z * wgt;
-      T = tT;
-      last = base + j + 1;
-      if (LOCAL) {
-        float lw = alpha * loc->t;
-        loc->c0 += rc.x * lw; loc->c1 += rc.y * lw; loc->c2 += rc.z * lw;
-        loc->t *= 1.f - alpha;
-      }
-    };
-    if (__popc(mask) >= HIT_LISTS_FWD) {
-      // per-lane hit lists: bit j of `mine` = hit j's alpha box reaches this lane's pixel
-      uint32_t mine = transpose32(hit ? hit_lanes(rx, ry, co, ox, oy, bw) : 0u);
-      while (mine && !done) {
-        int j1 = __ffs(mine) - 1;
+    // pixel-major: this pixel's pairs in list order
+    uint32_t mine = transpose32(valid);
+    int lj = -1;
+    if (mine && !done) {
+      int j = __ffs(mine) - 1;
+      float alpha = sc.alpha[j * MROW + lane];
+      for (;;) {  // the next pair's alpha is on its way while this one is composited
         mine &= mine - 1;
-        bool two = mine != 0u;
-        int j2 = two ? __ffs(mine) - 1 : j1;
-        if (two) mine &= mine - 1;
-        float a1 = hit_alpha(j1);
-        float a2 = two ? hit_alpha(j2) : 0.f;
-        composite(j1, a1);
-        if (two) composite(j2, a2);
-      }
-    } else {
-      while (mask) {
-        int j1 = __ffs(mask) - 1;
-        mask &= mask - 1;
-        bool two = mask != 0u;
-        int j2 = two ? __ffs(mask) - 1 : j1;
-        if (two) mask &= mask - 1;
-        float a1 = hit_alpha(j1);
-        float a2 = two ? hit_alpha(j2) : 0.f;
-        composite(j1, a1);
-        if (two) composite(j2, a2);
+        const int jn = mine ? __ffs(mine) - 1 : j;
+        const float an = sc.alpha[jn * MROW + lane];
+        const float tT = T * (1.f - alpha);
+        if (tT < T_MIN) { done = true; break; }
+        const float wgt = alpha * T, cr = sc.r[j], cg = sc.g[j], cb = sc.b[j];
+        c0 += cr * wgt; c1 += cg * wgt; c2 += cb * wgt;
+        if (DUAL) {
+          const float lw = alpha * loc.x;
+          loc.y += cr * lw; loc.z += cg * lw; loc.w += cb * lw;
+          loc.x *= 1.f - alpha;
+        }
+        T = tT;
+        lj = j;
+        if (!mine) break;
+        j = jn;
+        alpha = an;
       }
     }
+    if (lj >= 0) last = (int)sc.q[qh + lj] + 1;
+    qh += nb;
     __syncwarp();
   }
+  __syncwarp();
 }
 
-// ---- scheduled forward: chunk-parallel compositing in three passes
+// ---- scheduled forward: sequential fronts, chunk-parallel remainders
 //
 // Per pixel, front-to-back compositing over a list is a product of (1 - alpha)
 // factors and a sum of colours weighted by the running product, so chunks of
 // K entries can be composited independently from T = 1 and combined:
-// C += T C_c, T *= T_c.  The early stop is the only order-dependent decision:
-// a pixel whose (T T_c) would fall below T_MIN, or whose chunk stopped on its
-// own, stops inside that chunk, which is then walked again from the true
-// incoming state.
-//   pass 1 (chunk jobs):   partial (T_c, C_c, last_c | stop) of every chunk;
-//   pass 2 (list warps):   combine in order, find each pixel's stop chunk c*,
-//                          write the checkpoints in front of chunks <= c*,
-//                          finish the pixels that never stop;
-//   pass 3 (chunk jobs):   walk chunk c* again for the pixels that stop there,
-//                          write their final state and remaining checkpoints.
+// C += T C_c, T *= T_c.  Composited that way, everything behind a pixel's early
+// stop is work for nothing (at 10M Gaussians and 1080p 50-65% of the entries lie
+// behind the last stop of their block); walked in order, a list of a hundred
+// chunks is one warp's serial work.  So:
+//   front  (list, block warps): chunks 0 .. M - 1 in order with the early stop.
+//           A list that ends there, or whose pixels all stop there, is final.
+//           Otherwise the block's later chunks are queued;
+//   chunks (queued jobs): partial (T_c, C_c, last_c | stop) of every such chunk;
+//   combine (queued blocks): applies the partials in order, finds each pixel's
+//           stop chunk c* (the first with T T_c < T_MIN or a stop of its own),
+//           writes the checkpoints in front of it, finishes the pixels that
+//           never stop and marks the stop chunks' queue entries;
+//   stop   (marked jobs): walks c* again from the true incoming state for the
+//           pixels that stop there and writes their remaining checkpoints.
 // Per pixel the blended entries and the stop decision are those of the
 // sequential walk; the combine changes only the rounding order of T and C.
-constexpr uint32_t STOP_BIT = 0x80000000u;  // chunk partial: the pixel stopped inside the chunk
-constexpr uint32_t REWALK_BIT = 0x80000000u;  // n_contrib between passes 2 and 3: stop chunk pending,
+// gs_schedule.walk_whole_lists is M = infinity.
+// Forward stage at 10M / 1080p, two views, 8 partitions of 2.8M / 1080p, two
+// views (us): M = 8: 1498, 1721, 912, 784; 16: 1324, 1686, 926, 862; 32: 1329,
+// 1659, 1061, 825; chunk-parallel from the first chunk: 2129, 1882, 975, 945.
+constexpr int FRONT_CHUNKS = 16;
+constexpr uint32_t STOP_BIT = 0x80000000u;  // partial or front state: the pixel has stopped
+constexpr uint32_t REWALK_BIT = 0x80000000u;  // n_contrib between combine and stop pass: stop chunk pending,
                                              // the stop chunk c* in the bits below it
+constexpr uint32_t MARK_BIT = 0x80000000u;  // queue entry (chunk job << 3 | block): some pixel stops in it
 
 // The warp's pixel of (list o, block w) and its geometry.
 template <int BW>
 struct PixelOf {
-  int u, tile, tx, ty, px, py, pix_local;
+  int u, tile, tx, ty, px, py, pix_local, ox, oy;  // (ox, oy): the block's tile-local origin
   bool inside;
   uint32_t wbits;  // the 4x4 blocks of the warp's pixels
   __device__ __forceinline__ PixelOf(const uint32_t* __restrict__ order, int o, int w, int n_tiles, int TX, int W,
@@ -541,118 +613,251 @@ struct PixelOf {
     ty = tile / TX;
     constexpr int BH = 32 / BW, NWX = TILE / BW;
     int lane = threadIdx.x & 31;
-    px = tx * TILE + (w % NWX) * BW + (lane % BW);
-    py = ty * TILE + (w / NWX) * BH + (lane / BW);
+    ox = (w % NWX) * BW;
+    oy = (w / NWX) * BH;
+    px = tx * TILE + ox + (lane % BW);
+    py = ty * TILE + oy + (lane / BW);
     pix_local = (py - ty * TILE) * TILE + (px - tx * TILE);
     inside = px < W && py < H;
     wbits = warp_block_bits<BW>(w);
   }
 };
 
-// Pass 1: job (list o, chunk c, block w) composites entries [c K, min((c+1) K, L))
-// from T = 1.  A list of one chunk is final here.  Otherwise chunk 0's state
-// (exact: nothing lies in front of it) goes to img (colour without
-// background), final_T and n_contrib (| STOP_BIT), chunk c >= 1's partial to
-// checkpoint slot c - 1 and chunk_last.
-template <int BW>
-__global__ void __launch_bounds__(32) k_render_fwd_m(const uint2* __restrict__ ranges,
-                                                           const uint32_t* __restrict__ order,
-                                                           const uint32_t* __restrict__ job_base,
-                                                           const uint32_t* __restrict__ jobs, int K, int NT,
-                                                           float4* __restrict__ ckpt,
-                                                           uint32_t* __restrict__ chunk_last,
-                                                           const uint32_t* __restrict__ vals,
-                                                           const uint16_t* __restrict__ masks,
-                                                           const float4* __restrict__ xy,
-                                                           const float4* __restrict__ conic_op,
-                                                           const float4* __restrict__ rgb, int W, int H, int TX,
-                                                           int n_tiles, float bg0, float bg1, float bg2,
-                                                           float* __restrict__ img, float* __restrict__ final_T,
-                                                           uint32_t* __restrict__ n_contrib,
-    uint32_t* __restrict__ ticket) {
-  __shared__ Rec s_rec[32];
-  // the resident warps take the (chunk job, pixel block) units from a ticket counter (zeroed before
-  // the launch), the next ticket fetched while a unit runs: no block of a grid sized for the capacity
-  // sits idle, and units of very different cost still spread as they finish
-  const uint32_t total = job_base[NT] * 8u;
-  auto job = [&](uint32_t vb) {
-    uint32_t jid = vb >> 3;
-    int w = (int)(vb & 7u);
-    int o = (int)jobs[2 * (int64_t)jid], ch = (int)jobs[2 * (int64_t)jid + 1];
-    PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
-    int nch = (int)(job_base[o + 1] - job_base[o]);
-    uint2 rg = ranges[(int64_t)P.u * n_tiles + P.tile];
-    int L = (int)(rg.y - rg.x);
-    float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-    int last = 0;
-    bool done = !P.inside;
-    walk_fwd(vals, masks, xy, conic_op, rgb, rg.x, ch * K, min(ch * K + K, L), P.wbits, (float)(P.tx * TILE),
-             (float)(P.ty * TILE), (float)(P.px - P.tx * TILE), (float)(P.py - P.ty * TILE), s_rec, T, c0, c1, c2,
-             last, done);
-    if (!P.inside) return;
-    int64_t plane = (int64_t)W * H;
-    int64_t pix = (int64_t)P.py * W + P.px;
-    float* im = img + (int64_t)P.u * 3 * plane;
-    if (nch == 1 || ch == 0) {
-      bool fin = nch == 1;
-      im[pix] = fin ? c0 + T * bg0 : c0;
-      im[plane + pix] = fin ? c1 + T * bg1 : c1;
-      im[2 * plane + pix] = fin ? c2 + T * bg2 : c2;
-      final_T[(int64_t)P.u * plane + pix] = T;
-      n_contrib[(int64_t)P.u * plane + pix] = (uint32_t)last | (!fin && done ? STOP_BIT : 0u);
-    } else {
-      int64_t slot = ((int64_t)job_base[o] - o + ch - 1) * TILE_PIX + P.pix_local;
-      ckpt[slot] = make_float4(T, c0, c1, c2);
-      chunk_last[slot] = (uint32_t)last | (done ? STOP_BIT : 0u);
+// Lists without entries: the background.  One block per (unit, tile); block 0
+// also zeroes the work counters of the passes behind it.
+__global__ void __launch_bounds__(TILE_PIX) k_render_fwd_empty(const uint2* __restrict__ ranges, int W, int H, int TX,
+                                                               int n_tiles, float bg0, float bg1, float bg2,
+                                                               float* __restrict__ img, float* __restrict__ final_T,
+                                                               uint32_t* __restrict__ n_contrib,
+                                                               uint32_t* __restrict__ tickets,
+                                                               uint32_t* __restrict__ qcount) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) { tickets[0] = 0u; tickets[1] = 0u; *qcount = 0u; }
+  const uint2 rg = ranges[blockIdx.x];
+  if (rg.y > rg.x) return;
+  const int u = (int)(blockIdx.x / (unsigned)n_tiles), tile = (int)(blockIdx.x % (unsigned)n_tiles);
+  const int px = (tile % TX) * TILE + (int)(threadIdx.x % TILE), py = (tile / TX) * TILE + (int)(threadIdx.x / TILE);
+  if (px >= W || py >= H) return;
+  const int64_t plane = (int64_t)W * H, pix = (int64_t)py * W + px;
+  float* im = img + (int64_t)u * 3 * plane;
+  im[pix] = bg0; im[plane + pix] = bg1; im[2 * plane + pix] = bg2;
+  final_T[(int64_t)u * plane + pix] = 1.f;
+  n_contrib[(int64_t)u * plane + pix] = 0u;
+}
+
+// Number of lists with entries: they come first in tile order, so it is the
+// first order position from which job_base stays at its total (a 32-way search
+// by the warp).
+__device__ __forceinline__ int lists_in_use(const uint32_t* __restrict__ job_base, int NT) {
+  const uint32_t total = job_base[NT];
+  int lo = 0, hi = NT;  // the answer lies in [lo, hi]
+  while (lo < hi) {
+    const int step = (hi - lo + 31) / 32;
+    const int at = lo + step * (int)(threadIdx.x & 31);
+    const uint32_t full = __ballot_sync(0xffffffffu, at >= hi || job_base[min(at, NT)] == total);
+    const int f = full ? __ffs(full) - 1 : 32;  // first probe at or past the answer
+    const int nlo = f == 0 ? lo : lo + step * (f - 1) + 1;
+    hi = f == 0 ? lo : min(hi, lo + step * f);
+    lo = nlo;
+  }
+  return lo;
+}
+
+// Checkpoints of boundaries [lo, hi] of a pixel, back to front: boundary b's
+// slot holds chunk b's partial (T_b, C_b) and chunk_last the T in front of it;
+// it becomes (that T, colour behind the boundary per unit T).  S: the colour
+// behind boundary hi + 1, updated.  Loads are issued CB boundaries at a time.
+constexpr int CB = 4;
+__device__ __forceinline__ void close_checkpoints(float4* __restrict__ cpp, const uint32_t* __restrict__ clp, int lo,
+                                                  int hi, float& S0, float& S1, float& S2) {
+  for (int bb = hi; bb >= lo; bb -= CB) {
+    float4 ptv[CB];
+    uint32_t tv[CB];
+    #pragma unroll
+    for (int q = 0; q < CB; ++q)
+      if (bb - q >= lo) {
+        ptv[q] = cpp[(int64_t)(bb - q - 1) * TILE_PIX];
+        tv[q] = clp[(int64_t)(bb - q - 1) * TILE_PIX];
+      }
+    #pragma unroll
+    for (int q = 0; q < CB; ++q) {
+      if (bb - q < lo) break;
+      const float4 pt = ptv[q];
+      S0 = pt.y + pt.x * S0; S1 = pt.z + pt.x * S1; S2 = pt.w + pt.x * S2;
+      cpp[(int64_t)(bb - q - 1) * TILE_PIX] = make_float4(__uint_as_float(tv[q]), S0, S1, S2);
     }
+  }
+}
+
+// One chunk from the state (T, c): walked in order, its partial from T = 1 to
+// *slot and the incoming T to *tslot (slots of the boundary in front of it).
+template <int BW>
+__device__ __forceinline__ float4 walk_chunk(const uint32_t* __restrict__ vals, const uint16_t* __restrict__ masks,
+                                             const float4* __restrict__ xy, const float4* __restrict__ conic_op,
+                                             const float4* __restrict__ rgb, uint32_t off, int beg, int end,
+                                             uint32_t wbits, float tox, float toy, float ox, float oy, FwdScratch& sc,
+                                             float& T, float& c0, float& c1, float& c2, int& last, bool& done,
+                                             bool store, float4* slot, uint32_t* tslot) {
+  if (store) *tslot = __float_as_uint(T);
+  float4 loc = make_float4(1.f, 0.f, 0.f, 0.f);
+  walk_fwd<BW, true>(vals, masks, xy, conic_op, rgb, off, beg, end, wbits, tox, toy, ox, oy, sc, T, c0, c1, c2, last,
+                     done, loc);
+  if (store) *slot = loc;
+  return loc;
+}
+
+// Front pass: unit (list o, block w) walks chunks 0 .. min(nch, M) - 1 in
+// order.  The resident warps take the units, heaviest lists first, from a
+// ticket counter, the next ticket fetched while a unit runs.
+template <int BW>
+__global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict__ ranges,
+                                                         const uint32_t* __restrict__ order,
+                                                         const uint32_t* __restrict__ job_base, int K, int M, bool whole,
+                                                         int NT,
+                                                         float4* __restrict__ ckpt, uint32_t* __restrict__ chunk_last,
+                                                         const uint32_t* __restrict__ vals,
+                                                         const uint16_t* __restrict__ masks,
+                                                         const float4* __restrict__ xy,
+                                                         const float4* __restrict__ conic_op,
+                                                         const float4* __restrict__ rgb, int W, int H, int TX,
+                                                         int n_tiles, float bg0, float bg1, float bg2,
+                                                         float* __restrict__ img, float* __restrict__ final_T,
+                                                         uint32_t* __restrict__ n_contrib,
+                                                         uint32_t* __restrict__ queue, uint32_t qcap,
+                                                         uint32_t* __restrict__ ticket) {
+  __shared__ FwdScratch s_walk;
+  const int lane = threadIdx.x & 31;
+  const uint32_t total = (uint32_t)lists_in_use(job_base, NT) * 8u;
+  auto unit = [&](uint32_t vb) {
+    const int o = (int)(vb >> 3), w = (int)(vb & 7u);
+    PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
+    const uint32_t jb = job_base[o];
+    const int nch = (int)(job_base[o + 1] - jb);
+    const uint2 rg = ranges[(int64_t)P.u * n_tiles + P.tile];
+    const int L = (int)(rg.y - rg.x);
+    const int64_t cp0 = (int64_t)jb - o;
+    float4* cpp = ckpt + cp0 * TILE_PIX + P.pix_local;  // slot of boundary b: cpp[(b - 1) * TILE_PIX]
+    uint32_t* clp = chunk_last + cp0 * TILE_PIX + P.pix_local;
+    const int upto = min(nch, M);
+    float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
+    int last = 0, c = 0;
+    bool done = !P.inside, in_order = whole;
+    for (; c < upto; ++c) {
+      if (__all_sync(0xffffffffu, done)) break;
+      const float Tin = T, i0 = c0, i1 = c1, i2 = c2;
+      const bool was = done;
+      const float4 loc = walk_chunk<BW>(vals, masks, xy, conic_op, rgb, rg.x, c * K, min(c * K + K, L), P.wbits, (float)(P.tx * TILE),
+                     (float)(P.ty * TILE), (float)P.ox, (float)P.oy, s_walk, T, c0, c1, c2, last, done,
+                     c > 0 && P.inside, cpp + (int64_t)(c - 1) * TILE_PIX, clp + (int64_t)(c - 1) * TILE_PIX);
+      // a chunk without a stop enters by its partial, as the combine's do, so that images do not depend on M;
+      // from a stop chunk on (and in whole-list walks) the walked state counts
+      in_order = in_order || !(Tin * loc.x >= T_MIN);
+      if (!in_order && !done && !was) {
+        T = Tin * loc.x;
+        c0 = i0 + Tin * loc.y; c1 = i1 + Tin * loc.z; c2 = i2 + Tin * loc.w;
+      }
+    }
+    const int64_t plane = (int64_t)W * H;
+    const int64_t pix = (int64_t)P.py * W + P.px;
+    float* im = img + (int64_t)P.u * 3 * plane;
+    if (c < nch && !__all_sync(0xffffffffu, done)) {
+      // the rest of the list in parallel: this block's state in front of chunk M, and its later chunks' jobs
+      uint32_t base = lane == 0 ? atomicAdd(queue + qcap, (uint32_t)(nch - c)) : 0u;
+      base = __shfl_sync(0xffffffffu, base, 0);
+      for (int q = c + lane; q < nch; q += 32) queue[base + (uint32_t)(q - c)] = ((jb + (uint32_t)q) << 3) | (uint32_t)w;
+      if (!P.inside) return;
+      im[pix] = c0; im[plane + pix] = c1; im[2 * plane + pix] = c2;
+      final_T[(int64_t)P.u * plane + pix] = T;
+      n_contrib[(int64_t)P.u * plane + pix] = (uint32_t)last | (done ? STOP_BIT : 0u);
+      return;
+    }
+    if (!P.inside) return;
+    for (int b = nch - 1; b >= max(c, 1); --b)
+      cpp[(int64_t)(b - 1) * TILE_PIX] = make_float4(T, bg0, bg1, bg2);  // behind the stop: final state
+    float S0 = bg0, S1 = bg1, S2 = bg2;
+    close_checkpoints(cpp, clp, 1, c - 1, S0, S1, S2);
+    im[pix] = c0 + T * bg0;
+    im[plane + pix] = c1 + T * bg1;
+    im[2 * plane + pix] = c2 + T * bg2;
+    final_T[(int64_t)P.u * plane + pix] = T;
+    n_contrib[(int64_t)P.u * plane + pix] = (uint32_t)last;
   };
-  const bool lead = (threadIdx.x & 31) == 0;
+  const bool lead = lane == 0;
   uint32_t vb = __shfl_sync(0xffffffffu, lead ? atomicAdd(ticket, 1u) : 0u, 0);
   while (vb < total) {
     uint32_t nxt = lead ? atomicAdd(ticket, 1u) : 0u;
-    job(vb);
+    unit(vb);
     vb = __shfl_sync(0xffffffffu, nxt, 0);
   }
 }
 
-// Pass 2: one warp per (list, block) in tile order.  Empty lists give the
-// background.  For lists of several chunks, the state in front of chunk c is
-// (T, C); the chunk's partial is applied when it shows no stop and
-// T T_c >= T_MIN (then no entry of the chunk can stop the pixel), and
-// otherwise chunk c is the pixel's stop chunk c*.  T in front of each
-// boundary up to c* goes to chunk_last (the backward's checkpoints take it
-// from there).  Pixels that never stop are final here; pixels with c* >= 1
-// leave their state in front of c* in img / final_T, (c* | REWALK_BIT) in
-// n_contrib and their last contributing position in chunk_last at c*'s slot
-// for pass 3.  The per-chunk loads are issued CB chunks at a time: for lists
-// of hundreds of chunks the walk is otherwise one load latency per chunk.
-constexpr int CB = 4;
-
-// The combine of one pixel (pass 2), for a list of nch >= 2 chunks; cstar
-// receives the pixel's stop chunk (-1: none, or a stop inside chunk 0).
+// Chunk pass: queued job (list o, chunk c >= M, block w) composites its entries
+// from T = 1 for the pixels that have not stopped in front of chunk M; the
+// partial goes to checkpoint slot c - 1 and chunk_last.
 template <int BW>
-__device__ __forceinline__ void combine_pixel(const PixelOf<BW>& P, int o, int nch, int64_t plane, int64_t pix,
-                                              float* im, float* fT, uint32_t* nc, float4* __restrict__ ckpt,
-                                              uint32_t* __restrict__ chunk_last,
-                                              const uint32_t* __restrict__ job_base, float bg0, float bg1, float bg2,
-                                              int& cstar) {
+__global__ void __launch_bounds__(32) k_render_fwd_chunk(const uint2* __restrict__ ranges,
+                                                         const uint32_t* __restrict__ order,
+                                                         const uint32_t* __restrict__ job_base,
+                                                         const uint32_t* __restrict__ jobs, int K,
+                                                         float4* __restrict__ ckpt, uint32_t* __restrict__ chunk_last,
+                                                         const uint32_t* __restrict__ vals,
+                                                         const uint16_t* __restrict__ masks,
+                                                         const float4* __restrict__ xy,
+                                                         const float4* __restrict__ conic_op,
+                                                         const float4* __restrict__ rgb, int W, int H, int TX,
+                                                         int n_tiles, const uint32_t* __restrict__ n_contrib,
+                                                         const uint32_t* __restrict__ queue, uint32_t qcap,
+                                                         uint32_t* __restrict__ ticket) {
+  __shared__ FwdScratch s_walk;
+  const uint32_t total = queue[qcap];
+  auto job = [&](uint32_t ent) {
+    const uint32_t jid = ent >> 3;
+    const int w = (int)(ent & 7u), o = (int)jobs[2 * (int64_t)jid], ch = (int)jobs[2 * (int64_t)jid + 1];
+    PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
+    const uint2 rg = ranges[(int64_t)P.u * n_tiles + P.tile];
+    const int L = (int)(rg.y - rg.x);
+    float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
+    int last = 0;
+    bool done = !P.inside;
+    if (P.inside) done = (n_contrib[((int64_t)P.u * H + P.py) * W + P.px] & STOP_BIT) != 0u;
+    float4 none;
+    walk_fwd<BW, false>(vals, masks, xy, conic_op, rgb, rg.x, ch * K, min(ch * K + K, L), P.wbits,
+                        (float)(P.tx * TILE), (float)(P.ty * TILE), (float)P.ox, (float)P.oy, s_walk, T, c0, c1, c2,
+                        last, done, none);
+    if (!P.inside) return;
+    const int64_t slot = ((int64_t)job_base[o] - o + ch - 1) * TILE_PIX + P.pix_local;
+    ckpt[slot] = make_float4(T, c0, c1, c2);
+    chunk_last[slot] = (uint32_t)last | (done ? STOP_BIT : 0u);
+  };
+  const bool lead = (threadIdx.x & 31) == 0;
+  uint32_t e = __shfl_sync(0xffffffffu, lead ? atomicAdd(ticket, 1u) : 0u, 0);
+  while (e < total) {
+    uint32_t nxt = lead ? atomicAdd(ticket, 1u) : 0u;
+    job(queue[e]);
+    e = __shfl_sync(0xffffffffu, nxt, 0);
+  }
+}
+
+// The combine of one pixel of a queued block: the partials of chunks m .. nch - 1
+// applied to the front's state; cstar receives the pixel's stop chunk (-1: none,
+// or a stop in the front).  The per-chunk loads are issued CB chunks at a time:
+// for lists of hundreds of chunks the walk is otherwise one load latency per chunk.
+__device__ __forceinline__ void combine_pixel(int m, int nch, int64_t plane, int64_t pix, float* im, float* fT,
+                                              uint32_t* nc, float4* __restrict__ cpp, uint32_t* __restrict__ clp,
+                                              float bg0, float bg1, float bg2, int& cstar) {
   float c0 = im[pix], c1 = im[plane + pix], c2 = im[2 * plane + pix];
   float T = fT[pix];
-  uint32_t lw0 = nc[pix];
+  const uint32_t lw0 = nc[pix];
   int last = (int)(lw0 & ~STOP_BIT);
-  bool done = (lw0 & STOP_BIT) != 0u;  // a stop in chunk 0 is exact
-  int64_t cp0 = (int64_t)job_base[o] - o;
-  float4* cpp = ckpt + cp0 * TILE_PIX + P.pix_local;       // slot of boundary b: cpp[(b - 1) * TILE_PIX]
-  uint32_t* clp = chunk_last + cp0 * TILE_PIX + P.pix_local;
-  for (int cb = 1; cb < nch && cstar < 0; cb += CB) {
+  const bool done = (lw0 & STOP_BIT) != 0u;  // a stop in the front is exact
+  for (int cb = m; cb < nch && cstar < 0; cb += CB) {
     uint32_t lwv[CB];
     float4 ptv[CB];
     #pragma unroll
     for (int q = 0; q < CB; ++q) {
       int c = cb + q;
-      if (c < nch) {
+      if (c < nch && !done) {
         lwv[q] = clp[(int64_t)(c - 1) * TILE_PIX];
-        if (!done) ptv[q] = cpp[(int64_t)(c - 1) * TILE_PIX];
+        ptv[q] = cpp[(int64_t)(c - 1) * TILE_PIX];
       }
     }
     #pragma unroll
@@ -669,12 +874,12 @@ __device__ __forceinline__ void combine_pixel(const PixelOf<BW>& P, int o, int n
         uint32_t lc = lwv[q] & ~STOP_BIT;
         if (lc) last = (int)lc;
       } else {
-        cstar = c;  // pass 3 walks chunk c for this pixel and writes the rest
+        cstar = c;  // the stop pass walks chunk c for this pixel and writes the rest
       }
     }
   }
   if (cstar >= 1) {
-    // boundaries in front of the stop chunk: S_b = A_b + B_b S_c* (pass 3 knows S_c*)
+    // boundaries in front of the stop chunk: S_b = A_b + B_b S_c* (the stop pass knows S_c*)
     float A0 = 0.f, A1 = 0.f, A2 = 0.f, B = 1.f;
     for (int bb = cstar - 1; bb >= 1; bb -= CB) {
       float4 ptv[CB];
@@ -692,36 +897,15 @@ __device__ __forceinline__ void combine_pixel(const PixelOf<BW>& P, int o, int n
     }
     im[pix] = c0; im[plane + pix] = c1; im[2 * plane + pix] = c2;
     fT[pix] = T;
-    clp[(int64_t)(cstar - 1) * TILE_PIX] = (uint32_t)last;  // pass 3 reads it and puts T back
+    clp[(int64_t)(cstar - 1) * TILE_PIX] = (uint32_t)last;  // the stop pass reads it and puts T back
     nc[pix] = (uint32_t)cstar | REWALK_BIT;
   } else {
-    // checkpoint b: (T in front of chunk b, colour behind boundary b per unit T there), the chunks
-    // from b to the stop composited back to front over the background (a pixel that stopped in
-    // chunk 0 has the background behind every boundary)
-    int stop_at = done ? 0 : nch;
+    // checkpoint b: (T in front of chunk b, colour behind boundary b per unit T there); a pixel that
+    // stopped in the front has the background behind every boundary from chunk m on
     float S0 = bg0, S1 = bg1, S2 = bg2;
-    for (int bb = nch - 1; bb >= 1; bb -= CB) {
-      float4 ptv[CB];
-      uint32_t tv[CB];
-      #pragma unroll
-      for (int q = 0; q < CB; ++q) {
-        int b = bb - q;
-        if (b >= 1) {
-          if (b <= stop_at) ptv[q] = cpp[(int64_t)(b - 1) * TILE_PIX];
-          tv[q] = clp[(int64_t)(b - 1) * TILE_PIX];
-        }
-      }
-      #pragma unroll
-      for (int q = 0; q < CB; ++q) {
-        int b = bb - q;
-        if (b < 1) break;
-        if (b <= stop_at) {
-          float4 pt = ptv[q];
-          S0 = pt.y + pt.x * S0; S1 = pt.z + pt.x * S1; S2 = pt.w + pt.x * S2;
-        }
-        cpp[(int64_t)(b - 1) * TILE_PIX] = make_float4(__uint_as_float(tv[q]), S0, S1, S2);
-      }
-    }
+    if (done)
+      for (int b = nch - 1; b >= m; --b) cpp[(int64_t)(b - 1) * TILE_PIX] = make_float4(T, bg0, bg1, bg2);
+    close_checkpoints(cpp, clp, 1, done ? m - 1 : nch - 1, S0, S1, S2);
     im[pix] = c0 + T * bg0;
     im[plane + pix] = c1 + T * bg1;
     im[2 * plane + pix] = c2 + T * bg2;
@@ -730,55 +914,47 @@ __device__ __forceinline__ void combine_pixel(const PixelOf<BW>& P, int o, int n
   }
 }
 
+// Combine pass: one warp per queued block; the entry of its first queued chunk
+// (chunk M) stands for it.  The first block also zeroes the stop pass's ticket.
 template <int BW>
-__global__ void __launch_bounds__(32) k_render_fwd_combine(const uint2* __restrict__ ranges,
-                                                                 const uint32_t* __restrict__ order,
-                                                                 const uint32_t* __restrict__ job_base, int K,
-                                                                 float4* __restrict__ ckpt,
-                                                                 uint32_t* __restrict__ chunk_last, int W, int H,
-                                                                 int TX, int n_tiles, float bg0, float bg1, float bg2,
-                                                                 float* __restrict__ img, float* __restrict__ final_T,
-                                                                 uint32_t* __restrict__ n_contrib,
-                                                                 uint32_t* __restrict__ queue, uint32_t qcap) {
-  int o = (int)(blockIdx.x >> 3), w = (int)(blockIdx.x & 7u);
-  int nch = (int)(job_base[o + 1] - job_base[o]);
-  if (nch == 1) return;
-  PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
-  int64_t plane = (int64_t)W * H;
-  int64_t pix = (int64_t)P.py * W + P.px;
-  float* im = img + (int64_t)P.u * 3 * plane;
-  float* fT = final_T + (int64_t)P.u * plane;
-  uint32_t* nc = n_contrib + (int64_t)P.u * plane;
-  if (nch == 0) {  // the whole warp returns here
-    if (P.inside) {
-      im[pix] = bg0; im[plane + pix] = bg1; im[2 * plane + pix] = bg2;
-      fT[pix] = 1.f;
-      nc[pix] = 0u;
-    }
-    return;
-  }
-  int cstar = -1;
-  if (P.inside) combine_pixel(P, o, nch, plane, pix, im, fT, nc, ckpt, chunk_last, job_base, bg0, bg1, bg2, cstar);
-  // queue the units pass 3 walks: one (stop chunk, pixel block) per distinct stop chunk of the warp's pixels
-  int key = cstar >= 1 ? cstar : -1;
-  unsigned peers = __match_any_sync(0xffffffffu, key);
-  if (key >= 1 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) {
-    uint32_t slot = atomicAdd(queue + qcap, 1u);
-    queue[slot] = ((job_base[o] + (uint32_t)key) << 3) | (uint32_t)w;
+__global__ void __launch_bounds__(32) k_render_fwd_combine(const uint32_t* __restrict__ order,
+                                                           const uint32_t* __restrict__ job_base,
+                                                           const uint32_t* __restrict__ jobs, int M,
+                                                           float4* __restrict__ ckpt,
+                                                           uint32_t* __restrict__ chunk_last, int W, int H, int TX,
+                                                           int n_tiles, float bg0, float bg1, float bg2,
+                                                           float* __restrict__ img, float* __restrict__ final_T,
+                                                           uint32_t* __restrict__ n_contrib,
+                                                           uint32_t* __restrict__ queue, uint32_t qcap,
+                                                           uint32_t* __restrict__ ticket) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0u;
+  const uint32_t total = queue[qcap];
+  for (uint32_t e = blockIdx.x; e < total; e += gridDim.x) {
+    const uint32_t jid = (queue[e] & ~MARK_BIT) >> 3;  // (a mark is set on later entries of a block only by its warp)
+    if ((int)jobs[2 * (int64_t)jid + 1] != M) continue;
+    const int w = (int)(queue[e] & 7u), o = (int)jobs[2 * (int64_t)jid];
+    const uint32_t jb = job_base[o];
+    const int nch = (int)(job_base[o + 1] - jb);
+    PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
+    const int64_t plane = (int64_t)W * H, pix = (int64_t)P.py * W + P.px, cp0 = (int64_t)jb - o;
+    int cstar = -1;
+    if (P.inside)
+      combine_pixel(M, nch, plane, pix, img + (int64_t)P.u * 3 * plane, final_T + (int64_t)P.u * plane,
+                    n_contrib + (int64_t)P.u * plane, ckpt + cp0 * TILE_PIX + P.pix_local,
+                    chunk_last + cp0 * TILE_PIX + P.pix_local, bg0, bg1, bg2, cstar);
+    // mark the block's queue entries the stop pass walks: one per distinct stop chunk of its pixels
+    const unsigned peers = __match_any_sync(0xffffffffu, cstar);
+    if (cstar >= 1 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) queue[e + (uint32_t)(cstar - M)] |= MARK_BIT;
+    __syncwarp();
   }
 }
 
-// Pass 3: the units pass 2 queued, (list o, chunk c, block w) with some pixel
-// of block w stopping in chunk c: walks chunk c again for those pixels from
-// the state pass 2 left, and writes their final image, final_T, n_contrib and
-// the checkpoints after c (final state).  A resident grid takes the queued
-// units from a ticket counter (zeroed before the launch), so no block is
-// launched for a chunk in which nothing stops.  Bounded to 64 registers (32
-// resident warps per SM, the one-warp block limit): the body needs ~114 and
-// spills ~200 bytes of its checkpoint loops, which costs less than the
-// occupancy it gains (forward 1.69 -> 1.63 ms at 10M/1080p).
+// Stop pass: the marked queue entries, (list o, chunk c, block w) with some
+// pixel of block w stopping in chunk c: walks chunk c again for those pixels
+// from the state the combine left, and writes their final image, final_T,
+// n_contrib and the checkpoints after c (final state).
 template <int BW>
-__global__ void __launch_bounds__(32, 32) k_render_fwd_stop(const uint2* __restrict__ ranges,
+__global__ void __launch_bounds__(32) k_render_fwd_stop(const uint2* __restrict__ ranges,
                                                               const uint32_t* __restrict__ order,
                                                               const uint32_t* __restrict__ job_base,
                                                               const uint32_t* __restrict__ jobs, int K,
@@ -794,7 +970,7 @@ __global__ void __launch_bounds__(32, 32) k_render_fwd_stop(const uint2* __restr
                                                               uint32_t* __restrict__ n_contrib,
                                                               const uint32_t* __restrict__ queue, uint32_t qcap,
                                                               uint32_t* __restrict__ ticket) {
-  __shared__ Rec s_rec[32];
+  __shared__ FwdScratch s_walk;
   const uint32_t total = queue[qcap];
   auto job = [&](uint32_t ent) {
   uint32_t jid = ent >> 3;
@@ -818,7 +994,7 @@ __global__ void __launch_bounds__(32, 32) k_render_fwd_stop(const uint2* __restr
     uint32_t lw = nc[pix];
     mine = (lw & REWALK_BIT) != 0u && (int)(lw & ~REWALK_BIT) == ch;
     if (mine) {
-      last = (int)chunk_last[(cp0 + ch - 1) * TILE_PIX + P.pix_local];  // left there by pass 2
+      last = (int)chunk_last[(cp0 + ch - 1) * TILE_PIX + P.pix_local];  // left there by the combine
       c0 = im[pix]; c1 = im[plane + pix]; c2 = im[2 * plane + pix];
       T = fT[pix];
     }
@@ -833,16 +1009,9 @@ __global__ void __launch_bounds__(32, 32) k_render_fwd_stop(const uint2* __restr
   // walked chunk's partial and the T in front of it; chunks behind the stop get the identity partial
   int c = ch;
   for (; c < nch; ++c) {
-    LocalAcc la = {1.f, 0.f, 0.f, 0.f};
-    float Tin = T;
-    walk_fwd<true>(vals, masks, xy, conic_op, rgb, rg.x, c * K, min(c * K + K, L), wbits, (float)(P.tx * TILE),
-                   (float)(P.ty * TILE), (float)(P.px - P.tx * TILE), (float)(P.py - P.ty * TILE), s_rec, T, c0, c1,
-                   c2, last, done, &la);
-    if (mine) {
-      int64_t slot = (cp0 + c - 1) * TILE_PIX + P.pix_local;
-      ckpt[slot] = make_float4(la.t, la.c0, la.c1, la.c2);
-      chunk_last[slot] = __float_as_uint(Tin);
-    }
+    walk_chunk<BW>(vals, masks, xy, conic_op, rgb, rg.x, c * K, min(c * K + K, L), wbits, (float)(P.tx * TILE),
+                   (float)(P.ty * TILE), (float)P.ox, (float)P.oy, s_walk, T, c0, c1, c2, last, done, mine,
+                   ckpt + (cp0 + c - 1) * TILE_PIX + P.pix_local, chunk_last + (cp0 + c - 1) * TILE_PIX + P.pix_local);
     if (__all_sync(0xffffffffu, done)) break;
   }
   if (!mine) return;
@@ -852,21 +1021,8 @@ __global__ void __launch_bounds__(32, 32) k_render_fwd_stop(const uint2* __restr
   for (int b = nch - 1; b > c; --b)
     cpp[(int64_t)(b - 1) * TILE_PIX] = make_float4(T, bg0, bg1, bg2);  // behind the stop: final state
   float S0 = bg0, S1 = bg1, S2 = bg2;
-  for (int bb = min(c, nch - 1); bb >= ch; bb -= CB) {  // walked chunks, back to front
-    float4 ptv[CB];
-    uint32_t tv[CB];
-    #pragma unroll
-    for (int q = 0; q < CB; ++q)
-      if (bb - q >= ch) { ptv[q] = cpp[(int64_t)(bb - q - 1) * TILE_PIX]; tv[q] = clp[(int64_t)(bb - q - 1) * TILE_PIX]; }
-    #pragma unroll
-    for (int q = 0; q < CB; ++q) {
-      if (bb - q < ch) break;
-      float4 pt = ptv[q];
-      S0 = pt.y + pt.x * S0; S1 = pt.z + pt.x * S1; S2 = pt.w + pt.x * S2;
-      cpp[(int64_t)(bb - q - 1) * TILE_PIX] = make_float4(__uint_as_float(tv[q]), S0, S1, S2);
-    }
-  }
-  for (int bb = 1; bb < ch; bb += CB) {  // in front of c*: S_b = A_b + B_b S_c* as left by pass 2
+  close_checkpoints(cpp, clp, ch, min(c, nch - 1), S0, S1, S2);  // walked chunks
+  for (int bb = 1; bb < ch; bb += CB) {  // in front of c*: S_b = A_b + B_b S_c* as left by the combine
     float4 abv[CB];
     uint32_t tv[CB];
     #pragma unroll
@@ -890,82 +1046,31 @@ __global__ void __launch_bounds__(32, 32) k_render_fwd_stop(const uint2* __restr
   uint32_t e = __shfl_sync(0xffffffffu, lead ? atomicAdd(ticket, 1u) : 0u, 0);
   while (e < total) {
     uint32_t nxt = lead ? atomicAdd(ticket, 1u) : 0u;
-    job(queue[e]);
+    const uint32_t ent = queue[e];
+    if (ent & MARK_BIT) job(ent & ~MARK_BIT);
     e = __shfl_sync(0xffffffffu, nxt, 0);
   }
 }
 
 
-// Forward walking whole lists: one warp per (list, pixel block) in tile order
-// composites its list chunk after chunk and stores (T, C) of each pixel in
-// front of every interior chunk boundary (the backward's checkpoints); after
-// an early exit the remaining checkpoints hold the final state.  No work
-// follows a block's last stop, which suits renders whose pixels mostly stop
-// near the front of their lists (opaque, trained scenes).
-template <int BW>
-__global__ void __launch_bounds__(32) k_render_fwd_seq(const uint2* __restrict__ ranges,
-                                                             const uint32_t* __restrict__ order,
-                                                             const uint32_t* __restrict__ job_base, int K,
-                                                             float4* __restrict__ ckpt,
-                                                             uint32_t* __restrict__ chunk_last,
-                                                             const uint32_t* __restrict__ vals,
-                                                             const uint16_t* __restrict__ masks,
-                                                             const float4* __restrict__ xy,
-                                                             const float4* __restrict__ conic_op,
-                                                             const float4* __restrict__ rgb, int W, int H, int TX,
-                                                             int n_tiles, float bg0, float bg1, float bg2,
-                                                             float* __restrict__ img, float* __restrict__ final_T,
-                                                             uint32_t* __restrict__ n_contrib) {
-  __shared__ Rec s_rec[32];
-  int o = (int)(blockIdx.x >> 3), w = (int)(blockIdx.x & 7u);
-  PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
-  uint2 rg = ranges[(int64_t)P.u * n_tiles + P.tile];
-  int L = (int)(rg.y - rg.x);
-  int nch = (int)(job_base[o + 1] - job_base[o]);
-  int64_t cp0 = (int64_t)job_base[o] - o;
-  float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-  int last = 0;
-  bool done = !P.inside;
-  for (int c = 0; c < max(nch, 1); ++c) {
-    LocalAcc la = {1.f, 0.f, 0.f, 0.f};
-    float Tin = T;
-    walk_fwd<true>(vals, masks, xy, conic_op, rgb, rg.x, c * K, min(c * K + K, L), P.wbits, (float)(P.tx * TILE),
-                   (float)(P.ty * TILE), (float)(P.px - P.tx * TILE), (float)(P.py - P.ty * TILE), s_rec, T, c0, c1,
-                   c2, last, done, &la);
-    if (c > 0 && P.inside) {  // the chunk's partial and the T in front of it
-      int64_t slot = (cp0 + c - 1) * TILE_PIX + P.pix_local;
-      ckpt[slot] = make_float4(la.t, la.c0, la.c1, la.c2);
-      chunk_last[slot] = __float_as_uint(Tin);
-    }
-  }
-  if (P.inside) {
-    // checkpoints: (T in front of boundary b, colour behind it per unit T), composited back to front
-    float4* cpp = ckpt + cp0 * TILE_PIX + P.pix_local;  // slot of boundary b: cpp[(b - 1) * TILE_PIX]
-    const uint32_t* clp = chunk_last + cp0 * TILE_PIX + P.pix_local;
-    float S0 = bg0, S1 = bg1, S2 = bg2;
-    for (int bb = nch - 1; bb >= 1; bb -= CB) {
-      float4 ptv[CB];
-      uint32_t tv[CB];
-      #pragma unroll
-      for (int q = 0; q < CB; ++q)
-        if (bb - q >= 1) { ptv[q] = cpp[(int64_t)(bb - q - 1) * TILE_PIX]; tv[q] = clp[(int64_t)(bb - q - 1) * TILE_PIX]; }
-      #pragma unroll
-      for (int q = 0; q < CB; ++q) {
-        if (bb - q < 1) break;
-        float4 pt = ptv[q];
-        S0 = pt.y + pt.x * S0; S1 = pt.z + pt.x * S1; S2 = pt.w + pt.x * S2;
-        cpp[(int64_t)(bb - q - 1) * TILE_PIX] = make_float4(__uint_as_float(tv[q]), S0, S1, S2);
-      }
-    }
-    int64_t plane = (int64_t)W * H;
-    int64_t pix = (int64_t)P.py * W + P.px;
-    float* im = img + (int64_t)P.u * 3 * plane;
-    im[pix] = c0 + T * bg0;
-    im[plane + pix] = c1 + T * bg1;
-    im[2 * plane + pix] = c2 + T * bg2;
-    final_T[(int64_t)P.u * plane + pix] = T;
-    n_contrib[(int64_t)P.u * plane + pix] = (uint32_t)last;
-  }
+// Lanes of a warp's pixel block (bw x 32 / bw pixels from tile-local origin
+// (ox, oy), lane = row bw + column) whose pixel centre lies in a record's
+// alpha >= 1/255 box (alpha_box: conservative, so every pixel outside it has
+// alpha < 1/255 and would be skipped by the blend).  (rx, ry): the record's
+// tile-local position; co: conic and opacity.
+__device__ __forceinline__ uint32_t hit_lanes(float rx, float ry, float4 co, float ox, float oy, int bw) {
+  float pm;
+  const float4 b = alpha_box(make_float2(rx, ry), co, pm);
+  if (!(b.x <= b.y)) return 0u;
+  const int bh = 32 / bw;
+  const float c0 = fmaxf(ceilf(b.x - ox), 0.f), c1 = fminf(floorf(b.y - ox), (float)(bw - 1));
+  const float r0 = fmaxf(ceilf(b.z - oy), 0.f), r1 = fminf(floorf(b.w - oy), (float)(bh - 1));
+  if (!(c0 <= c1) || !(r0 <= r1)) return 0u;
+  const int lo = (int)c0, rl = (int)r0, rh = (int)r1;
+  const uint32_t cm = ((2u << ((int)c1 - lo)) - 1u) << lo;
+  uint32_t m = 0u;
+  for (int r = rl; r <= rh; ++r) m |= cm << (r * bw);
+  return m;
 }
 
 // Contributing lanes up to which the scheduled backward skips the warp
@@ -985,6 +1090,12 @@ __device__ __forceinline__ void pos_conic_terms(float dx, float dy, float dp, fl
   v[0] = -(A * dx + B * dy) * dp;
   v[1] = -(Cc * dy + B * dx) * dp;
 }
+
+// Rounds with at least this many hits walk per-lane hit lists: each lane takes
+// only the hits whose alpha box reaches its pixel.  Below it the box and the
+// transpose cost more than the hits they spare (10M Gaussians at 1080p,
+// thresholds swept over 1-24).
+constexpr int HIT_LISTS_BWD = 8;
 
 // Ring of deferred (pixel, record) pairs of the scheduled backward, per warp.
 constexpr int QCAP = 64;
@@ -1010,10 +1121,9 @@ __device__ __forceinline__ void bwd_queue_flush(const float4* s_q, int head, int
 // forward's checkpoint at the chunk's end (T in front of it and the colour
 // behind it per unit T), or from final_T and the background for the last
 // chunk.  Headers two rounds ahead, hit records one round ahead, as in the
-// forward.  QUEUE (float accumulation) defers the gradient terms of sparse
-// hits to a per-warp ring; the deterministic mode (fixed != NULL) runs
-// without it.
-template <int BW, bool QUEUE>
+// forward.  The gradient terms of sparse hits go through a per-warp ring (float
+// accumulation; k_render_bwd_det has the deterministic one).
+template <int BW>
 __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict__ ranges,
                                                            const uint32_t* __restrict__ order,
                                                            const uint32_t* __restrict__ job_base,
@@ -1031,8 +1141,7 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
                                                            const float* __restrict__ dimg,
                                                            const float* __restrict__ dLdT, float* __restrict__ dxy,
                                                            float* __restrict__ dco, float* __restrict__ drgb,
-                                                           unsigned long long* __restrict__ fixed,
-    uint32_t* __restrict__ ticket) {
+                                                           uint32_t* __restrict__ ticket) {
   const unsigned FULL = 0xffffffffu;
   __shared__ Rec s_rec[32];
   // the resident warps take the (chunk job, pixel block) units from a ticket counter (zeroed before
@@ -1062,8 +1171,11 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
     float T = 1.f, g0 = 0.f, g1 = 0.f, g2 = 0.f, S0 = bg0, S1 = bg1, S2 = bg2;
     float qT = 0.f;  // dL/dT_final x T_final: a blended entry adds -qT / (1 - alpha) to dL/dalpha
     int last = 0;
+    if (inside) last = (int)n_contrib[(int64_t)u * plane + pix];
+    // entries this warp replays: [cbeg, min(cend, max over its pixels of last)); a chunk behind the last stop has none
+    const int n = min(__reduce_max_sync(FULL, last), cend);
+    if (n <= cbeg) return;
     if (inside) {
-      last = (int)n_contrib[(int64_t)u * plane + pix];
       const float* d = dimg + (int64_t)u * 3 * plane;
       g0 = d[pix]; g1 = d[plane + pix]; g2 = d[2 * plane + pix];
       if (dLdT) qT = dLdT[(int64_t)u * plane + pix] * final_T[(int64_t)u * plane + pix];
@@ -1077,8 +1189,6 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
         T = final_T[(int64_t)u * plane + pix];
       }
     }
-    // entries this warp replays: [cbeg, min(cend, max over its pixels of last))
-    int n = min(__reduce_max_sync(FULL, last), cend);
     Rec* my = &s_rec[0];
     int q = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
     bool h1 = false;
@@ -1098,11 +1208,11 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
       int k2 = n - 64 + lane;
       if (n - 32 > cbeg && k2 >= cbeg) { mk2 = masks[rg.x + k2]; pk2 = vals[rg.x + k2]; }
     }
-    // QUEUE: pairs of hits with at most DIRECT_LANES contributing lanes go to a ring of
+    // pairs of hits with at most DIRECT_LANES contributing lanes go to a ring of
     // (dx, dy, dp, dopacity | A, B, C, id | dr, dg, db) entries; every 32 entries all
     // lanes finish one pair each (conic and position terms, vector atomics).  The
     // per-pixel state (T, colour behind) is still updated at the hit in list order.
-    __shared__ float4 s_q[QUEUE ? 3 * QCAP : 1];
+    __shared__ float4 s_q[3 * QCAP];
     int qh = 0, qt = 0;  // ring head and tail (warp-uniform)
     for (int top = n; top > cbeg; top -= 32) {
       int base = top - 32;
@@ -1123,7 +1233,7 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
         my[lane].c = c;
       }
       __syncwarp();
-      if (QUEUE && __popc(mask) >= HIT_LISTS_BWD) {
+      if (__popc(mask) >= HIT_LISTS_BWD) {
         // per-lane hit lists, back to front: bit j of `mine` = hit j's alpha box reaches this lane's
         // pixel and the entry lies in front of the pixel's last contribution; every pair goes to the ring
         uint32_t mine = transpose32(hit ? hit_lanes(rx, ry, co, (float)((w % NWX) * BW), (float)((w / NWX) * BH), BW)
@@ -1217,7 +1327,7 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
         unsigned cm = __ballot_sync(FULL, contrib);
         if (!cm) continue;
         int nc = __popc(cm);
-        if (QUEUE && nc <= DIRECT_LANES) {
+        if (nc <= DIRECT_LANES) {
           if (contrib) {
             int e = (qt + __popc(cm & ((1u << lane) - 1u))) & (QCAP - 1);
             s_q[e] = make_float4(dx, dy, dp, v5);
@@ -1237,26 +1347,193 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
         float v[9];
         pos_conic_terms(dx, dy, dp, ra.z, ra.w, rb.x, v);
         v[5] = v5; v[6] = v6; v[7] = v7; v[8] = v8;
-        // fixed point: nine scalar int64 atomics per lane, so reduce unless one lane contributes
-        if (nc <= (fixed ? 1 : DIRECT_LANES)) {
-          // few contributing lanes (small splats): each issues its own three vector
-          // atomics, which costs fewer instructions and atomic operations than a reduction
-          if (contrib) add_lane(dxy, dco, drgb, fixed, pr, v);
-        } else {
+        {
           float tot = reduce8(v, lane);
           float e8 = v[8];
           #pragma unroll
           for (int oo = 16; oo > 0; oo >>= 1) e8 += __shfl_xor_sync(FULL, e8, oo);
           if ((lane & 3) == 0) {
-            add_one(dxy, dco, drgb, fixed, pr, q, tot);
+            add_one(dxy, dco, drgb, nullptr, pr, q, tot);
           } else if (lane == 1) {
-            add_one(dxy, dco, drgb, fixed, pr, 8, e8);
+            add_one(dxy, dco, drgb, nullptr, pr, 8, e8);
           }
         }
       }
       __syncwarp();
     }
-    if (QUEUE && qt > qh) bwd_queue_flush(s_q, qh, qt - qh, lane, dxy, dco, drgb);
+    if (qt > qh) bwd_queue_flush(s_q, qh, qt - qh, lane, dxy, dco, drgb);
+  };
+  const bool lead = (threadIdx.x & 31) == 0;
+  uint32_t vb = __shfl_sync(0xffffffffu, lead ? atomicAdd(ticket, 1u) : 0u, 0);
+  while (vb < total) {
+    uint32_t nxt = lead ? atomicAdd(ticket, 1u) : 0u;
+    job(vb);
+    vb = __shfl_sync(0xffffffffu, nxt, 0);
+  }
+}
+
+struct BwdScratch {
+  float w[32 * MROW];   // o G of an accepted (hit, pixel) pair, then its colour weight alpha T
+  float dp[32 * MROW];  // dL/dpower of the pair (0 when alpha was clamped)
+  float r[32], g[32], b[32];     // the batch's colours
+  float g0[32], g1[32], g2[32];  // dL/dimg of the block's pixels
+  uint32_t q[QUEUE_CAP];
+};
+
+// The deterministic backward over the same chunk jobs.  Its cost is the int64
+// atomics, nine per record and addition, so it sums each hit over the block's
+// pixels first: hits are gathered back to front into batches of 32 and
+// evaluated record-major, then replayed pixel-major, as in the forward walk;
+// the replay leaves each pair's colour weight alpha T and dL/dpower in shared
+// memory, and a third, record-major phase forms the pairs' gradients and sums
+// them in its lane's registers, in pixel order, so that nothing depends on
+// scheduling.  700k at 1011x757: 578 us with a warp reduction per hit, 240 us.
+template <int BW>
+__global__ void __launch_bounds__(32, 20) k_render_bwd_det(const uint2* __restrict__ ranges,
+                                                           const uint32_t* __restrict__ order,
+                                                           const uint32_t* __restrict__ job_base,
+                                                           const uint32_t* __restrict__ jobs, int K,
+                                                           const float4* __restrict__ ckpt,
+                                                           const uint32_t* __restrict__ vals,
+                                                           const uint16_t* __restrict__ masks,
+                                                           const float4* __restrict__ xy,
+                                                           const float4* __restrict__ conic_op,
+                                                           const float4* __restrict__ rgb, int W, int H, int TX,
+                                                           int n_tiles, int NT, float bg0, float bg1, float bg2,
+                                                           const float* __restrict__ img,
+                                                           const float* __restrict__ final_T,
+                                                           const uint32_t* __restrict__ n_contrib,
+                                                           const float* __restrict__ dimg,
+                                                           const float* __restrict__ dLdT,
+                                                           unsigned long long* __restrict__ fixed,
+                                                           uint32_t* __restrict__ ticket) {
+  const unsigned FULL = 0xffffffffu;
+  __shared__ BwdScratch sc;
+  // the resident warps take the (chunk job, pixel block) units from a ticket counter (zeroed before
+  // the launch), the next ticket fetched while a unit runs: no block of a grid sized for the capacity
+  // sits idle, and units of very different cost still spread as they finish
+  const uint32_t total = job_base[NT] * 8u;
+  auto job = [&](uint32_t vb) {
+    uint32_t jid = vb >> 3;
+    int w = (int)(vb & 7u);
+    int o = (int)jobs[2 * (int64_t)jid], ch = (int)jobs[2 * (int64_t)jid + 1];
+    PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
+    int nch = (int)(job_base[o + 1] - job_base[o]);
+    const int lane = threadIdx.x & 31;
+    const float tox = (float)(P.tx * TILE), toy = (float)(P.ty * TILE);  // origin of the record positions
+    const float ox = (float)P.ox, oy = (float)P.oy, bx = 8388608.f - ox, by = 8388608.f - oy;
+    uint2 rg = ranges[(int64_t)P.u * n_tiles + P.tile];
+    int L = (int)(rg.y - rg.x);
+    int cbeg = ch * K, cend = min(cbeg + K, L);
+    int64_t plane = (int64_t)W * H;
+    int64_t pix = (int64_t)P.py * W + P.px;
+    float T = 1.f, g0 = 0.f, g1 = 0.f, g2 = 0.f, S0 = bg0, S1 = bg1, S2 = bg2;
+    float qT = 0.f;  // dL/dT_final x T_final: a blended entry adds -qT / (1 - alpha) to dL/dalpha
+    // entries this warp replays: [cbeg, min(cend, max over its pixels of last))
+    const int last = P.inside ? (int)n_contrib[(int64_t)P.u * plane + pix] : 0;
+    const int n = min(__reduce_max_sync(FULL, last), cend);
+    if (n <= cbeg) return;
+    if (P.inside) {
+      const float* d = dimg + (int64_t)P.u * 3 * plane;
+      g0 = d[pix]; g1 = d[plane + pix]; g2 = d[2 * plane + pix];
+      if (dLdT) qT = dLdT[(int64_t)P.u * plane + pix] * final_T[(int64_t)P.u * plane + pix];
+      if (ch + 1 < nch && last > cbeg) {
+        // the forward's checkpoint at the chunk's end: T there and the colour behind it per unit T
+        float4 cp = ckpt[((int64_t)job_base[o] - o + ch) * TILE_PIX + P.pix_local];
+        T = cp.x;
+        S0 = cp.y; S1 = cp.z; S2 = cp.w;
+      } else {
+        T = final_T[(int64_t)P.u * plane + pix];
+      }
+    }
+    sc.g0[lane] = g0; sc.g1[lane] = g1; sc.g2[lane] = g2;
+    const uint32_t act = __ballot_sync(FULL, last > cbeg);  // pixels with an entry to replay
+    const uint32_t* lv = vals + rg.x;
+    const uint16_t* lm = masks + rg.x;
+    int scan = n - 1, qn = 0, qh = 0;  // next entry to scan (downwards); queued entries are q[qh .. qn)
+    for (;;) {
+      if (qn - qh < 32 && scan >= cbeg) {
+        const uint32_t keep = qh + lane < qn ? sc.q[qh + lane] : 0u;
+        __syncwarp();
+        qn -= qh;
+        qh = 0;
+        if (lane < qn) sc.q[lane] = keep;
+        do {
+          qn = scan_hits<true>(lm, scan, cbeg, P.wbits, sc.q, qn);
+          scan -= SCAN;
+        } while (qn < 32 && scan >= cbeg);
+        __syncwarp();
+      }
+      const int nb = min(32, qn - qh);
+      if (nb == 0) break;
+      // record-major: o G of hit `lane` at the pixels its box reaches
+      uint32_t pr = 0u, valid = 0u;
+      float rx = 0.f, ry = 0.f;
+      float4 co = make_float4(0.f, 0.f, 0.f, 1.f);
+      if (lane < nb) {
+        pr = lv[sc.q[qh + lane]];
+        const float4 m = xy[pr], c = rgb[pr];
+        co = conic_op[pr];
+        rx = rel_pos(m.x, m.z, tox); ry = rel_pos(m.y, m.w, toy);
+        sc.r[lane] = c.x; sc.g[lane] = c.y; sc.b[lane] = c.z;
+        valid = eval_hit<BW, false>(rx, ry, co, c.w, ox, oy, act, sc.w + lane * MROW);
+      }
+      __syncwarp();
+      // pixel-major: this pixel's pairs back to front, those in front of its last contribution
+      uint32_t mine = transpose32(valid);
+      if (mine && (int)sc.q[qh] >= last) {
+        int a = 0, b = nb;  // first hit with an entry below `last` (entries fall with j)
+        while (a < b) {
+          const int mid = (a + b) >> 1;
+          if ((int)sc.q[qh + mid] >= last) a = mid + 1; else b = mid;
+        }
+        mine &= a < 32 ? 0xffffffffu << a : 0u;
+      }
+      const uint32_t con = mine;
+      while (mine) {
+        const int j = __ffs(mine) - 1;
+        mine &= mine - 1;
+        const float araw = sc.w[j * MROW + lane];
+        const bool clamped = araw > ALPHA_MAX;  // a clamped alpha passes no gradient to opacity, conic or position
+        const float alpha = clamped ? ALPHA_MAX : araw;
+        const float om = 1.f - alpha;
+        T = __fdividef(T, om);  // transmittance in front of this entry
+        const float cr = sc.r[j], cg = sc.g[j], cb = sc.b[j];
+        float dalpha = T * ((cr - S0) * g0 + (cg - S1) * g1 + (cb - S2) * g2);
+        if (qT != 0.f) dalpha -= __fdividef(qT, om);
+        S0 = alpha * cr + om * S0; S1 = alpha * cg + om * S1; S2 = alpha * cb + om * S2;
+        sc.w[j * MROW + lane] = alpha * T;
+        sc.dp[j * MROW + lane] = clamped ? 0.f : araw * dalpha;
+      }
+      __syncwarp();
+      // record-major: the sums over hit `lane`'s pixels, then its atomics
+      uint32_t pm = transpose32(con);
+      if (pm) {
+        float v[9];
+        #pragma unroll
+        for (int q = 0; q < 9; ++q) v[q] = 0.f;
+        while (pm) {
+          const int px = __ffs(pm) - 1;
+          pm &= pm - 1;
+          const float wgt = sc.w[lane * MROW + px], dp = sc.dp[lane * MROW + px];
+          // 2^23 + integer, minus the origin's offset: the pixel's coordinates without an integer conversion
+          const float dx = rx - (__int_as_float(0x4b000000 | (px & (BW - 1))) - bx);
+          const float dy = ry - (__int_as_float(0x4b000000 | (px / BW)) - by);
+          v[0] += (co.x * dx + co.y * dy) * dp;
+          v[1] += (co.z * dy + co.y * dx) * dp;
+          v[2] += dx * dx * dp; v[3] += dx * dy * dp; v[4] += dy * dy * dp;
+          v[5] += dp;
+          v[6] += wgt * sc.g0[px]; v[7] += wgt * sc.g1[px]; v[8] += wgt * sc.g2[px];
+        }
+        v[0] = -v[0]; v[1] = -v[1];
+        v[2] *= -0.5f; v[3] = -v[3]; v[4] *= -0.5f;
+        v[5] /= co.w;
+        add_lane(nullptr, nullptr, nullptr, fixed, (int64_t)pr, v);
+      }
+      qh += nb;
+      __syncwarp();
+    }
+    __syncwarp();
   };
   const bool lead = (threadIdx.x & 31) == 0;
   uint32_t vb = __shfl_sync(0xffffffffu, lead ? atomicAdd(ticket, 1u) : 0u, 0);
@@ -1391,7 +1668,7 @@ unsigned resident_grid(K kernel, int64_t units) {
   return (unsigned)(g < units ? g : units);
 }
 
-// The ticket word of the scheduled blend kernels: the jobs array's last entry, which no job uses
+// The two ticket words of the scheduled blend kernels: the jobs array's last entry, which no job uses
 // (a list of L entries has ceil(L / K) < L / K + 1 jobs, so there are fewer than max_jobs - 1).
 inline uint32_t* sched_ticket(const gs_schedule* sched) {
   return sched->jobs + 2 * (sched->max_jobs - 1);
@@ -1408,32 +1685,34 @@ int gs_render_fwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const u
     return GS_ERR_INVALID;
   int TX = (width + TILE - 1) / TILE, TY = (height + TILE - 1) / TILE;
   dim3 grid(TX * TY * n_units);
-  // the re-walk queue holds at most one entry per (chunk job, pixel block); its count follows it
+  // the queue of the forward's later passes holds at most one entry per (chunk job, pixel block); its count follows it
   const uint32_t qcap = sched ? (uint32_t)(8 * sched->max_jobs) : 0u;
 #define GS_FWD(BW)                                                                                                  \
-  if (sched && sched->walk_whole_lists) {                                                                          \
-    k_render_fwd_seq<BW><<<dim3(grid.x * 8), 32, 0, s>>>(                                                           \
-        (const uint2*)ranges, sched->tile_order, sched->job_base, sched->chunk, (float4*)sched->checkpoints,        \
-        sched->chunk_last, sorted_vals, sched->block_masks, (const float4*)proj->xy, (const float4*)proj->conic_op,                    \
-        (const float4*)proj->rgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib);        \
-  } else if (sched) {                                                                                               \
-    if (cudaMemsetAsync(sched_ticket(sched), 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;          \
-    k_render_fwd_m<BW><<<dim3(resident_grid(k_render_fwd_m<BW>, sched->max_jobs * 8)), 32, 0, s>>>(                 \
-        (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, (int)grid.x,            \
-        (float4*)sched->checkpoints, sched->chunk_last, sorted_vals, sched->block_masks, (const float4*)proj->xy,   \
-        (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2],  \
-        img, final_T, n_contrib, sched_ticket(sched));                                                              \
-    if (cudaMemsetAsync(sched->stop_queue + qcap, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;     \
-    k_render_fwd_combine<BW><<<dim3(grid.x * 8), 32, 0, s>>>(                                                       \
-        (const uint2*)ranges, sched->tile_order, sched->job_base, sched->chunk, (float4*)sched->checkpoints,        \
-        sched->chunk_last, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib,               \
-        sched->stop_queue, qcap);                                                                                   \
-    if (cudaMemsetAsync(sched_ticket(sched), 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;          \
-    k_render_fwd_stop<BW><<<dim3(resident_grid(k_render_fwd_stop<BW>, (int64_t)qcap)), 32, 0, s>>>(                 \
-        (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                        \
-        (float4*)sched->checkpoints, sched->chunk_last, sorted_vals, sched->block_masks, (const float4*)proj->xy,    \
-        (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2],  \
-        img, final_T, n_contrib, sched->stop_queue, qcap, sched_ticket(sched));                                     \
+  if (sched) {                                                                                                        \
+    const int M = sched->walk_whole_lists ? INT_MAX : FRONT_CHUNKS;                                                   \
+    uint32_t* tk = sched_ticket(sched);                                                                               \
+    uint32_t* q = sched->stop_queue;                                                                                  \
+    float4* ck = (float4*)sched->checkpoints;                                                                         \
+    const float4 *pxy = (const float4*)proj->xy, *pco = (const float4*)proj->conic_op, *prgb = (const float4*)proj->rgb;\
+    const uint2* rg = (const uint2*)ranges;                                                                           \
+    k_render_fwd_empty<<<grid, TILE_PIX, 0, s>>>(rg, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T,   \
+                                                 n_contrib, tk, q + qcap);                                            \
+    k_render_fwd_front<BW><<<resident_grid(k_render_fwd_front<BW>, (int64_t)grid.x * 8), 32, 0, s>>>(                 \
+        rg, sched->tile_order, sched->job_base, sched->chunk, M, sched->walk_whole_lists != 0, (int)grid.x, ck, sched->chunk_last, sorted_vals,     \
+        sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib, \
+        q, qcap, tk);                                                                                                 \
+    if (!sched->walk_whole_lists) {                                                                                   \
+      k_render_fwd_chunk<BW><<<resident_grid(k_render_fwd_chunk<BW>, (int64_t)qcap), 32, 0, s>>>(                     \
+          rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last, sorted_vals,      \
+          sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, n_contrib, q, qcap, tk + 1);                \
+      k_render_fwd_combine<BW><<<resident_grid(k_render_fwd_combine<BW>, (int64_t)qcap), 32, 0, s>>>(                 \
+          sched->tile_order, sched->job_base, sched->jobs, M, ck, sched->chunk_last, width, height, TX, TX * TY, bg[0],\
+          bg[1], bg[2], img, final_T, n_contrib, q, qcap, tk);                                                        \
+      k_render_fwd_stop<BW><<<resident_grid(k_render_fwd_stop<BW>, (int64_t)qcap), 32, 0, s>>>(                       \
+          rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last, sorted_vals,      \
+          sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib,\
+          q, qcap, tk);                                                                                               \
+    }                                                                                                                 \
   } else                                                                                                            \
     k_render_fwd<BW><<<grid, TILE_PIX, 0, s>>>((const uint2*)ranges, nullptr, sorted_vals, (const float4*)proj->xy, \
                                                (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, \
@@ -1474,14 +1753,20 @@ int gs_blend_bwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const ui
   if (sched)                                                                                                         \
     {                                                                                                              \
       if (cudaMemsetAsync(sched_ticket(sched), 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;        \
-      auto kb = fixed ? k_render_bwd_m<BW, false> : k_render_bwd_m<BW, true>;                                      \
-      kb<<<dim3(resident_grid(kb, sched->max_jobs * 8)), 32, 0, s>>>(                                               \
-          (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                       \
-          (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,               \
-          (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, TX * TY * n_units,   \
-          bg[0], bg[1], bg[2],                                                                                       \
-          img, final_T, n_contrib, dL_dimg, dL_dT, g2d->dxy, g2d->dconic_op, g2d->drgb, fixed,                       \
-          sched_ticket(sched));                                                                                      \
+      if (fixed) {                                                                                                   \
+        k_render_bwd_det<BW><<<dim3(resident_grid(k_render_bwd_det<BW>, sched->max_jobs * 8)), 32, 0, s>>>(          \
+            (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                     \
+            (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,             \
+            (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, TX * TY * n_units,  \
+            bg[0], bg[1], bg[2], img, final_T, n_contrib, dL_dimg, dL_dT, fixed, sched_ticket(sched));               \
+      } else {                                                                                                       \
+        k_render_bwd_m<BW><<<dim3(resident_grid(k_render_bwd_m<BW>, sched->max_jobs * 8)), 32, 0, s>>>(              \
+            (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                     \
+            (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,             \
+            (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, TX * TY * n_units,  \
+            bg[0], bg[1], bg[2], img, final_T, n_contrib, dL_dimg, dL_dT, g2d->dxy, g2d->dconic_op, g2d->drgb,       \
+            sched_ticket(sched));                                                                                    \
+      }                                                                                                              \
     }                                                                                                              \
   else                                                                                                               \
     k_render_bwd<BW><<<grid, TILE_PIX, 0, s>>>((const uint2*)ranges, nullptr, sorted_vals, (const float4*)proj->xy, \
