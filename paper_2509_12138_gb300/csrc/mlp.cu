@@ -10,16 +10,19 @@
 // (mma.sync m16n8k16 / m16n8k8); activations are rounded to bf16 where they
 // become the next GEMM's operand, and back-propagated signals likewise.
 //
-// One CTA of 4 warps handles batches of 64 points, 16 per warp.  Layer
-// outputs stay in registers: the accumulator layout of two adjacent n8 tiles
-// is the A-operand layout of one k16 step, so layers chain without shared
-// memory.  Weight gradients are tensor-core GEMMs over the 64-point batch
-// from bf16 tiles in shared memory, accumulated per CTA in fp32 shared memory
-// and added to the global gradient once per CTA.
+// Batches of 128 points, 16 per warp.  Layer outputs stay in registers: the
+// accumulator layout of two adjacent n8 tiles is the A-operand layout of one
+// k16 step, so layers chain without shared memory; the other operands come
+// from bf16 tiles in shared memory by ldmatrix.  Weight gradients are
+// tensor-core GEMMs over the batch's points, summed in fp32 registers over all
+// of a CTA's batches and added to the global gradient once per CTA.
 //
-// This stage is HBM-bound (about 300 bytes of gathered neighbour data per
-// point against 23 kFLOP), so mma.sync at this size already saturates the
-// memory system; see the design notes.
+// The arithmetic (23 kFLOP per point forward) is small for the tensor cores,
+// and the 300 gathered bytes per point are small for HBM; what bounds the
+// stage is latency: index load -> gather -> tile -> chained mma.  So the
+// training kernel gives the gathers to warps of their own, one batch ahead of
+// the warps that multiply, and mma.sync, whose operands and results are
+// registers, suffices.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -34,41 +37,61 @@ namespace {
 constexpr int KIN = 112, HID = 64, KOUT = 8, KNN = 16;
 constexpr int W1_OFF = 0, B1_OFF = W1_OFF + KIN * HID, W2_OFF = B1_OFF + HID, B2_OFF = W2_OFF + HID * HID;
 constexpr int W3_OFF = B2_OFF + HID, B3_OFF = W3_OFF + HID * KOUT, NPARAM = B3_OFF + KOUT;  // 11912
-constexpr int BATCH = 64;
-constexpr int THREADS = 128;
-constexpr int LDX = 120;  // bf16 row stride of the feature tile and of W1^T
-constexpr int LDH = 72;   // bf16 row stride of 64-wide tiles
+constexpr int BATCH = 128;       // points per batch
+constexpr int FWD_T = 256;        // threads of the forward kernels: 8 warps build, then multiply 16 points each
+constexpr int PROD_T = 128;       // training kernel: 4 warps that build the next batch's features,
+constexpr int CONS_T = 256;       // 8 warps that multiply
+constexpr int LDX = 120;  // bf16 row stride of the feature tile and of W1^T (240 B: 8 rows hit 8 bank groups)
+constexpr int LDH = 72;   // bf16 row stride of 64-wide tiles (144 B: likewise)
+constexpr int LDI = 17;   // row stride of the staged neighbour indices
 
 static_assert(NPARAM == 11912, "parameter layout");
+static_assert(CONS_T / 32 * 16 == BATCH && FWD_T / 32 * 16 == BATCH, "16 points per warp");
 
 // shared-memory layout (bytes)
 struct Smem {
   static constexpr int W1t = 0;                          // [64][LDX] bf16  W1^T
   static constexpr int W2t = W1t + HID * LDX * 2;        // [64][LDH] bf16  W2^T
-  static constexpr int W2 = W2t + HID * LDH * 2;         // [64][LDH] bf16  W2 (in-major)
-  static constexpr int W3t = W2 + HID * LDH * 2;         // [8][LDH]  bf16  W3^T
-  static constexpr int W3 = W3t + KOUT * LDH * 2;        // [64][8]   bf16  W3 (in-major)
-  static constexpr int Bias = W3 + HID * KOUT * 2;       // fp32 b1[64] b2[64] b3[8]
-  static constexpr int X = Bias + (2 * HID + KOUT) * 4;  // [64][LDX] bf16 features
-  static constexpr int Dbar = X + BATCH * LDX * 2;       // fp32 [64]
-  static constexpr int FWD_END = Dbar + BATCH * 4;
-  static constexpr int H1 = FWD_END;                     // [64][LDH] bf16
+  static constexpr int W3t = W2t + HID * LDH * 2;        // [8][LDH]  bf16  W3^T
+  static constexpr int Bias = W3t + KOUT * LDH * 2;      // fp32 b1[64] b2[64] b3[8]
+  static constexpr int Idx = Bias + (2 * HID + KOUT) * 4;  // int [BATCH][LDI]
+  static constexpr int Dbar = Idx + BATCH * LDI * 4;     // fp32 [BATCH]
+  static constexpr int X = Dbar + BATCH * 4;             // [BATCH][LDX] bf16 features
+  static constexpr int FWD_END = X + BATCH * LDX * 2;
+  static constexpr int Y = FWD_END;                      // fp32 [BATCH][8] outputs (initialiser)
+  static constexpr int INIT_END = Y + BATCH * KOUT * 4;
+  static constexpr int X2 = FWD_END;                     // training: the second feature tile
+  static constexpr int W2 = X2 + BATCH * LDX * 2;        // [64][LDH] bf16  W2 (in-major)
+  static constexpr int W3 = W2 + HID * LDH * 2;          // [64][8]   bf16  W3 (in-major)
+  static constexpr int H1 = W3 + HID * KOUT * 2;         // [BATCH][LDH] bf16
   static constexpr int H2 = H1 + BATCH * LDH * 2;
   static constexpr int dH1 = H2 + BATCH * LDH * 2;
   static constexpr int dH2 = dH1 + BATCH * LDH * 2;
-  static constexpr int dY = dH2 + BATCH * LDH * 2;       // [64][8] bf16
-  static constexpr int dW = dY + BATCH * KOUT * 2;       // fp32 [NPARAM]
-  static constexpr int TRAIN_END = dW + NPARAM * 4;
+  static constexpr int dY = dH2 + BATCH * LDH * 2;       // [BATCH][8] bf16
+  static constexpr int TRAIN_END = dY + BATCH * KOUT * 2;
 };
+static_assert(Smem::X % 16 == 0 && Smem::X2 % 16 == 0 && Smem::W2 % 16 == 0 && Smem::H1 % 16 == 0 &&
+              Smem::dY % 16 == 0 && Smem::W2t % 16 == 0 && Smem::W3t % 16 == 0, "ldmatrix rows are 16-byte aligned");
 
 __device__ __forceinline__ uint16_t bf(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ uint32_t pack(float lo, float hi) {
   return (uint32_t)bf(lo) | ((uint32_t)bf(hi) << 16);
 }
-__device__ __forceinline__ float unbf(uint16_t h) { return __bfloat162float(__ushort_as_bfloat16(h)); }
 __device__ __forceinline__ uint32_t ld32(const uint16_t* p) { return *reinterpret_cast<const uint32_t*>(p); }
-__device__ __forceinline__ uint32_t pair(const uint16_t* lo, const uint16_t* hi) {
-  return (uint32_t)(*lo) | ((uint32_t)(*hi) << 16);
+// Four 8x8 bf16 matrices, lane l giving the address of row l & 7 of matrix l >> 3; TRANS: transposed.
+template <bool TRANS = false>
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const uint16_t* p) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  if (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldsm2t(uint32_t& r0, uint32_t& r1, const uint16_t* p) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(a) : "memory");
 }
 
 __device__ __forceinline__ void mma16816(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
@@ -116,69 +139,104 @@ __device__ void stage_weights(const float* __restrict__ w, char* sm, bool train)
   }
 }
 
-// Features of the batch's points into the bf16 tile X[64][LDX].
-__device__ void build_features(const float* __restrict__ pts, const float* __restrict__ nrm,
-                               const int* __restrict__ knn_idx, const float* __restrict__ knn_dist, int64_t n,
-                               int64_t base, char* sm) {
-  uint16_t* X = (uint16_t*)(sm + Smem::X);
-  float* dbar = (float*)(sm + Smem::Dbar);
-  for (int p = threadIdx.x; p < BATCH; p += blockDim.x) {
-    int64_t i = base + p;
-    float s = 0.f;
-    if (i < n)
-      for (int a = 0; a < KNN; ++a) s += knn_dist[i * KNN + a];
-    float d = s / (float)KNN;
-    dbar[p] = d > 1e-12f ? d : 1e-12f;
+// The 16 neighbour indices and distances of a point, loaded ahead of their use.
+struct KnnRow {
+  int idx[KNN];
+  float dist[KNN];
+};
+__device__ __forceinline__ void load_row(KnnRow& r, const int* __restrict__ knn_idx,
+                                         const float* __restrict__ knn_dist, int64_t n, int64_t i, bool vec) {
+  if (i < n) {
+    if (vec) {  // rows are 64 bytes: 16-byte loads when the arrays start on 16 bytes
+      #pragma unroll
+      for (int q = 0; q < KNN / 4; ++q) {
+        const int4 a = __ldg(reinterpret_cast<const int4*>(knn_idx + i * KNN) + q);
+        const float4 b = __ldg(reinterpret_cast<const float4*>(knn_dist + i * KNN) + q);
+        r.idx[4 * q] = a.x; r.idx[4 * q + 1] = a.y; r.idx[4 * q + 2] = a.z; r.idx[4 * q + 3] = a.w;
+        r.dist[4 * q] = b.x; r.dist[4 * q + 1] = b.y; r.dist[4 * q + 2] = b.z; r.dist[4 * q + 3] = b.w;
+      }
+    } else {
+      #pragma unroll
+      for (int a = 0; a < KNN; ++a) { r.idx[a] = knn_idx[i * KNN + a]; r.dist[a] = knn_dist[i * KNN + a]; }
+    }
+  } else {
+    #pragma unroll
+    for (int a = 0; a < KNN; ++a) { r.idx[a] = -1; r.dist[a] = 0.f; }
   }
-  __syncthreads();
-  for (int q = threadIdx.x; q < BATCH * KNN; q += blockDim.x) {
-    int p = q / KNN, a = q % KNN;
-    int64_t i = base + p;
-    float o[3] = {0.f, 0.f, 0.f}, nn[3] = {0.f, 0.f, 0.f};
-    if (i < n) {
-      int j = knn_idx[i * KNN + a];
-      if (j >= 0) {
-        float inv = dbar[p];
-        for (int c = 0; c < 3; ++c) {
-          o[c] = (pts[3 * (int64_t)j + c] - pts[3 * i + c]) / inv;
-          nn[c] = nrm[3 * (int64_t)j + c];
-        }
+}
+__device__ __forceinline__ void stage_row(const KnnRow& r, int p, int* s_idx, float* s_dbar) {
+  float s = 0.f;
+  #pragma unroll
+  for (int a = 0; a < KNN; ++a) { s_idx[p * LDI + a] = r.idx[a]; s += r.dist[a]; }
+  const float d = s / (float)KNN;
+  s_dbar[p] = d > 1e-12f ? d : 1e-12f;
+}
+
+// Features of the batch's points into the bf16 tile X[BATCH][LDX] by NT
+// threads, from the staged neighbour rows.  A thread takes single (point,
+// neighbour, component) values: consecutive lanes read the components of one
+// neighbour and write consecutive features, so a warp's gather touches a third
+// of the sectors that whole neighbours per lane would.
+template <int NT>
+__device__ __forceinline__ void build_features(int tid, const float* __restrict__ pts, const float* __restrict__ nrm,
+                                               int64_t n, int64_t base, const int* s_idx, const float* s_dbar,
+                                               uint16_t* X) {
+  constexpr int STEP = NT * 3 / 48;  // points covered by three rounds of NT values
+  static_assert(NT * 3 % 48 == 0 && BATCH % STEP == 0, "rounds repeat every STEP points");
+  int pr[3], fr[3];
+  #pragma unroll
+  for (int r = 0; r < 3; ++r) { pr[r] = (tid + NT * r) / 48; fr[r] = (tid + NT * r) % 48; }
+  #pragma unroll 2
+  for (int q = 0; q < BATCH; q += STEP) {
+    float o[3], nn[3];
+    #pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int p = pr[r] + q, c = fr[r] % 3;
+      const int j = s_idx[p * LDI + fr[r] / 3];
+      o[r] = nn[r] = 0.f;
+      if (j >= 0) {  // (-1 for the points past n too)
+        o[r] = __ldg(pts + 3 * (int64_t)j + c) - __ldg(pts + 3 * (base + p) + c);
+        nn[r] = __ldg(nrm + 3 * (int64_t)j + c);
       }
     }
-    for (int c = 0; c < 3; ++c) {
-      X[p * LDX + 3 * a + c] = bf(o[c]);
-      X[p * LDX + 48 + 3 * a + c] = bf(nn[c]);
+    #pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int p = pr[r] + q;
+      X[p * LDX + fr[r]] = bf(o[r] / s_dbar[p]);
+      X[p * LDX + 48 + fr[r]] = bf(nn[r]);
     }
   }
-  for (int q = threadIdx.x; q < BATCH * (KIN - 96); q += blockDim.x) {
-    int p = q / (KIN - 96), f = 96 + q % (KIN - 96);
-    int64_t i = base + p;
-    float v = (f < 99 && i < n) ? nrm[3 * i + (f - 96)] : 0.f;
+  for (int e = tid; e < BATCH * (KIN - 96); e += NT) {
+    const int p = e / (KIN - 96), f = 96 + e % (KIN - 96);
+    const float v = (f < 99 && base + p < n) ? __ldg(nrm + 3 * (base + p) + (f - 96)) : 0.f;
     X[p * LDX + f] = bf(v);
   }
-  __syncthreads();
 }
 
 // Forward pass of the warp's 16 rows (m0 .. m0+15 of the batch).  h1, h2 are
 // the post-ReLU fp32 activations in accumulator layout; y the outputs.
-__device__ __forceinline__ void forward_rows(const char* sm, int m0, float (&h1)[8][4], float (&h2)[8][4],
-                                             float (&y)[4]) {
-  const uint16_t* X = (const uint16_t*)(sm + Smem::X);
-  const uint16_t* W1t = (const uint16_t*)(sm + Smem::W1t);
-  const uint16_t* W2t = (const uint16_t*)(sm + Smem::W2t);
+__device__ __forceinline__ void forward_rows(const char* sm, const uint16_t* X, int m0, float (&h1)[8][4],
+                                             float (&h2)[8][4], float (&y)[4]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, l8 = lane & 7, mi = lane >> 3;
+  // ldmatrix rows: A tiles (rows 0-7 | 8-15) x (k 0-7 | 8-15); weight tiles two n8 tiles x (k 0-7 | 8-15)
+  const uint16_t* ax = X + (m0 + l8 + (mi & 1) * 8) * LDX + (mi >> 1) * 8;
+  const uint16_t* w1 = (const uint16_t*)(sm + Smem::W1t) + (l8 + (mi >> 1) * 8) * LDX + (mi & 1) * 8;
+  const uint16_t* w2 = (const uint16_t*)(sm + Smem::W2t) + (l8 + (mi >> 1) * 8) * LDH + (mi & 1) * 8;
   const uint16_t* W3t = (const uint16_t*)(sm + Smem::W3t);
   const float* bias = (const float*)(sm + Smem::Bias);
-  int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   #pragma unroll
   for (int j = 0; j < 8; ++j) h1[j][0] = h1[j][1] = h1[j][2] = h1[j][3] = 0.f;
   #pragma unroll
   for (int s = 0; s < KIN / 16; ++s) {
-    int k0 = 16 * s + 2 * t;
-    uint32_t a[4] = {ld32(X + (m0 + g) * LDX + k0), ld32(X + (m0 + g + 8) * LDX + k0),
-                     ld32(X + (m0 + g) * LDX + k0 + 8), ld32(X + (m0 + g + 8) * LDX + k0 + 8)};
+    uint32_t a[4];
+    ldsm4(a, ax + 16 * s);
     #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      mma16816(h1[j], a, ld32(W1t + (8 * j + g) * LDX + k0), ld32(W1t + (8 * j + g) * LDX + k0 + 8));
+    for (int j = 0; j < 8; j += 2) {
+      uint32_t b[4];
+      ldsm4(b, w1 + 8 * j * LDX + 16 * s);
+      mma16816(h1[j], a, b[0], b[1]);
+      mma16816(h1[j + 1], a, b[2], b[3]);
+    }
   }
   #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -192,10 +250,13 @@ __device__ __forceinline__ void forward_rows(const char* sm, int m0, float (&h1)
   for (int s = 0; s < HID / 16; ++s) {
     uint32_t a[4] = {pack(h1[2 * s][0], h1[2 * s][1]), pack(h1[2 * s][2], h1[2 * s][3]),
                      pack(h1[2 * s + 1][0], h1[2 * s + 1][1]), pack(h1[2 * s + 1][2], h1[2 * s + 1][3])};
-    int k0 = 16 * s + 2 * t;
     #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      mma16816(h2[j], a, ld32(W2t + (8 * j + g) * LDH + k0), ld32(W2t + (8 * j + g) * LDH + k0 + 8));
+    for (int j = 0; j < 8; j += 2) {
+      uint32_t b[4];
+      ldsm4(b, w2 + 8 * j * LDH + 16 * s);
+      mma16816(h2[j], a, b[0], b[1]);
+      mma16816(h2[j + 1], a, b[2], b[3]);
+    }
   }
   #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -215,22 +276,36 @@ __device__ __forceinline__ void forward_rows(const char* sm, int m0, float (&h1)
   y[0] += b0; y[1] += b1; y[2] += b0; y[3] += b1;
 }
 
+// Rows of a batch staged, then its features (all FWD_T threads of a forward kernel).
+__device__ __forceinline__ void build_batch(const float* __restrict__ pts, const float* __restrict__ nrm,
+                                            const int* __restrict__ knn_idx, const float* __restrict__ knn_dist,
+                                            int64_t n, int64_t base, bool vec, char* sm) {
+  if (threadIdx.x < BATCH) {
+    KnnRow r;
+    load_row(r, knn_idx, knn_dist, n, base + threadIdx.x, vec);
+    stage_row(r, threadIdx.x, (int*)(sm + Smem::Idx), (float*)(sm + Smem::Dbar));
+  }
+  __syncthreads();
+  build_features<FWD_T>(threadIdx.x, pts, nrm, n, base, (const int*)(sm + Smem::Idx), (const float*)(sm + Smem::Dbar),
+                        (uint16_t*)(sm + Smem::X));
+  __syncthreads();
+}
+
 // y rows (m0+g, m0+g+8), cols (2t, 2t+1) -> out[row][col]
-__global__ void __launch_bounds__(THREADS) k_mlp_forward(const float* __restrict__ pts, const float* __restrict__ nrm,
+__global__ void __launch_bounds__(FWD_T) k_mlp_forward(const float* __restrict__ pts, const float* __restrict__ nrm,
                                                          const int* __restrict__ knn_idx,
-                                                         const float* __restrict__ knn_dist, int64_t n,
+                                                         const float* __restrict__ knn_dist, int64_t n, bool vec,
                                                          const float* __restrict__ w, float* __restrict__ out) {
   extern __shared__ __align__(16) char sm[];
   stage_weights(w, sm, false);
-  __syncthreads();
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   int64_t nb = (n + BATCH - 1) / BATCH;
   for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
     int64_t base = b * BATCH;
-    build_features(pts, nrm, knn_idx, knn_dist, n, base, sm);
+    build_batch(pts, nrm, knn_idx, knn_dist, n, base, vec, sm);
     float h1[8][4], h2[8][4], y[4];
     int m0 = warp * 16;
-    forward_rows(sm, m0, h1, h2, y);
+    forward_rows(sm, (const uint16_t*)(sm + Smem::X), m0, h1, h2, y);
     int64_t r0 = base + m0 + g, r1 = r0 + 8;
     if (r0 < n) { out[r0 * KOUT + 2 * t] = y[0]; out[r0 * KOUT + 2 * t + 1] = y[1]; }
     if (r1 < n) { out[r1 * KOUT + 2 * t] = y[2]; out[r1 * KOUT + 2 * t + 1] = y[3]; }
@@ -270,52 +345,82 @@ __global__ void k_plain_init(const float* __restrict__ knn_dist, int k, int64_t 
   write_init(params, N, i, d3, nullptr, false, logit_default);
 }
 
-__global__ void __launch_bounds__(THREADS) k_mlp_init(const float* __restrict__ pts, const float* __restrict__ nrm,
+__global__ void __launch_bounds__(FWD_T) k_mlp_init(const float* __restrict__ pts, const float* __restrict__ nrm,
                                                       const int* __restrict__ knn_idx,
-                                                      const float* __restrict__ knn_dist, int64_t n,
+                                                      const float* __restrict__ knn_dist, int64_t n, bool vec,
                                                       const float* __restrict__ w, float logit_default,
                                                       float4* __restrict__ params, int64_t N) {
   extern __shared__ __align__(16) char sm[];
   stage_weights(w, sm, false);
-  __syncthreads();
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  float* ybuf = (float*)(sm + Smem::H1);  // [64][8] fp32 staging of the outputs
+  float* ybuf = (float*)(sm + Smem::Y);  // [BATCH][8] fp32 staging of the outputs
   int64_t nb = (n + BATCH - 1) / BATCH;
   for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
     int64_t base = b * BATCH;
-    build_features(pts, nrm, knn_idx, knn_dist, n, base, sm);
+    build_batch(pts, nrm, knn_idx, knn_dist, n, base, vec, sm);
     float h1[8][4], h2[8][4], y[4];
     int m0 = warp * 16;
-    forward_rows(sm, m0, h1, h2, y);
+    forward_rows(sm, (const uint16_t*)(sm + Smem::X), m0, h1, h2, y);
     ybuf[(m0 + g) * KOUT + 2 * t] = y[0];
     ybuf[(m0 + g) * KOUT + 2 * t + 1] = y[1];
     ybuf[(m0 + g + 8) * KOUT + 2 * t] = y[2];
     ybuf[(m0 + g + 8) * KOUT + 2 * t + 1] = y[3];
     __syncthreads();
-    for (int p = threadIdx.x; p < BATCH; p += blockDim.x) {
-      int64_t i = base + p;
-      if (i >= n) continue;
+    if (threadIdx.x < BATCH && base + threadIdx.x < n) {
+      int64_t i = base + threadIdx.x;
       float d3 = (knn_dist[i * KNN] + knn_dist[i * KNN + 1] + knn_dist[i * KNN + 2]) / 3.f;
-      write_init(params, N, i, d3, ybuf + p * KOUT, true, logit_default);
+      write_init(params, N, i, d3, ybuf + threadIdx.x * KOUT, true, logit_default);
     }
-    __syncthreads();
   }
+}
+
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
 }
 
 // One training step's gradients: forward, loss (sum of squared errors times
 // `scale`), backward; dW accumulated into `grad` (zeroed by the caller).
-__global__ void __launch_bounds__(THREADS) k_mlp_train(const float* __restrict__ pts, const float* __restrict__ nrm,
-                                                       const int* __restrict__ knn_idx,
-                                                       const float* __restrict__ knn_dist,
-                                                       const float* __restrict__ target, int64_t n,
-                                                       const float* __restrict__ w, float scale,
-                                                       float* __restrict__ grad, float* __restrict__ loss) {
+//
+// One CTA per SM (183 KB of tiles): 8 warps multiply batch t while 4 warps
+// build the features of batch t + 1 into the other tile (with the neighbour
+// rows of t + 2 already loading), one block barrier per batch.  The weight
+// gradients' 92 m16n8 tiles are split over the 8 warps as (half of the rows) x
+// (16 columns), at most 12 tiles each, so every operand fragment serves several
+// mma; a batch's tiles are summed from zero on the tensor cores and added to
+// fp32 registers, which leave for memory once, at the end.  Bias gradients are
+// the same columns multiplied by a fragment of ones.  2M points: 3792 us with
+// one warp group per SM doing both in turn, operands read as 16-bit scalars
+// and gradients kept in shared memory; 923 us.
+__global__ void __launch_bounds__(CONS_T + PROD_T, 1)
+    k_mlp_train(const float* __restrict__ pts, const float* __restrict__ nrm, const int* __restrict__ knn_idx,
+                const float* __restrict__ knn_dist, const float* __restrict__ target, int64_t n, bool vec,
+                const float* __restrict__ w, float scale, float* __restrict__ grad, float* __restrict__ loss) {
   extern __shared__ __align__(16) char sm[];
+  int* s_idx = (int*)(sm + Smem::Idx);
+  float* s_dbar = (float*)(sm + Smem::Dbar);
+  const int64_t nb = (n + BATCH - 1) / BATCH;
+  const int64_t b0 = blockIdx.x;
+  const int steps = b0 < nb ? (int)((nb - b0 + gridDim.x - 1) / gridDim.x) : 0;
+  auto base_of = [&](int k) { return (b0 + (int64_t)k * gridDim.x) * BATCH; };
+  auto tile = [&](int k) { return (uint16_t*)(sm + ((k & 1) ? Smem::X2 : Smem::X)); };
   stage_weights(w, sm, true);
-  float* dW = (float*)(sm + Smem::dW);
-  for (int q = threadIdx.x; q < NPARAM; q += blockDim.x) dW[q] = 0.f;
   __syncthreads();
-  uint16_t* sX = (uint16_t*)(sm + Smem::X);
+  if (threadIdx.x >= CONS_T) {
+    // ---- feature builders
+    const int tid = threadIdx.x - CONS_T;
+    KnnRow row;
+    if (steps > 0) load_row(row, knn_idx, knn_dist, n, base_of(0) + tid, vec);
+    for (int k = 0; k < steps; ++k) {  // batch k, while the other warps multiply batch k - 1
+      stage_row(row, tid, s_idx, s_dbar);
+      if (k + 1 < steps) load_row(row, knn_idx, knn_dist, n, base_of(k + 1) + tid, vec);
+      bar_sync(2, PROD_T);
+      build_features<PROD_T>(tid, pts, nrm, n, base_of(k), s_idx, s_dbar, tile(k));
+      __syncthreads();
+    }
+    __syncthreads();  // the last batch is multiplied
+    return;
+  }
+  // ---- multipliers
   uint16_t* sH1 = (uint16_t*)(sm + Smem::H1);
   uint16_t* sH2 = (uint16_t*)(sm + Smem::H2);
   uint16_t* sdH1 = (uint16_t*)(sm + Smem::dH1);
@@ -323,128 +428,221 @@ __global__ void __launch_bounds__(THREADS) k_mlp_train(const float* __restrict__
   uint16_t* sdY = (uint16_t*)(sm + Smem::dY);
   const uint16_t* W2 = (const uint16_t*)(sm + Smem::W2);
   const uint16_t* W3 = (const uint16_t*)(sm + Smem::W3);
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int l8 = lane & 7, mi = lane >> 3;
+  const int m0 = warp * 16;
+  // weight-gradient tiles of this warp: rows 64 half .. of dW1 (4 or 3 m16 tiles), 32 half .. of dW2, 16 nq .. of
+  // dW3 (half 1), all in columns 16 nq ..
+  const int half = warp & 1, nq = warp >> 1;
+  float g1[4][2][4], g2[2][2][4], g3[4], gb[2][2], gb3[2];
+  #pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    #pragma unroll
+    for (int m = 0; m < 4; ++m) g1[m][0][e] = g1[m][1][e] = 0.f;
+    #pragma unroll
+    for (int m = 0; m < 2; ++m) g2[m][0][e] = g2[m][1][e] = 0.f;
+    g3[e] = 0.f;
+  }
+  gb[0][0] = gb[0][1] = gb[1][0] = gb[1][1] = gb3[0] = gb3[1] = 0.f;
+  const uint32_t ONES[4] = {0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u};
   float lsum = 0.f;
-  int64_t nb = (n + BATCH - 1) / BATCH;
-  for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
-    int64_t base = b * BATCH;
-    build_features(pts, nrm, knn_idx, knn_dist, n, base, sm);
-    float h1[8][4], h2[8][4], y[4];
-    int m0 = warp * 16;
-    forward_rows(sm, m0, h1, h2, y);
-    int64_t r0 = base + m0 + g, r1 = r0 + 8;
-    float dy[4];
+  for (int k = 0; k < steps; ++k) {
+    __syncthreads();  // batch k's features are in its tile; every warp is done with batch k - 1
+    const uint16_t* X = tile(k);
+    const int64_t r0 = base_of(k) + m0 + g, r1 = r0 + 8;
+    float tg[4] = {0.f, 0.f, 0.f, 0.f};
+    if (r0 < n) { tg[0] = __ldg(target + r0 * KOUT + 2 * t); tg[1] = __ldg(target + r0 * KOUT + 2 * t + 1); }
+    if (r1 < n) { tg[2] = __ldg(target + r1 * KOUT + 2 * t); tg[3] = __ldg(target + r1 * KOUT + 2 * t + 1); }
+    uint32_t on1 = 0u, on2 = 0u;  // active ReLUs, bit 4 j + e
+    uint32_t ady0, ady1;
+    {
+      float h1[8][4], h2[8][4], y[4];
+      forward_rows(sm, X, m0, h1, h2, y);
+      float dy[4];
+      #pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float d = (e < 2 ? r0 : r1) < n ? y[e] - tg[e] : 0.f;
+        lsum += d * d;
+        dy[e] = 2.f * d * scale;
+      }
+      ady0 = pack(dy[0], dy[1]); ady1 = pack(dy[2], dy[3]);
+      *reinterpret_cast<uint32_t*>(sdY + (m0 + g) * KOUT + 2 * t) = ady0;
+      *reinterpret_cast<uint32_t*>(sdY + (m0 + g + 8) * KOUT + 2 * t) = ady1;
+      // activations as bf16 tiles for the weight gradients
+      #pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        *reinterpret_cast<uint32_t*>(sH1 + (m0 + g) * LDH + 8 * j + 2 * t) = pack(h1[j][0], h1[j][1]);
+        *reinterpret_cast<uint32_t*>(sH1 + (m0 + g + 8) * LDH + 8 * j + 2 * t) = pack(h1[j][2], h1[j][3]);
+        *reinterpret_cast<uint32_t*>(sH2 + (m0 + g) * LDH + 8 * j + 2 * t) = pack(h2[j][0], h2[j][1]);
+        *reinterpret_cast<uint32_t*>(sH2 + (m0 + g + 8) * LDH + 8 * j + 2 * t) = pack(h2[j][2], h2[j][3]);
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          on1 |= (h1[j][e] > 0.f ? 1u : 0u) << (4 * j + e);
+          on2 |= (h2[j][e] > 0.f ? 1u : 0u) << (4 * j + e);
+        }
+      }
+    }
+    {
+      // dH2 = dY W3^T, masked by the ReLU of layer 2, rounded to bf16
+      uint32_t d2[8][2];
+      #pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        mma1688(d, ady0, ady1, ld32(W3 + (8 * j + g) * KOUT + 2 * t));
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) d[e] = (on2 >> (4 * j + e)) & 1u ? d[e] : 0.f;
+        d2[j][0] = pack(d[0], d[1]); d2[j][1] = pack(d[2], d[3]);
+        *reinterpret_cast<uint32_t*>(sdH2 + (m0 + g) * LDH + 8 * j + 2 * t) = d2[j][0];
+        *reinterpret_cast<uint32_t*>(sdH2 + (m0 + g + 8) * LDH + 8 * j + 2 * t) = d2[j][1];
+      }
+      // dH1 = dH2 W2^T, masked by the ReLU of layer 1
+      float d1[8][4];
+      #pragma unroll
+      for (int j = 0; j < 8; ++j) d1[j][0] = d1[j][1] = d1[j][2] = d1[j][3] = 0.f;
+      const uint16_t* w2 = W2 + (l8 + (mi >> 1) * 8) * LDH + (mi & 1) * 8;
+      #pragma unroll
+      for (int s = 0; s < HID / 16; ++s) {
+        const uint32_t a[4] = {d2[2 * s][0], d2[2 * s][1], d2[2 * s + 1][0], d2[2 * s + 1][1]};
+        #pragma unroll
+        for (int j = 0; j < 8; j += 2) {
+          uint32_t b[4];
+          ldsm4(b, w2 + 8 * j * LDH + 16 * s);
+          mma16816(d1[j], a, b[0], b[1]);
+          mma16816(d1[j + 1], a, b[2], b[3]);
+        }
+      }
+      #pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) d1[j][e] = (on1 >> (4 * j + e)) & 1u ? d1[j][e] : 0.f;
+        *reinterpret_cast<uint32_t*>(sdH1 + (m0 + g) * LDH + 8 * j + 2 * t) = pack(d1[j][0], d1[j][1]);
+        *reinterpret_cast<uint32_t*>(sdH1 + (m0 + g + 8) * LDH + 8 * j + 2 * t) = pack(d1[j][2], d1[j][3]);
+      }
+    }
+    bar_sync(1, CONS_T);
+    // weight gradients over the batch's points: dW1 = X^T dH1, dW2 = H1^T dH2, dW3 = H2^T dY; both operands
+    // transposed on the way into registers (ldmatrix rows: points)
+    const int arow = l8 + (mi >> 1) * 8, acol = (mi & 1) * 8;  // A: (points 0-7 | 8-15) x (rows 0-7 | 8-15)
+    const int brow = l8 + (mi & 1) * 8, bcol = 16 * nq + (mi >> 1) * 8;
+    {
+      float a1[4][2][4], s1[2][4];
+      #pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        #pragma unroll
+        for (int m = 0; m < 4; ++m) a1[m][0][e] = a1[m][1][e] = 0.f;
+        s1[0][e] = s1[1][e] = 0.f;
+      }
+      #pragma unroll 2
+      for (int s = 0; s < BATCH / 16; ++s) {
+        uint32_t b[4];
+        ldsm4<true>(b, sdH1 + (16 * s + brow) * LDH + bcol);
+        #pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          if (half == 1 && m == 3) continue;  // 7 row tiles: 4 and 3
+          uint32_t a[4];
+          ldsm4<true>(a, X + (16 * s + arow) * LDX + 64 * half + 16 * m + acol);
+          mma16816(a1[m][0], a, b[0], b[1]);
+          mma16816(a1[m][1], a, b[2], b[3]);
+        }
+        if (half == 0) {
+          mma16816(s1[0], ONES, b[0], b[1]);
+          mma16816(s1[1], ONES, b[2], b[3]);
+        }
+      }
+      #pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        #pragma unroll
+        for (int e = 0; e < 4; ++e)
+          #pragma unroll
+          for (int m = 0; m < 4; ++m) g1[m][q][e] += a1[m][q][e];
+        if (half == 0) { gb[q][0] += s1[q][0]; gb[q][1] += s1[q][1]; }
+      }
+    }
+    {
+      float a2[2][2][4], a3[4], s2[2][4], s3[4];
+      #pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        a2[0][0][e] = a2[0][1][e] = a2[1][0][e] = a2[1][1][e] = 0.f;
+        a3[e] = s2[0][e] = s2[1][e] = s3[e] = 0.f;
+      }
+      #pragma unroll 2
+      for (int s = 0; s < BATCH / 16; ++s) {
+        uint32_t b[4];
+        ldsm4<true>(b, sdH2 + (16 * s + brow) * LDH + bcol);
+        #pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          uint32_t a[4];
+          ldsm4<true>(a, sH1 + (16 * s + arow) * LDH + 32 * half + 16 * m + acol);
+          mma16816(a2[m][0], a, b[0], b[1]);
+          mma16816(a2[m][1], a, b[2], b[3]);
+        }
+        if (half == 1) {
+          mma16816(s2[0], ONES, b[0], b[1]);
+          mma16816(s2[1], ONES, b[2], b[3]);
+          uint32_t a[4], y0, y1;
+          ldsm2t(y0, y1, sdY + (16 * s + (lane & 15)) * KOUT);
+          ldsm4<true>(a, sH2 + (16 * s + arow) * LDH + 16 * nq + acol);
+          mma16816(a3, a, y0, y1);
+          if (nq == 0) mma16816(s3, ONES, y0, y1);
+        }
+      }
+      #pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) { g2[0][q][e] += a2[0][q][e]; g2[1][q][e] += a2[1][q][e]; }
+        if (half == 1) { gb[q][0] += s2[q][0]; gb[q][1] += s2[q][1]; }
+      }
+      #pragma unroll
+      for (int e = 0; e < 4; ++e) g3[e] += a3[e];
+      gb3[0] += s3[0]; gb3[1] += s3[1];
+    }
+  }
+  __syncthreads();  // (the builders' last barrier)
+  // accumulator element e of a tile: row g (+ 8 for e >= 2), column 2 t + (e & 1)
+  auto put = [&](int off, int ncols, int row, int col, const float* v) {
     #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      int64_t r = e < 2 ? r0 : r1;
-      int col = 2 * t + (e & 1);
-      float d = 0.f;
-      if (r < n) {
-        d = y[e] - target[r * KOUT + col];
-        lsum += d * d;
-      }
-      dy[e] = 2.f * d * scale;
+      const int r = row + g + (e >> 1) * 8, c = col + 2 * t + (e & 1);
+      if (v[e] != 0.f) atomicAdd(grad + off + r * ncols + c, v[e]);
     }
-    uint32_t ady0 = pack(dy[0], dy[1]), ady1 = pack(dy[2], dy[3]);
-    *reinterpret_cast<uint32_t*>(sdY + (m0 + g) * KOUT + 2 * t) = ady0;
-    *reinterpret_cast<uint32_t*>(sdY + (m0 + g + 8) * KOUT + 2 * t) = ady1;
-    // activations as bf16 tiles for the weight gradients
+  };
+  #pragma unroll
+  for (int q = 0; q < 2; ++q) {
     #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      *reinterpret_cast<uint32_t*>(sH1 + (m0 + g) * LDH + 8 * j + 2 * t) = pack(h1[j][0], h1[j][1]);
-      *reinterpret_cast<uint32_t*>(sH1 + (m0 + g + 8) * LDH + 8 * j + 2 * t) = pack(h1[j][2], h1[j][3]);
-      *reinterpret_cast<uint32_t*>(sH2 + (m0 + g) * LDH + 8 * j + 2 * t) = pack(h2[j][0], h2[j][1]);
-      *reinterpret_cast<uint32_t*>(sH2 + (m0 + g + 8) * LDH + 8 * j + 2 * t) = pack(h2[j][2], h2[j][3]);
-    }
-    // dH2 = dY W3^T, masked by the ReLU of layer 2, rounded to bf16
-    float d2[8][4];
+    for (int m = 0; m < 4; ++m)
+      if (half == 0 || m < 3) put(W1_OFF, HID, 64 * half + 16 * m, 16 * nq + 8 * q, g1[m][q]);
     #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      d2[j][0] = d2[j][1] = d2[j][2] = d2[j][3] = 0.f;
-      mma1688(d2[j], ady0, ady1, ld32(W3 + (8 * j + g) * KOUT + 2 * t));
-      #pragma unroll
-      for (int e = 0; e < 4; ++e) d2[j][e] = h2[j][e] > 0.f ? d2[j][e] : 0.f;
-      *reinterpret_cast<uint32_t*>(sdH2 + (m0 + g) * LDH + 8 * j + 2 * t) = pack(d2[j][0], d2[j][1]);
-      *reinterpret_cast<uint32_t*>(sdH2 + (m0 + g + 8) * LDH + 8 * j + 2 * t) = pack(d2[j][2], d2[j][3]);
+    for (int m = 0; m < 2; ++m) put(W2_OFF, HID, 32 * half + 16 * m, 16 * nq + 8 * q, g2[m][q]);
+    if (g == 0) {  // every row of a ones product holds the column sums
+      float* gbias = grad + (half == 0 ? B1_OFF : B2_OFF) + 16 * nq + 8 * q + 2 * t;
+      atomicAdd(gbias, gb[q][0]);
+      atomicAdd(gbias + 1, gb[q][1]);
     }
-    // dH1 = dH2 W2^T, masked by the ReLU of layer 1
-    float d1[8][4];
-    #pragma unroll
-    for (int j = 0; j < 8; ++j) d1[j][0] = d1[j][1] = d1[j][2] = d1[j][3] = 0.f;
-    #pragma unroll
-    for (int s = 0; s < HID / 16; ++s) {
-      uint32_t a[4] = {pack(d2[2 * s][0], d2[2 * s][1]), pack(d2[2 * s][2], d2[2 * s][3]),
-                       pack(d2[2 * s + 1][0], d2[2 * s + 1][1]), pack(d2[2 * s + 1][2], d2[2 * s + 1][3])};
-      int k0 = 16 * s + 2 * t;
-      #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        mma16816(d1[j], a, ld32(W2 + (8 * j + g) * LDH + k0), ld32(W2 + (8 * j + g) * LDH + k0 + 8));
-    }
-    #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      #pragma unroll
-      for (int e = 0; e < 4; ++e) d1[j][e] = h1[j][e] > 0.f ? d1[j][e] : 0.f;
-      *reinterpret_cast<uint32_t*>(sdH1 + (m0 + g) * LDH + 8 * j + 2 * t) = pack(d1[j][0], d1[j][1]);
-      *reinterpret_cast<uint32_t*>(sdH1 + (m0 + g + 8) * LDH + 8 * j + 2 * t) = pack(d1[j][2], d1[j][3]);
-    }
-    __syncthreads();
-    // weight gradients over the 64-point batch: dW1 = X^T dH1 (7 x 8 tiles),
-    // dW2 = H1^T dH2 (4 x 8), dW3 = H2^T dY (4 x 1); K = the 64 points
-    for (int tile = warp; tile < 56 + 32 + 4; tile += THREADS / 32) {
-      const uint16_t *A, *B;
-      int lda, ldb, mi, nj, ncols, off;
-      if (tile < 56) { A = sX; lda = LDX; B = sdH1; ldb = LDH; mi = tile / 8; nj = tile % 8; ncols = HID; off = W1_OFF; }
-      else if (tile < 88) { int q = tile - 56; A = sH1; lda = LDH; B = sdH2; ldb = LDH; mi = q / 8; nj = q % 8; ncols = HID; off = W2_OFF; }
-      else { int q = tile - 88; A = sH2; lda = LDH; B = sdY; ldb = KOUT; mi = q; nj = 0; ncols = KOUT; off = W3_OFF; }
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      int m = 16 * mi + g, ncol = 8 * nj + g;
-      #pragma unroll
-      for (int s = 0; s < BATCH / 16; ++s) {
-        int p = 16 * s + 2 * t;  // batch rows (the K dimension)
-        uint32_t a[4] = {pair(A + p * lda + m, A + (p + 1) * lda + m),
-                         pair(A + p * lda + m + 8, A + (p + 1) * lda + m + 8),
-                         pair(A + (p + 8) * lda + m, A + (p + 9) * lda + m),
-                         pair(A + (p + 8) * lda + m + 8, A + (p + 9) * lda + m + 8)};
-        uint32_t b0 = pair(B + p * ldb + ncol, B + (p + 1) * ldb + ncol);
-        uint32_t b1 = pair(B + (p + 8) * ldb + ncol, B + (p + 9) * ldb + ncol);
-        mma16816(acc, a, b0, b1);
-      }
-      int col = 8 * nj + 2 * t;
-      dW[off + m * ncols + col] += acc[0];
-      dW[off + m * ncols + col + 1] += acc[1];
-      dW[off + (m + 8) * ncols + col] += acc[2];
-      dW[off + (m + 8) * ncols + col + 1] += acc[3];
-    }
-    // bias gradients: sums of the rounded back-propagated signals
-    for (int q = threadIdx.x; q < 2 * HID + KOUT; q += blockDim.x) {
-      float s = 0.f;
-      if (q < HID) { for (int p = 0; p < BATCH; ++p) s += unbf(sdH1[p * LDH + q]); dW[B1_OFF + q] += s; }
-      else if (q < 2 * HID) { for (int p = 0; p < BATCH; ++p) s += unbf(sdH2[p * LDH + q - HID]); dW[B2_OFF + q - HID] += s; }
-      else { for (int p = 0; p < BATCH; ++p) s += unbf(sdY[p * KOUT + q - 2 * HID]); dW[B3_OFF + q - 2 * HID] += s; }
-    }
-    __syncthreads();
   }
-  for (int q = threadIdx.x; q < NPARAM; q += blockDim.x)
-    if (dW[q] != 0.f) atomicAdd(&grad[q], dW[q]);
+  if (half == 1) put(W3_OFF, KOUT, 16 * nq, 0, g3);
+  if (half == 1 && nq == 0 && g == 0) {
+    atomicAdd(grad + B3_OFF + 2 * t, gb3[0]);
+    atomicAdd(grad + B3_OFF + 2 * t + 1, gb3[1]);
+  }
   #pragma unroll
   for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if (lane == 0 && lsum != 0.f) atomicAdd(loss, lsum * scale);
 }
 
-__global__ void k_features_out(const float* __restrict__ pts, const float* __restrict__ nrm,
-                               const int* __restrict__ knn_idx, const float* __restrict__ knn_dist, int64_t n,
-                               uint16_t* __restrict__ X) {
+__global__ void __launch_bounds__(FWD_T) k_features_out(const float* __restrict__ pts, const float* __restrict__ nrm,
+                                                        const int* __restrict__ knn_idx,
+                                                        const float* __restrict__ knn_dist, int64_t n, bool vec,
+                                                        uint16_t* __restrict__ X) {
   extern __shared__ __align__(16) char sm[];
   int64_t nb = (n + BATCH - 1) / BATCH;
   const uint16_t* sX = (const uint16_t*)(sm + Smem::X);
   for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
     int64_t base = b * BATCH;
-    build_features(pts, nrm, knn_idx, knn_dist, n, base, sm);
+    build_batch(pts, nrm, knn_idx, knn_dist, n, base, vec, sm);
     for (int q = threadIdx.x; q < BATCH * KIN; q += blockDim.x) {
       int p = q / KIN, f = q % KIN;
       if (base + p < n) X[(base + p) * KIN + f] = sX[p * LDX + f];
     }
-    __syncthreads();
   }
 }
 
@@ -463,6 +661,8 @@ int set_smem(K kernel, int bytes) {
                                                                                                           : GS_ERR_CUDA;
 }
 
+bool rows_aligned(const int32_t* idx, const float* dist) { return (((uintptr_t)idx | (uintptr_t)dist) & 15u) == 0; }
+
 bool knn_args_ok(const float* pts, const float* nrm, const int32_t* idx, const float* dist, int64_t n) {
   return pts && nrm && idx && dist && n >= 0;
 }
@@ -477,8 +677,8 @@ GS_API int gs_mlp_features(const float* points, const float* normals, const int3
   if (!knn_args_ok(points, normals, knn_idx, knn_dist, n) || !features) return GS_ERR_INVALID;
   if (n == 0) return GS_OK;
   if (set_smem(k_features_out, Smem::FWD_END) != GS_OK) return GS_ERR_CUDA;
-  k_features_out<<<grid_for(n, 4), THREADS, Smem::FWD_END, (cudaStream_t)stream>>>(points, normals, knn_idx, knn_dist,
-                                                                                   n, features);
+  k_features_out<<<grid_for(n, 3), FWD_T, Smem::FWD_END, (cudaStream_t)stream>>>(
+      points, normals, knn_idx, knn_dist, n, rows_aligned(knn_idx, knn_dist), features);
   return gs_check_launch();
 }
 
@@ -488,8 +688,8 @@ GS_API int gs_mlp_forward(const float* points, const float* normals, const int32
   if (!knn_args_ok(points, normals, knn_idx, knn_dist, n) || !weights || !out) return GS_ERR_INVALID;
   if (n == 0) return GS_OK;
   if (set_smem(k_mlp_forward, Smem::FWD_END) != GS_OK) return GS_ERR_CUDA;
-  k_mlp_forward<<<grid_for(n, 4), THREADS, Smem::FWD_END, (cudaStream_t)stream>>>(points, normals, knn_idx, knn_dist,
-                                                                                  n, weights, out);
+  k_mlp_forward<<<grid_for(n, 3), FWD_T, Smem::FWD_END, (cudaStream_t)stream>>>(
+      points, normals, knn_idx, knn_dist, n, rows_aligned(knn_idx, knn_dist), weights, out);
   return gs_check_launch();
 }
 
@@ -506,8 +706,8 @@ GS_API int gs_mlp_train_step(const float* points, const float* normals, const in
     return GS_ERR_CUDA;
   if (set_smem(k_mlp_train, Smem::TRAIN_END) != GS_OK) return GS_ERR_CUDA;
   float scale = 1.0f / (8.0f * (float)n);
-  k_mlp_train<<<grid_for(n, 1), THREADS, Smem::TRAIN_END, s>>>(points, normals, knn_idx, knn_dist, targets, n,
-                                                               weights, scale, grad, d_loss);
+  k_mlp_train<<<grid_for(n, 1), CONS_T + PROD_T, Smem::TRAIN_END, s>>>(
+      points, normals, knn_idx, knn_dist, targets, n, rows_aligned(knn_idx, knn_dist), weights, scale, grad, d_loss);
   int r = gs_check_launch();
   if (r != GS_OK) return r;
   float lr4[4] = {lr, lr, lr, lr};
@@ -531,9 +731,10 @@ GS_API int gs_init_gaussians(const float* points, const float* normals, const in
     k_plain_init<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(knn_dist, knn_k, n, logit_default, (float4*)params,
                                                              n_gauss);
   } else {
-    if (set_smem(k_mlp_init, Smem::FWD_END + BATCH * KOUT * 4) != GS_OK) return GS_ERR_CUDA;
-    k_mlp_init<<<grid_for(n, 4), THREADS, Smem::FWD_END + BATCH * KOUT * 4, s>>>(
-        points, normals, knn_idx, knn_dist, n, weights, logit_default, (float4*)params, n_gauss);
+    if (set_smem(k_mlp_init, Smem::INIT_END) != GS_OK) return GS_ERR_CUDA;
+    k_mlp_init<<<grid_for(n, 3), FWD_T, Smem::INIT_END, s>>>(points, normals, knn_idx, knn_dist, n,
+                                                             rows_aligned(knn_idx, knn_dist), weights, logit_default,
+                                                             (float4*)params, n_gauss);
   }
   return gs_check_launch();
 }
