@@ -2,8 +2,8 @@
 //
 // The mask restricts the loss to the pixels a partition owns (paper Sec. II,
 // "Image Rendering and Masking").  SSIM uses the 11x11 Gaussian window
-// (sigma 1.5) as a separable, zero-padded "same" convolution; each 16x16
-// output tile stages its (16+10)^2 input halo in shared memory.  The SSIM
+// (sigma 1.5) as a separable, zero-padded "same" convolution; each 32x32
+// output tile stages its (32+10)^2 input halo in shared memory.  The SSIM
 // gradient w.r.t. the rendered image is the adjoint convolution of three
 // per-pixel factor maps (dS/dmu_x, dS/dE[x^2], dS/dE[xy] times the mask
 // weight), again separable and zero padded.
@@ -17,9 +17,13 @@ using namespace gs;
 
 namespace {
 
-constexpr int LT = 16;           // output tile edge
+constexpr int LT = 32;           // output tile edge
 constexpr int R = 5;             // window radius
-constexpr int HT = LT + 2 * R;   // halo tile edge (26)
+constexpr int HT = LT + 2 * R;   // halo tile edge (42)
+constexpr int HS = 44;           // halo row stride: rows start on 16 bytes
+constexpr int SEG = 4;           // outputs per thread along each pass
+constexpr int LOSS_T = 256;      // LT columns x (LT / SEG) strips
+static_assert(LT * (LT / SEG) == LOSS_T && HS % 4 == 0 && HS >= HT, "thread layout");
 constexpr float C1 = 0.01f * 0.01f;
 constexpr float C2 = 0.03f * 0.03f;
 
@@ -62,12 +66,22 @@ __device__ __forceinline__ float block_sum(float v, float* s) {
   return t;  // valid in thread 0
 }
 
-__global__ void k_mask_count(const uint8_t* __restrict__ mask, int64_t plane, uint32_t* msum) {
+// Mask pixels per unit.  vec: the units' masks start on 16 bytes and hold a multiple of 16 (16-byte loads).
+__global__ void k_mask_count(const uint8_t* __restrict__ mask, int64_t plane, int vec, uint32_t* msum) {
   __shared__ float s[32];
   int u = blockIdx.y;
   uint32_t c = 0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < plane; k += (int64_t)gridDim.x * blockDim.x)
-    c += mask[(int64_t)u * plane + k] ? 1u : 0u;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (vec) {
+    const uint4* m4 = reinterpret_cast<const uint4*>(mask + (int64_t)u * plane);
+    auto nonzero = [](uint32_t x) { return (uint32_t)__popc(__vcmpne4(x, 0u)) >> 3; };
+    for (int64_t k = first; k < plane / 16; k += stride) {
+      const uint4 x = __ldg(m4 + k);
+      c += nonzero(x.x) + nonzero(x.y) + nonzero(x.z) + nonzero(x.w);
+    }
+  } else {
+    for (int64_t k = first; k < plane; k += stride) c += mask[(int64_t)u * plane + k] ? 1u : 0u;
+  }
   float t = block_sum((float)c, s);
   if (threadIdx.x == 0 && t > 0.f) atomicAdd(&msum[u], (uint32_t)t);
 }
@@ -96,93 +110,123 @@ __global__ void k_l1(const float* __restrict__ img, const float* __restrict__ gt
   if (threadIdx.x == 0 && t != 0.f) atomicAdd(&l1sum[u], (double)t);
 }
 
-// Separable 11-tap window over a (HT x HT) halo tile of NQ quantities held in
-// shared memory; result for output pixel (ly, lx) of each quantity.
-template <int NQ>
-__device__ __forceinline__ void conv_tile(float (*in)[HT][HT], float (*tmp)[HT][LT], float* out, int lx, int ly,
-                                          const float* c_win) {
-  // horizontal: rows 0..HT-1, output columns 0..LT-1
-  for (int k = threadIdx.x; k < HT * LT; k += blockDim.x) {
-    int r = k / LT, cx = k % LT;
-    #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      float a = 0.f;
-      #pragma unroll
-      for (int t = 0; t < 11; ++t) a += c_win[t] * in[q][r][cx + t];
-      tmp[q][r][cx] = a;
-    }
-  }
-  __syncthreads();
+// Separable 11-tap window, SEG outputs per thread along each pass: a thread
+// reads its 14 inputs once and multiplies from registers, where one output per
+// thread would read 11 values for 11 multiplications.  Taps are added in
+// ascending order from zero, one fused multiply-add each.
+__device__ __forceinline__ void taps(const float* w, const float* in, float* out) {
   #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
+  for (int e = 0; e < SEG; ++e) {
     float a = 0.f;
     #pragma unroll
-    for (int t = 0; t < 11; ++t) a += c_win[t] * tmp[q][ly + t][lx];
-    out[q] = a;
+    for (int t = 0; t < 11; ++t) a = fmaf(w[t], in[e + t], a);
+    out[e] = a;
   }
 }
+// the 16 halo values from column SEG g of a row (the 14 used and two of the row's padding)
+__device__ __forceinline__ void load_seg(const float* row, int g, float* v) {
+  #pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float4 x = reinterpret_cast<const float4*>(row + SEG * g)[q];
+    v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+  }
+}
+__device__ __forceinline__ void store_seg(float* row, int g, const float* v) {
+  reinterpret_cast<float4*>(row)[g] = make_float4(v[0], v[1], v[2], v[3]);
+}
+// vertical pass: the SEG outputs of column lx from row SEG strip of one quantity's horizontal sums
+__device__ __forceinline__ void taps_down(const float* w, const float (*tmp)[LT], int lx, int strip, float* out) {
+  float v[SEG + 10];
+  #pragma unroll
+  for (int t = 0; t < SEG + 10; ++t) v[t] = tmp[SEG * strip + t][lx];
+  taps(w, v, out);
+}
 
-// SSIM statistics, loss sums and the three factor maps.
-__global__ void __launch_bounds__(256) k_ssim_stats(const float* __restrict__ img, const float* __restrict__ gt,
-                                                    const uint8_t* __restrict__ mask, int W, int H,
-                                                    const uint32_t* __restrict__ msum, float lam, float invU,
-                                                    double* l1sum, double* ssum, float* __restrict__ fac) {
-  __shared__ float s_in[5][HT][HT];
-  __shared__ float s_tmp[5][HT][LT];
+// SSIM statistics, loss sums and the three factor maps.  Bound by fp32 issue
+// (127 multiply-adds per pixel and channel with the halo rows): 2048x2048,
+// whole mask: 272 us at one output per thread.
+__global__ void __launch_bounds__(LOSS_T) k_ssim_stats(const float* __restrict__ img, const float* __restrict__ gt,
+                                                       const uint8_t* __restrict__ mask, int W, int H,
+                                                       const uint32_t* __restrict__ msum, float lam, float invU,
+                                                       double* l1sum, double* ssum, float* __restrict__ fac) {
+  __shared__ __align__(16) float s_x[HT][HS], s_y[HT][HS];
+  __shared__ __align__(16) float s_tmp[5][HT][LT];
   __shared__ float s_red[32];
   __shared__ float s_win[11];
   int tiles_x = (W + LT - 1) / LT;
   int bx = blockIdx.x % tiles_x, by = blockIdx.x / tiles_x;
   int c = blockIdx.y, u = blockIdx.z;
   int64_t plane = (int64_t)W * H;
-  {
-    // a tile without mask pixels adds nothing to the loss and has no factor map entries
-    int qx = bx * LT + (int)(threadIdx.x % LT), qy = by * LT + (int)(threadIdx.x / LT);
-    bool m = qx < W && qy < H && mask[(int64_t)u * plane + (int64_t)qy * W + qx] != 0;
-    if (!__syncthreads_or(m)) return;
+  const int lx = threadIdx.x % LT, strip = threadIdx.x / LT;
+  const int px = bx * LT + lx, py = by * LT + SEG * strip;  // this thread's outputs: rows py .. py + SEG - 1
+  bool in[SEG], any = false;
+  #pragma unroll
+  for (int e = 0; e < SEG; ++e) {
+    in[e] = px < W && py + e < H && mask[(int64_t)u * plane + (int64_t)(py + e) * W + px] != 0;
+    any = any || in[e];
   }
+  // a tile without mask pixels adds nothing to the loss and has no factor map entries
+  if (!__syncthreads_or(any)) return;
   load_window(s_win);
   const float* X = img + ((int64_t)u * 3 + c) * plane;
   const float* Y = gt + ((int64_t)u * 3 + c) * plane;
-  int x0 = bx * LT - R, y0 = by * LT - R;
-  for (int k = threadIdx.x; k < HT * HT; k += blockDim.x) {
-    int r = k / HT, q = k % HT;
+  const int x0 = bx * LT - R, y0 = by * LT - R;
+  for (int k = threadIdx.x; k < HT * HS; k += LOSS_T) {
+    int r = k / HS, q = k % HS;
     int gx = x0 + q, gy = y0 + r;
     float a = 0.f, b = 0.f;
-    if (gx >= 0 && gx < W && gy >= 0 && gy < H) { a = X[(int64_t)gy * W + gx]; b = Y[(int64_t)gy * W + gx]; }
-    s_in[0][r][q] = a; s_in[1][r][q] = b; s_in[2][r][q] = a * a; s_in[3][r][q] = b * b; s_in[4][r][q] = a * b;
+    if (q < HT && gx >= 0 && gx < W && gy >= 0 && gy < H) { a = X[(int64_t)gy * W + gx]; b = Y[(int64_t)gy * W + gx]; }
+    s_x[r][q] = a; s_y[r][q] = b;
   }
   __syncthreads();
-  int lx = threadIdx.x % LT, ly = threadIdx.x / LT;
-  float st[5];
-  conv_tile<5>(s_in, s_tmp, st, lx, ly, s_win);
-  int px = bx * LT + lx, py = by * LT + ly;
+  float w[11];
+  #pragma unroll
+  for (int t = 0; t < 11; ++t) w[t] = s_win[t];
+  for (int k = threadIdx.x; k < HT * (LT / SEG); k += LOSS_T) {
+    const int r = k / (LT / SEG), g = k % (LT / SEG);
+    float a[16], b[16], p[16], o[SEG];
+    load_seg(s_x[r], g, a);
+    load_seg(s_y[r], g, b);
+    taps(w, a, o); store_seg(s_tmp[0][r], g, o);
+    taps(w, b, o); store_seg(s_tmp[1][r], g, o);
+    #pragma unroll
+    for (int t = 0; t < SEG + 10; ++t) p[t] = __fmul_rn(a[t], a[t]);
+    taps(w, p, o); store_seg(s_tmp[2][r], g, o);
+    #pragma unroll
+    for (int t = 0; t < SEG + 10; ++t) p[t] = __fmul_rn(b[t], b[t]);
+    taps(w, p, o); store_seg(s_tmp[3][r], g, o);
+    #pragma unroll
+    for (int t = 0; t < SEG + 10; ++t) p[t] = __fmul_rn(a[t], b[t]);
+    taps(w, p, o); store_seg(s_tmp[4][r], g, o);
+  }
+  __syncthreads();
+  float st[5][SEG];
+  #pragma unroll
+  for (int q = 0; q < 5; ++q) taps_down(w, s_tmp[q], lx, strip, st[q]);
   float nm = (float)msum[u];
   float sacc = 0.f, lacc = 0.f;
-  if (px < W && py < H) {
-    int64_t pix = (int64_t)py * W + px;
-    bool in = mask[(int64_t)u * plane + pix] != 0;
+  #pragma unroll
+  for (int e = 0; e < SEG; ++e) {
+    if (!in[e]) continue;  // the factor maps are zero off the mask; only mask pixels are stored and read
     float fmu = 0.f, fxx = 0.f, fxy = 0.f;
-    if (in && nm > 0.f) {
-      float ux = st[0], uy = st[1];
-      float vx = st[2] - ux * ux, vy = st[3] - uy * uy, cxy = st[4] - ux * uy;
+    if (nm > 0.f) {
+      float ux = st[0][e], uy = st[1][e];
+      float vx = st[2][e] - ux * ux, vy = st[3][e] - uy * uy, cxy = st[4][e] - ux * uy;
       float A1 = 2.f * ux * uy + C1, A2 = 2.f * cxy + C2;
       float B1 = ux * ux + uy * uy + C1, B2 = vx + vy + C2;
       float S = (A1 * A2) / (B1 * B2);
-      sacc = S;
-      lacc = fabsf(X[pix] - Y[pix]);
+      sacc += S;
+      lacc += fabsf(s_x[SEG * strip + e + R][lx + R] - s_y[SEG * strip + e + R][lx + R]);
       float wp = -lam * invU / (3.f * nm);  // d loss / d S_p
       fmu = wp * S * (2.f * uy / A1 - 2.f * ux / B1 - 2.f * uy / A2 + 2.f * ux / B2);
       fxx = wp * S * (-1.f / B2);
       fxy = wp * S * (2.f / A2);
     }
-    if (in) {  // the factor maps are zero off the mask; only mask pixels are stored and read
-      int64_t base = ((int64_t)u * 3 + c) * plane + pix;
-      int64_t fs = (int64_t)3 * plane * gridDim.z;  // stride between the three factor maps
-      fac[base] = fmu;
-      fac[fs + base] = fxx;
-      fac[2 * fs + base] = fxy;
-    }
+    int64_t base = ((int64_t)u * 3 + c) * plane + (int64_t)(py + e) * W + px;
+    int64_t fs = (int64_t)3 * plane * gridDim.z;  // stride between the three factor maps
+    fac[base] = fmu;
+    fac[fs + base] = fxx;
+    fac[2 * fs + base] = fxy;
   }
   float ts = block_sum(sacc, s_red);
   if (threadIdx.x == 0 && ts != 0.f) atomicAdd(&ssum[u], (double)ts);
@@ -190,13 +234,15 @@ __global__ void __launch_bounds__(256) k_ssim_stats(const float* __restrict__ im
   if (threadIdx.x == 0 && tl != 0.f) atomicAdd(&l1sum[u], (double)tl);
 }
 
-// dL/dimg = L1 part + conv(fmu) + 2 x conv(fxx) + y conv(fxy)
-__global__ void __launch_bounds__(256) k_ssim_grad(const float* __restrict__ img, const float* __restrict__ gt,
-                                                   const uint8_t* __restrict__ mask, int W, int H,
-                                                   const uint32_t* __restrict__ msum, float w1, float invU,
-                                                   const float* __restrict__ fac, float* __restrict__ dimg) {
-  __shared__ float s_in[3][HT][HT];
-  __shared__ float s_tmp[3][HT][LT];
+// dL/dimg = L1 part + conv(fmu) + 2 x conv(fxx) + y conv(fxy).  76
+// multiply-adds per pixel and channel; 2048x2048, whole mask: 230 us at one
+// output per thread.
+__global__ void __launch_bounds__(LOSS_T) k_ssim_grad(const float* __restrict__ img, const float* __restrict__ gt,
+                                                      const uint8_t* __restrict__ mask, int W, int H,
+                                                      const uint32_t* __restrict__ msum, float w1, float invU,
+                                                      const float* __restrict__ fac, float* __restrict__ dimg) {
+  __shared__ __align__(16) float s_in[3][HT][HS];
+  __shared__ __align__(16) float s_tmp[3][HT][LT];
   __shared__ float s_win[11];
   int tiles_x = (W + LT - 1) / LT;
   int bx = blockIdx.x % tiles_x, by = blockIdx.x / tiles_x;
@@ -204,14 +250,17 @@ __global__ void __launch_bounds__(256) k_ssim_grad(const float* __restrict__ img
   int64_t plane = (int64_t)W * H;
   int64_t off = ((int64_t)u * 3 + c) * plane;
   int64_t fs = (int64_t)3 * plane * gridDim.z;
-  int x0 = bx * LT - R, y0 = by * LT - R;
+  const int x0 = bx * LT - R, y0 = by * LT - R;
+  const int lx = threadIdx.x % LT, strip = threadIdx.x / LT;
+  const int px = bx * LT + lx, py = by * LT + SEG * strip;
   // factor maps are nonzero only at mask pixels: read them there, zero elsewhere
   bool any = false;
-  for (int k = threadIdx.x; k < HT * HT; k += blockDim.x) {
-    int r = k / HT, q = k % HT;
+  for (int k = threadIdx.x; k < HT * HS; k += LOSS_T) {
+    int r = k / HS, q = k % HS;
     int gx = x0 + q, gy = y0 + r;
     float a = 0.f, b = 0.f, d = 0.f;
-    if (gx >= 0 && gx < W && gy >= 0 && gy < H && mask[(int64_t)u * plane + (int64_t)gy * W + gx] != 0) {
+    if (q < HT && gx >= 0 && gx < W && gy >= 0 && gy < H &&
+        mask[(int64_t)u * plane + (int64_t)gy * W + gx] != 0) {
       int64_t pix = off + (int64_t)gy * W + gx;
       a = fac[pix]; b = fac[fs + pix]; d = fac[2 * fs + pix];
       any = true;
@@ -220,32 +269,49 @@ __global__ void __launch_bounds__(256) k_ssim_grad(const float* __restrict__ img
   }
   if (!__syncthreads_or(any)) {
     // no mask pixel within the window's reach: both gradient terms vanish
-    int px = bx * LT + (int)(threadIdx.x % LT), py = by * LT + (int)(threadIdx.x / LT);
-    if (px < W && py < H) dimg[off + (int64_t)py * W + px] = 0.f;
+    #pragma unroll
+    for (int e = 0; e < SEG; ++e)
+      if (px < W && py + e < H) dimg[off + (int64_t)(py + e) * W + px] = 0.f;
     return;
   }
   load_window(s_win);
   __syncthreads();
-  int lx = threadIdx.x % LT, ly = threadIdx.x / LT;
-  float cv[3];
-  conv_tile<3>(s_in, s_tmp, cv, lx, ly, s_win);
-  int px = bx * LT + lx, py = by * LT + ly;
-  if (px < W && py < H) {
-    int64_t pix = (int64_t)py * W + px;
+  float w[11];
+  #pragma unroll
+  for (int t = 0; t < 11; ++t) w[t] = s_win[t];
+  for (int k = threadIdx.x; k < HT * (LT / SEG); k += LOSS_T) {
+    const int r = k / (LT / SEG), g = k % (LT / SEG);
+    #pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      float a[16], o[SEG];
+      load_seg(s_in[q][r], g, a);
+      taps(w, a, o);
+      store_seg(s_tmp[q][r], g, o);
+    }
+  }
+  __syncthreads();
+  float cv[3][SEG];
+  #pragma unroll
+  for (int q = 0; q < 3; ++q) taps_down(w, s_tmp[q], lx, strip, cv[q]);
+  float nm = (float)msum[u];
+  #pragma unroll
+  for (int e = 0; e < SEG; ++e) {
+    if (!(px < W && py + e < H)) continue;
+    int64_t pix = (int64_t)(py + e) * W + px;
     float x = img[off + pix], y = gt[off + pix];
-    float nm = (float)msum[u];
     bool in = mask[(int64_t)u * plane + pix] != 0;
     float d = x - y;
     float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
     float gl1 = (in && nm > 0.f) ? w1 * invU / (3.f * nm) * sg : 0.f;
-    dimg[off + pix] = gl1 + cv[0] + 2.f * x * cv[1] + y * cv[2];
+    dimg[off + pix] = gl1 + cv[0][e] + 2.f * x * cv[1][e] + y * cv[2][e];
   }
 }
 
-__global__ void k_loss_final(const uint32_t* msum, const double* l1sum, const double* ssum, int U, float lam,
-                             float* out) {
+// the units' losses, one per lane (a thread summing them alone waits for each unit's loads in turn)
+__global__ void __launch_bounds__(32) k_loss_final(const uint32_t* msum, const double* l1sum, const double* ssum, int U,
+                                                   float lam, float* out) {
   double acc = 0.0;
-  for (int u = 0; u < U; ++u) {
+  for (int u = threadIdx.x; u < U; u += 32) {
     double nm = (double)msum[u];
     if (nm <= 0.0) continue;
     double l1 = l1sum[u] / (3.0 * nm);
@@ -253,7 +319,9 @@ __global__ void k_loss_final(const uint32_t* msum, const double* l1sum, const do
     if (lam > 0.f) v += lam * (1.0 - ssum[u] / (3.0 * nm));
     acc += v;
   }
-  *out = (float)(acc / U);
+  #pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (threadIdx.x == 0) *out = (float)(acc / U);
 }
 
 // Background-opacity penalty (variant of the mask): per unit, the number of pixels outside the mask
@@ -352,16 +420,17 @@ GS_API int gs_loss(const float* img, const float* gt, const uint8_t* mask, int n
   float invU = 1.f / n_units;
   int gx = (int)((plane + 255) / 256);
   if (gx > 1024) gx = 1024;
-  k_mask_count<<<dim3(gx, n_units), 256, 0, s>>>(mask, plane, msum);
+  const int vec = ((uintptr_t)mask & 15u) == 0 && plane % 16 == 0;
+  k_mask_count<<<dim3(gx, n_units), 256, 0, s>>>(mask, plane, vec, msum);
   if (lambda_ssim == 0.f) {
     k_l1<<<dim3(gx, n_units), 256, 0, s>>>(img, gt, mask, plane, msum, 1.f, invU, l1, dL_dimg);
   } else {
     int tiles = ((width + LT - 1) / LT) * ((height + LT - 1) / LT);
     dim3 grid(tiles, 3, n_units);
-    k_ssim_stats<<<grid, 256, 0, s>>>(img, gt, mask, width, height, msum, lambda_ssim, invU, l1, ss, fac);
-    k_ssim_grad<<<grid, 256, 0, s>>>(img, gt, mask, width, height, msum, 1.f - lambda_ssim, invU, fac, dL_dimg);
+    k_ssim_stats<<<grid, LOSS_T, 0, s>>>(img, gt, mask, width, height, msum, lambda_ssim, invU, l1, ss, fac);
+    k_ssim_grad<<<grid, LOSS_T, 0, s>>>(img, gt, mask, width, height, msum, 1.f - lambda_ssim, invU, fac, dL_dimg);
   }
-  k_loss_final<<<1, 1, 0, s>>>(msum, l1, ss, n_units, lambda_ssim, d_loss);
+  k_loss_final<<<1, 32, 0, s>>>(msum, l1, ss, n_units, lambda_ssim, d_loss);
   return gs_check_launch();
 }
 
