@@ -2,12 +2,19 @@
 // uniform grid.  Their distances give the plain initial scale (mean 3-NN
 // distance) and, with k = 16, the geometry features of the learned initialiser.
 //
-// Build: count points per cell, exclusive scan, scatter the points (as float4
-// with the index in .w) into cell order.  Query: one thread per point keeps
-// the k best (squared distance, index) pairs in registers and visits cubic
-// shells of cells of growing radius R until the k-th best distance is no
-// larger than the distance from the point to the outside of the searched cube.
-// Ties in distance are broken by the smaller index, so the result is unique.
+// Build: count points per cell (each point keeping its rank in its cell),
+// exclusive scan, scatter the points (as float4 with the index in .w) into cell
+// order.  Query: one thread per point, taken in cell order so that a warp's
+// points search the same cells; the cells of one (z, y) row are consecutive, so
+// a run of them is one range of the sorted points.  Cubes of cells of growing
+// radius R are searched, rows that lie farther than the k-th best skipped,
+// until the k-th best distance is smaller than the distance from the point to
+// the outside of the cube.  A first search keeps the k smallest squared
+// distances alone, in registers (two min / max per slot and candidate, where
+// (distance, index) pairs would cost compares and selects); a second one over
+// the same rows collects the points within the k-th distance, and one sort
+// orders them.  Ties in distance are broken by the smaller index, so the result
+// is unique.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -24,20 +31,19 @@ struct Grid {
   float lo[3];
   float h, inv_h;
   int dim[3];
+  float slack;  // bounds the rounding of cell boundaries and of the points' cells
 };
 
 struct KnnWs {
-  size_t count, start, cursor, scan, sorted, total_cnt, total;
+  size_t start, rank, scan, sorted, total;
 };
 KnnWs knn_ws(int64_t n, int64_t cells) {
   KnnWs L;
   size_t o = 0;
-  L.count = o; o += a256(sizeof(uint32_t) * (size_t)cells);
   L.start = o; o += a256(sizeof(uint32_t) * (size_t)(cells + 1));
-  L.cursor = o; o += a256(sizeof(uint32_t) * (size_t)cells);
+  L.rank = o; o += a256(sizeof(uint32_t) * (size_t)(n > 0 ? n : 1));
   L.scan = o; o += a256(gs_scan_ws_bytes(cells));
   L.sorted = o; o += a256(sizeof(float4) * (size_t)(n > 0 ? n : 1));
-  L.total_cnt = o; o += a256(sizeof(uint32_t));
   L.total = o;
   return L;
 }
@@ -47,84 +53,106 @@ __device__ __forceinline__ int cell_coord(float x, float lo, float inv_h, int di
   return min(max(c, 0), dim - 1);
 }
 
-__global__ void k_cell_count(const float* __restrict__ pts, int64_t n, Grid g, uint32_t* __restrict__ count) {
+__device__ __forceinline__ int64_t cell_of(const Grid& g, float x, float y, float z) {
+  const int cx = cell_coord(x, g.lo[0], g.inv_h, g.dim[0]);
+  const int cy = cell_coord(y, g.lo[1], g.inv_h, g.dim[1]);
+  const int cz = cell_coord(z, g.lo[2], g.inv_h, g.dim[2]);
+  return ((int64_t)cz * g.dim[1] + cy) * g.dim[0] + cx;
+}
+
+__global__ void k_cell_count(const float* __restrict__ pts, int64_t n, Grid g, uint32_t* __restrict__ count,
+                             uint32_t* __restrict__ rank) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
-  int cx = cell_coord(pts[3 * i], g.lo[0], g.inv_h, g.dim[0]);
-  int cy = cell_coord(pts[3 * i + 1], g.lo[1], g.inv_h, g.dim[1]);
-  int cz = cell_coord(pts[3 * i + 2], g.lo[2], g.inv_h, g.dim[2]);
-  atomicAdd(&count[((int64_t)cz * g.dim[1] + cy) * g.dim[0] + cx], 1u);
+  rank[i] = atomicAdd(&count[cell_of(g, pts[3 * i], pts[3 * i + 1], pts[3 * i + 2])], 1u);
 }
 
 __global__ void k_cell_scatter(const float* __restrict__ pts, int64_t n, Grid g, const uint32_t* __restrict__ start,
-                               uint32_t* __restrict__ cursor, float4* __restrict__ sorted) {
+                               const uint32_t* __restrict__ rank, float4* __restrict__ sorted) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
-  int cx = cell_coord(x, g.lo[0], g.inv_h, g.dim[0]);
-  int cy = cell_coord(y, g.lo[1], g.inv_h, g.dim[1]);
-  int cz = cell_coord(z, g.lo[2], g.inv_h, g.dim[2]);
-  int64_t c = ((int64_t)cz * g.dim[1] + cy) * g.dim[0] + cx;
-  uint32_t pos = start[c] + atomicAdd(&cursor[c], 1u);
-  sorted[pos] = make_float4(x, y, z, __int_as_float((int)i));
+  sorted[start[cell_of(g, x, y, z)] + rank[i]] = make_float4(x, y, z, __int_as_float((int)i));
 }
 
-template <int K>
-__device__ __forceinline__ void offer(float d, int j, float* bd, int* bi) {
-  if (d > bd[K - 1] || (d == bd[K - 1] && j > bi[K - 1])) return;
-  float cd = d;
-  int ci = j;
-  #pragma unroll
-  for (int q = 0; q < K; ++q) {
-    bool less = cd < bd[q] || (cd == bd[q] && ci < bi[q]);
-    if (less) {
-      float td = bd[q]; bd[q] = cd; cd = td;
-      int ti = bi[q]; bi[q] = ci; ci = ti;
+// squared distance, one rounding order for both searches
+__device__ __forceinline__ float dist2(float4 a, float4 b) {
+  const float ex = a.x - b.x, ey = a.y - b.y, ez = a.z - b.z;
+  return __fmaf_rn(ez, ez, __fmaf_rn(ey, ey, __fmul_rn(ex, ex)));
+}
+
+// distance along one axis from p to cells c + lo .. c + hi (0 inside)
+__device__ __forceinline__ float axis_gap(float p, float lo, const Grid& g, int c0, int c1) {
+  return fmaxf(0.f, fmaxf(lo + (float)c0 * g.h - p, p - (lo + (float)(c1 + 1) * g.h)) - g.slack);
+}
+
+// Calls f(point) for the points of the cells that cube radius R adds to radius
+// R - 1 (all of the cube when `whole`), except runs of cells farther from p
+// than the squared distance limit().
+template <typename F, typename L>
+__device__ __forceinline__ void visit(const Grid& g, const uint32_t* __restrict__ start,
+                                      const float4* __restrict__ sorted, const int* c, const float* p, int R,
+                                      bool whole, L limit, F f) {
+  auto run = [&](int64_t row, float d2yz, int xa, int xb) {
+    xa = max(xa, 0);
+    xb = min(xb, g.dim[0] - 1);
+    if (xa > xb) return;
+    const float gx = axis_gap(p[0], g.lo[0], g, xa, xb);
+    if ((d2yz + gx * gx) * 0.999f > limit()) return;
+    const uint32_t e = start[row + xb + 1];
+    for (uint32_t q = start[row + xa]; q < e; ++q) f(sorted[q]);
+  };
+  for (int dz = -R; dz <= R; ++dz) {
+    const int z = c[2] + dz;
+    if (z < 0 || z >= g.dim[2]) continue;
+    const float gz = axis_gap(p[2], g.lo[2], g, z, z);
+    for (int dy = -R; dy <= R; ++dy) {
+      const int y = c[1] + dy;
+      if (y < 0 || y >= g.dim[1]) continue;
+      const float gy = axis_gap(p[1], g.lo[1], g, y, y);
+      const float d2 = gz * gz + gy * gy;
+      const int64_t row = ((int64_t)z * g.dim[1] + y) * g.dim[0];
+      if (whole || dz == -R || dz == R || dy == -R || dy == R) {
+        run(row, d2, c[0] - R, c[0] + R);
+      } else {
+        run(row, d2, c[0] - R, c[0] - R);
+        run(row, d2, c[0] + R, c[0] + R);
+      }
     }
   }
 }
 
+// 1M points of an interface, k = 16: 1721 us with sorted (distance, index)
+// insertions, cells visited one by one and points in input order.
+constexpr int KNN_T = 128;
 template <int K>
-__global__ void __launch_bounds__(128) k_knn_query(const float* __restrict__ pts, int64_t n, Grid g,
-                                                   const uint32_t* __restrict__ start,
-                                                   const float4* __restrict__ sorted, int* __restrict__ out_idx,
-                                                   float* __restrict__ out_dist) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float px = pts[3 * i], py = pts[3 * i + 1], pz = pts[3 * i + 2];
-  int c[3] = {cell_coord(px, g.lo[0], g.inv_h, g.dim[0]), cell_coord(py, g.lo[1], g.inv_h, g.dim[1]),
-              cell_coord(pz, g.lo[2], g.inv_h, g.dim[2])};
-  float bd[K];
-  int bi[K];
+__global__ void __launch_bounds__(KNN_T) k_knn_query(int64_t n, Grid g, const uint32_t* __restrict__ start,
+                                                     const float4* __restrict__ sorted, int vec,
+                                                     int* __restrict__ out_idx, float* __restrict__ out_dist) {
+  __shared__ unsigned long long s_best[K][KNN_T];
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const float4 me = sorted[t];
+  const int i = __float_as_int(me.w);
+  const float p[3] = {me.x, me.y, me.z};
+  int c[3];
   #pragma unroll
-  for (int q = 0; q < K; ++q) { bd[q] = INFINITY; bi[q] = 0x7fffffff; }
-  int maxdim = max(g.dim[0], max(g.dim[1], g.dim[2]));
-  float p[3] = {px, py, pz};
-  for (int R = 0; R <= maxdim; ++R) {
-    for (int dz = -R; dz <= R; ++dz) {
-      int z = c[2] + dz;
-      if (z < 0 || z >= g.dim[2]) continue;
-      for (int dy = -R; dy <= R; ++dy) {
-        int y = c[1] + dy;
-        if (y < 0 || y >= g.dim[1]) continue;
-        bool face = (dz == -R || dz == R || dy == -R || dy == R);
-        for (int dx = -R; dx <= R; dx += (face ? 1 : 2 * R)) {
-          int x = c[0] + dx;
-          if (x >= 0 && x < g.dim[0]) {
-            int64_t cell = ((int64_t)z * g.dim[1] + y) * g.dim[0] + x;
-            uint32_t s = start[cell], e = start[cell + 1];
-            for (uint32_t q = s; q < e; ++q) {
-              float4 o = sorted[q];
-              int j = __float_as_int(o.w);
-              if (j == (int)i) continue;
-              float ex = o.x - px, ey = o.y - py, ez = o.z - pz;
-              offer<K>(ex * ex + ey * ey + ez * ez, j, bd, bi);
-            }
-          }
-          if (R == 0) break;
-        }
+  for (int a = 0; a < 3; ++a) c[a] = cell_coord(p[a], g.lo[a], g.inv_h, g.dim[a]);
+  float b[K];  // the K smallest squared distances so far, ascending
+  #pragma unroll
+  for (int q = 0; q < K; ++q) b[q] = INFINITY;
+  auto kth = [&]() { return b[K - 1]; };
+  const int maxdim = max(g.dim[0], max(g.dim[1], g.dim[2]));
+  int R = 1;
+  for (;; ++R) {
+    visit(g, start, sorted, c, p, R, R == 1, kth, [&](float4 o) {
+      const float d = dist2(o, me);
+      if (d < b[K - 1] && __float_as_int(o.w) != i) {
+        #pragma unroll
+        for (int q = K - 1; q > 0; --q) b[q] = fminf(b[q], fmaxf(b[q - 1], d));
+        b[0] = fminf(b[0], d);
       }
-    }
+    });
     // distance from p to the outside of the searched cube of cells
     float guard = INFINITY;
     bool whole = true;
@@ -135,15 +163,79 @@ __global__ void __launch_bounds__(128) k_knn_query(const float* __restrict__ pts
       if (hi < g.dim[a] - 1) guard = fminf(guard, (g.lo[a] + (hi + 1) * g.h) - p[a]);
       whole = whole && lo <= 0 && hi >= g.dim[a] - 1;
     }
-    if (whole) break;
     // the k-th best must be strictly inside: a point outside the cube is at least `guard` away
-    if (bd[K - 1] < guard * guard * 0.999f) break;
+    if (whole || R >= maxdim || b[K - 1] < guard * guard * 0.999f) break;
   }
+  // the points within the k-th distance: `below` nearer ones, and the smallest indices at it in the other slots
+  const float last = b[K - 1];
+  int below = 0;
+  #pragma unroll
+  for (int q = 0; q < K; ++q) below += b[q] < last ? 1 : 0;
+  #pragma unroll
+  for (int q = 0; q < K; ++q) s_best[q][threadIdx.x] = ~0ull;
+  int n1 = 0, n2 = 0;
+  visit(g, start, sorted, c, p, R, true, kth, [&](float4 o) {
+    const float d = dist2(o, me);
+    const int j = __float_as_int(o.w);
+    if (!(d <= last) || j == i) return;
+    const unsigned long long key = ((unsigned long long)__float_as_uint(d) << 32) | (uint32_t)j;
+    if (d < last) {
+      if (n1 < K) s_best[n1++][threadIdx.x] = key;
+    } else if (below + n2 < K) {
+      s_best[below + n2++][threadIdx.x] = key;
+    } else {  // more ties than slots: replace the largest index held
+      int w = below;
+      for (int q = below + 1; q < K; ++q)
+        if (s_best[q][threadIdx.x] > s_best[w][threadIdx.x]) w = q;
+      if (w < K && key < s_best[w][threadIdx.x]) s_best[w][threadIdx.x] = key;
+    }
+  });
+  // ascending (distance, index): odd-even transposition for K = 3, a bitonic network otherwise
+  unsigned long long v[K];
+  #pragma unroll
+  for (int q = 0; q < K; ++q) v[q] = s_best[q][threadIdx.x];
+  auto order = [&](unsigned long long& x, unsigned long long& y) {
+    const bool sw = y < x;
+    const unsigned long long lo = sw ? y : x, hi = sw ? x : y;
+    x = lo; y = hi;
+  };
+  if ((K & (K - 1)) != 0) {
+    #pragma unroll
+    for (int r = 0; r < K; ++r)
+      #pragma unroll
+      for (int q = r & 1; q + 1 < K; q += 2) order(v[q], v[q + 1]);
+  } else {
+    #pragma unroll
+    for (int k = 2; k <= K; k *= 2)
+      #pragma unroll
+      for (int j = k / 2; j > 0; j /= 2)
+        #pragma unroll
+        for (int q = 0; q < K; ++q) {
+          const int o = q ^ j;
+          if (o > q) {
+            if ((q & k) == 0) order(v[q], v[o]); else order(v[o], v[q]);
+          }
+        }
+  }
+  int ri[K];
+  float rd[K];
   #pragma unroll
   for (int q = 0; q < K; ++q) {
-    bool ok = bd[q] < INFINITY;
-    out_idx[i * K + q] = ok ? bi[q] : -1;
-    out_dist[i * K + q] = ok ? sqrtf(bd[q]) : INFINITY;
+    const bool ok = v[q] != ~0ull;
+    ri[q] = ok ? (int)(uint32_t)v[q] : -1;
+    rd[q] = ok ? sqrtf(__uint_as_float((uint32_t)(v[q] >> 32))) : INFINITY;
+  }
+  int* oi = out_idx + (int64_t)i * K;
+  float* od = out_dist + (int64_t)i * K;
+  if (K % 4 == 0 && vec) {
+    #pragma unroll
+    for (int q = 0; q + 3 < K; q += 4) {
+      reinterpret_cast<int4*>(oi)[q / 4] = make_int4(ri[q], ri[q + 1], ri[q + 2], ri[q + 3]);
+      reinterpret_cast<float4*>(od)[q / 4] = make_float4(rd[q], rd[q + 1], rd[q + 2], rd[q + 3]);
+    }
+  } else {
+    #pragma unroll
+    for (int q = 0; q < K; ++q) { oi[q] = ri[q]; od[q] = rd[q]; }
   }
 }
 
@@ -170,6 +262,8 @@ GS_API int gs_knn(const float* points, int64_t n, int k, const float* grid_lo, f
   }
   g.h = cell_size;
   g.inv_h = 1.0f / cell_size;
+  g.slack = 0.f;
+  for (int a = 0; a < 3; ++a) g.slack = fmaxf(g.slack, 1e-6f * (fabsf(g.lo[a]) + (float)g.dim[a] * cell_size));
   int64_t cells = (int64_t)g.dim[0] * g.dim[1] * g.dim[2];
   if (cells >= (int64_t)UINT32_MAX) return GS_ERR_INVALID;
   KnnWs L = knn_ws(n, cells);
@@ -177,21 +271,19 @@ GS_API int gs_knn(const float* points, int64_t n, int k, const float* grid_lo, f
   if (n == 0) return GS_OK;
   cudaStream_t s = (cudaStream_t)stream;
   char* ws = (char*)workspace;
-  uint32_t* count = (uint32_t*)(ws + L.count);
   uint32_t* start = (uint32_t*)(ws + L.start);
-  uint32_t* cursor = (uint32_t*)(ws + L.cursor);
+  uint32_t* rank = (uint32_t*)(ws + L.rank);
   float4* sorted = (float4*)(ws + L.sorted);
-  if (cudaMemsetAsync(count, 0, sizeof(uint32_t) * cells, s) != cudaSuccess ||
-      cudaMemsetAsync(cursor, 0, sizeof(uint32_t) * cells, s) != cudaSuccess)
-    return GS_ERR_CUDA;
+  if (cudaMemsetAsync(start, 0, sizeof(uint32_t) * cells, s) != cudaSuccess) return GS_ERR_CUDA;
   unsigned nb = (unsigned)((n + 255) / 256);
-  k_cell_count<<<nb, 256, 0, s>>>(points, n, g, count);
-  // start[c] = exclusive prefix; start[cells] = n
-  int r = gs_scan_u32(count, start, cells, ws + L.scan, start + cells, s);
+  k_cell_count<<<nb, 256, 0, s>>>(points, n, g, start, rank);
+  // start[c] = exclusive prefix (in place); start[cells] = n
+  int r = gs_scan_u32(start, start, cells, ws + L.scan, start + cells, s);
   if (r != GS_OK) return r;
-  k_cell_scatter<<<nb, 256, 0, s>>>(points, n, g, start, cursor, sorted);
-  unsigned qb = (unsigned)((n + 127) / 128);
-#define GS_KQ(K) k_knn_query<K><<<qb, 128, 0, s>>>(points, n, g, start, sorted, idx, dist)
+  k_cell_scatter<<<nb, 256, 0, s>>>(points, n, g, start, rank, sorted);
+  unsigned qb = (unsigned)((n + KNN_T - 1) / KNN_T);
+  const int vec = (((uintptr_t)idx | (uintptr_t)dist) & 15u) == 0;
+#define GS_KQ(K) k_knn_query<K><<<qb, KNN_T, 0, s>>>(n, g, start, sorted, vec, idx, dist)
   switch (k) {
     case 3: GS_KQ(3); break;
     case 8: GS_KQ(8); break;
