@@ -877,9 +877,15 @@ static int depth_first_sort(const UnitTable& U, int64_t P, const gs_proj* proj, 
   return gs_check_launch();
 }
 
+bool gs_small_sort_applies(const UnitTable& U, int64_t P, int n_tiles);
+size_t gs_small_sort_ctrl_words();
+int gs_small_sort(const UnitTable& U, const gs_proj* proj, int width, int height, int64_t cap, uint32_t* rec,
+                  uint2* rect, uint32_t* count, void* ctrl_ws, uint32_t* sorted_vals, uint32_t* ranges,
+                  uint32_t* d_num_instances, const gs_schedule* sched, int* d_status, cudaStream_t s);
+
 // method 0: the global LSD radix sort of (unit | tile | depth) keys; 1: the bucketed sort (sort_seg.cu);
-// 2: the depth-first design (falls back to 0 when unit | tile needs more than 16 bits).  All give the
-// same lists, ranges and masks.
+// 2: the small design (sort_small.cu) where it applies, else the depth-first design (falls back to 0 when
+// unit | tile needs more than 16 bits).  All give the same lists, ranges and masks.
 int gs_bin_sort_impl(const gs_proj* proj, const gs_units* units, int width, int height, int64_t max_instances,
                      void* workspace, size_t workspace_bytes, uint32_t* sorted_vals, uint32_t* ranges,
                      uint32_t* d_num_instances, const gs_schedule* sched, int* d_status, cudaStream_t s,
@@ -919,6 +925,12 @@ int gs_bin_sort_impl(const gs_proj* proj, const gs_units* units, int width, int 
   int64_t stride = ((max_instances > P ? max_instances : P) + RS_TILE - 1) / RS_TILE;
   if (stride < 1) stride = 1;
 
+  // its buffers: rectangles and records in the key buffers (8 bytes per record each), list lengths in the digit
+  // totals (4096 words), control words in the schedule's scan scratch (over 4000 words)
+  static_assert(RS_BINS_MAX * MAX_PASSES >= 4096 && MAX_SCHED_TILES / SCAN_BLOCK > 1024, "small sort's scratch");
+  if (method == 2 && P > 0 && max_instances > 0 && gs_small_sort_applies(U, P, n_tiles))
+    return gs_small_sort(U, proj, width, height, max_instances, (uint32_t*)k1, (uint2*)k0, totals, ws + L.jscan,
+                         sorted_vals, ranges, d_num_instances, sched, d_status, s);
   if (cudaMemsetAsync(ranges, 0, sizeof(uint32_t) * 2 * (size_t)n_tiles * U.n, s) != cudaSuccess ||
       cudaMemsetAsync(totals, 0, sizeof(uint32_t) * RS_BINS_MAX * MAX_PASSES, s) != cudaSuccess ||
       cudaMemsetAsync(cur, 0, sizeof(int32_t) * 2 * (MAX_PASSES + 1), s) != cudaSuccess ||

@@ -1,0 +1,167 @@
+"""Sizes at which the tiled kernels can go wrong: partial batches, tiles and rows, ties, unaligned arrays (GPU)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from paper_2509_12138_gb300 import Frame, Units
+from paper_2509_12138_gb300 import init as gi
+
+pytestmark = pytest.mark.gpu
+
+
+def _points(n, seed):
+    pts, nrm, _ = synth.interface_points(n, 8, seed)
+    p, m = torch.from_numpy(pts).cuda(), torch.from_numpy(nrm).cuda()
+    return (p, m) + gi.knn(p, 16)
+
+
+def _weights(seed):
+    w = gi.init_weights(seed)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    w[7168 + 64 + 4096 + 64:-8] = 0.1 * torch.randn(512, generator=g, device="cuda")
+    return w
+
+
+def _off_by_one(t):
+    """The same rows in storage that starts 4 bytes past a 16-byte boundary."""
+    s = torch.empty(t.numel() + 1, dtype=t.dtype, device=t.device)
+    v = s[1:].view(t.shape)
+    v.copy_(t)
+    return v
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 300])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_mlp_forward_partial_batches(n, aligned):
+    """A point's outputs and features do not depend on the points behind it, nor on how its rows are aligned."""
+    p, m, idx, dist = _points(700, 1)
+    w = _weights(2)
+    full, feat = gi.mlp_forward(w, p, m, idx, dist), gi.mlp_features(p, m, idx, dist)
+    # neighbours may lie past the first n points: the point arrays stay whole, the rows end at n
+    i, d = (idx[:n], dist[:n]) if aligned else (_off_by_one(idx[:n]), _off_by_one(dist[:n]))
+    L = gi._lib.load()
+    out = torch.empty((n, 8), device="cuda")
+    gi.check(L.gs_mlp_forward(gi._ptr(p), gi._ptr(m), gi._ptr(i), gi._ptr(d), n, gi._ptr(w), gi._ptr(out),
+                              gi._stream()), "gs_mlp_forward")
+    x = torch.empty((n, 112), dtype=torch.int16, device="cuda")
+    gi.check(L.gs_mlp_features(gi._ptr(p), gi._ptr(m), gi._ptr(i), gi._ptr(d), n, gi._ptr(x), gi._stream()),
+             "gs_mlp_features")
+    assert torch.equal(out, full[:n]) and torch.equal(x, feat[:n])
+
+
+@pytest.mark.parametrize("n,aligned", [(1, True), (127, True), (129, False), (128 * 152 + 3, True)])
+def test_mlp_train_partial_batches(n, aligned):
+    """Gradients and loss of one step against torch in 64 bits.  Every GEMM operand is rounded to bf16 (2^-9
+    relative each; activation, signal and weight along three layers), so a gradient of random-signed terms lies
+    within a few 2^-9 of the 64-bit one in norm; 2^-6 leaves a factor of about 3.  A point left out or counted
+    twice changes it by about n^-1/2 (the small sizes), a CTA's share by more."""
+    p, m, idx, dist = _points(max(n, 200), 3)
+    w, g = _weights(4), torch.Generator(device="cuda")
+    g.manual_seed(n)
+    t = 0.5 * torch.randn((n, 8), generator=g, device="cuda")
+    i, d = (idx[:n], dist[:n]) if aligned else (_off_by_one(idx[:n]), _off_by_one(dist[:n]))
+    tr = gi.MLPTrainer(w.clone())
+    loss = float(tr.step(p, m, i, d, t, n=n))
+    q = w.double().requires_grad_(True)
+    W1, b1, W2, b2, W3, b3 = torch.split(q, [7168, 64, 4096, 64, 512, 8])
+    P, N, J, D = p.double(), m.double(), idx[:n].long(), dist[:n].double()
+    X = torch.cat([((P[J] - P[:n, None]) / D.mean(1)[:, None, None]).reshape(n, 48), N[J].reshape(n, 48), N[:n]], 1)
+    h = torch.relu(X @ W1.reshape(112, 64)[:99] + b1)
+    h = torch.relu(h @ W2.reshape(64, 64) + b2)
+    ref = (h @ W3.reshape(64, 8) + b3 - t).square().sum() / (8 * n)
+    ref.backward()
+    err = ((tr.grad - q.grad).norm() / q.grad.norm()).item()
+    print(f"n {n}: gradient error {err:.2e}, loss {loss:.6f} against {ref.item():.6f}")
+    assert err <= 2.0 ** -6 and abs(loss - ref.item()) <= 2.0 ** -6 * ref.item()
+
+
+@pytest.mark.parametrize("n,k", [(2, 3), (5, 8), (17, 16), (4096, 16), (4096, 8), (4096, 3)])
+def test_knn_ties_exact(n, k):
+    """Points of a small lattice, many of them repeated: squared distances are exact in float32 and tie in large
+    groups, so the neighbours are exactly the first k by (distance, index)."""
+    g = np.random.default_rng(n + k)
+    pts = (g.integers(0, 9, (n, 3)) / 8.0).astype(np.float32)
+    idx, dist = (a.cpu().numpy() for a in gi.knn(torch.from_numpy(pts).cuda(), k))
+    q = (pts * 8).astype(np.int64)
+    for i in range(0, n, max(1, n // 200)):
+        d2 = ((q - q[i]) ** 2).sum(1)
+        o = np.lexsort((np.arange(n), d2))
+        o = o[o != i][:k]
+        want = np.full(k, -1)
+        want[:len(o)] = o
+        wd = np.full(k, np.inf, np.float32)
+        wd[:len(o)] = np.sqrt((d2[o] / 64.0).astype(np.float32))
+        assert np.array_equal(idx[i], want) and np.array_equal(dist[i], wd)
+
+
+@pytest.mark.parametrize("W,H,units", [(1, 1, 1), (31, 33, 2), (32, 32, 1), (65, 10, 3), (100, 71, 2)])
+def test_loss_partial_tiles(W, H, units):
+    """Image edges inside the loss kernels' tiles, planes that are no multiple of 16 bytes, several units; bounds
+    as for the larger images: 1e-5 of the loss, 1e-3 of the largest gradient."""
+    g = np.random.default_rng(W * H)
+    img, gt = (g.uniform(0, 1, (units, 3, H, W)).astype(np.float32) for _ in range(2))
+    mask = (g.uniform(0, 1, (units, H, W)) < 0.6).astype(np.uint8)
+    mask[:, 0, 0] = 1
+    fr = Frame(1, Units.single(1, units), W, H, 0, with_backward=False)
+    fr.img.copy_(torch.from_numpy(img))
+    loss = float(fr.loss(torch.from_numpy(gt).cuda(), torch.from_numpy(mask).cuda(), 0.2))
+    ref = [oracle.loss(img[u].astype(np.float64), gt[u].astype(np.float64), mask[u], 0.2) for u in range(units)]
+    assert loss == pytest.approx(np.mean([r[0] for r in ref]), rel=1e-5)
+    d = np.stack([r[1] for r in ref]) / units
+    assert np.abs(fr.dimg.cpu().numpy() - d).max() <= 1e-3 * np.abs(d).max()
+
+
+def _lists_by_numpy(fr, cap):
+    """The lists gs_bin_sort documents, from the projected records: instances in (depth, record index, tile) order,
+    the first cap of them kept, each list in that order."""
+    t = lambda a: a.cpu().numpy()  # noqa: E731
+    P = fr.P
+    tiles, depth, rad, xy = t(fr.tiles)[:P], t(fr.depth)[:P], t(fr.radius)[:P].astype(np.int64), fr.xy64()[:P]
+    fu, fv = np.floor(xy[:, 0]).astype(np.int64), np.floor(xy[:, 1]).astype(np.int64)
+    x0, x1 = (np.clip((fu + s) // 16, 0, fr.TX) for s in (-rad, rad + 15))
+    y0, y1 = (np.clip((fv + s) // 16, 0, fr.TY) for s in (-rad, rad + 15))
+    unit = np.searchsorted(fr.units.proj_base, np.arange(P), side="right") - 1
+    lists = [[] for _ in range(fr.units.n * fr.n_tiles)]
+    left = cap
+    for p in np.lexsort((np.arange(P), depth.view(np.uint32))):
+        if tiles[p] == 0:
+            continue
+        for ty in range(y0[p], y1[p]):
+            for tx in range(x0[p], x1[p]):
+                if left > 0:
+                    lists[unit[p] * fr.n_tiles + ty * fr.TX + tx].append(p)
+                    left -= 1
+    return lists, cap - left
+
+
+@pytest.mark.parametrize("n,views,W,H,cap", [
+    (1, 1, 16, 16, 64), (33, 2, 40, 24, 1000), (1025, 3, 100, 60, 1 << 15), (1500, 2, 64, 64, 2000),
+    (1500, 2, 64, 64, 1), (16384, 1, 48, 48, 1 << 17), (16385, 1, 48, 48, 1 << 17), (700, 1, 1024, 1024, 1 << 15),
+    (300, 1, 1040, 1024, 1 << 15)])
+def test_sort_lists_at_design_limits(n, views, W, H, cap):
+    """Both sides of the small sort's limits (records per unit, number of lists), partial warps and rounds, several
+    units, and a capacity that runs out, inside a record too: lists, ranges, counts and the chunk jobs."""
+    g = synth.random_gaussians(n, 0, n + views, extent=0.8, log_scale_range=(-4.0, -2.0))
+    cams = synth.orbital_cameras(8, 3.0, width=W, height=H).subset(list(range(views)))
+    import paper_2509_12138_gb300 as gs
+    fr = Frame(n, Units.single(n, views), W, H, 0, max_instances=cap, with_backward=False, with_loss=False, chunk=32)
+    fr.preprocess(gs.pack_params(g, 0), gs.pack_cameras(cams))
+    total = fr.total_instances()
+    fr.sort()
+    want, kept = _lists_by_numpy(fr, cap)
+    assert fr.read_status() == (2 if total > cap else 0) and fr.instances() == kept == min(total, cap)
+    vals, ranges = fr.sorted_lists()
+    lens = ranges[:, 1] - ranges[:, 0]
+    assert np.array_equal(lens, [len(w) for w in want])
+    assert sorted(ranges[lens > 0, 0].tolist()) == np.cumsum([0] + [len(w) for w in want if w])[:-1].tolist()
+    for (a, b), w in zip(ranges, want):
+        assert vals[a:b].tolist() == w
+    order, base = fr.tile_order.cpu().numpy(), fr.job_base.cpu().numpy()
+    jobs = fr.jobs.cpu().numpy()[:2 * base[-1]].reshape(-1, 2)
+    chunks = (lens[order] + 31) // 32
+    assert sorted(order.tolist()) == list(range(len(lens))) and np.array_equal(np.diff(base), chunks)
+    assert np.array_equal(jobs[:, 0], np.repeat(np.arange(len(order)), chunks))
+    assert np.array_equal(jobs[:, 1], np.concatenate([np.arange(c) for c in chunks]))
