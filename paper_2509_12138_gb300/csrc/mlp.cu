@@ -55,8 +55,8 @@ struct Smem {
   static constexpr int W3t = W2t + HID * LDH * 2;        // [8][LDH]  bf16  W3^T
   static constexpr int Bias = W3t + KOUT * LDH * 2;      // fp32 b1[64] b2[64] b3[8]
   static constexpr int Idx = Bias + (2 * HID + KOUT) * 4;  // int [BATCH][LDI]
-  static constexpr int Dbar = Idx + BATCH * LDI * 4;     // fp32 [BATCH]
-  static constexpr int X = Dbar + BATCH * 4;             // [BATCH][LDX] bf16 features
+  static constexpr int Dbar = Idx + BATCH * LDI * 4;     // float2 [BATCH]: mean distance, its reciprocal
+  static constexpr int X = Dbar + BATCH * 8;             // [BATCH][LDX] bf16 features
   static constexpr int FWD_END = X + BATCH * LDX * 2;
   static constexpr int Y = FWD_END;                      // fp32 [BATCH][8] outputs (initialiser)
   static constexpr int INIT_END = Y + BATCH * KOUT * 4;
@@ -164,46 +164,69 @@ __device__ __forceinline__ void load_row(KnnRow& r, const int* __restrict__ knn_
     for (int a = 0; a < KNN; ++a) { r.idx[a] = -1; r.dist[a] = 0.f; }
   }
 }
-__device__ __forceinline__ void stage_row(const KnnRow& r, int p, int* s_idx, float* s_dbar) {
+__device__ __forceinline__ void stage_row(const KnnRow& r, int p, int* s_idx, float2* s_dbar) {
   float s = 0.f;
   #pragma unroll
   for (int a = 0; a < KNN; ++a) { s_idx[p * LDI + a] = r.idx[a]; s += r.dist[a]; }
-  const float d = s / (float)KNN;
-  s_dbar[p] = d > 1e-12f ? d : 1e-12f;
+  float d = s / (float)KNN;
+  d = d > 1e-12f ? d : 1e-12f;
+  s_dbar[p] = make_float2(d, 1.f / d);
+}
+
+// bf16 of the float quotient o / d, given r = 1 / d: the product o r is within
+// two units in the last place of the quotient, so both round to the same bf16
+// unless the product lies within a few units of the midpoint of two bf16
+// values; only then (about one value in 4000) the division is carried out.
+__device__ __forceinline__ uint16_t bf_quotient(float o, float d, float r) {
+  float q = o * r;
+  if (((__float_as_uint(q) & 0xffffu) - 0x7ff8u) < 0x11u) q = o / d;
+  return bf(q);
 }
 
 // Features of the batch's points into the bf16 tile X[BATCH][LDX] by NT
 // threads, from the staged neighbour rows.  A thread takes single (point,
 // neighbour, component) values: consecutive lanes read the components of one
 // neighbour and write consecutive features, so a warp's gather touches a third
-// of the sectors that whole neighbours per lane would.
+// of the sectors that whole neighbours per lane would.  Three rounds of NT
+// values cover STEP points, so a round's neighbour and component are the same
+// for all of a thread's points; GRP gathers are in flight per thread, since the
+// builders' time is the gathers' latency (a step of 2M points: 4 in flight 842
+// us, 16 784 us; with the division of every value 923 us).
 template <int NT>
 __device__ __forceinline__ void build_features(int tid, const float* __restrict__ pts, const float* __restrict__ nrm,
-                                               int64_t n, int64_t base, const int* s_idx, const float* s_dbar,
+                                               int64_t n, int64_t base, const int* s_idx, const float2* s_dbar,
                                                uint16_t* X) {
-  constexpr int STEP = NT * 3 / 48;  // points covered by three rounds of NT values
-  static_assert(NT * 3 % 48 == 0 && BATCH % STEP == 0, "rounds repeat every STEP points");
-  int pr[3], fr[3];
-  #pragma unroll
-  for (int r = 0; r < 3; ++r) { pr[r] = (tid + NT * r) / 48; fr[r] = (tid + NT * r) % 48; }
-  #pragma unroll 2
-  for (int q = 0; q < BATCH; q += STEP) {
-    float o[3], nn[3];
-    #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const int p = pr[r] + q, c = fr[r] % 3;
-      const int j = s_idx[p * LDI + fr[r] / 3];
-      o[r] = nn[r] = 0.f;
-      if (j >= 0) {  // (-1 for the points past n too)
-        o[r] = __ldg(pts + 3 * (int64_t)j + c) - __ldg(pts + 3 * (base + p) + c);
-        nn[r] = __ldg(nrm + 3 * (int64_t)j + c);
+  constexpr int STEP = NT * 3 / 48, GRP = BATCH / STEP < 16 ? BATCH / STEP : 16;
+  static_assert(NT * 3 % 48 == 0 && BATCH % (STEP * GRP) == 0, "rounds repeat every STEP points");
+  #pragma unroll 1
+  for (int r = 0; r < 3; ++r) {
+    const int p0 = (tid + NT * r) / 48, f = (tid + NT * r) % 48, c = f % 3;
+    const int* idx = s_idx + p0 * LDI + f / 3;
+    const float2* dbar = s_dbar + p0;
+    const float* own = pts + 3 * (base + p0) + c;
+    uint16_t* x = X + p0 * LDX + f;
+    #pragma unroll 1
+    for (int q = 0; q < BATCH / STEP; q += GRP) {
+      float o[GRP], nn[GRP];
+      #pragma unroll
+      for (int e = 0; e < GRP; ++e) {
+        const int j = idx[e * STEP * LDI];
+        o[e] = nn[e] = 0.f;
+        if (j >= 0) {  // (-1 for the points past n too)
+          o[e] = __ldg(pts + 3 * (int64_t)j + c) - __ldg(own + e * STEP * 3);
+          nn[e] = __ldg(nrm + 3 * (int64_t)j + c);
+        }
       }
-    }
-    #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const int p = pr[r] + q;
-      X[p * LDX + fr[r]] = bf(o[r] / s_dbar[p]);
-      X[p * LDX + 48 + fr[r]] = bf(nn[r]);
+      #pragma unroll
+      for (int e = 0; e < GRP; ++e) {
+        const float2 d = dbar[e * STEP];  // mean neighbour distance and its reciprocal
+        x[e * STEP * LDX] = bf_quotient(o[e], d.x, d.y);
+        x[e * STEP * LDX + 48] = bf(nn[e]);
+      }
+      idx += GRP * STEP * LDI;
+      dbar += GRP * STEP;
+      own += GRP * STEP * 3;
+      x += GRP * STEP * LDX;
     }
   }
   for (int e = tid; e < BATCH * (KIN - 96); e += NT) {
@@ -283,16 +306,16 @@ __device__ __forceinline__ void build_batch(const float* __restrict__ pts, const
   if (threadIdx.x < BATCH) {
     KnnRow r;
     load_row(r, knn_idx, knn_dist, n, base + threadIdx.x, vec);
-    stage_row(r, threadIdx.x, (int*)(sm + Smem::Idx), (float*)(sm + Smem::Dbar));
+    stage_row(r, threadIdx.x, (int*)(sm + Smem::Idx), (float2*)(sm + Smem::Dbar));
   }
   __syncthreads();
-  build_features<FWD_T>(threadIdx.x, pts, nrm, n, base, (const int*)(sm + Smem::Idx), (const float*)(sm + Smem::Dbar),
+  build_features<FWD_T>(threadIdx.x, pts, nrm, n, base, (const int*)(sm + Smem::Idx), (const float2*)(sm + Smem::Dbar),
                         (uint16_t*)(sm + Smem::X));
   __syncthreads();
 }
 
 // y rows (m0+g, m0+g+8), cols (2t, 2t+1) -> out[row][col]
-__global__ void __launch_bounds__(FWD_T) k_mlp_forward(const float* __restrict__ pts, const float* __restrict__ nrm,
+__global__ void __launch_bounds__(FWD_T, 3) k_mlp_forward(const float* __restrict__ pts, const float* __restrict__ nrm,
                                                          const int* __restrict__ knn_idx,
                                                          const float* __restrict__ knn_dist, int64_t n, bool vec,
                                                          const float* __restrict__ w, float* __restrict__ out) {
@@ -345,7 +368,7 @@ __global__ void k_plain_init(const float* __restrict__ knn_dist, int k, int64_t 
   write_init(params, N, i, d3, nullptr, false, logit_default);
 }
 
-__global__ void __launch_bounds__(FWD_T) k_mlp_init(const float* __restrict__ pts, const float* __restrict__ nrm,
+__global__ void __launch_bounds__(FWD_T, 3) k_mlp_init(const float* __restrict__ pts, const float* __restrict__ nrm,
                                                       const int* __restrict__ knn_idx,
                                                       const float* __restrict__ knn_dist, int64_t n, bool vec,
                                                       const float* __restrict__ w, float logit_default,
@@ -390,14 +413,14 @@ __device__ __forceinline__ void bar_sync(int id, int threads) {
 // fp32 registers, which leave for memory once, at the end.  Bias gradients are
 // the same columns multiplied by a fragment of ones.  2M points: 3792 us with
 // one warp group per SM doing both in turn, operands read as 16-bit scalars
-// and gradients kept in shared memory; 923 us.
+// and gradients kept in shared memory; 784 us.
 __global__ void __launch_bounds__(CONS_T + PROD_T, 1)
     k_mlp_train(const float* __restrict__ pts, const float* __restrict__ nrm, const int* __restrict__ knn_idx,
                 const float* __restrict__ knn_dist, const float* __restrict__ target, int64_t n, bool vec,
                 const float* __restrict__ w, float scale, float* __restrict__ grad, float* __restrict__ loss) {
   extern __shared__ __align__(16) char sm[];
   int* s_idx = (int*)(sm + Smem::Idx);
-  float* s_dbar = (float*)(sm + Smem::Dbar);
+  float2* s_dbar = (float2*)(sm + Smem::Dbar);
   const int64_t nb = (n + BATCH - 1) / BATCH;
   const int64_t b0 = blockIdx.x;
   const int steps = b0 < nb ? (int)((nb - b0 + gridDim.x - 1) / gridDim.x) : 0;
