@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "gs.h"
 #include <nvtx3/nvToolsExt.h>
 
@@ -171,6 +173,29 @@ struct GsRange {
   GsRange& operator=(const GsRange&) = delete;
 };
 #define GS_RANGE(name) GsRange gs_range_guard_(name)
+
+// Blocks of `threads` threads and `smem` dynamic bytes of a kernel that stay resident on the current device,
+// at most `units`: the grid of a kernel whose blocks take units of work in turn (a grid sized for the capacity
+// would mostly hold blocks that find nothing to do).  The occupancy query costs a microsecond or two of host time
+// and its answer is a property of the kernel and the device, so it is asked once per device.
+template <auto Kernel>
+unsigned gs_resident_grid(int threads, size_t smem, int64_t units) {
+  constexpr int DEVICES = 64;
+  static std::atomic<int> known[DEVICES];  // 0: not asked yet
+  if (units < 1) return 1u;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return (unsigned)units;
+  int g = dev < DEVICES ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (g == 0) {
+    int sms = 0, per = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, Kernel, threads, smem) != cudaSuccess || sms < 1 || per < 1)
+      return (unsigned)units;
+    g = sms * per;
+    if (dev < DEVICES) known[dev].store(g, std::memory_order_relaxed);
+  }
+  return (unsigned)(g < units ? g : units);
+}
 
 // host-side helpers
 int gs_fill_units(const gs_units* u, gs::UnitTable& t, int64_t* total);

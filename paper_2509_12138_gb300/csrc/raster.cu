@@ -419,13 +419,13 @@ __device__ __forceinline__ uint32_t eval_hit(float rx, float ry, float4 co, floa
   const float x0 = ox + (float)h.c0, x1 = ox + (float)h.c1;
   float x = x0, y = oy + (float)h.r0;
   int px = h.r0 * BW + h.c0;
+  #pragma unroll 2
   for (int k = 0; k < n; ++k) {
     const float power = splat_power(co.x, co.y, co.z, rx - x, ry - y);
     const float a = co.w * __expf(power), alpha = fminf(ALPHA_MAX, a);
-    if (!(power > 0.f) && !(alpha < ALPHA_MIN)) {
-      row[px] = CLAMP ? alpha : a;
-      valid |= 1u << px;
-    }
+    const bool hit = !(power > 0.f) && !(alpha < ALPHA_MIN);
+    if (hit) row[px] = CLAMP ? alpha : a;
+    valid |= (hit ? 1u : 0u) << px;
     const bool wrap = x >= x1;  // next column, or the next row's first
     x = wrap ? x0 : x + 1.f;
     y = wrap ? y + 1.f : y;
@@ -537,27 +537,38 @@ __device__ __forceinline__ void walk_fwd(const uint32_t* __restrict__ vals, cons
     // pixel-major: this pixel's pairs in list order
     uint32_t mine = transpose32(valid);
     int lj = -1;
-    if (mine && !done) {
-      int j = __ffs(mine) - 1;
-      float alpha = sc.alpha[j * MROW + lane];
-      for (;;) {  // the next pair's alpha is on its way while this one is composited
+    if (done) mine = 0u;
+    // as many steps as the busiest lane has pairs, two at a time; a lane without one takes alpha 0.  No branch
+    // inside, so the loads and bit scans of the next pairs overlap this one's chain through T.
+    for (int it = (int)__reduce_max_sync(FULL, (uint32_t)__popc(mine)); it > 0; it -= 2) {
+      int j[2];
+      float al[2], cr[2], cg[2], cb[2];
+      #pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        j[e] = mine ? __ffs(mine) - 1 : 0;
+        al[e] = mine ? sc.alpha[j[e] * MROW + lane] : 0.f;
+        cr[e] = sc.r[j[e]]; cg[e] = sc.g[j[e]]; cb[e] = sc.b[j[e]];
         mine &= mine - 1;
-        const int jn = mine ? __ffs(mine) - 1 : j;
-        const float an = sc.alpha[jn * MROW + lane];
-        const float tT = T * (1.f - alpha);
-        if (tT < T_MIN) { done = true; break; }
-        const float wgt = alpha * T, cr = sc.r[j], cg = sc.g[j], cb = sc.b[j];
-        c0 += cr * wgt; c1 += cg * wgt; c2 += cb * wgt;
-        if (DUAL) {
-          const float lw = alpha * loc.x;
-          loc.y += cr * lw; loc.z += cg * lw; loc.w += cb * lw;
-          loc.x *= 1.f - alpha;
+      }
+      #pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float om = 1.f - al[e], tT = T * om;
+        const bool pair = al[e] > 0.f && !done;
+        const bool blend = pair && !(tT < T_MIN);
+        done = done || (pair && tT < T_MIN);
+        const float wgt = blend ? al[e] * T : 0.f;
+        if (blend) {
+          c0 += cr[e] * wgt; c1 += cg[e] * wgt; c2 += cb[e] * wgt;
+          T = tT;
+          lj = j[e];
         }
-        T = tT;
-        lj = j;
-        if (!mine) break;
-        j = jn;
-        alpha = an;
+        if (DUAL) {
+          const float lw = al[e] * loc.x;
+          if (blend) {
+            loc.y += cr[e] * lw; loc.z += cg[e] * lw; loc.w += cb[e] * lw;
+            loc.x *= om;
+          }
+        }
       }
     }
     if (lj >= 0) last = (int)sc.q[qh + lj] + 1;
@@ -589,10 +600,36 @@ __device__ __forceinline__ void walk_fwd(const uint32_t* __restrict__ vals, cons
 // Per pixel the blended entries and the stop decision are those of the
 // sequential walk; the combine changes only the rounding order of T and C.
 // gs_schedule.walk_whole_lists is M = infinity.
-// Forward stage at 10M / 1080p, two views, 8 partitions of 2.8M / 1080p, two
-// views (us): M = 8: 1498, 1721, 912, 784; 16: 1324, 1686, 926, 862; 32: 1329,
-// 1659, 1061, 825; chunk-parallel from the first chunk: 2129, 1882, 975, 945.
+// M depends on the lists alone (a split that followed the timing would change
+// the rounding of the checkpoints from run to run):
+//   all lists of at most 8 chunks (by the heaviest's class): no split, the
+//     passes behind the front would cost more than its last blocks' walks;
+//   fewer blocks than resident warps: 1, a serial walk leaves warps idle;
+//   else the chunks or blocks a resident warp gets, the fewer, 4 to 16, so that
+//     a serial walk is no longer than the whole pass; the parallel passes walk
+//     chunks behind stops, so as much as that bound allows stays in front.
+// Forward stage, two views each (us), M = 1 / 4 / 16 -> by this rule: 10M at
+// 1080p 1997, 1773 / 1822, 1755 / 1223, 1503 -> 1250, 1526; 1M at 1080p 292,
+// 329 / 195, 312 / 194, 249 -> 195, 254; 8 partitions of 2.8M at 1080p 771, 726
+// / 769, 728 / 879, 804 -> 859, 777; 4M at 1800x1300 731, 803 / 694, 754 / 551,
+// 772 -> 556, 764; 3M in 3 partitions at 400x300, two views, 1265, 1222 / 1398,
+// 1356 / 2075, 1841 -> 1248, 1241; 6M at 400x300 1260, 1206 / 1457, 1403 /
+// 1926, 1853 -> 1274, 1211; 1M there 396, 395 / 465, 494 / 542, 619 -> 390, 390.
+// Where the capacity bounds every list to FRONT_CHUNKS chunks, the passes behind
+// the front are not launched at all (5 us each with nothing to do).
+// 88 registers, 22 warps per SM; held to 80, 72 and 64 the 10M views took 1275,
+// 1265 and 1423 us.
 constexpr int FRONT_CHUNKS = 16;
+__device__ __forceinline__ int front_chunks(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
+                                            uint32_t jobs, uint32_t lists, uint32_t warps, int K) {
+  if (lists == 0u) return FRONT_CHUNKS;
+  const uint32_t units = 8u * lists;
+  const uint2 first = ranges[order[0]];  // of the heaviest lists' class: less than twice its length is the longest
+  const uint32_t longest = 2u << (31 - __clz((int)max(first.y - first.x, 1u)));
+  if (longest <= 8u * (uint32_t)K) return FRONT_CHUNKS;
+  if (units < warps) return 1;
+  return (int)min((uint32_t)FRONT_CHUNKS, max(4u, 8u * min(jobs, units) / warps));
+}
 constexpr uint32_t STOP_BIT = 0x80000000u;  // partial or front state: the pixel has stopped
 constexpr uint32_t REWALK_BIT = 0x80000000u;  // n_contrib between combine and stop pass: stop chunk pending,
                                              // the stop chunk c* in the bits below it
@@ -711,7 +748,7 @@ __device__ __forceinline__ float4 walk_chunk(const uint32_t* __restrict__ vals, 
 template <int BW>
 __global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict__ ranges,
                                                          const uint32_t* __restrict__ order,
-                                                         const uint32_t* __restrict__ job_base, int K, int M, bool whole,
+                                                         const uint32_t* __restrict__ job_base, int K, bool whole, bool later,
                                                          int NT,
                                                          float4* __restrict__ ckpt, uint32_t* __restrict__ chunk_last,
                                                          const uint32_t* __restrict__ vals,
@@ -726,7 +763,9 @@ __global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict
                                                          uint32_t* __restrict__ ticket) {
   __shared__ FwdScratch s_walk;
   const int lane = threadIdx.x & 31;
-  const uint32_t total = (uint32_t)lists_in_use(job_base, NT) * 8u;
+  const int lists = lists_in_use(job_base, NT);
+  const uint32_t total = (uint32_t)lists * 8u;
+  const int M = later ? front_chunks(ranges, order, job_base[NT], (uint32_t)lists, gridDim.x, K) : INT_MAX;
   auto unit = [&](uint32_t vb) {
     const int o = (int)(vb >> 3), w = (int)(vb & 7u);
     PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
@@ -790,7 +829,7 @@ __global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict
   }
 }
 
-// Chunk pass: queued job (list o, chunk c >= M, block w) composites its entries
+// Chunk pass: queued job (list o, chunk c, block w) composites its entries
 // from T = 1 for the pixels that have not stopped in front of chunk M; the
 // partial goes to checkpoint slot c - 1 and chunk_last.
 template <int BW>
@@ -915,11 +954,13 @@ __device__ __forceinline__ void combine_pixel(int m, int nch, int64_t plane, int
 }
 
 // Combine pass: one warp per queued block; the entry of its first queued chunk
-// (chunk M) stands for it.  The first block also zeroes the stop pass's ticket.
+// stands for it (a block's entries are consecutive, so it is one whose
+// predecessor is not the same block's previous chunk).  The first block also
+// zeroes the stop pass's ticket.
 template <int BW>
 __global__ void __launch_bounds__(32) k_render_fwd_combine(const uint32_t* __restrict__ order,
                                                            const uint32_t* __restrict__ job_base,
-                                                           const uint32_t* __restrict__ jobs, int M,
+                                                           const uint32_t* __restrict__ jobs,
                                                            float4* __restrict__ ckpt,
                                                            uint32_t* __restrict__ chunk_last, int W, int H, int TX,
                                                            int n_tiles, float bg0, float bg1, float bg2,
@@ -930,21 +971,22 @@ __global__ void __launch_bounds__(32) k_render_fwd_combine(const uint32_t* __res
   if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0u;
   const uint32_t total = queue[qcap];
   for (uint32_t e = blockIdx.x; e < total; e += gridDim.x) {
-    const uint32_t jid = (queue[e] & ~MARK_BIT) >> 3;  // (a mark is set on later entries of a block only by its warp)
-    if ((int)jobs[2 * (int64_t)jid + 1] != M) continue;
-    const int w = (int)(queue[e] & 7u), o = (int)jobs[2 * (int64_t)jid];
+    const uint32_t ent = queue[e] & ~MARK_BIT;  // (marks are set by the warp of the entry's block)
+    if (e > 0 && ((queue[e - 1] & ~MARK_BIT) + 8u) == ent) continue;
+    const uint32_t jid = ent >> 3;
+    const int w = (int)(ent & 7u), o = (int)jobs[2 * (int64_t)jid], m = (int)jobs[2 * (int64_t)jid + 1];
     const uint32_t jb = job_base[o];
     const int nch = (int)(job_base[o + 1] - jb);
     PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
     const int64_t plane = (int64_t)W * H, pix = (int64_t)P.py * W + P.px, cp0 = (int64_t)jb - o;
     int cstar = -1;
     if (P.inside)
-      combine_pixel(M, nch, plane, pix, img + (int64_t)P.u * 3 * plane, final_T + (int64_t)P.u * plane,
+      combine_pixel(m, nch, plane, pix, img + (int64_t)P.u * 3 * plane, final_T + (int64_t)P.u * plane,
                     n_contrib + (int64_t)P.u * plane, ckpt + cp0 * TILE_PIX + P.pix_local,
                     chunk_last + cp0 * TILE_PIX + P.pix_local, bg0, bg1, bg2, cstar);
     // mark the block's queue entries the stop pass walks: one per distinct stop chunk of its pixels
     const unsigned peers = __match_any_sync(0xffffffffu, cstar);
-    if (cstar >= 1 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) queue[e + (uint32_t)(cstar - M)] |= MARK_BIT;
+    if (cstar >= 1 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) queue[e + (uint32_t)(cstar - m)] |= MARK_BIT;
     __syncwarp();
   }
 }
@@ -1655,19 +1697,6 @@ __global__ void k_fixed_to_grad2d(const unsigned long long* __restrict__ fixed, 
   reinterpret_cast<float4*>(drgb)[p] = make_float4(g[6], g[7], g[8], 0.f);
 }
 
-// Grid of a one-warp kernel whose blocks take units of work from a ticket counter: as many blocks as
-// stay resident on the device, at most one per unit.
-template <typename K>
-unsigned resident_grid(K kernel, int64_t units) {
-  int dev = 0, sms = 0, per = 0;
-  if (units < 1) return 1u;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 32, 0) != cudaSuccess || sms < 1 || per < 1)
-    return (unsigned)units;
-  int64_t g = (int64_t)sms * per;
-  return (unsigned)(g < units ? g : units);
-}
-
 // The two ticket words of the scheduled blend kernels: the jobs array's last entry, which no job uses
 // (a list of L entries has ceil(L / K) < L / K + 1 jobs, so there are fewer than max_jobs - 1).
 inline uint32_t* sched_ticket(const gs_schedule* sched) {
@@ -1689,7 +1718,7 @@ int gs_render_fwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const u
   const uint32_t qcap = sched ? (uint32_t)(8 * sched->max_jobs) : 0u;
 #define GS_FWD(BW)                                                                                                  \
   if (sched) {                                                                                                        \
-    const int M = sched->walk_whole_lists ? INT_MAX : FRONT_CHUNKS;                                                   \
+    const bool later = !sched->walk_whole_lists && sched->max_checkpoints > FRONT_CHUNKS;                             \
     uint32_t* tk = sched_ticket(sched);                                                                               \
     uint32_t* q = sched->stop_queue;                                                                                  \
     float4* ck = (float4*)sched->checkpoints;                                                                         \
@@ -1697,18 +1726,19 @@ int gs_render_fwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const u
     const uint2* rg = (const uint2*)ranges;                                                                           \
     k_render_fwd_empty<<<grid, TILE_PIX, 0, s>>>(rg, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T,   \
                                                  n_contrib, tk, q + qcap);                                            \
-    k_render_fwd_front<BW><<<resident_grid(k_render_fwd_front<BW>, (int64_t)grid.x * 8), 32, 0, s>>>(                 \
-        rg, sched->tile_order, sched->job_base, sched->chunk, M, sched->walk_whole_lists != 0, (int)grid.x, ck, sched->chunk_last, sorted_vals,     \
+    k_render_fwd_front<BW><<<gs_resident_grid<k_render_fwd_front<BW>>(32, 0, (int64_t)grid.x * 8), 32, 0, s>>>(                 \
+        rg, sched->tile_order, sched->job_base, sched->chunk, sched->walk_whole_lists != 0, later, (int)grid.x, ck,   \
+        sched->chunk_last, sorted_vals,                                                                               \
         sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib, \
         q, qcap, tk);                                                                                                 \
-    if (!sched->walk_whole_lists) {                                                                                   \
-      k_render_fwd_chunk<BW><<<resident_grid(k_render_fwd_chunk<BW>, (int64_t)qcap), 32, 0, s>>>(                     \
+    if (later) {                                                                                                      \
+      k_render_fwd_chunk<BW><<<gs_resident_grid<k_render_fwd_chunk<BW>>(32, 0, (int64_t)qcap), 32, 0, s>>>(                     \
           rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last, sorted_vals,      \
           sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, n_contrib, q, qcap, tk + 1);                \
-      k_render_fwd_combine<BW><<<resident_grid(k_render_fwd_combine<BW>, (int64_t)qcap), 32, 0, s>>>(                 \
-          sched->tile_order, sched->job_base, sched->jobs, M, ck, sched->chunk_last, width, height, TX, TX * TY, bg[0],\
+      k_render_fwd_combine<BW><<<gs_resident_grid<k_render_fwd_combine<BW>>(32, 0, (int64_t)qcap), 32, 0, s>>>(                 \
+          sched->tile_order, sched->job_base, sched->jobs, ck, sched->chunk_last, width, height, TX, TX * TY, bg[0],\
           bg[1], bg[2], img, final_T, n_contrib, q, qcap, tk);                                                        \
-      k_render_fwd_stop<BW><<<resident_grid(k_render_fwd_stop<BW>, (int64_t)qcap), 32, 0, s>>>(                       \
+      k_render_fwd_stop<BW><<<gs_resident_grid<k_render_fwd_stop<BW>>(32, 0, (int64_t)qcap), 32, 0, s>>>(                       \
           rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last, sorted_vals,      \
           sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib,\
           q, qcap, tk);                                                                                               \
@@ -1754,13 +1784,13 @@ int gs_blend_bwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const ui
     {                                                                                                              \
       if (cudaMemsetAsync(sched_ticket(sched), 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;        \
       if (fixed) {                                                                                                   \
-        k_render_bwd_det<BW><<<dim3(resident_grid(k_render_bwd_det<BW>, sched->max_jobs * 8)), 32, 0, s>>>(          \
+        k_render_bwd_det<BW><<<gs_resident_grid<k_render_bwd_det<BW>>(32, 0, sched->max_jobs * 8), 32, 0, s>>>(          \
             (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                     \
             (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,             \
             (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, TX * TY * n_units,  \
             bg[0], bg[1], bg[2], img, final_T, n_contrib, dL_dimg, dL_dT, fixed, sched_ticket(sched));               \
       } else {                                                                                                       \
-        k_render_bwd_m<BW><<<dim3(resident_grid(k_render_bwd_m<BW>, sched->max_jobs * 8)), 32, 0, s>>>(              \
+        k_render_bwd_m<BW><<<gs_resident_grid<k_render_bwd_m<BW>>(32, 0, sched->max_jobs * 8), 32, 0, s>>>(              \
             (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                     \
             (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,             \
             (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, TX * TY * n_units,  \

@@ -165,3 +165,38 @@ def test_sort_lists_at_design_limits(n, views, W, H, cap):
     assert sorted(order.tolist()) == list(range(len(lens))) and np.array_equal(np.diff(base), chunks)
     assert np.array_equal(jobs[:, 0], np.repeat(np.arange(len(order)), chunks))
     assert np.array_equal(jobs[:, 1], np.concatenate([np.arange(c) for c in chunks]))
+
+
+@pytest.mark.parametrize("n,W,H,log_scales", [
+    (3000, 100, 60, (-4.0, -2.5)),    # few short lists: no split
+    (30000, 100, 60, (-3.5, -2.5)),   # fewer blocks than warps, long lists: everything behind the first chunk
+    (60000, 500, 500, (-3.5, -2.0)),  # more blocks than warps: 4 to 16 chunks in front
+])
+def test_front_split_rules(n, W, H, log_scales):
+    """A list's chunks composited by either pass: images within the rounding of a sum of n_contrib terms grouped by
+    chunks of 32, against whole-list walks.  A pixel whose stop falls on the other side of the rounding differs by at most
+    what the one that stopped left over."""
+    import paper_2509_12138_gb300 as gs
+    g = synth.random_gaussians(n, 0, 3, extent=1.0, log_scale_range=log_scales)
+    cams = gs.pack_cameras(synth.orbital_cameras(8, 3.0, width=W, height=H).subset([0]))
+    params = gs.pack_params(g, 0)
+    fr = Frame(n, Units.single(n, 1), W, H, 0, with_backward=False, with_loss=False, chunk=32)
+    fr.fit_capacity(params, cams)
+    out = []
+    for whole in (False, True):
+        fr.walk_whole_lists = whole
+        fr.preprocess(params, cams)
+        fr.sort()
+        fr.render((0.2, 0.4, 0.6))
+        assert fr.read_status() == 0
+        out.append((fr.img.double().cpu().reshape(3, -1), fr.final_T.double().cpu().reshape(-1),
+                    fr.n_contrib.cpu().reshape(-1)))
+    (ia, ta, na), (ib, tb, nb) = out
+    same = na == nb
+    colour = max(1.0, float(fr.rgb[:, :3].abs().max()))
+    # T: a product of n_contrib factors, each pair of groupings n_contrib roundings apart; C: the sum of weights is 1
+    eps = 2.0 ** -23 * (nb.double() + 64)
+    assert float(same.double().mean()) > 0.99
+    assert bool(((ta - tb).abs() <= eps * tb.clamp_min(1e-6))[same].all())
+    assert bool(((ia - ib).abs() <= eps * colour)[:, same].all())
+    assert bool(((ia - ib).abs() <= (2 * torch.maximum(ta, tb) + eps) * colour).all())
