@@ -167,6 +167,31 @@ def test_sort_lists_at_design_limits(n, views, W, H, cap):
     assert np.array_equal(jobs[:, 1], np.concatenate([np.arange(c) for c in chunks]))
 
 
+@pytest.mark.parametrize("wide", [False, True])
+def test_sort_of_many_records_equals_global(wide):
+    """2^24 records on: with room for two instances a record the emission reads packed rectangles (wide: some are
+    too wide to pack), with one less it reads the records; both give the global sort's lists, bit for bit."""
+    import paper_2509_12138_gb300 as gs
+    n = (1 << 24) + 77
+    g = synth.random_gaussians(n, 0, 5, extent=0.9, log_scale_range=(-7.5, -6.0))
+    if wide:
+        g["log_scales"][::200_003] = -1.0
+    cams = gs.pack_cameras(synth.orbital_cameras(8, 3.0, width=333, height=250).subset([1]))
+    params = gs.pack_params(g, 0)
+    del g
+    got = []
+    for cap, design in ((2 * n, "depth_first"), (2 * n - 1, "depth_first"), (2 * n, "global")):
+        fr = Frame(n, Units.single(n, 1), 333, 250, 0, max_instances=cap, with_backward=False, with_loss=False)
+        fr.preprocess(params, cams)
+        fr.sort(design)
+        count = fr.instances()
+        assert fr.read_status() == 0 and 0 < count <= cap
+        got.append([fr.sorted_vals[:count].cpu(), fr.ranges.cpu(), fr.block_masks[:count].cpu()])
+        del fr
+    for other in got[:2]:
+        assert all(torch.equal(a, b) for a, b in zip(other, got[2]))
+
+
 @pytest.mark.parametrize("n,W,H,log_scales", [
     (3000, 100, 60, (-4.0, -2.5)),    # few short lists: no split
     (30000, 100, 60, (-3.5, -2.5)),   # fewer blocks than warps, long lists: everything behind the first chunk
