@@ -9,8 +9,9 @@
 // its tile: records x tiles tests in all, so the design is for small products
 // of the two (gs_small_sort_applies).  A list comes out in (depth, record index)
 // order without any sort of the instances.  What bounds it is latency, not
-// bytes.  Sort and schedule of 500 records on 16 tiles: 150 -> 43 us; of 8 units
-// of 2,000 records on 64 tiles: 204 -> 90 us.
+// bytes.  Sort and schedule of 500 records on 16 tiles: 150 -> 37 us; of 8 units
+// of 2,000 records on 64 tiles: 204 -> 66 us (43 and 90 us with 32 records per
+// step of a list's warp instead of 128, and 8 lists per block instead of 4).
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -241,36 +242,49 @@ __global__ void __launch_bounds__(ST, 1) k_small_units(UnitTable U, const float4
   }
 }
 
-// Calls f(hit, record) 32 records at a time, in depth order, for one (unit,
-// tile) list; hit: the record has an instance in the list.
-template <typename F>
-__device__ __forceinline__ void for_hits(const UnitTable& U, int u, int tx, int ty, const uint32_t* __restrict__ rec,
-                                         const uint2* __restrict__ rect, const float* __restrict__ depth,
-                                         const Ctrl* __restrict__ ctrl, F f) {
-  const int lane = threadIdx.x & 31;
-  const int64_t base = U.proj_base[u];
-  const int m = (int)ctrl->vis[u];
-  const bool over = ctrl->over != 0u;
-  for (int i = 0; i < m; i += 32) {
-    bool hit = false;
-    uint32_t p = 0u;
-    if (i + lane < m) {
-      const uint2 r = rect[base + i + lane];
-      const int x0 = (int)(r.x & 0xffffu), y0 = (int)(r.x >> 16), x1 = (int)(r.y & 0xffffu), y1 = (int)(r.y >> 16);
-      hit = tx >= x0 && tx < x1 && ty >= y0 && ty < y1;
-      if (hit) {
-        p = rec[base + i + lane];
-        if (over) {  // instances are numbered row by row within a record
-          const unsigned long long k = ((unsigned long long)__float_as_uint(depth[p]) << 32) | p;
-          hit = k < ctrl->cut || (k == ctrl->cut && (uint32_t)((ty - y0) * (x1 - x0) + tx - x0) < ctrl->cut_m);
-        }
+// The records of one (unit, tile) list, 32 GROUP at a time in depth order:
+// whether record i + 32 q + lane has an instance in it, and its id.  The loads
+// of a group are independent, so a warp waits for memory once per group.
+constexpr int GROUP = 4;
+struct Hits {
+  const uint32_t* rec;
+  const uint2* rect;
+  const float* depth;
+  const Ctrl* ctrl;
+  int tx, ty, m;
+  bool over;
+  unsigned long long cut;
+  uint32_t cut_m;
+  __device__ __forceinline__ Hits(const UnitTable& U, int u, int tx_, int ty_, const uint32_t* rec_, const uint2* rect_,
+                                  const float* depth_, const Ctrl* ctrl_)
+      : rec(rec_ + U.proj_base[u]), rect(rect_ + U.proj_base[u]), depth(depth_), ctrl(ctrl_), tx(tx_), ty(ty_) {
+    m = (int)ctrl->vis[u];
+    over = ctrl->over != 0u;
+    cut = ctrl->cut;
+    cut_m = ctrl->cut_m;
+  }
+  __device__ __forceinline__ void load(int i, bool* hit, uint32_t* p) const {
+    uint2 r[GROUP];
+    #pragma unroll
+    for (int q = 0; q < GROUP; ++q) {
+      const int k = i + 32 * q + (int)(threadIdx.x & 31);
+      r[q] = k < m ? __ldg(rect + k) : make_uint2(0u, 0u);  // (an empty rectangle)
+      p[q] = k < m ? __ldg(rec + k) : 0u;
+    }
+    #pragma unroll
+    for (int q = 0; q < GROUP; ++q) {
+      const int x0 = (int)(r[q].x & 0xffffu), y0 = (int)(r[q].x >> 16);
+      const int x1 = (int)(r[q].y & 0xffffu), y1 = (int)(r[q].y >> 16);
+      hit[q] = tx >= x0 && tx < x1 && ty >= y0 && ty < y1;
+      if (over && hit[q]) {  // instances are numbered row by row within a record
+        const unsigned long long k = ((unsigned long long)__float_as_uint(depth[p[q]]) << 32) | p[q];
+        hit[q] = k < cut || (k == cut && (uint32_t)((ty - y0) * (x1 - x0) + tx - x0) < cut_m);
       }
     }
-    f(hit, p);
   }
-}
+};
 
-constexpr int LW = 8;  // lists (warps) per block
+constexpr int LW = 4;  // lists (warps) per block
 
 __global__ void __launch_bounds__(LW * 32) k_small_count(UnitTable U, int W, int n_tiles, int NT,
                                                          const uint32_t* __restrict__ rec,
@@ -280,9 +294,16 @@ __global__ void __launch_bounds__(LW * 32) k_small_count(UnitTable U, int W, int
   const int f = blockIdx.x * LW + (threadIdx.x >> 5);
   if (f >= NT) return;
   const int TX = (W + TILE - 1) / TILE, tile = f % n_tiles;
+  const Hits H(U, f / n_tiles, tile % TX, tile / TX, rec, rect, depth, ctrl);
   uint32_t c = 0u;
-  for_hits(U, f / n_tiles, tile % TX, tile / TX, rec, rect, depth, ctrl,
-           [&](bool hit, uint32_t) { c += __popc(__ballot_sync(0xffffffffu, hit)); });
+  for (int i = 0; i < H.m; i += 32 * GROUP) {
+    bool hit[GROUP];
+    uint32_t p[GROUP];
+    H.load(i, hit, p);
+    #pragma unroll
+    for (int q = 0; q < GROUP; ++q) c += hit[q] ? 1u : 0u;
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
   if ((threadIdx.x & 31) == 0) count[f] = c;
 }
 
@@ -378,20 +399,34 @@ __global__ void __launch_bounds__(LW * 32) k_small_fill(UnitTable U, int W, int 
   if (rg.x == rg.y) return;
   const int TX = (W + TILE - 1) / TILE, tile = f % n_tiles, tx = tile % TX, ty = tile / TX;
   const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
+  const Hits H(U, f / n_tiles, tx, ty, rec, rect, depth, ctrl);
   uint32_t at = rg.x;
-  for_hits(U, f / n_tiles, tx, ty, rec, rect, depth, ctrl, [&](bool hit, uint32_t p) {
-    const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-    if (hit) {
-      const uint32_t k = at + __popc(bal & lt);
-      vals[k] = p;
-      if (masks) {
-        const float4 m = xy[p];
+  for (int i = 0; i < H.m; i += 32 * GROUP) {
+    bool hit[GROUP];
+    uint32_t p[GROUP], mk[GROUP];
+    H.load(i, hit, p);
+    if (masks) {
+      float4 m[GROUP], co[GROUP];
+      #pragma unroll
+      for (int q = 0; q < GROUP; ++q)
+        if (hit[q]) { m[q] = xy[p[q]]; co[q] = conic_op[p[q]]; }
+      #pragma unroll
+      for (int q = 0; q < GROUP; ++q) {
         float pm;
-        masks[k] = (uint16_t)block_mask(alpha_box(make_float2(m.x, m.y), conic_op[p], pm), tx, ty);
+        mk[q] = hit[q] ? block_mask(alpha_box(make_float2(m[q].x, m[q].y), co[q], pm), tx, ty) : 0u;
       }
     }
-    at += __popc(bal);
-  });
+    #pragma unroll
+    for (int q = 0; q < GROUP; ++q) {
+      const uint32_t bal = __ballot_sync(0xffffffffu, hit[q]);
+      if (hit[q]) {
+        const uint32_t k = at + __popc(bal & lt);
+        vals[k] = p[q];
+        if (masks) masks[k] = (uint16_t)mk[q];
+      }
+      at += __popc(bal);
+    }
+  }
 }
 
 }  // namespace
