@@ -20,10 +20,15 @@ namespace {
 constexpr int LT = 32;           // output tile edge
 constexpr int R = 5;             // window radius
 constexpr int HT = LT + 2 * R;   // halo tile edge (42)
-constexpr int HS = 44;           // halo row stride: rows start on 16 bytes
+constexpr int PAD = 8;           // columns staged in front of the output tile: a multiple of 4 pixels, at least R
+constexpr int HW = LT + 2 * PAD; // staged columns (48), in groups of 4
 constexpr int SEG = 4;           // outputs per thread along each pass
 constexpr int LOSS_T = 256;      // LT columns x (LT / SEG) strips
-static_assert(LT * (LT / SEG) == LOSS_T && HS % 4 == 0 && HS >= HT, "thread layout");
+// Row strides in shared memory: 8 threads of a 16-byte access take 4 segments of 2 rows (seg_task), whose banks
+// differ when the rows of pairs (8 bytes) start 4 banks apart and those of single values 16 banks apart.
+constexpr int HS2 = 50, TS2 = 34;  // pairs: staged rows, horizontal sums
+constexpr int HS1 = 48, TS1 = 48;  // single values
+static_assert(LT * (LT / SEG) == LOSS_T && HT % 2 == 0 && PAD >= R + 2 && HW <= HS2 && HW <= HS1, "thread layout");
 constexpr float C1 = 0.01f * 0.01f;
 constexpr float C2 = 0.03f * 0.03f;
 
@@ -110,6 +115,31 @@ __global__ void k_l1(const float* __restrict__ img, const float* __restrict__ gt
   if (threadIdx.x == 0 && t != 0.f) atomicAdd(&l1sum[u], (double)t);
 }
 
+// Two quantities that go through the same window travel as a pair, which
+// Blackwell multiplies and adds in one instruction (each half rounded as the
+// scalar operation would).
+using pair = unsigned long long;
+__device__ __forceinline__ pair make_pair(float a, float b) {
+  pair r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 halves(pair v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ pair fma2(pair a, pair b, pair c) {
+  pair r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ pair mul2(pair a, pair b) {
+  pair r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // Separable 11-tap window, SEG outputs per thread along each pass: a thread
 // reads its 14 inputs once and multiplies from registers, where one output per
 // thread would read 11 values for 11 multiplications.  Taps are added in
@@ -123,34 +153,88 @@ __device__ __forceinline__ void taps(const float* w, const float* in, float* out
     out[e] = a;
   }
 }
-// the 16 halo values from column SEG g of a row (the 14 used and two of the row's padding)
+__device__ __forceinline__ void taps2(const pair* w, const pair* in, pair* out) {
+  #pragma unroll
+  for (int e = 0; e < SEG; ++e) {
+    pair a = 0ull;
+    #pragma unroll
+    for (int t = 0; t < 11; ++t) a = fma2(w[t], in[e + t], a);
+    out[e] = a;
+  }
+}
+// the window's inputs of the outputs SEG g .. SEG g + 3 of a staged row: columns SEG g + PAD - R on, from the aligned
+// column in front of them (v[1] and v[3] are the first)
+__device__ __forceinline__ void load_seg2(const pair* row, int g, pair* v) {
+  #pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const ulonglong2 x = reinterpret_cast<const ulonglong2*>(row + SEG * g + 2)[q];
+    v[2 * q] = x.x; v[2 * q + 1] = x.y;
+  }
+}
 __device__ __forceinline__ void load_seg(const float* row, int g, float* v) {
   #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < 5; ++q) {
     const float4 x = reinterpret_cast<const float4*>(row + SEG * g)[q];
     v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
   }
 }
+__device__ __forceinline__ void store_seg2(pair* row, int g, const pair* v) {
+  ulonglong2* r = reinterpret_cast<ulonglong2*>(row + SEG * g);
+  r[0] = make_ulonglong2(v[0], v[1]);
+  r[1] = make_ulonglong2(v[2], v[3]);
+}
 __device__ __forceinline__ void store_seg(float* row, int g, const float* v) {
   reinterpret_cast<float4*>(row)[g] = make_float4(v[0], v[1], v[2], v[3]);
 }
-// vertical pass: the SEG outputs of column lx from row SEG strip of one quantity's horizontal sums
-__device__ __forceinline__ void taps_down(const float* w, const float (*tmp)[LT], int lx, int strip, float* out) {
+// horizontal task k: (halo row, segment), so that 8 threads in a row take 2 rows x 4 segments
+constexpr int SEG_TASKS = HT * (LT / SEG);
+__device__ __forceinline__ void seg_task(int k, int& r, int& g) {
+  const int hi = k >> 3;
+  r = 2 * (hi >> 1) + ((k >> 2) & 1);
+  g = 4 * (hi & 1) + (k & 3);
+}
+static_assert(LT / SEG == 8, "seg_task");
+
+// vertical pass: the SEG outputs of column lx from row SEG strip of the horizontal sums
+__device__ __forceinline__ void taps_down(const float* w, const float (*tmp)[TS1], int lx, int strip, float* out) {
   float v[SEG + 10];
   #pragma unroll
   for (int t = 0; t < SEG + 10; ++t) v[t] = tmp[SEG * strip + t][lx];
   taps(w, v, out);
 }
+__device__ __forceinline__ void taps_down2(const pair* w, const pair (*tmp)[TS2], int lx, int strip, pair* out) {
+  pair v[SEG + 10];
+  #pragma unroll
+  for (int t = 0; t < SEG + 10; ++t) v[t] = tmp[SEG * strip + t][lx];
+  taps2(w, v, out);
+}
+
+// Calls f(staged row, first staged column, image column, row in the image?,
+// offset in the plane) for every group of 4 staged pixels.  Where the plane's
+// rows start on 16 bytes (vec) a group lies inside the image or outside and is
+// one load per array; otherwise its pixels are read one at a time.
+template <typename F>
+__device__ __forceinline__ void for_groups(int bx, int by, int W, int H, F f) {
+  for (int k = threadIdx.x; k < HT * (HW / 4); k += LOSS_T) {
+    const int r = k / (HW / 4), q = 4 * (k % (HW / 4));
+    const int gx = bx * LT - PAD + q, gy = by * LT - R + r;
+    f(r, q, gx, gy >= 0 && gy < H, (int64_t)gy * W + gx);
+  }
+}
 
 // SSIM statistics, loss sums and the three factor maps.  Bound by fp32 issue
-// (127 multiply-adds per pixel and channel with the halo rows): 2048x2048,
-// whole mask: 272 us at one output per thread.
+// (127 multiply-adds per pixel and channel with the halo rows, 76 instructions
+// as pairs); the rest is staging and the divisions of the epilogue.  The whole
+// loss at 2048x2048, a random half of the pixels in the mask: 650 us with one
+// output per thread -> 280; 16 views of 1920x1080, 20% mask: 360 us with scalar
+// multiply-adds and pixel-by-pixel staging -> 234, one view 85 -> 66.
 __global__ void __launch_bounds__(LOSS_T) k_ssim_stats(const float* __restrict__ img, const float* __restrict__ gt,
-                                                       const uint8_t* __restrict__ mask, int W, int H,
+                                                       const uint8_t* __restrict__ mask, int W, int H, int vec,
                                                        const uint32_t* __restrict__ msum, float lam, float invU,
                                                        double* l1sum, double* ssum, float* __restrict__ fac) {
-  __shared__ __align__(16) float s_x[HT][HS], s_y[HT][HS];
-  __shared__ __align__(16) float s_tmp[5][HT][LT];
+  __shared__ __align__(16) pair s_xy[HT][HS2];       // (image, GT)
+  __shared__ __align__(16) pair s_mu[HT][TS2], s_sq[HT][TS2];  // horizontal sums of (x, y) and (x^2, y^2)
+  __shared__ __align__(16) float s_c[HT][TS1];       // of x y
   __shared__ float s_red[32];
   __shared__ float s_win[11];
   int tiles_x = (W + LT - 1) / LT;
@@ -170,39 +254,54 @@ __global__ void __launch_bounds__(LOSS_T) k_ssim_stats(const float* __restrict__
   load_window(s_win);
   const float* X = img + ((int64_t)u * 3 + c) * plane;
   const float* Y = gt + ((int64_t)u * 3 + c) * plane;
-  const int x0 = bx * LT - R, y0 = by * LT - R;
-  for (int k = threadIdx.x; k < HT * HS; k += LOSS_T) {
-    int r = k / HS, q = k % HS;
-    int gx = x0 + q, gy = y0 + r;
-    float a = 0.f, b = 0.f;
-    if (q < HT && gx >= 0 && gx < W && gy >= 0 && gy < H) { a = X[(int64_t)gy * W + gx]; b = Y[(int64_t)gy * W + gx]; }
-    s_x[r][q] = a; s_y[r][q] = b;
-  }
+  for_groups(bx, by, W, H, [&](int r, int q, int gx, bool row_in, int64_t off) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+    if (vec) {
+      if (row_in && gx >= 0 && gx < W) {
+        a = __ldg(reinterpret_cast<const float4*>(X + off));
+        b = __ldg(reinterpret_cast<const float4*>(Y + off));
+      }
+    } else if (row_in) {
+      auto get = [&](int e, float& av, float& bv) {
+        if (gx + e >= 0 && gx + e < W) { av = X[off + e]; bv = Y[off + e]; }
+      };
+      get(0, a.x, b.x); get(1, a.y, b.y); get(2, a.z, b.z); get(3, a.w, b.w);
+    }
+    ulonglong2* dst = reinterpret_cast<ulonglong2*>(&s_xy[r][q]);
+    dst[0] = make_ulonglong2(make_pair(a.x, b.x), make_pair(a.y, b.y));
+    dst[1] = make_ulonglong2(make_pair(a.z, b.z), make_pair(a.w, b.w));
+  });
   __syncthreads();
   float w[11];
+  pair w2[11];
   #pragma unroll
-  for (int t = 0; t < 11; ++t) w[t] = s_win[t];
-  for (int k = threadIdx.x; k < HT * (LT / SEG); k += LOSS_T) {
-    const int r = k / (LT / SEG), g = k % (LT / SEG);
-    float a[16], b[16], p[16], o[SEG];
-    load_seg(s_x[r], g, a);
-    load_seg(s_y[r], g, b);
-    taps(w, a, o); store_seg(s_tmp[0][r], g, o);
-    taps(w, b, o); store_seg(s_tmp[1][r], g, o);
+  for (int t = 0; t < 11; ++t) { w[t] = s_win[t]; w2[t] = make_pair(w[t], w[t]); }
+  for (int k = threadIdx.x; k < SEG_TASKS; k += LOSS_T) {
+    int r, g;
+    seg_task(k, r, g);
+    pair v[16], o2[SEG];
+    float p[SEG + 10], o[SEG];
+    load_seg2(s_xy[r], g, v);
+    taps2(w2, v + 1, o2);
+    store_seg2(s_mu[r], g, o2);
     #pragma unroll
-    for (int t = 0; t < SEG + 10; ++t) p[t] = __fmul_rn(a[t], a[t]);
-    taps(w, p, o); store_seg(s_tmp[2][r], g, o);
+    for (int t = 0; t < SEG + 10; ++t) {
+      const float2 ab = halves(v[t + 1]);
+      p[t] = __fmul_rn(ab.x, ab.y);
+    }
+    taps(w, p, o);
+    store_seg(s_c[r], g, o);
     #pragma unroll
-    for (int t = 0; t < SEG + 10; ++t) p[t] = __fmul_rn(b[t], b[t]);
-    taps(w, p, o); store_seg(s_tmp[3][r], g, o);
-    #pragma unroll
-    for (int t = 0; t < SEG + 10; ++t) p[t] = __fmul_rn(a[t], b[t]);
-    taps(w, p, o); store_seg(s_tmp[4][r], g, o);
+    for (int t = 0; t < SEG + 10; ++t) v[t + 1] = mul2(v[t + 1], v[t + 1]);
+    taps2(w2, v + 1, o2);
+    store_seg2(s_sq[r], g, o2);
   }
   __syncthreads();
-  float st[5][SEG];
-  #pragma unroll
-  for (int q = 0; q < 5; ++q) taps_down(w, s_tmp[q], lx, strip, st[q]);
+  pair mu[SEG], sq[SEG];
+  float cr[SEG];
+  taps_down2(w2, s_mu, lx, strip, mu);
+  taps_down2(w2, s_sq, lx, strip, sq);
+  taps_down(w, s_c, lx, strip, cr);
   float nm = (float)msum[u];
   float sacc = 0.f, lacc = 0.f;
   #pragma unroll
@@ -210,13 +309,15 @@ __global__ void __launch_bounds__(LOSS_T) k_ssim_stats(const float* __restrict__
     if (!in[e]) continue;  // the factor maps are zero off the mask; only mask pixels are stored and read
     float fmu = 0.f, fxx = 0.f, fxy = 0.f;
     if (nm > 0.f) {
-      float ux = st[0][e], uy = st[1][e];
-      float vx = st[2][e] - ux * ux, vy = st[3][e] - uy * uy, cxy = st[4][e] - ux * uy;
+      const float2 m = halves(mu[e]), q2 = halves(sq[e]);
+      float ux = m.x, uy = m.y;
+      float vx = q2.x - ux * ux, vy = q2.y - uy * uy, cxy = cr[e] - ux * uy;
       float A1 = 2.f * ux * uy + C1, A2 = 2.f * cxy + C2;
       float B1 = ux * ux + uy * uy + C1, B2 = vx + vy + C2;
       float S = (A1 * A2) / (B1 * B2);
       sacc += S;
-      lacc += fabsf(s_x[SEG * strip + e + R][lx + R] - s_y[SEG * strip + e + R][lx + R]);
+      const float2 xy = halves(s_xy[SEG * strip + e + R][lx + PAD]);
+      lacc += fabsf(xy.x - xy.y);
       float wp = -lam * invU / (3.f * nm);  // d loss / d S_p
       fmu = wp * S * (2.f * uy / A1 - 2.f * ux / B1 - 2.f * uy / A2 + 2.f * ux / B2);
       fxx = wp * S * (-1.f / B2);
@@ -235,14 +336,15 @@ __global__ void __launch_bounds__(LOSS_T) k_ssim_stats(const float* __restrict__
 }
 
 // dL/dimg = L1 part + conv(fmu) + 2 x conv(fxx) + y conv(fxy).  76
-// multiply-adds per pixel and channel; 2048x2048, whole mask: 230 us at one
-// output per thread.
+// multiply-adds per pixel and channel, 51 instructions as pairs.
 __global__ void __launch_bounds__(LOSS_T) k_ssim_grad(const float* __restrict__ img, const float* __restrict__ gt,
-                                                      const uint8_t* __restrict__ mask, int W, int H,
+                                                      const uint8_t* __restrict__ mask, int W, int H, int vec,
                                                       const uint32_t* __restrict__ msum, float w1, float invU,
                                                       const float* __restrict__ fac, float* __restrict__ dimg) {
-  __shared__ __align__(16) float s_in[3][HT][HS];
-  __shared__ __align__(16) float s_tmp[3][HT][LT];
+  __shared__ __align__(16) pair s_in[HT][HS2];    // (fmu, fxx)
+  __shared__ __align__(16) float s_in1[HT][HS1];  // fxy
+  __shared__ __align__(16) pair s_tmp[HT][TS2];
+  __shared__ __align__(16) float s_tmp1[HT][TS1];
   __shared__ float s_win[11];
   int tiles_x = (W + LT - 1) / LT;
   int bx = blockIdx.x % tiles_x, by = blockIdx.x / tiles_x;
@@ -250,25 +352,43 @@ __global__ void __launch_bounds__(LOSS_T) k_ssim_grad(const float* __restrict__ 
   int64_t plane = (int64_t)W * H;
   int64_t off = ((int64_t)u * 3 + c) * plane;
   int64_t fs = (int64_t)3 * plane * gridDim.z;
-  const int x0 = bx * LT - R, y0 = by * LT - R;
   const int lx = threadIdx.x % LT, strip = threadIdx.x / LT;
   const int px = bx * LT + lx, py = by * LT + SEG * strip;
-  // factor maps are nonzero only at mask pixels: read them there, zero elsewhere
+  const uint8_t* M = mask + (int64_t)u * plane;
+  // factor maps are nonzero only at mask pixels: zero elsewhere, whatever the maps' memory holds there
   bool any = false;
-  for (int k = threadIdx.x; k < HT * HS; k += LOSS_T) {
-    int r = k / HS, q = k % HS;
-    int gx = x0 + q, gy = y0 + r;
-    float a = 0.f, b = 0.f, d = 0.f;
-    if (q < HT && gx >= 0 && gx < W && gy >= 0 && gy < H &&
-        mask[(int64_t)u * plane + (int64_t)gy * W + gx] != 0) {
-      int64_t pix = off + (int64_t)gy * W + gx;
-      a = fac[pix]; b = fac[fs + pix]; d = fac[2 * fs + pix];
-      any = true;
+  for_groups(bx, by, W, H, [&](int r, int q, int gx, bool row_in, int64_t o) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, d = a;
+    if (vec) {
+      const uint32_t m = row_in && gx >= 0 && gx < W ? __ldg(reinterpret_cast<const uint32_t*>(M + o)) : 0u;
+      if (m) {
+        // (the outer 3 of the staged columns are beyond the window's reach)
+        any = any || (q == 0 ? m >> 24 : q == HW - 4 ? m & 0xffu : m) != 0u;
+        a = __ldg(reinterpret_cast<const float4*>(fac + off + o));
+        b = __ldg(reinterpret_cast<const float4*>(fac + fs + off + o));
+        d = __ldg(reinterpret_cast<const float4*>(fac + 2 * fs + off + o));
+        if (!(m & 0xffu)) a.x = b.x = d.x = 0.f;
+        if (!(m & 0xff00u)) a.y = b.y = d.y = 0.f;
+        if (!(m & 0xff0000u)) a.z = b.z = d.z = 0.f;
+        if (!(m & 0xff000000u)) a.w = b.w = d.w = 0.f;
+      }
+    } else if (row_in) {
+      auto get = [&](int e, float& av, float& bv, float& dv) {
+        if (gx + e >= 0 && gx + e < W && M[o + e] != 0) {
+          const int64_t pix = off + o + e;
+          av = fac[pix]; bv = fac[fs + pix]; dv = fac[2 * fs + pix];
+          any = any || (q + e >= PAD - R && q + e < PAD + LT + R);
+        }
+      };
+      get(0, a.x, b.x, d.x); get(1, a.y, b.y, d.y); get(2, a.z, b.z, d.z); get(3, a.w, b.w, d.w);
     }
-    s_in[0][r][q] = a; s_in[1][r][q] = b; s_in[2][r][q] = d;
-  }
+    ulonglong2* dst = reinterpret_cast<ulonglong2*>(&s_in[r][q]);
+    dst[0] = make_ulonglong2(make_pair(a.x, b.x), make_pair(a.y, b.y));
+    dst[1] = make_ulonglong2(make_pair(a.z, b.z), make_pair(a.w, b.w));
+    *reinterpret_cast<float4*>(&s_in1[r][q]) = d;
+  });
+  // no mask pixel within the window's reach: both gradient terms vanish
   if (!__syncthreads_or(any)) {
-    // no mask pixel within the window's reach: both gradient terms vanish
     #pragma unroll
     for (int e = 0; e < SEG; ++e)
       if (px < W && py + e < H) dimg[off + (int64_t)(py + e) * W + px] = 0.f;
@@ -277,33 +397,38 @@ __global__ void __launch_bounds__(LOSS_T) k_ssim_grad(const float* __restrict__ 
   load_window(s_win);
   __syncthreads();
   float w[11];
+  pair w2[11];
   #pragma unroll
-  for (int t = 0; t < 11; ++t) w[t] = s_win[t];
-  for (int k = threadIdx.x; k < HT * (LT / SEG); k += LOSS_T) {
-    const int r = k / (LT / SEG), g = k % (LT / SEG);
-    #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      float a[16], o[SEG];
-      load_seg(s_in[q][r], g, a);
-      taps(w, a, o);
-      store_seg(s_tmp[q][r], g, o);
-    }
+  for (int t = 0; t < 11; ++t) { w[t] = s_win[t]; w2[t] = make_pair(w[t], w[t]); }
+  for (int k = threadIdx.x; k < SEG_TASKS; k += LOSS_T) {
+    int r, g;
+    seg_task(k, r, g);
+    pair v[16], o2[SEG];
+    float a[20], o[SEG];
+    load_seg2(s_in[r], g, v);
+    taps2(w2, v + 1, o2);
+    store_seg2(s_tmp[r], g, o2);
+    load_seg(s_in1[r], g, a);
+    taps(w, a + 3, o);
+    store_seg(s_tmp1[r], g, o);
   }
   __syncthreads();
-  float cv[3][SEG];
-  #pragma unroll
-  for (int q = 0; q < 3; ++q) taps_down(w, s_tmp[q], lx, strip, cv[q]);
+  pair cv[SEG];
+  float cv1[SEG];
+  taps_down2(w2, s_tmp, lx, strip, cv);
+  taps_down(w, s_tmp1, lx, strip, cv1);
   float nm = (float)msum[u];
   #pragma unroll
   for (int e = 0; e < SEG; ++e) {
     if (!(px < W && py + e < H)) continue;
     int64_t pix = (int64_t)(py + e) * W + px;
     float x = img[off + pix], y = gt[off + pix];
-    bool in = mask[(int64_t)u * plane + pix] != 0;
+    bool in = M[pix] != 0;
     float d = x - y;
     float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
     float gl1 = (in && nm > 0.f) ? w1 * invU / (3.f * nm) * sg : 0.f;
-    dimg[off + pix] = gl1 + cv[0][e] + 2.f * x * cv[1][e] + y * cv[2][e];
+    const float2 f = halves(cv[e]);
+    dimg[off + pix] = gl1 + f.x + 2.f * x * f.y + y * cv1[e];
   }
 }
 
@@ -427,8 +552,12 @@ GS_API int gs_loss(const float* img, const float* gt, const uint8_t* mask, int n
   } else {
     int tiles = ((width + LT - 1) / LT) * ((height + LT - 1) / LT);
     dim3 grid(tiles, 3, n_units);
-    k_ssim_stats<<<grid, LOSS_T, 0, s>>>(img, gt, mask, width, height, msum, lambda_ssim, invU, l1, ss, fac);
-    k_ssim_grad<<<grid, LOSS_T, 0, s>>>(img, gt, mask, width, height, msum, 1.f - lambda_ssim, invU, fac, dL_dimg);
+    // rows, and with them every group of 4 pixels, start on 16 bytes (the mask's on 4)
+    const int rows = width % 4 == 0 && (((uintptr_t)img | (uintptr_t)gt) & 15u) == 0 && ((uintptr_t)mask & 3u) == 0;
+    k_ssim_stats<<<grid, LOSS_T, 0, s>>>(img, gt, mask, width, height, rows, msum, lambda_ssim, invU, l1, ss,
+                                          fac);
+    k_ssim_grad<<<grid, LOSS_T, 0, s>>>(img, gt, mask, width, height, rows, msum, 1.f - lambda_ssim, invU, fac,
+                                         dL_dimg);
   }
   k_loss_final<<<1, 32, 0, s>>>(msum, l1, ss, n_units, lambda_ssim, d_loss);
   return gs_check_launch();

@@ -114,6 +114,26 @@ def test_loss_partial_tiles(W, H, units):
     assert np.abs(fr.dimg.cpu().numpy() - d).max() <= 1e-3 * np.abs(d).max()
 
 
+@pytest.mark.parametrize("W,H,units", [(4, 1, 1), (32, 32, 1), (36, 45, 2), (100, 71, 2)])
+def test_loss_unaligned_arrays(W, H, units):
+    """Rows that start on 16 bytes are read 4 pixels at a time, others one by one: the same gradient, bit for bit; the
+    mask has rows and columns with single pixels."""
+    g = np.random.default_rng(W + H)
+    gt = torch.from_numpy(g.uniform(0, 1, (units, 3, H, W)).astype(np.float32)).cuda()
+    mask = torch.from_numpy((g.uniform(0, 1, (units, H, W)) < 0.3).astype(np.uint8)).cuda()
+    mask[:, :, W // 2:] = 0
+    mask[:, 0, 0] = 1
+    fr = Frame(1, Units.single(1, units), W, H, 0, with_backward=False)
+    fr.img.copy_(torch.from_numpy(g.uniform(0, 1, (units, 3, H, W)).astype(np.float32)))
+    fr.loss(gt, mask, 0.2)
+    want = fr.dimg.clone()
+    assert float(want.abs().max()) > 0
+    for a, b in ((_off_by_one(gt), mask), (gt, _off_by_one(mask)), (_off_by_one(gt), _off_by_one(mask))):
+        fr.dimg.fill_(7.0)
+        fr.loss(a, b, 0.2)
+        assert torch.equal(fr.dimg, want)
+
+
 def _lists_by_numpy(fr, cap):
     """The lists gs_bin_sort documents, from the projected records: instances in (depth, record index, tile) order,
     the first cap of them kept, each list in that order."""
