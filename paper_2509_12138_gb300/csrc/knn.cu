@@ -62,6 +62,7 @@ __device__ __forceinline__ int64_t cell_of(const Grid& g, float x, float y, floa
 
 __global__ void k_cell_count(const float* __restrict__ pts, int64_t n, Grid g, uint32_t* __restrict__ count,
                              uint32_t* __restrict__ rank) {
+  gs_wait_previous();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   rank[i] = atomicAdd(&count[cell_of(g, pts[3 * i], pts[3 * i + 1], pts[3 * i + 2])], 1u);
@@ -69,6 +70,7 @@ __global__ void k_cell_count(const float* __restrict__ pts, int64_t n, Grid g, u
 
 __global__ void k_cell_scatter(const float* __restrict__ pts, int64_t n, Grid g, const uint32_t* __restrict__ start,
                                const uint32_t* __restrict__ rank, float4* __restrict__ sorted) {
+  gs_wait_previous();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
@@ -129,6 +131,7 @@ template <int K>
 __global__ void __launch_bounds__(KNN_T) k_knn_query(int64_t n, Grid g, const uint32_t* __restrict__ start,
                                                      const float4* __restrict__ sorted, int vec,
                                                      int* __restrict__ out_idx, float* __restrict__ out_dist) {
+  gs_wait_previous();
   __shared__ unsigned long long s_best[K][KNN_T];
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= n) return;
@@ -276,14 +279,14 @@ GS_API int gs_knn(const float* points, int64_t n, int k, const float* grid_lo, f
   float4* sorted = (float4*)(ws + L.sorted);
   if (cudaMemsetAsync(start, 0, sizeof(uint32_t) * cells, s) != cudaSuccess) return GS_ERR_CUDA;
   unsigned nb = (unsigned)((n + 255) / 256);
-  k_cell_count<<<nb, 256, 0, s>>>(points, n, g, start, rank);
+  gs_launch(k_cell_count, nb, 256, 0, s, points, n, g, start, rank);
   // start[c] = exclusive prefix (in place); start[cells] = n
   int r = gs_scan_u32(start, start, cells, ws + L.scan, start + cells, s);
   if (r != GS_OK) return r;
-  k_cell_scatter<<<nb, 256, 0, s>>>(points, n, g, start, rank, sorted);
+  gs_launch(k_cell_scatter, nb, 256, 0, s, points, n, g, start, rank, sorted);
   unsigned qb = (unsigned)((n + KNN_T - 1) / KNN_T);
   const int vec = (((uintptr_t)idx | (uintptr_t)dist) & 15u) == 0;
-#define GS_KQ(K) k_knn_query<K><<<qb, KNN_T, 0, s>>>(n, g, start, sorted, vec, idx, dist)
+#define GS_KQ(K) gs_launch(k_knn_query<K>, qb, KNN_T, 0, s, n, g, start, sorted, vec, idx, dist)
   switch (k) {
     case 3: GS_KQ(3); break;
     case 8: GS_KQ(8); break;

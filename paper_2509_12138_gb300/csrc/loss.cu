@@ -73,6 +73,7 @@ __device__ __forceinline__ float block_sum(float v, float* s) {
 
 // Mask pixels per unit.  vec: the units' masks start on 16 bytes and hold a multiple of 16 (16-byte loads).
 __global__ void k_mask_count(const uint8_t* __restrict__ mask, int64_t plane, int vec, uint32_t* msum) {
+  gs_wait_previous();
   __shared__ float s[32];
   int u = blockIdx.y;
   uint32_t c = 0;
@@ -95,6 +96,7 @@ __global__ void k_mask_count(const uint8_t* __restrict__ mask, int64_t plane, in
 __global__ void k_l1(const float* __restrict__ img, const float* __restrict__ gt, const uint8_t* __restrict__ mask,
                      int64_t plane, const uint32_t* __restrict__ msum, float w1, float invU, double* l1sum,
                      float* __restrict__ dimg) {
+  gs_wait_previous();
   __shared__ float s[32];
   int u = blockIdx.y;
   float acc = 0.f;
@@ -226,12 +228,13 @@ __device__ __forceinline__ void for_groups(int bx, int by, int W, int H, F f) {
 // (127 multiply-adds per pixel and channel with the halo rows, 76 instructions
 // as pairs); the rest is staging and the divisions of the epilogue.  The whole
 // loss at 2048x2048, a random half of the pixels in the mask: 650 us with one
-// output per thread -> 280; 16 views of 1920x1080, 20% mask: 360 us with scalar
+// output per thread -> 280; 8 views of 1920x1080, 20% mask: 360 us with scalar
 // multiply-adds and pixel-by-pixel staging -> 234, one view 85 -> 66.
 __global__ void __launch_bounds__(LOSS_T) k_ssim_stats(const float* __restrict__ img, const float* __restrict__ gt,
                                                        const uint8_t* __restrict__ mask, int W, int H, int vec,
                                                        const uint32_t* __restrict__ msum, float lam, float invU,
                                                        double* l1sum, double* ssum, float* __restrict__ fac) {
+  gs_wait_previous();
   __shared__ __align__(16) pair s_xy[HT][HS2];       // (image, GT)
   __shared__ __align__(16) pair s_mu[HT][TS2], s_sq[HT][TS2];  // horizontal sums of (x, y) and (x^2, y^2)
   __shared__ __align__(16) float s_c[HT][TS1];       // of x y
@@ -341,6 +344,7 @@ __global__ void __launch_bounds__(LOSS_T) k_ssim_grad(const float* __restrict__ 
                                                       const uint8_t* __restrict__ mask, int W, int H, int vec,
                                                       const uint32_t* __restrict__ msum, float w1, float invU,
                                                       const float* __restrict__ fac, float* __restrict__ dimg) {
+  gs_wait_previous();
   __shared__ __align__(16) pair s_in[HT][HS2];    // (fmu, fxx)
   __shared__ __align__(16) float s_in1[HT][HS1];  // fxy
   __shared__ __align__(16) pair s_tmp[HT][TS2];
@@ -435,6 +439,7 @@ __global__ void __launch_bounds__(LOSS_T) k_ssim_grad(const float* __restrict__ 
 // the units' losses, one per lane (a thread summing them alone waits for each unit's loads in turn)
 __global__ void __launch_bounds__(32) k_loss_final(const uint32_t* msum, const double* l1sum, const double* ssum, int U,
                                                    float lam, float* out) {
+  gs_wait_previous();
   double acc = 0.0;
   for (int u = threadIdx.x; u < U; u += 32) {
     double nm = (double)msum[u];
@@ -454,6 +459,7 @@ __global__ void __launch_bounds__(32) k_loss_final(const uint32_t* msum, const d
 __global__ void __launch_bounds__(256) k_bg_sum(const float* __restrict__ final_T, const uint8_t* __restrict__ mask,
                                                 int64_t plane, unsigned long long* __restrict__ cnt,
                                                 double* __restrict__ sum) {
+  gs_wait_previous();
   int u = blockIdx.y;
   const float* T = final_T + (int64_t)u * plane;
   const uint8_t* m = mask + (int64_t)u * plane;
@@ -475,6 +481,7 @@ __global__ void __launch_bounds__(256) k_bg_sum(const float* __restrict__ final_
 __global__ void __launch_bounds__(256) k_bg_grad(const uint8_t* __restrict__ mask, int64_t plane,
                                                  const unsigned long long* __restrict__ cnt, float lam, float invU,
                                                  float* __restrict__ dLdT) {
+  gs_wait_previous();
   int u = blockIdx.y;
   unsigned long long n = cnt[u];
   float g = n ? -lam * invU / (float)n : 0.f;
@@ -485,6 +492,7 @@ __global__ void __launch_bounds__(256) k_bg_grad(const uint8_t* __restrict__ mas
 }
 
 __global__ void k_bg_final(const unsigned long long* cnt, const double* sum, int U, float lam, float* out) {
+  gs_wait_previous();
   double acc = 0.0;
   for (int u = 0; u < U; ++u)
     if (cnt[u]) acc += sum[u] / (double)cnt[u];
@@ -514,9 +522,9 @@ GS_API int gs_bg_penalty(const float* final_T, const uint8_t* mask, int n_units,
   int64_t plane = (int64_t)width * height;
   int gx = (int)((plane + 255) / 256);
   if (gx > 1024) gx = 1024;
-  k_bg_sum<<<dim3(gx, n_units), 256, 0, s>>>(final_T, mask, plane, cnt, sum);
-  k_bg_grad<<<dim3(gx, n_units), 256, 0, s>>>(mask, plane, cnt, lambda_bg, 1.f / n_units, dL_dT);
-  k_bg_final<<<1, 1, 0, s>>>(cnt, sum, n_units, lambda_bg, d_loss);
+  gs_launch(k_bg_sum, dim3(gx, n_units), 256, 0, s, final_T, mask, plane, cnt, sum);
+  gs_launch(k_bg_grad, dim3(gx, n_units), 256, 0, s, mask, plane, cnt, lambda_bg, 1.f / n_units, dL_dT);
+  gs_launch(k_bg_final, 1, 1, 0, s, cnt, sum, n_units, lambda_bg, d_loss);
   return gs_check_launch();
 }
 
@@ -546,20 +554,20 @@ GS_API int gs_loss(const float* img, const float* gt, const uint8_t* mask, int n
   int gx = (int)((plane + 255) / 256);
   if (gx > 1024) gx = 1024;
   const int vec = ((uintptr_t)mask & 15u) == 0 && plane % 16 == 0;
-  k_mask_count<<<dim3(gx, n_units), 256, 0, s>>>(mask, plane, vec, msum);
+  gs_launch(k_mask_count, dim3(gx, n_units), 256, 0, s, mask, plane, vec, msum);
   if (lambda_ssim == 0.f) {
-    k_l1<<<dim3(gx, n_units), 256, 0, s>>>(img, gt, mask, plane, msum, 1.f, invU, l1, dL_dimg);
+    gs_launch(k_l1, dim3(gx, n_units), 256, 0, s, img, gt, mask, plane, msum, 1.f, invU, l1, dL_dimg);
   } else {
     int tiles = ((width + LT - 1) / LT) * ((height + LT - 1) / LT);
     dim3 grid(tiles, 3, n_units);
     // rows, and with them every group of 4 pixels, start on 16 bytes (the mask's on 4)
     const int rows = width % 4 == 0 && (((uintptr_t)img | (uintptr_t)gt) & 15u) == 0 && ((uintptr_t)mask & 3u) == 0;
-    k_ssim_stats<<<grid, LOSS_T, 0, s>>>(img, gt, mask, width, height, rows, msum, lambda_ssim, invU, l1, ss,
-                                          fac);
-    k_ssim_grad<<<grid, LOSS_T, 0, s>>>(img, gt, mask, width, height, rows, msum, 1.f - lambda_ssim, invU, fac,
-                                         dL_dimg);
+    gs_launch(k_ssim_stats, grid, LOSS_T, 0, s, img, gt, mask, width, height, rows, msum, lambda_ssim, invU, l1, ss,
+        fac);
+    gs_launch(k_ssim_grad, grid, LOSS_T, 0, s, img, gt, mask, width, height, rows, msum, 1.f - lambda_ssim, invU,
+        fac, dL_dimg);
   }
-  k_loss_final<<<1, 32, 0, s>>>(msum, l1, ss, n_units, lambda_ssim, d_loss);
+  gs_launch(k_loss_final, 1, 32, 0, s, msum, l1, ss, n_units, lambda_ssim, d_loss);
   return gs_check_launch();
 }
 

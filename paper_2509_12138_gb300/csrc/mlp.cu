@@ -319,6 +319,7 @@ __global__ void __launch_bounds__(FWD_T, 3) k_mlp_forward(const float* __restric
                                                          const int* __restrict__ knn_idx,
                                                          const float* __restrict__ knn_dist, int64_t n, bool vec,
                                                          const float* __restrict__ w, float* __restrict__ out) {
+  gs_wait_previous();
   extern __shared__ __align__(16) char sm[];
   stage_weights(w, sm, false);
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -362,6 +363,7 @@ __device__ __forceinline__ void write_init(float4* __restrict__ params, int64_t 
 
 __global__ void k_plain_init(const float* __restrict__ knn_dist, int k, int64_t n, float logit_default,
                              float4* __restrict__ params, int64_t N) {
+  gs_wait_previous();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   float d3 = (knn_dist[i * k] + knn_dist[i * k + 1] + knn_dist[i * k + 2]) / 3.f;
@@ -373,6 +375,7 @@ __global__ void __launch_bounds__(FWD_T, 3) k_mlp_init(const float* __restrict__
                                                       const float* __restrict__ knn_dist, int64_t n, bool vec,
                                                       const float* __restrict__ w, float logit_default,
                                                       float4* __restrict__ params, int64_t N) {
+  gs_wait_previous();
   extern __shared__ __align__(16) char sm[];
   stage_weights(w, sm, false);
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -418,6 +421,7 @@ __global__ void __launch_bounds__(CONS_T + PROD_T, 1)
     k_mlp_train(const float* __restrict__ pts, const float* __restrict__ nrm, const int* __restrict__ knn_idx,
                 const float* __restrict__ knn_dist, const float* __restrict__ target, int64_t n, bool vec,
                 const float* __restrict__ w, float scale, float* __restrict__ grad, float* __restrict__ loss) {
+  gs_wait_previous();
   extern __shared__ __align__(16) char sm[];
   int* s_idx = (int*)(sm + Smem::Idx);
   float2* s_dbar = (float2*)(sm + Smem::Dbar);
@@ -656,6 +660,7 @@ __global__ void __launch_bounds__(FWD_T) k_features_out(const float* __restrict_
                                                         const int* __restrict__ knn_idx,
                                                         const float* __restrict__ knn_dist, int64_t n, bool vec,
                                                         uint16_t* __restrict__ X) {
+  gs_wait_previous();
   extern __shared__ __align__(16) char sm[];
   int64_t nb = (n + BATCH - 1) / BATCH;
   const uint16_t* sX = (const uint16_t*)(sm + Smem::X);
@@ -700,8 +705,8 @@ GS_API int gs_mlp_features(const float* points, const float* normals, const int3
   if (!knn_args_ok(points, normals, knn_idx, knn_dist, n) || !features) return GS_ERR_INVALID;
   if (n == 0) return GS_OK;
   if (set_smem(k_features_out, Smem::FWD_END) != GS_OK) return GS_ERR_CUDA;
-  k_features_out<<<grid_for(n, 3), FWD_T, Smem::FWD_END, (cudaStream_t)stream>>>(
-      points, normals, knn_idx, knn_dist, n, rows_aligned(knn_idx, knn_dist), features);
+  gs_launch(k_features_out, grid_for(n, 3), FWD_T, Smem::FWD_END, (cudaStream_t)stream, points, normals, knn_idx,
+      knn_dist, n, rows_aligned(knn_idx, knn_dist), features);
   return gs_check_launch();
 }
 
@@ -711,8 +716,8 @@ GS_API int gs_mlp_forward(const float* points, const float* normals, const int32
   if (!knn_args_ok(points, normals, knn_idx, knn_dist, n) || !weights || !out) return GS_ERR_INVALID;
   if (n == 0) return GS_OK;
   if (set_smem(k_mlp_forward, Smem::FWD_END) != GS_OK) return GS_ERR_CUDA;
-  k_mlp_forward<<<grid_for(n, 3), FWD_T, Smem::FWD_END, (cudaStream_t)stream>>>(
-      points, normals, knn_idx, knn_dist, n, rows_aligned(knn_idx, knn_dist), weights, out);
+  gs_launch(k_mlp_forward, grid_for(n, 3), FWD_T, Smem::FWD_END, (cudaStream_t)stream, points, normals, knn_idx,
+      knn_dist, n, rows_aligned(knn_idx, knn_dist), weights, out);
   return gs_check_launch();
 }
 
@@ -729,8 +734,8 @@ GS_API int gs_mlp_train_step(const float* points, const float* normals, const in
     return GS_ERR_CUDA;
   if (set_smem(k_mlp_train, Smem::TRAIN_END) != GS_OK) return GS_ERR_CUDA;
   float scale = 1.0f / (8.0f * (float)n);
-  k_mlp_train<<<grid_for(n, 1), CONS_T + PROD_T, Smem::TRAIN_END, s>>>(
-      points, normals, knn_idx, knn_dist, targets, n, rows_aligned(knn_idx, knn_dist), weights, scale, grad, d_loss);
+  gs_launch(k_mlp_train, grid_for(n, 1), CONS_T + PROD_T, Smem::TRAIN_END, s, points, normals, knn_idx, knn_dist,
+      targets, n, rows_aligned(knn_idx, knn_dist), weights, scale, grad, d_loss);
   int r = gs_check_launch();
   if (r != GS_OK) return r;
   float lr4[4] = {lr, lr, lr, lr};
@@ -751,13 +756,12 @@ GS_API int gs_init_gaussians(const float* points, const float* normals, const in
                         cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return GS_ERR_CUDA;
   if (!weights) {
-    k_plain_init<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(knn_dist, knn_k, n, logit_default, (float4*)params,
-                                                             n_gauss);
+    gs_launch(k_plain_init, (unsigned)((n + 255) / 256), 256, 0, s, knn_dist, knn_k, n, logit_default,
+        (float4*)params, n_gauss);
   } else {
     if (set_smem(k_mlp_init, Smem::INIT_END) != GS_OK) return GS_ERR_CUDA;
-    k_mlp_init<<<grid_for(n, 3), FWD_T, Smem::INIT_END, s>>>(points, normals, knn_idx, knn_dist, n,
-                                                             rows_aligned(knn_idx, knn_dist), weights, logit_default,
-                                                             (float4*)params, n_gauss);
+    gs_launch(k_mlp_init, grid_for(n, 3), FWD_T, Smem::INIT_END, s, points, normals, knn_idx, knn_dist, n,
+        rows_aligned(knn_idx, knn_dist), weights, logit_default, (float4*)params, n_gauss);
   }
   return gs_check_launch();
 }

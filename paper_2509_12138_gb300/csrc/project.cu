@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(256) k_preprocess(const float4* __restrict__ p
                                                     float4* __restrict__ rgb, float* __restrict__ depth,
                                                     int* __restrict__ radius, uint32_t* __restrict__ tiles,
                                                     int* status) {
+  gs_wait_previous();
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= U.proj_base[U.n]) return;
   int u = unit_of(U, p);
@@ -519,6 +520,7 @@ __global__ void __launch_bounds__(128) k_project_bwd(const float4* __restrict__ 
                                                      const float4* __restrict__ gco,
                                                      const float4* __restrict__ grgb,
                                                      float4* __restrict__ grads) {
+  gs_wait_previous();
   constexpr int NP = ShCount<DEG>::NP;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
@@ -551,6 +553,7 @@ __global__ void __launch_bounds__(256) k_adam(float4* __restrict__ p, float4* __
                                               int n_planes, AdamLR lr, int lr_steps, float b1, float b2,
                                               float eps, const int32_t* __restrict__ d_step, int zero,
                                               int* __restrict__ status) {
+  gs_wait_previous();
   __shared__ float4 s_lr[16];
   int t = *d_step + 1;
   if (threadIdx.x < n_planes) {
@@ -610,6 +613,7 @@ __global__ void __launch_bounds__(128) k_project_bwd_adam(float4* __restrict__ p
                                                           float b2, float eps, const int32_t* __restrict__ d_step,
                                                           float4* __restrict__ grads, int sparse,
                                                           int* __restrict__ status) {
+  gs_wait_previous();
   constexpr int NP = ShCount<DEG>::NP;
   constexpr int NPL = 3 + NP;
   __shared__ float4 s_lr[16];
@@ -715,6 +719,7 @@ __global__ void __launch_bounds__(PBA_T) k_project_bwd_adam1(float4* __restrict_
                                                            float b2, float eps, const int32_t* __restrict__ d_step,
                                                            float4* __restrict__ grads, int sparse,
                                                            int* __restrict__ status, NextProj nx) {
+  gs_wait_previous();
   constexpr int NC = ShCount<DEG>::NC;
   constexpr int NP = ShCount<DEG>::NP;
   constexpr int NPL = 3 + NP;
@@ -978,7 +983,8 @@ __global__ void __launch_bounds__(PBA_T) k_project_bwd_adam1(float4* __restrict_
                         nx.rgb + pidx, nx.depth + pidx, nx.radius + pidx, nx.tiles + pidx, status);
 }
 
-__global__ void k_step_advance(int32_t* s) { *s += 1; }
+__global__ void k_step_advance(int32_t* s) {
+  gs_wait_previous(); *s += 1; }
 
 }  // namespace
 
@@ -1062,9 +1068,8 @@ GS_API int gs_preprocess(const float* params, int64_t n_gauss, int sh_degree, co
   cudaStream_t s = (cudaStream_t)stream;
   const float4* p4 = (const float4*)params;
 #define GS_PRE(D)                                                                                   \
-  k_preprocess<D><<<grid, block, 0, s>>>(p4, n_gauss, U, O, cams, width, height, (float4*)proj->xy, \
-                                         (float4*)proj->conic_op, (float4*)proj->rgb, proj->depth,   \
-                                         proj->radius, proj->tiles, d_status)
+  gs_launch(k_preprocess<D>, grid, block, 0, s, p4, n_gauss, U, O, cams, width, height, (float4*)proj->xy,         \
+      (float4*)proj->conic_op, (float4*)proj->rgb, proj->depth, proj->radius, proj->tiles, d_status)
   switch (sh_degree) {
     case 0: GS_PRE(0); break;
     case 1: GS_PRE(1); break;
@@ -1090,9 +1095,8 @@ GS_API int gs_project_bwd(const float* params, int64_t n_gauss, int sh_degree, c
   dim3 block(128), grid((unsigned)((n_gauss + 127) / 128));
   cudaStream_t s = (cudaStream_t)stream;
 #define GS_PB(D)                                                                                           \
-  k_project_bwd<D><<<grid, block, 0, s>>>((const float4*)params, n_gauss, U, cams, proj->radius,          \
-                                          (const float2*)g2d->dxy, (const float4*)g2d->dconic_op,         \
-                                          (const float4*)g2d->drgb, (float4*)grads)
+  gs_launch(k_project_bwd<D>, grid, block, 0, s, (const float4*)params, n_gauss, U, cams, proj->radius,            \
+      (const float2*)g2d->dxy, (const float4*)g2d->dconic_op, (const float4*)g2d->drgb, (float4*)grads)
   switch (sh_degree) {
     case 0: GS_PB(0); break;
     case 1: GS_PB(1); break;
@@ -1125,16 +1129,15 @@ GS_API int gs_adam_step(float* params, float* grads, float* m, float* v, int64_t
   int64_t want = (total + 255) / 256;
   int64_t cap = (int64_t)sms * 8;
   unsigned grid = (unsigned)(want < cap ? want : cap);
-  k_adam<<<grid, 256, 0, (cudaStream_t)stream>>>((float4*)params, (float4*)grads, (float4*)m, (float4*)v, n_gauss,
-                                                 n_planes, lr, lr_steps, beta1, beta2, eps, d_step, zero_grad,
-                                                 d_status);
+  gs_launch(k_adam, grid, 256, 0, (cudaStream_t)stream, (float4*)params, (float4*)grads, (float4*)m, (float4*)v,
+      n_gauss, n_planes, lr, lr_steps, beta1, beta2, eps, d_step, zero_grad, d_status);
   return gs_check_launch();
 }
 
 GS_API int gs_step_advance(int32_t* d_step, gs_stream_t stream) {
   GS_RANGE("gs_step_advance");
   if (!d_step) return GS_ERR_INVALID;
-  k_step_advance<<<1, 1, 0, (cudaStream_t)stream>>>(d_step);
+  gs_launch(k_step_advance, 1, 1, 0, (cudaStream_t)stream, d_step);
   return gs_check_launch();
 }
 
@@ -1183,10 +1186,9 @@ static int project_bwd_adam_impl(float* params, int64_t n_gauss, int sh_degree, 
     dim3 grid1((unsigned)((n_gauss + PBA_T - 1) / PBA_T));
     size_t smem1 = sizeof(float4) * ((size_t)npl + 2 * PBA_R) * PBA_T;  // 23,552 B at degree 3
 #define GS_PBA1(D)                                                                                                \
-  k_project_bwd_adam1<D><<<grid1, PBA_T, smem1, s>>>((float4*)params, n_gauss, U, cams, proj->radius,            \
-                                                (const float2*)g2d->dxy, (const float4*)g2d->dconic_op,          \
-                                                (const float4*)g2d->drgb, (float4*)m, (float4*)v, lr, lr_steps,   \
-                                                beta1, beta2, eps, d_step, (float4*)grads, sparse, d_status, nx)
+  gs_launch(k_project_bwd_adam1<D>, grid1, PBA_T, smem1, s, (float4*)params, n_gauss, U, cams, proj->radius,       \
+      (const float2*)g2d->dxy, (const float4*)g2d->dconic_op, (const float4*)g2d->drgb, (float4*)m, (float4*)v,    \
+      lr, lr_steps, beta1, beta2, eps, d_step, (float4*)grads, sparse, d_status, nx)
     switch (sh_degree) {
       case 0: GS_PBA1(0); break;
       case 1: GS_PBA1(1); break;
@@ -1197,10 +1199,9 @@ static int project_bwd_adam_impl(float* params, int64_t n_gauss, int sh_degree, 
     return gs_check_launch();
   }
 #define GS_PBA(D)                                                                                                \
-  k_project_bwd_adam<D><<<grid, block, 0, s>>>((float4*)params, n_gauss, U, cams, proj->radius,                 \
-                                               (const float2*)g2d->dxy, (const float4*)g2d->dconic_op,          \
-                                               (const float4*)g2d->drgb, (float4*)m, (float4*)v, lr, lr_steps,   \
-                                               beta1, beta2, eps, d_step, (float4*)grads, sparse, d_status)
+  gs_launch(k_project_bwd_adam<D>, grid, block, 0, s, (float4*)params, n_gauss, U, cams, proj->radius,             \
+      (const float2*)g2d->dxy, (const float4*)g2d->dconic_op, (const float4*)g2d->drgb, (float4*)m, (float4*)v,    \
+      lr, lr_steps, beta1, beta2, eps, d_step, (float4*)grads, sparse, d_status)
   switch (sh_degree) {
     case 0: GS_PBA(0); break;
     case 1: GS_PBA(1); break;

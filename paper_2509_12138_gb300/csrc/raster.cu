@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(TILE_PIX) k_render_fwd(const uint2* __restrict
                                                          int n_tiles, float bg0, float bg1, float bg2,
                                                          float* __restrict__ img, float* __restrict__ final_T,
                                                          uint32_t* __restrict__ n_contrib) {
+  gs_wait_previous();
   const unsigned FULL = 0xffffffffu;
   __shared__ Rec s_rec[TILE_PIX / 32][32];
   int u, tile;
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(TILE_PIX) k_render_bwd(const uint2* __restrict
                                                          const float* __restrict__ dLdT, float* __restrict__ dxy,
                                                          float* __restrict__ dco, float* __restrict__ drgb,
                                                            unsigned long long* __restrict__ fixed) {
+  gs_wait_previous();
   const unsigned FULL = 0xffffffffu;
   __shared__ Rec s_rec[TILE_PIX / 32][32];
   int u, tile;
@@ -668,6 +670,7 @@ __global__ void __launch_bounds__(TILE_PIX) k_render_fwd_empty(const uint2* __re
                                                                uint32_t* __restrict__ n_contrib,
                                                                uint32_t* __restrict__ tickets,
                                                                uint32_t* __restrict__ qcount) {
+  gs_wait_previous();
   if (blockIdx.x == 0 && threadIdx.x == 0) { tickets[0] = 0u; tickets[1] = 0u; *qcount = 0u; }
   const uint2 rg = ranges[blockIdx.x];
   if (rg.y > rg.x) return;
@@ -761,6 +764,7 @@ __global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict
                                                          uint32_t* __restrict__ n_contrib,
                                                          uint32_t* __restrict__ queue, uint32_t qcap,
                                                          uint32_t* __restrict__ ticket) {
+  gs_wait_previous();
   __shared__ FwdScratch s_walk;
   const int lane = threadIdx.x & 31;
   const int lists = lists_in_use(job_base, NT);
@@ -846,6 +850,7 @@ __global__ void __launch_bounds__(32) k_render_fwd_chunk(const uint2* __restrict
                                                          int n_tiles, const uint32_t* __restrict__ n_contrib,
                                                          const uint32_t* __restrict__ queue, uint32_t qcap,
                                                          uint32_t* __restrict__ ticket) {
+  gs_wait_previous();
   __shared__ FwdScratch s_walk;
   const uint32_t total = queue[qcap];
   auto job = [&](uint32_t ent) {
@@ -968,6 +973,7 @@ __global__ void __launch_bounds__(32) k_render_fwd_combine(const uint32_t* __res
                                                            uint32_t* __restrict__ n_contrib,
                                                            uint32_t* __restrict__ queue, uint32_t qcap,
                                                            uint32_t* __restrict__ ticket) {
+  gs_wait_previous();
   if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0u;
   const uint32_t total = queue[qcap];
   for (uint32_t e = blockIdx.x; e < total; e += gridDim.x) {
@@ -1012,6 +1018,7 @@ __global__ void __launch_bounds__(32) k_render_fwd_stop(const uint2* __restrict_
                                                               uint32_t* __restrict__ n_contrib,
                                                               const uint32_t* __restrict__ queue, uint32_t qcap,
                                                               uint32_t* __restrict__ ticket) {
+  gs_wait_previous();
   __shared__ FwdScratch s_walk;
   const uint32_t total = queue[qcap];
   auto job = [&](uint32_t ent) {
@@ -1184,6 +1191,7 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
                                                            const float* __restrict__ dLdT, float* __restrict__ dxy,
                                                            float* __restrict__ dco, float* __restrict__ drgb,
                                                            uint32_t* __restrict__ ticket) {
+  gs_wait_previous();
   const unsigned FULL = 0xffffffffu;
   __shared__ Rec s_rec[32];
   // the resident warps take the (chunk job, pixel block) units from a ticket counter (zeroed before
@@ -1449,6 +1457,7 @@ __global__ void __launch_bounds__(32, 20) k_render_bwd_det(const uint2* __restri
                                                            const float* __restrict__ dLdT,
                                                            unsigned long long* __restrict__ fixed,
                                                            uint32_t* __restrict__ ticket) {
+  gs_wait_previous();
   const unsigned FULL = 0xffffffffu;
   __shared__ BwdScratch sc;
   // the resident warps take the (chunk job, pixel block) units from a ticket counter (zeroed before
@@ -1590,6 +1599,7 @@ __global__ void __launch_bounds__(32, 20) k_render_bwd_det(const uint2* __restri
 // bit length of the list length; order within a class is arbitrary and the
 // blend results do not depend on it).
 __global__ void k_order_hist(const uint2* __restrict__ ranges, int n, uint32_t* __restrict__ hist) {
+  gs_wait_previous();
   __shared__ uint32_t s[33];
   if (threadIdx.x < 33) s[threadIdx.x] = 0;
   __syncthreads();
@@ -1605,6 +1615,7 @@ __global__ void k_order_hist(const uint2* __restrict__ ranges, int n, uint32_t* 
 
 __global__ void k_order_scatter(const uint2* __restrict__ ranges, int n, const uint32_t* __restrict__ hist,
                                 uint32_t* __restrict__ cursor, uint32_t* __restrict__ order) {
+  gs_wait_previous();
   __shared__ uint32_t s_base[33];
   if (threadIdx.x == 0) {
     uint32_t acc = 0;
@@ -1633,6 +1644,7 @@ __global__ void __launch_bounds__(TILE_PIX) k_blend_pairs(const uint2* __restric
                                                           int n_tiles, const uint32_t* __restrict__ n_contrib,
                                                           const uint16_t* __restrict__ masks,
                                                           unsigned long long* __restrict__ counts) {
+  gs_wait_previous();
   int tile = blockIdx.x, u = blockIdx.y;
   int tx = tile % TX, ty = tile / TX;
   int px = tx * TILE + (threadIdx.x & 15), py = ty * TILE + (threadIdx.x >> 4);
@@ -1687,6 +1699,7 @@ __global__ void __launch_bounds__(TILE_PIX) k_blend_pairs(const uint2* __restric
 // Deterministic mode: the int64 fixed-point sums back to the float screen-space gradients.
 __global__ void k_fixed_to_grad2d(const unsigned long long* __restrict__ fixed, int64_t P, float* __restrict__ dxy,
                                   float* __restrict__ dco, float* __restrict__ drgb) {
+  gs_wait_previous();
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= P) return;
   float g[9];
@@ -1724,29 +1737,29 @@ int gs_render_fwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const u
     float4* ck = (float4*)sched->checkpoints;                                                                         \
     const float4 *pxy = (const float4*)proj->xy, *pco = (const float4*)proj->conic_op, *prgb = (const float4*)proj->rgb;\
     const uint2* rg = (const uint2*)ranges;                                                                           \
-    k_render_fwd_empty<<<grid, TILE_PIX, 0, s>>>(rg, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T,   \
-                                                 n_contrib, tk, q + qcap);                                            \
-    k_render_fwd_front<BW><<<gs_resident_grid<k_render_fwd_front<BW>>(32, 0, (int64_t)grid.x * 8), 32, 0, s>>>(                 \
-        rg, sched->tile_order, sched->job_base, sched->chunk, sched->walk_whole_lists != 0, later, (int)grid.x, ck,   \
-        sched->chunk_last, sorted_vals,                                                                               \
-        sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib, \
-        q, qcap, tk);                                                                                                 \
+    gs_launch(k_render_fwd_empty, grid, TILE_PIX, 0, s, rg, width, height, TX, TX * TY, bg[0], bg[1], bg[2],       \
+        img, final_T, n_contrib, tk, q + qcap);                                                                    \
+    gs_launch(k_render_fwd_front<BW>, gs_resident_grid<k_render_fwd_front<BW>>(32, 0, (int64_t)grid.x * 8), 32,    \
+        0, s, rg, sched->tile_order, sched->job_base, sched->chunk, sched->walk_whole_lists != 0, later,           \
+        (int)grid.x, ck, sched->chunk_last, sorted_vals, sched->block_masks, pxy, pco, prgb, width, height, TX,    \
+        TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib, q, qcap, tk);                                       \
     if (later) {                                                                                                      \
-      k_render_fwd_chunk<BW><<<gs_resident_grid<k_render_fwd_chunk<BW>>(32, 0, (int64_t)qcap), 32, 0, s>>>(                     \
-          rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last, sorted_vals,      \
-          sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, n_contrib, q, qcap, tk + 1);                \
-      k_render_fwd_combine<BW><<<gs_resident_grid<k_render_fwd_combine<BW>>(32, 0, (int64_t)qcap), 32, 0, s>>>(                 \
-          sched->tile_order, sched->job_base, sched->jobs, ck, sched->chunk_last, width, height, TX, TX * TY, bg[0],\
-          bg[1], bg[2], img, final_T, n_contrib, q, qcap, tk);                                                        \
-      k_render_fwd_stop<BW><<<gs_resident_grid<k_render_fwd_stop<BW>>(32, 0, (int64_t)qcap), 32, 0, s>>>(                       \
-          rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last, sorted_vals,      \
-          sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib,\
-          q, qcap, tk);                                                                                               \
+      gs_launch(k_render_fwd_chunk<BW>, gs_resident_grid<k_render_fwd_chunk<BW>>(32, 0, (int64_t)qcap), 32, 0,     \
+          s, rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last,             \
+          sorted_vals, sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, n_contrib, q, qcap,         \
+          tk + 1);                                                                                                 \
+      gs_launch(k_render_fwd_combine<BW>, gs_resident_grid<k_render_fwd_combine<BW>>(32, 0, (int64_t)qcap), 32,    \
+          0, s, sched->tile_order, sched->job_base, sched->jobs, ck, sched->chunk_last, width, height, TX,         \
+          TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib, q, qcap, tk);                                     \
+      gs_launch(k_render_fwd_stop<BW>, gs_resident_grid<k_render_fwd_stop<BW>>(32, 0, (int64_t)qcap), 32, 0, s,    \
+          rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last,                \
+          sorted_vals, sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2],        \
+          img, final_T, n_contrib, q, qcap, tk);                                                                   \
     }                                                                                                                 \
   } else                                                                                                            \
-    k_render_fwd<BW><<<grid, TILE_PIX, 0, s>>>((const uint2*)ranges, nullptr, sorted_vals, (const float4*)proj->xy, \
-                                               (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, \
-                                               TX, TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib)
+    gs_launch(k_render_fwd<BW>, grid, TILE_PIX, 0, s, (const uint2*)ranges, nullptr, sorted_vals,                  \
+        (const float4*)proj->xy, (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX,       \
+        TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib)
   if (variant == 0) { GS_FWD(8); } else if (variant == 1) { GS_FWD(16); } else { GS_FWD(4); }
 #undef GS_FWD
   return gs_check_launch();
@@ -1784,30 +1797,31 @@ int gs_blend_bwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const ui
     {                                                                                                              \
       if (cudaMemsetAsync(sched_ticket(sched), 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;        \
       if (fixed) {                                                                                                   \
-        k_render_bwd_det<BW><<<gs_resident_grid<k_render_bwd_det<BW>>(32, 0, sched->max_jobs * 8), 32, 0, s>>>(          \
-            (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                     \
-            (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,             \
-            (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, TX * TY * n_units,  \
-            bg[0], bg[1], bg[2], img, final_T, n_contrib, dL_dimg, dL_dT, fixed, sched_ticket(sched));               \
+        gs_launch(k_render_bwd_det<BW>, gs_resident_grid<k_render_bwd_det<BW>>(32, 0, sched->max_jobs * 8), 32,    \
+            0, s, (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,             \
+            (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,           \
+            (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY,                   \
+            TX * TY * n_units, bg[0], bg[1], bg[2], img, final_T, n_contrib, dL_dimg, dL_dT, fixed,                \
+            sched_ticket(sched));                                                                                  \
       } else {                                                                                                       \
-        k_render_bwd_m<BW><<<gs_resident_grid<k_render_bwd_m<BW>>(32, 0, sched->max_jobs * 8), 32, 0, s>>>(              \
-            (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                     \
-            (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,             \
-            (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY, TX * TY * n_units,  \
-            bg[0], bg[1], bg[2], img, final_T, n_contrib, dL_dimg, dL_dT, g2d->dxy, g2d->dconic_op, g2d->drgb,       \
-            sched_ticket(sched));                                                                                    \
+        gs_launch(k_render_bwd_m<BW>, gs_resident_grid<k_render_bwd_m<BW>>(32, 0, sched->max_jobs * 8), 32, 0,     \
+            s, (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                \
+            (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,           \
+            (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY,                   \
+            TX * TY * n_units, bg[0], bg[1], bg[2], img, final_T, n_contrib, dL_dimg, dL_dT, g2d->dxy,             \
+            g2d->dconic_op, g2d->drgb, sched_ticket(sched));                                                       \
       }                                                                                                              \
     }                                                                                                              \
   else                                                                                                               \
-    k_render_bwd<BW><<<grid, TILE_PIX, 0, s>>>((const uint2*)ranges, nullptr, sorted_vals, (const float4*)proj->xy, \
-                                               (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height,  \
-                                               TX, TX * TY, bg[0], bg[1], bg[2], final_T, n_contrib, dL_dimg, dL_dT,    \
-                                               g2d->dxy, g2d->dconic_op, g2d->drgb, fixed)
+    gs_launch(k_render_bwd<BW>, grid, TILE_PIX, 0, s, (const uint2*)ranges, nullptr, sorted_vals,                  \
+        (const float4*)proj->xy, (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX,       \
+        TX * TY, bg[0], bg[1], bg[2], final_T, n_contrib, dL_dimg, dL_dT, g2d->dxy, g2d->dconic_op, g2d->drgb,     \
+        fixed)
   if (variant == 0) { GS_BWD(8); } else if (variant == 1) { GS_BWD(16); } else { GS_BWD(4); }
 #undef GS_BWD
   if (fixed && n_proj > 0)
-    k_fixed_to_grad2d<<<(unsigned)((n_proj + 255) / 256), 256, 0, s>>>(fixed, n_proj, g2d->dxy, g2d->dconic_op,
-                                                                       g2d->drgb);
+    gs_launch(k_fixed_to_grad2d, (unsigned)((n_proj + 255) / 256), 256, 0, s, fixed, n_proj, g2d->dxy,
+        g2d->dconic_op, g2d->drgb);
   return gs_check_launch();
 }
 
@@ -1821,9 +1835,9 @@ GS_API int gs_blend_pairs(const gs_proj* proj, const uint32_t* sorted_vals, cons
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaMemsetAsync(d_count, 0, 5 * sizeof(unsigned long long), s) != cudaSuccess) return GS_ERR_CUDA;
   int TX = (width + TILE - 1) / TILE, TY = (height + TILE - 1) / TILE;
-  k_blend_pairs<<<dim3(TX * TY, n_units), TILE_PIX, 0, s>>>((const uint2*)ranges, sorted_vals, (const float4*)proj->xy,
-                                                            (const float4*)proj->conic_op, width, height, TX, TX * TY,
-                                                            n_contrib, block_masks, d_count);
+  gs_launch(k_blend_pairs, dim3(TX * TY, n_units), TILE_PIX, 0, s, (const uint2*)ranges, sorted_vals,
+      (const float4*)proj->xy, (const float4*)proj->conic_op, width, height, TX, TX * TY, n_contrib, block_masks,
+      d_count);
   return gs_check_launch();
 }
 
@@ -1832,7 +1846,7 @@ GS_API int gs_blend_pairs(const gs_proj* proj, const uint32_t* sorted_vals, cons
 int gs_tile_order_impl(const uint32_t* ranges, int n, uint32_t* ws, uint32_t* order, cudaStream_t s) {
   if (cudaMemsetAsync(ws, 0, sizeof(uint32_t) * 66, s) != cudaSuccess) return GS_ERR_CUDA;
   unsigned nb = (unsigned)((n + 255) / 256);
-  k_order_hist<<<nb, 256, 0, s>>>((const uint2*)ranges, n, ws);
-  k_order_scatter<<<nb, 256, 0, s>>>((const uint2*)ranges, n, ws, ws + 33, order);
+  gs_launch(k_order_hist, nb, 256, 0, s, (const uint2*)ranges, n, ws);
+  gs_launch(k_order_scatter, nb, 256, 0, s, (const uint2*)ranges, n, ws, ws + 33, order);
   return gs_check_launch();
 }

@@ -106,6 +106,7 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* s_warp
 // ---- exclusive scan of tiles_touched -> instance offsets
 __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* __restrict__ in, int64_t P,
                                                         uint32_t* __restrict__ bsums) {
+  gs_wait_previous();
   __shared__ uint32_t s_warp[33];
   int64_t base = (int64_t)blockIdx.x * SCAN_BLOCK;
   uint32_t s = 0;
@@ -122,6 +123,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* __restri
 // bmins (may be NULL): per-block minima reduced on the way into *dmin
 __global__ void __launch_bounds__(1024) k_scan_bsums(uint32_t* bsums, int64_t nb, const uint32_t* bmins,
                                                      uint32_t* dmin) {
+  gs_wait_previous();
   __shared__ uint32_t s_warp[33];
   __shared__ uint32_t s_carry;
   __shared__ uint32_t s_min;
@@ -152,6 +154,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_down(const uint32_t* __restrict
                                                       const uint32_t* __restrict__ bsums, int64_t nb,
                                                       uint32_t* __restrict__ out, int64_t cap,
                                                       uint32_t* d_count, int* status) {
+  gs_wait_previous();
   __shared__ uint32_t s_warp[33];
   __shared__ uint32_t s_items[SCAN_BLOCK];
   int64_t base = (int64_t)blockIdx.x * SCAN_BLOCK;
@@ -200,6 +203,7 @@ __global__ void __launch_bounds__(256) k_duplicate(UnitTable U, const float4* __
                                                    const uint32_t* __restrict__ offsets, int W, int H,
                                                    int tile_bits, int64_t cap, int key_masks,
                                                    uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  gs_wait_previous();
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int64_t P = U.proj_base[U.n];
   if (p >= P) return;
@@ -240,6 +244,7 @@ __global__ void __launch_bounds__(RS_T) k_radix_hist(const KT* __restrict__ k0, 
                                                      const uint32_t* __restrict__ d_count, int shift,
                                                      uint32_t* __restrict__ hist, int64_t stride,
                                                      uint32_t* __restrict__ totals) {
+  gs_wait_previous();
   constexpr int BINS = 1 << BITS;
   __shared__ uint32_t s_h[RS_T / 32][BINS];
   int64_t I = *d_count;
@@ -297,6 +302,7 @@ __global__ void __launch_bounds__(1024) k_radix_scan(uint32_t* __restrict__ hist
                                                      const uint32_t* __restrict__ totals, int pass, int bins,
                                                      const uint32_t* __restrict__ d_count,
                                                      int32_t* __restrict__ cur) {
+  gs_wait_previous();
   __shared__ uint32_t s_warp[33];
   __shared__ uint32_t s_carry;
   __shared__ int s_skip;
@@ -344,6 +350,7 @@ __global__ void __launch_bounds__(RS_T, sizeof(KT) == 4 ? 3 : 2) k_radix_scatter
                                                         const uint32_t* __restrict__ d_count, int shift,
                                                         const uint32_t* __restrict__ hist, int64_t stride,
                                                         uint32_t* __restrict__ vfinal, uint16_t* __restrict__ mfinal) {
+  gs_wait_previous();
   // FINAL: the values go to vfinal instead of the other value buffer (the last pass of a sort writes the
   // caller's output directly), and bits 16-31 of each key (the block mask) to mfinal unless it is NULL
   constexpr int BINS = 1 << BITS;
@@ -476,6 +483,7 @@ __global__ void __launch_bounds__(256) k_ranges(const uint64_t* __restrict__ k0,
                                                 uint32_t* __restrict__ out_vals, const float4* __restrict__ xy,
                                                 const float4* __restrict__ conic_op, uint16_t* __restrict__ masks,
                                                 int key_masks) {
+  gs_wait_previous();
   int64_t I = *d_count;
   int c = cur[final_pass];
   const uint64_t* keys = c ? k1 : k0;
@@ -515,6 +523,7 @@ __global__ void __launch_bounds__(256) k_ranges(const uint64_t* __restrict__ k0,
 __global__ void __launch_bounds__(SCAN_T) k_vis_reduce(const uint32_t* __restrict__ tiles,
                                                        const float* __restrict__ depth, int64_t P, int vec,
                                                        uint32_t* __restrict__ bsums, uint32_t* __restrict__ bmins) {
+  gs_wait_previous();
   __shared__ uint32_t s_warp[33];
   __shared__ uint32_t s_min;
   if (threadIdx.x == 0) s_min = 0xffffffffu;
@@ -632,6 +641,7 @@ __global__ void __launch_bounds__(SCAN_T) k_vis_compact(const uint32_t* __restri
                                                         const float4* __restrict__ conic_op,
                                                         const int* __restrict__ radius, int TX, int TY, int masks,
                                                         uint64_t* __restrict__ desc) {
+  gs_wait_previous();
   // desc (may be NULL): also the visible records' packed rectangles, by record
   constexpr int NW = SCAN_T / 32;
   static_assert(SCAN_ITEMS * NW == 64, "one warp scans the (round, warp) counts two per lane");
@@ -675,6 +685,7 @@ __global__ void __launch_bounds__(SCAN_T) k_dup_reduce(const uint32_t* __restric
                                                        const uint32_t* __restrict__ d_vis,
                                                        const uint32_t* __restrict__ tiles,
                                                        uint32_t* __restrict__ bsums) {
+  gs_wait_previous();
   __shared__ uint32_t s_warp[33];
   const uint32_t* v = cur[final_pass] ? vB : vA;
   int64_t V = *d_vis;
@@ -709,6 +720,7 @@ __global__ void __launch_bounds__(SCAN_T, 4) k_dup_emit(UnitTable U, const float
                                                      int tile_bits, int64_t cap, int key_masks,
                                                      uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
                                                      uint32_t* __restrict__ d_count, int* __restrict__ status) {
+  gs_wait_previous();
   __shared__ uint32_t s_warp[33];
   __shared__ uint32_t s_p[SCAN_BLOCK];
   __shared__ uint32_t s_key[EMIT_WIN];
@@ -809,6 +821,7 @@ __global__ void __launch_bounds__(256) k_ranges32(const uint32_t* __restrict__ k
                                                   const uint32_t* __restrict__ d_count, int tile_bits, int n_tiles,
                                                   uint32_t* __restrict__ ranges, uint32_t* __restrict__ out_vals,
                                                   uint16_t* __restrict__ masks) {
+  gs_wait_previous();
   int64_t I = *d_count;
   int c = cur[final_pass];
   const bool copy = final_pass < 1 || cur[final_pass - 1] == c;  // the last pass was skipped
@@ -846,6 +859,7 @@ __global__ void __launch_bounds__(256) k_ranges32(const uint32_t* __restrict__ k
 // number of chunks of each list, in tile order
 __global__ void k_chunk_count(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order, int NT, int K,
                               uint32_t* __restrict__ counts) {
+  gs_wait_previous();
   int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= NT) return;
   uint2 r = ranges[order[o]];
@@ -855,6 +869,7 @@ __global__ void k_chunk_count(const uint2* __restrict__ ranges, const uint32_t* 
 // (order position, chunk) of every chunk job
 __global__ void k_chunk_jobs(const uint32_t* __restrict__ job_base, int NT, int64_t max_jobs,
                              uint32_t* __restrict__ jobs) {
+  gs_wait_previous();
   int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= NT) return;
   uint32_t b = job_base[o], e = job_base[o + 1];
@@ -880,9 +895,9 @@ int gs_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, void* ws, uint32_t
   if (n <= 0) return cudaMemsetAsync(d_total, 0, sizeof(uint32_t), s) == cudaSuccess ? GS_OK : GS_ERR_CUDA;
   int64_t nsb = (n + SCAN_BLOCK - 1) / SCAN_BLOCK;
   uint32_t* bsums = (uint32_t*)ws;
-  k_scan_reduce<<<(unsigned)nsb, SCAN_T, 0, s>>>(in, n, bsums);
-  k_scan_bsums<<<1, 1024, 0, s>>>(bsums, nsb, nullptr, nullptr);
-  k_scan_down<<<(unsigned)nsb, SCAN_T, 0, s>>>(in, n, bsums, nsb, out, INT64_MAX, d_total, nullptr);
+  gs_launch(k_scan_reduce, (unsigned)nsb, SCAN_T, 0, s, in, n, bsums);
+  gs_launch(k_scan_bsums, 1, 1024, 0, s, bsums, nsb, nullptr, nullptr);
+  gs_launch(k_scan_down, (unsigned)nsb, SCAN_T, 0, s, in, n, bsums, nsb, out, INT64_MAX, d_total, nullptr);
   return gs_check_launch();
 }
 
@@ -900,10 +915,10 @@ int gs_schedule_jobs(const uint32_t* ranges, int NT, char* order_ws, char* scan_
   int r = order_done ? GS_OK : gs_tile_order_impl(ranges, NT, (uint32_t*)order_ws, sched->tile_order, s);
   if (r != GS_OK) return r;
   unsigned nb = (unsigned)((NT + 255) / 256);
-  k_chunk_count<<<nb, 256, 0, s>>>((const uint2*)ranges, sched->tile_order, NT, sched->chunk, sched->job_base);
+  gs_launch(k_chunk_count, nb, 256, 0, s, (const uint2*)ranges, sched->tile_order, NT, sched->chunk, sched->job_base);
   r = gs_scan_u32(sched->job_base, sched->job_base, NT, scan_ws, sched->job_base + NT, s);
   if (r != GS_OK) return r;
-  k_chunk_jobs<<<nb, 256, 0, s>>>(sched->job_base, NT, sched->max_jobs, sched->jobs);
+  gs_launch(k_chunk_jobs, nb, 256, 0, s, sched->job_base, NT, sched->max_jobs, sched->jobs);
   return gs_check_launch();
 }
 
@@ -960,50 +975,48 @@ static int depth_first_sort(const UnitTable& U, int64_t P, const gs_proj* proj, 
   // reads 36 bytes per record in order: at 10M records that costs what the gathers of the emission save (270 us
   // without, 301 us with it), at 107M it saves a fifth of the sort.
   uint64_t* desc = P >= DESC_RECORDS && cap >= 2 * P ? k0 + P : nullptr;
-  k_vis_reduce<<<(unsigned)nsb, SCAN_T, 0, s>>>(proj->tiles, proj->depth, P, vec, bsums, bmins);
-  k_scan_bsums<<<1, 1024, 0, s>>>(bsums, nsb, bmins, d_min);
-  k_vis_compact<<<(unsigned)nsb, SCAN_T, 0, s>>>(proj->tiles, proj->depth, P, bsums, nsb, d_min, dkA, dvA, d_vis,
-                                                 (const float4*)proj->xy, (const float4*)proj->conic_op, proj->radius,
-                                                 TX, TY, key_masks, desc);
+  gs_launch(k_vis_reduce, (unsigned)nsb, SCAN_T, 0, s, proj->tiles, proj->depth, P, vec, bsums, bmins);
+  gs_launch(k_scan_bsums, 1, 1024, 0, s, bsums, nsb, bmins, d_min);
+  gs_launch(k_vis_compact, (unsigned)nsb, SCAN_T, 0, s, proj->tiles, proj->depth, P, bsums, nsb, d_min, dkA, dvA,
+      d_vis, (const float4*)proj->xy, (const float4*)proj->conic_op, proj->radius, TX, TY, key_masks, desc);
   // (three 9-bit passes and a skipped top pass measured slower: a 9-bit scatter pass took 76 us against
   // 48 us for an 8-bit one at 10M records)
   constexpr int DEPTH_PASSES = 4;
   for (int pass = 0; pass < DEPTH_PASSES; ++pass) {
-    k_radix_hist<8, uint32_t><<<gh, RS_T, 0, s>>>(dkA, dkB, cur, pass, d_vis, 8 * pass, hist, stride, totals);
-    k_radix_scan<<<256, 1024, 0, s>>>(hist, stride, totals, pass, 256, d_vis, cur);
-    k_radix_scatter<8, uint32_t><<<gsc, RS_T, DYN32, s>>>(dkA, dkB, dvA, dvB, cur, pass, d_vis, 8 * pass, hist,
-                                                          stride, nullptr, nullptr);
+    gs_launch(k_radix_hist<8, uint32_t>, gh, RS_T, 0, s, dkA, dkB, cur, pass, d_vis, 8 * pass, hist, stride, totals);
+    gs_launch(k_radix_scan, 256, 1024, 0, s, hist, stride, totals, pass, 256, d_vis, cur);
+    gs_launch(k_radix_scatter<8, uint32_t>, gsc, RS_T, DYN32, s, dkA, dkB, dvA, dvB, cur, pass, d_vis, 8 * pass,
+        hist, stride, nullptr, nullptr);
   }
-  k_dup_reduce<<<(unsigned)nsb, SCAN_T, 0, s>>>(dvA, dvB, cur, DEPTH_PASSES, d_vis, proj->tiles, bsums);
-  k_scan_bsums<<<1, 1024, 0, s>>>(bsums, nsb, nullptr, nullptr);
+  gs_launch(k_dup_reduce, (unsigned)nsb, SCAN_T, 0, s, dvA, dvB, cur, DEPTH_PASSES, d_vis, proj->tiles, bsums);
+  gs_launch(k_scan_bsums, 1, 1024, 0, s, bsums, nsb, nullptr, nullptr);
   uint32_t* ikA = v0;
   uint32_t* ivA = v1;
   uint32_t* ikB = (uint32_t*)k0;
   uint32_t* ivB = (uint32_t*)k1;
-  k_dup_emit<<<(unsigned)nsb, SCAN_T, 0, s>>>(U, (const float4*)proj->xy, (const float4*)proj->conic_op,
-                                              proj->radius, desc, dvA, dvB, cur, DEPTH_PASSES, d_vis, bsums, nsb,
-                                              width, height, tile_bits, cap, key_masks, ikA, ivA, d_num_instances,
-                                              d_status);
+  gs_launch(k_dup_emit, (unsigned)nsb, SCAN_T, 0, s, U, (const float4*)proj->xy, (const float4*)proj->conic_op,
+      proj->radius, desc, dvA, dvB, cur, DEPTH_PASSES, d_vis, bsums, nsb, width, height, tile_bits, cap, key_masks,
+      ikA, ivA, d_num_instances, d_status);
   if (cap == 0) return gs_check_launch();
   // the instance passes keep their own buffer parity and digit totals
   int32_t* cur_t = cur + MAX_PASSES + 1;
   uint32_t* totals_t = totals + DEPTH_PASSES * RS_BINS_MAX;
   int tpasses = (ut_bits + 7) / 8;
   for (int pass = 0; pass < tpasses; ++pass) {
-    k_radix_hist<8, uint32_t><<<gh, RS_T, 0, s>>>(ikA, ikB, cur_t, pass, d_num_instances, 8 * pass, hist, stride,
-                                                  totals_t);
-    k_radix_scan<<<256, 1024, 0, s>>>(hist, stride, totals_t, pass, 256, d_num_instances, cur_t);
+    gs_launch(k_radix_hist<8, uint32_t>, gh, RS_T, 0, s, ikA, ikB, cur_t, pass, d_num_instances, 8 * pass, hist,
+        stride, totals_t);
+    gs_launch(k_radix_scan, 256, 1024, 0, s, hist, stride, totals_t, pass, 256, d_num_instances, cur_t);
     // the last pass writes the record ids and block masks to the outputs (k_ranges32 copies them only
     // when the device skips that pass)
     if (pass == tpasses - 1)
-      k_radix_scatter<8, uint32_t, true><<<gscf, RS_T, DYN32, s>>>(ikA, ikB, ivA, ivB, cur_t, pass, d_num_instances,
-                                                                   8 * pass, hist, stride, sorted_vals, block_masks);
+      gs_launch(k_radix_scatter<8, uint32_t, true>, gscf, RS_T, DYN32, s, ikA, ikB, ivA, ivB, cur_t, pass,
+          d_num_instances, 8 * pass, hist, stride, sorted_vals, block_masks);
     else
-      k_radix_scatter<8, uint32_t><<<gsc, RS_T, DYN32, s>>>(ikA, ikB, ivA, ivB, cur_t, pass, d_num_instances, 8 * pass,
-                                                            hist, stride, nullptr, nullptr);
+      gs_launch(k_radix_scatter<8, uint32_t>, gsc, RS_T, DYN32, s, ikA, ikB, ivA, ivB, cur_t, pass, d_num_instances,
+          8 * pass, hist, stride, nullptr, nullptr);
   }
-  k_ranges32<<<gs_resident_grid<k_ranges32>(256, 0, (cap + 1023) / 1024), 256, 0, s>>>(
-      ikA, ikB, ivA, ivB, cur_t, tpasses, d_num_instances, tile_bits, n_tiles, ranges, sorted_vals, block_masks);
+  gs_launch(k_ranges32, gs_resident_grid<k_ranges32>(256, 0, (cap + 1023) / 1024), 256, 0, s, ikA, ikB, ivA, ivB,
+      cur_t, tpasses, d_num_instances, tile_bits, n_tiles, ranges, sorted_vals, block_masks);
   return gs_check_launch();
 }
 
@@ -1079,10 +1092,10 @@ int gs_bin_sort_impl(const gs_proj* proj, const gs_units* units, int width, int 
     if (sched) return gs_schedule_jobs(ranges, n_tiles * U.n, ws + L.order, ws + L.jscan, sched, s);
     return gs_check_launch();
   }
-  k_scan_reduce<<<(unsigned)nsb, SCAN_T, 0, s>>>(proj->tiles, P, bsums);
-  k_scan_bsums<<<1, 1024, 0, s>>>(bsums, nsb, nullptr, nullptr);
-  k_scan_down<<<(unsigned)nsb, SCAN_T, 0, s>>>(proj->tiles, P, bsums, nsb, offsets, max_instances,
-                                               d_num_instances, d_status);
+  gs_launch(k_scan_reduce, (unsigned)nsb, SCAN_T, 0, s, proj->tiles, P, bsums);
+  gs_launch(k_scan_bsums, 1, 1024, 0, s, bsums, nsb, nullptr, nullptr);
+  gs_launch(k_scan_down, (unsigned)nsb, SCAN_T, 0, s, proj->tiles, P, bsums, nsb, offsets, max_instances,
+      d_num_instances, d_status);
   if (method == 1) {
     if ((int64_t)n_tiles * U.n > MAX_SCHED_TILES) return GS_ERR_INVALID;
     int r = gs_seg_sort(U, P, proj, width, height, max_instances, k0, k1, v0, v1, (uint32_t*)(ws + L.jscan),
@@ -1093,9 +1106,9 @@ int gs_bin_sort_impl(const gs_proj* proj, const gs_units* units, int width, int 
   }
   // block masks ride in the keys when unit | tile | depth leave bits 48..63 free
   int key_masks = (block_masks && key_bits <= 48) ? 1 : 0;
-  k_duplicate<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(U, (const float4*)proj->xy, (const float4*)proj->conic_op,
-                                                          proj->depth, proj->radius, proj->tiles, offsets, width,
-                                                          height, tile_bits, max_instances, key_masks, k0, v0);
+  gs_launch(k_duplicate, (unsigned)((P + 255) / 256), 256, 0, s, U, (const float4*)proj->xy,
+      (const float4*)proj->conic_op, proj->depth, proj->radius, proj->tiles, offsets, width, height, tile_bits,
+      max_instances, key_masks, k0, v0);
   if (max_instances > 0) {
     if (cudaFuncSetAttribute(k_radix_scatter<8, uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCATTER_DYN_SMEM) !=
             cudaSuccess ||
@@ -1109,20 +1122,22 @@ int gs_bin_sort_impl(const gs_proj* proj, const gs_units* units, int width, int 
     for (int pass = 0; pass < passes; ++pass) {
       int shift = digit * pass;
       if (digit == 9) {
-        k_radix_hist<9, uint64_t><<<gh, RS_T, 0, s>>>(k0, k1, cur, pass, d_num_instances, shift, hist, stride, totals);
-        k_radix_scan<<<512, 1024, 0, s>>>(hist, stride, totals, pass, 512, d_num_instances, cur);
-        k_radix_scatter<9, uint64_t><<<gs, RS_T, SCATTER_DYN_SMEM, s>>>(k0, k1, v0, v1, cur, pass, d_num_instances, shift,
-                                                               hist, stride, nullptr, nullptr);
+        gs_launch(k_radix_hist<9, uint64_t>, gh, RS_T, 0, s, k0, k1, cur, pass, d_num_instances, shift, hist, stride,
+            totals);
+        gs_launch(k_radix_scan, 512, 1024, 0, s, hist, stride, totals, pass, 512, d_num_instances, cur);
+        gs_launch(k_radix_scatter<9, uint64_t>, gs, RS_T, SCATTER_DYN_SMEM, s, k0, k1, v0, v1, cur, pass,
+            d_num_instances, shift, hist, stride, nullptr, nullptr);
       } else {
-        k_radix_hist<8, uint64_t><<<gh, RS_T, 0, s>>>(k0, k1, cur, pass, d_num_instances, shift, hist, stride, totals);
-        k_radix_scan<<<256, 1024, 0, s>>>(hist, stride, totals, pass, 256, d_num_instances, cur);
-        k_radix_scatter<8, uint64_t><<<gs, RS_T, SCATTER_DYN_SMEM, s>>>(k0, k1, v0, v1, cur, pass, d_num_instances, shift,
-                                                               hist, stride, nullptr, nullptr);
+        gs_launch(k_radix_hist<8, uint64_t>, gh, RS_T, 0, s, k0, k1, cur, pass, d_num_instances, shift, hist, stride,
+            totals);
+        gs_launch(k_radix_scan, 256, 1024, 0, s, hist, stride, totals, pass, 256, d_num_instances, cur);
+        gs_launch(k_radix_scatter<8, uint64_t>, gs, RS_T, SCATTER_DYN_SMEM, s, k0, k1, v0, v1, cur, pass,
+            d_num_instances, shift, hist, stride, nullptr, nullptr);
       }
     }
-    k_ranges<<<gs_resident_grid<k_ranges>(256, 0, (max_instances + 255) / 256), 256, 0, s>>>(
-        k0, k1, v0, v1, cur, passes, d_num_instances, tile_bits, n_tiles, TX, ranges, sorted_vals,
-        (const float4*)proj->xy, (const float4*)proj->conic_op, block_masks, key_masks);
+    gs_launch(k_ranges, gs_resident_grid<k_ranges>(256, 0, (max_instances + 255) / 256), 256, 0, s, k0, k1, v0, v1,
+        cur, passes, d_num_instances, tile_bits, n_tiles, TX, ranges, sorted_vals, (const float4*)proj->xy,
+        (const float4*)proj->conic_op, block_masks, key_masks);
   }
   if (sched) return gs_schedule_jobs(ranges, n_tiles * U.n, ws + L.order, ws + L.jscan, sched, s);
   return gs_check_launch();

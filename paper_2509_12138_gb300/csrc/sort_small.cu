@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(ST, 1) k_small_units(UnitTable U, const float4
                                                        const uint32_t* __restrict__ tiles, int W, int H, int64_t cap,
                                                        uint32_t* __restrict__ rec, uint2* __restrict__ rect,
                                                        Ctrl* __restrict__ ctrl, int* __restrict__ status) {
+  gs_wait_previous();
   extern __shared__ __align__(16) unsigned char s_raw[];
   UnitSmem& s = *reinterpret_cast<UnitSmem*>(s_raw);
   __shared__ uint64_t s_sum[SW];
@@ -291,6 +292,7 @@ __global__ void __launch_bounds__(LW * 32) k_small_count(UnitTable U, int W, int
                                                          const uint2* __restrict__ rect,
                                                          const float* __restrict__ depth,
                                                          const Ctrl* __restrict__ ctrl, uint32_t* __restrict__ count) {
+  gs_wait_previous();
   const int f = blockIdx.x * LW + (threadIdx.x >> 5);
   if (f >= NT) return;
   const int TX = (W + TILE - 1) / TILE, tile = f % n_tiles;
@@ -331,6 +333,7 @@ __global__ void __launch_bounds__(ST) k_small_ranges(int NT, const uint32_t* __r
                                                      uint2* __restrict__ ranges, uint32_t* __restrict__ d_count,
                                                      uint32_t* __restrict__ order, uint32_t* __restrict__ job_base,
                                                      uint32_t* __restrict__ jobs, int64_t max_jobs, int K) {
+  gs_wait_previous();
   constexpr int PER = LISTS_MAX / ST;
   __shared__ uint32_t s[SW], s_class[33], s_len[LISTS_MAX];
   const int t0 = threadIdx.x * PER;
@@ -393,6 +396,7 @@ __global__ void __launch_bounds__(LW * 32) k_small_fill(UnitTable U, int W, int 
                                                         const float4* __restrict__ conic_op,
                                                         const uint2* __restrict__ ranges,
                                                         uint32_t* __restrict__ vals, uint16_t* __restrict__ masks) {
+  gs_wait_previous();
   const int f = blockIdx.x * LW + (threadIdx.x >> 5);
   if (f >= NT) return;
   const uint2 rg = ranges[f];
@@ -453,16 +457,15 @@ int gs_small_sort(const UnitTable& U, const gs_proj* proj, int width, int height
       cudaFuncSetAttribute(k_small_units, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(UnitSmem)) !=
           cudaSuccess)
     return GS_ERR_CUDA;
-  k_small_units<<<(unsigned)U.n, ST, sizeof(UnitSmem), s>>>(U, (const float4*)proj->xy, proj->depth, proj->radius,
-                                                            proj->tiles, width, height, cap, rec, rect, ctrl,
-                                                            d_status);
+  gs_launch(k_small_units, (unsigned)U.n, ST, sizeof(UnitSmem), s, U, (const float4*)proj->xy, proj->depth,
+      proj->radius, proj->tiles, width, height, cap, rec, rect, ctrl, d_status);
   const unsigned lb = (unsigned)((NT + LW - 1) / LW);
-  k_small_count<<<lb, LW * 32, 0, s>>>(U, width, n_tiles, NT, rec, rect, proj->depth, ctrl, count);
-  k_small_ranges<<<1, ST, 0, s>>>(NT, count, (uint2*)ranges, d_num_instances, sched ? sched->tile_order : nullptr,
-                                  sched ? sched->job_base : nullptr, sched ? sched->jobs : nullptr,
-                                  sched ? sched->max_jobs : 0, sched ? sched->chunk : 32);
-  k_small_fill<<<lb, LW * 32, 0, s>>>(U, width, n_tiles, NT, rec, rect, proj->depth, ctrl, (const float4*)proj->xy,
-                                      (const float4*)proj->conic_op, (const uint2*)ranges, sorted_vals,
-                                      sched ? sched->block_masks : nullptr);
+  gs_launch(k_small_count, lb, LW * 32, 0, s, U, width, n_tiles, NT, rec, rect, proj->depth, ctrl, count);
+  gs_launch(k_small_ranges, 1, ST, 0, s, NT, count, (uint2*)ranges, d_num_instances,
+      sched ? sched->tile_order : nullptr, sched ? sched->job_base : nullptr, sched ? sched->jobs : nullptr,
+      sched ? sched->max_jobs : 0, sched ? sched->chunk : 32);
+  gs_launch(k_small_fill, lb, LW * 32, 0, s, U, width, n_tiles, NT, rec, rect, proj->depth, ctrl,
+      (const float4*)proj->xy, (const float4*)proj->conic_op, (const uint2*)ranges, sorted_vals,
+      sched ? sched->block_masks : nullptr);
   return gs_check_launch();
 }

@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(256) k_gather_views(const gs_camera* __restric
                                                       int n_views, int vps, const int32_t* __restrict__ d_step,
                                                       int64_t plane, int vec, gs_camera* __restrict__ cams_step,
                                                       float* __restrict__ gt_step, uint8_t* __restrict__ mask_step) {
+  gs_wait_previous();
   int u = blockIdx.y;
   int v = unit_view((int64_t)*d_step, u, vps, train_views, n_train);
   int k = u / vps;
@@ -78,9 +79,9 @@ GS_API int gs_gather_views(const gs_train_batch_desc* d, const int32_t* d_step, 
             (3 * plane) % 4 == 0 && plane % 16 == 0;
   int64_t per_unit = (3 * plane / 4 + 255) / 256;
   unsigned gx = (unsigned)(per_unit < 64 ? (per_unit > 0 ? per_unit : 1) : 64);
-  k_gather_views<<<dim3(gx, (unsigned)U), 256, 0, (cudaStream_t)stream>>>(
-      d->cam_pool, d->gt_pool, d->mask_pool, d->train_views, d->n_train, d->n_views, d->views_per_step, d_step, plane,
-      vec, d->cams_step, d->gt_step, d->mask_step);
+  gs_launch(k_gather_views, dim3(gx, (unsigned)U), 256, 0, (cudaStream_t)stream, d->cam_pool, d->gt_pool,
+      d->mask_pool, d->train_views, d->n_train, d->n_views, d->views_per_step, d_step, plane, vec, d->cams_step,
+      d->gt_step, d->mask_step);
   return gs_check_launch();
 }
 
