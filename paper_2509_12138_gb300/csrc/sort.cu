@@ -19,6 +19,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 using namespace gs;
@@ -343,6 +345,23 @@ __global__ void __launch_bounds__(1024) k_radix_scan(uint32_t* __restrict__ hist
 // counts are scanned across warps.  Keys are then placed in a block-local
 // digit-sorted buffer in shared memory and written out so that each digit's
 // run goes to consecutive global positions (coalesced stores).
+// The lanes whose digit equals this lane's are found MATCH rounds ahead of the
+// counters, with one vote per digit bit.  (The match instruction takes longer
+// the more digits there are: 69 us per pass over 10M records with it, 59 with
+// votes; but in the last pass, whose digits are a few bits, 68 against 99 us
+// over 17M instances.)
+constexpr int MATCH = 4;
+template <int BITS>
+__device__ __forceinline__ uint32_t same_digit(uint32_t d, bool valid) {
+  uint32_t peers = __ballot_sync(0xffffffffu, valid);
+  #pragma unroll
+  for (int b = 0; b < BITS; ++b) {
+    const bool bit = (d >> b) & 1u;
+    const uint32_t set = __ballot_sync(0xffffffffu, bit);
+    peers &= bit ? set : ~set;
+  }
+  return peers;
+}
 template <int BITS, typename KT, bool FINAL = false>
 __global__ void __launch_bounds__(RS_T, sizeof(KT) == 4 ? 3 : 2) k_radix_scatter(KT* __restrict__ k0, KT* __restrict__ k1,
                                                         uint32_t* __restrict__ v0, uint32_t* __restrict__ v1,
@@ -382,34 +401,49 @@ __global__ void __launch_bounds__(RS_T, sizeof(KT) == 4 ? 3 : 2) k_radix_scatter
       #pragma unroll
       for (int q = 0; q < NW; ++q) s_wc[q][dd] = 0u;
     }
-    uint32_t lt = (1u << lane) - 1u;
+    const uint32_t lt = (1u << lane) - 1u;
     KT key[RS_ITEMS];
     uint32_t val[RS_ITEMS];
     uint32_t rnk[RS_ITEMS / 2];  // ranks within the digit among this warp's keys, two 16-bit ranks a word
     int64_t wk = base + (int64_t)w * WKEYS + lane;  // this lane's key of round 0
     int64_t rem64 = I - wk;
-    int rem = rem64 > RS_TILE ? RS_TILE : (int)rem64;  // round j holds a key iff 32 j < rem
+    const int rem = rem64 > RS_TILE ? RS_TILE : (int)rem64;  // round j holds a key iff 32 j < rem
     const KT* kp = kin + wk;
     const uint32_t* vp = vin + wk;
-    #pragma unroll
-    for (int j = 0; j < RS_ITEMS; ++j) {
-      bool valid = j * 32 < rem;
-      key[j] = valid ? kp[j * 32] : (KT)0;
-      val[j] = valid ? vp[j * 32] : 0u;
-    }
-    __syncthreads();
-    #pragma unroll
-    for (int j = 0; j < RS_ITEMS; ++j) {
-      bool valid = j * 32 < rem;
-      uint32_t d = valid ? ((uint32_t)(key[j] >> shift) & (BINS - 1u)) : (uint32_t)BINS;
-      uint32_t peers = __match_any_sync(0xffffffffu, d);
-      uint32_t before = valid ? s_wc[w][d] : 0u;
-      uint32_t r = before + __popc(peers & lt);  // < WKEYS: fits 16 bits
-      if (j & 1) rnk[j >> 1] |= r << 16; else rnk[j >> 1] = r;
-      __syncwarp();
-      if (valid && (peers & lt) == 0u) s_wc[w][d] = before + __popc(peers);  // lowest lane of the group
-      __syncwarp();
-    }
+    auto rank_keys = [&](auto whole) {  // whole: a full tile, every round holds a key
+      constexpr bool WHOLE = decltype(whole)::value;
+      #pragma unroll
+      for (int j = 0; j < RS_ITEMS; ++j) {
+        const bool valid = WHOLE || j * 32 < rem;
+        key[j] = valid ? kp[j * 32] : (KT)0;
+        val[j] = valid ? vp[j * 32] : 0u;
+      }
+      __syncthreads();
+      #pragma unroll
+      for (int j0 = 0; j0 < RS_ITEMS; j0 += MATCH) {
+        uint32_t peers[MATCH];  // the lanes of round j0 + e with this lane's digit
+        #pragma unroll
+        for (int e = 0; e < MATCH; ++e) {
+          const bool valid = WHOLE || (j0 + e) * 32 < rem;
+          const uint32_t d = (uint32_t)(key[j0 + e] >> shift) & (BINS - 1u);
+          peers[e] = FINAL ? __match_any_sync(0xffffffffu, valid ? d : (uint32_t)BINS) : same_digit<BITS>(d, valid);
+        }
+        #pragma unroll
+        for (int e = 0; e < MATCH; ++e) {
+          const int j = j0 + e;
+          const bool valid = WHOLE || j * 32 < rem;
+          const uint32_t d = (uint32_t)(key[j] >> shift) & (BINS - 1u);
+          const uint32_t before = valid ? s_wc[w][d] : 0u;
+          const uint32_t r = before + __popc(peers[e] & lt);  // < WKEYS: fits 16 bits
+          if (j & 1) rnk[j >> 1] |= r << 16; else rnk[j >> 1] = r;
+          __syncwarp();
+          if (valid && (peers[e] & lt) == 0u) s_wc[w][d] = before + __popc(peers[e]);  // lowest lane of the group
+          __syncwarp();
+        }
+      }
+    };
+    if (base + RS_TILE <= I) rank_keys(std::true_type{});
+    else rank_keys(std::false_type{});
     __syncthreads();
     // per digit: exclusive scan of the warp counts (warp order = key order); thread tid
     // owns digits tid * DPT .. tid * DPT + DPT - 1, then a block scan gives digit starts
@@ -449,7 +483,11 @@ __global__ void __launch_bounds__(RS_T, sizeof(KT) == 4 ? 3 : 2) k_radix_scatter
       __syncthreads();
       uint32_t st = inc - cnt + s_warp[w];
       #pragma unroll
-      for (int e = 0; e < DPT; ++e) { s_lstart[tid * DPT + e] = st; st += cnts[e]; }
+      for (int e = 0; e < DPT; ++e) {
+        s_lstart[tid * DPT + e] = st;
+        s_off[tid * DPT + e] -= st;  // global position of block-local position 0 of the digit's run
+        st += cnts[e];
+      }
     }
     __syncthreads();
     #pragma unroll
@@ -466,7 +504,7 @@ __global__ void __launch_bounds__(RS_T, sizeof(KT) == 4 ? 3 : 2) k_radix_scatter
     for (int i = tid; i < n_here; i += RS_T) {
       KT kk = s_keys[i];
       uint32_t d = (uint32_t)(kk >> shift) & (BINS - 1u);
-      uint32_t gp = s_off[d] + (uint32_t)i - s_lstart[d];
+      uint32_t gp = s_off[d] + (uint32_t)i;
       kout[gp] = kk;
       vout[gp] = s_vals[i];
       if (FINAL && mfinal) mfinal[gp] = (uint16_t)((uint64_t)kk >> 16);
@@ -631,7 +669,11 @@ __device__ __forceinline__ uint32_t tile_blocks(int b, int e, int t) {
 // number.  Keys relative to the nearest visible depth keep the order and leave the top byte zero when the
 // view's depths stay within a factor of ~4 (then the device skips the top radix pass).
 // Round j of a block covers its records [256 j, 256 j + 256) (coalesced loads); a record's slot is the
-// block's base, the visible records of earlier (round, warp) pairs and those of lower lanes.
+// block's base, the visible records of earlier (round, warp) pairs and those of lower lanes.  Every load of a
+// thread's records is issued first, wanted or not: bound by the loads in flight (10M records 123 us with the
+// depth read behind the visibility test, the tests one after the other).
+// DESC: also the visible records' packed rectangles, by record.
+template <bool DESC>
 __global__ void __launch_bounds__(SCAN_T) k_vis_compact(const uint32_t* __restrict__ tiles,
                                                         const float* __restrict__ depth, int64_t P,
                                                         const uint32_t* __restrict__ bsums, int64_t nb,
@@ -642,17 +684,21 @@ __global__ void __launch_bounds__(SCAN_T) k_vis_compact(const uint32_t* __restri
                                                         const int* __restrict__ radius, int TX, int TY, int masks,
                                                         uint64_t* __restrict__ desc) {
   gs_wait_previous();
-  // desc (may be NULL): also the visible records' packed rectangles, by record
   constexpr int NW = SCAN_T / 32;
   static_assert(SCAN_ITEMS * NW == 64, "one warp scans the (round, warp) counts two per lane");
   __shared__ uint32_t s_cnt[SCAN_ITEMS * NW];
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int64_t base = (int64_t)blockIdx.x * SCAN_BLOCK;
-  uint32_t bal[SCAN_ITEMS];
+  uint32_t bal[SCAN_ITEMS], tk[SCAN_ITEMS], dk[SCAN_ITEMS];
   #pragma unroll
   for (int j = 0; j < SCAN_ITEMS; ++j) {
     int64_t k = base + (int64_t)j * SCAN_T + threadIdx.x;
-    bal[j] = __ballot_sync(0xffffffffu, k < P && tiles[k] > 0u);
+    tk[j] = k < P ? __ldg(tiles + k) : 0u;
+    dk[j] = k < P ? __float_as_uint(__ldg(depth + k)) : 0u;
+  }
+  #pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    bal[j] = __ballot_sync(0xffffffffu, tk[j] > 0u);
     if (lane == 0) s_cnt[j * NW + w] = __popc(bal[j]);
   }
   __syncthreads();
@@ -671,9 +717,9 @@ __global__ void __launch_bounds__(SCAN_T) k_vis_compact(const uint32_t* __restri
     if (bal[j] >> lane & 1u) {
       int64_t k = base + (int64_t)j * SCAN_T + threadIdx.x;
       uint32_t c = c0 + s_cnt[j * NW + w] + __popc(bal[j] & lt);
-      keys[c] = __float_as_uint(depth[k]) - d0;
+      keys[c] = dk[j] - d0;
       vals[c] = (uint32_t)k;
-      if (desc) desc[k] = pack_desc(record_rect(xy[k], radius[k], TX, TY, masks != 0, conic_op + k));
+      if (DESC) desc[k] = pack_desc(record_rect(xy[k], radius[k], TX, TY, masks != 0, conic_op + k));
     }
   if (blockIdx.x == 0 && threadIdx.x == 0) *d_vis = bsums[nb];
 }
@@ -707,13 +753,49 @@ __global__ void __launch_bounds__(SCAN_T) k_dup_reduce(const uint32_t* __restric
 // windows of EMIT_WIN and writes each window out with coalesced stores (a thread only visits the
 // instances of its records that fall in the window, so a window costs O(its instances + 8) per thread).
 // Block 0 also writes the instance count (clamped to the capacity, GS_ERR_CAPACITY beyond it).
-// desc: the packed rectangles, or NULL (the capacity leaves no room for them): computed from the arrays.
 constexpr int EMIT_WIN = 4096;
-__global__ void __launch_bounds__(SCAN_T, 4) k_dup_emit(UnitTable U, const float4* __restrict__ xy,
+struct EmitSmem {
+  uint32_t warp[33];
+  uint32_t p[SCAN_BLOCK];
+  uint32_t key[EMIT_WIN];
+  uint32_t val[EMIT_WIN];
+};
+__device__ __forceinline__ void emit_records(const uint32_t* __restrict__ v, int64_t V, EmitSmem& sm) {
+  int64_t base = (int64_t)blockIdx.x * SCAN_BLOCK;
+  #pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    int64_t i = base + (int64_t)j * SCAN_T + threadIdx.x;
+    sm.p[j * SCAN_T + threadIdx.x] = i < V ? v[i] : 0xffffffffu;
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void emit_write(const EmitSmem& sm, int64_t first, uint32_t count, int64_t cap,
+                                           uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < count; i += SCAN_T) {
+    int64_t g = first + i;
+    if (g < cap) {
+      keys[g] = sm.key[i];
+      vals[g] = sm.val[i];
+    }
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void emit_count(uint32_t total, int64_t cap, uint32_t* d_count, int* status) {
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  if ((int64_t)total > cap) {
+    set_status(status, GS_ERR_CAPACITY);
+    total = (uint32_t)cap;
+  }
+  *d_count = total;
+}
+
+// From the projected records.  Bound by instructions (a tile rectangle and an alpha box per record, 10M records
+// 246 us); packing the rectangles here and unpacking them per window (272 us in registers, 315 through shared
+// memory) was slower.
+__global__ void __launch_bounds__(SCAN_T, 3) k_dup_emit(UnitTable U, const float4* __restrict__ xy,
                                                      const float4* __restrict__ conic_op,
-                                                     const int* __restrict__ radius,
-                                                     const uint64_t* __restrict__ desc,
-                                                     const uint32_t* __restrict__ vA,
+                                                     const int* __restrict__ radius, const uint32_t* __restrict__ vA,
                                                      const uint32_t* __restrict__ vB, const int32_t* __restrict__ cur,
                                                      int final_pass, const uint32_t* __restrict__ d_vis,
                                                      const uint32_t* __restrict__ bsums, int64_t nb, int W, int H,
@@ -721,50 +803,91 @@ __global__ void __launch_bounds__(SCAN_T, 4) k_dup_emit(UnitTable U, const float
                                                      uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
                                                      uint32_t* __restrict__ d_count, int* __restrict__ status) {
   gs_wait_previous();
-  __shared__ uint32_t s_warp[33];
-  __shared__ uint32_t s_p[SCAN_BLOCK];
-  __shared__ uint32_t s_key[EMIT_WIN];
-  __shared__ uint32_t s_val[EMIT_WIN];
-  const uint32_t* v = cur[final_pass] ? vB : vA;
-  int64_t V = *d_vis;
-  int64_t base = (int64_t)blockIdx.x * SCAN_BLOCK;
+  __shared__ EmitSmem sm;
+  emit_records(cur[final_pass] ? vB : vA, *d_vis, sm);
+  int TX = (W + TILE - 1) / TILE, TY = (H + TILE - 1) / TILE;
+  int rx0[SCAN_ITEMS], ry0[SCAN_ITEMS], rw[SCAN_ITEMS], rh[SCAN_ITEMS];
+  float4 box[SCAN_ITEMS];
+  uint32_t n = 0;
   #pragma unroll
   for (int j = 0; j < SCAN_ITEMS; ++j) {
-    int64_t i = base + (int64_t)j * SCAN_T + threadIdx.x;
-    s_p[j * SCAN_T + threadIdx.x] = i < V ? v[i] : 0xffffffffu;
+    uint32_t p = sm.p[threadIdx.x * SCAN_ITEMS + j];
+    rx0[j] = ry0[j] = rw[j] = rh[j] = 0;
+    box[j] = make_float4(1.f, -1.f, 1.f, -1.f);
+    if (p != 0xffffffffu) {
+      float4 m = xy[p];
+      int x0, y0, x1, y1;
+      tile_rect(m, radius[p], TX, TY, x0, y0, x1, y1);
+      rx0[j] = x0; ry0[j] = y0; rw[j] = x1 - x0; rh[j] = y1 - y0;
+      n += (uint32_t)((x1 - x0) * (y1 - y0));
+      if (key_masks) {
+        float pm;
+        box[j] = alpha_box(make_float2(m.x, m.y), conic_op[p], pm);
+      }
+    }
   }
-  __syncthreads();
+  uint32_t tot;
+  uint32_t lo = block_excl_scan(n, sm.warp, &tot);  // this thread's first instance within the block
+  int64_t ob = (int64_t)bsums[blockIdx.x];           // the block's first instance
+  for (uint32_t win = 0; win < tot; win += EMIT_WIN) {
+    uint32_t a = lo;
+    #pragma unroll
+    for (int j = 0; j < SCAN_ITEMS; ++j) {
+      uint32_t c = (uint32_t)(rw[j] * rh[j]);
+      uint32_t k0 = a > win ? a : win;
+      uint32_t k1 = a + c < win + EMIT_WIN ? a + c : win + EMIT_WIN;
+      if (k0 < k1) {
+        uint32_t p = sm.p[threadIdx.x * SCAN_ITEMS + j];
+        uint32_t hi = (uint32_t)unit_of(U, p) << tile_bits;
+        uint32_t t = k0 - a;
+        int ty = ry0[j], tx = rx0[j];
+        if (t) { ty += (int)(t / (uint32_t)rw[j]); tx += (int)(t % (uint32_t)rw[j]); }  // from the window before
+        for (uint32_t k = k0; k < k1; ++k) {
+          uint32_t mk = key_masks ? block_mask(box[j], tx, ty) << 16 : 0u;
+          sm.key[k - win] = mk | hi | (uint32_t)(ty * TX + tx);
+          sm.val[k - win] = p;
+          if (++tx == rx0[j] + rw[j]) { tx = rx0[j]; ++ty; }
+        }
+      }
+      a += c;
+    }
+    emit_write(sm, ob + win, tot - win < (uint32_t)EMIT_WIN ? tot - win : (uint32_t)EMIT_WIN, cap, keys, vals);
+  }
+  emit_count(bsums[nb], cap, d_count, status);
+}
+
+// From the packed rectangles: one 8-byte gather per record.
+__global__ void __launch_bounds__(SCAN_T, 4) k_dup_emit_packed(
+    UnitTable U, const float4* __restrict__ xy, const float4* __restrict__ conic_op, const int* __restrict__ radius,
+    const uint64_t* __restrict__ desc, const uint32_t* __restrict__ vA, const uint32_t* __restrict__ vB,
+    const int32_t* __restrict__ cur, int final_pass, const uint32_t* __restrict__ d_vis,
+    const uint32_t* __restrict__ bsums, int64_t nb, int W, int H, int tile_bits, int64_t cap, int key_masks,
+    uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, uint32_t* __restrict__ d_count,
+    int* __restrict__ status) {
+  gs_wait_previous();
+  __shared__ EmitSmem sm;
+  emit_records(cur[final_pass] ? vB : vA, *d_vis, sm);
   int TX = (W + TILE - 1) / TILE, TY = (H + TILE - 1) / TILE;
   uint64_t d[SCAN_ITEMS];
   uint32_t cnt[SCAN_ITEMS];
   uint32_t n = 0;
   #pragma unroll
   for (int j = 0; j < SCAN_ITEMS; ++j) {
-    const uint32_t p = s_p[threadIdx.x * SCAN_ITEMS + j];
-    d[j] = p == 0xffffffffu ? 0ull : (desc ? __ldg(desc + p) : DESC_FAR);
+    const uint32_t p = sm.p[threadIdx.x * SCAN_ITEMS + j];
+    d[j] = p == 0xffffffffu ? 0ull : __ldg(desc + p);
   }
   auto rect_of = [&](int j, uint32_t p) {
     return d[j] & DESC_FAR ? record_rect(xy[p], radius[p], TX, TY, key_masks != 0, conic_op + p) : unpack_desc(d[j]);
   };
   #pragma unroll
   for (int j = 0; j < SCAN_ITEMS; ++j) {
-    const uint32_t p = s_p[threadIdx.x * SCAN_ITEMS + j];
-    cnt[j] = 0u;
-    if (p != 0xffffffffu) {
-      if (!desc) {  // every rectangle is computed once, and packed here where it fits
-        const RecordRect R = record_rect(xy[p], radius[p], TX, TY, key_masks != 0, conic_op + p);
-        d[j] = pack_desc(R);
-        cnt[j] = (uint32_t)(R.w * R.h);
-      } else {
-        const RecordRect R = rect_of(j, p);
-        cnt[j] = (uint32_t)(R.w * R.h);
-      }
-    }
+    const RecordRect R = rect_of(j, sm.p[threadIdx.x * SCAN_ITEMS + j]);
+    cnt[j] = (uint32_t)(R.w * R.h);
     n += cnt[j];
   }
   uint32_t tot;
-  uint32_t lo = block_excl_scan(n, s_warp, &tot);  // this thread's first instance within the block
-  int64_t ob = (int64_t)bsums[blockIdx.x];           // the block's first instance
+  uint32_t lo = block_excl_scan(n, sm.warp, &tot);
+  int64_t ob = (int64_t)bsums[blockIdx.x];
   for (uint32_t win = 0; win < tot; win += EMIT_WIN) {
     uint32_t a = lo;
     #pragma unroll
@@ -773,11 +896,12 @@ __global__ void __launch_bounds__(SCAN_T, 4) k_dup_emit(UnitTable U, const float
       uint32_t k0 = a > win ? a : win;
       uint32_t k1 = a + c < win + EMIT_WIN ? a + c : win + EMIT_WIN;
       if (k0 < k1) {
-        const uint32_t p = s_p[threadIdx.x * SCAN_ITEMS + j];
+        const uint32_t p = sm.p[threadIdx.x * SCAN_ITEMS + j];
         const uint32_t hi = (uint32_t)unit_of(U, p) << tile_bits;
         const RecordRect R = rect_of(j, p);
         const uint32_t t = k0 - a;
-        int dy = (int)(t / (uint32_t)R.w), dx = (int)(t % (uint32_t)R.w);
+        int dy = 0, dx = 0;
+        if (t) { dy = (int)(t / (uint32_t)R.w); dx = (int)(t % (uint32_t)R.w); }
         auto row_bits = [&](int y) {  // the row's reached blocks, spread to the first bit of each block row
           const uint32_t r = tile_blocks(R.rb, R.re, y);
           return (r & 1u) | ((r & 2u) << 3) | ((r & 4u) << 6) | ((r & 8u) << 9);
@@ -785,32 +909,16 @@ __global__ void __launch_bounds__(SCAN_T, 4) k_dup_emit(UnitTable U, const float
         uint32_t rows = row_bits(dy);
         for (uint32_t k = k0; k < k1; ++k) {
           const uint32_t mk = key_masks ? tile_blocks(R.cb, R.ce, dx) * rows << 16 : 0u;
-          s_key[k - win] = mk | hi | (uint32_t)((R.y0 + dy) * TX + R.x0 + dx);
-          s_val[k - win] = p;
+          sm.key[k - win] = mk | hi | (uint32_t)((R.y0 + dy) * TX + R.x0 + dx);
+          sm.val[k - win] = p;
           if (++dx == R.w) { dx = 0; rows = row_bits(++dy); }
         }
       }
       a += c;
     }
-    __syncthreads();
-    uint32_t wn = tot - win < (uint32_t)EMIT_WIN ? tot - win : (uint32_t)EMIT_WIN;
-    for (uint32_t i = threadIdx.x; i < wn; i += SCAN_T) {
-      int64_t g = ob + win + i;
-      if (g < cap) {
-        keys[g] = s_key[i];
-        vals[g] = s_val[i];
-      }
-    }
-    __syncthreads();
+    emit_write(sm, ob + win, tot - win < (uint32_t)EMIT_WIN ? tot - win : (uint32_t)EMIT_WIN, cap, keys, vals);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    uint32_t total = bsums[nb];
-    if ((int64_t)total > cap) {
-      set_status(status, GS_ERR_CAPACITY);
-      total = (uint32_t)cap;
-    }
-    *d_count = total;
-  }
+  emit_count(bsums[nb], cap, d_count, status);
 }
 
 // list ranges from the sorted 32-bit instance keys, and the record ids and block masks when the last
@@ -909,10 +1017,10 @@ GS_API size_t gs_bin_sort_workspace_size(int64_t n_proj, int64_t max_instances) 
 // The sort chain, shared by gs_bin_sort and the fixed-scratch variant.
 int gs_tile_order_impl(const uint32_t* ranges, int n, uint32_t* ws, uint32_t* order, cudaStream_t s);
 
-// Tile order (unless the sort already made it), then the chunk jobs in that order.
+// Tile order, then the chunk jobs in that order.
 int gs_schedule_jobs(const uint32_t* ranges, int NT, char* order_ws, char* scan_ws, const gs_schedule* sched,
-                     cudaStream_t s, bool order_done = false) {
-  int r = order_done ? GS_OK : gs_tile_order_impl(ranges, NT, (uint32_t*)order_ws, sched->tile_order, s);
+                     cudaStream_t s) {
+  int r = gs_tile_order_impl(ranges, NT, (uint32_t*)order_ws, sched->tile_order, s);
   if (r != GS_OK) return r;
   unsigned nb = (unsigned)((NT + 255) / 256);
   gs_launch(k_chunk_count, nb, 256, 0, s, (const uint2*)ranges, sched->tile_order, NT, sched->chunk, sched->job_base);
@@ -972,13 +1080,14 @@ static int depth_first_sort(const UnitTable& U, int64_t P, const gs_proj* proj, 
   const int key_masks = block_masks ? 1 : 0;
   const int TX = (width + TILE - 1) / TILE, TY = (height + TILE - 1) / TILE;
   // the packed rectangles lie behind the record pairs in keys0, which holds 8 bytes per instance.  Packing them
-  // reads 36 bytes per record in order: at 10M records that costs what the gathers of the emission save (270 us
-  // without, 301 us with it), at 107M it saves a fifth of the sort.
+  // reads 36 bytes per record in order: compaction and emission of 10M records take 269 us without and 301 us
+  // with it (the gathered arrays are not much larger than L2), of 107M 4044 and 3025 us.
   uint64_t* desc = P >= DESC_RECORDS && cap >= 2 * P ? k0 + P : nullptr;
   gs_launch(k_vis_reduce, (unsigned)nsb, SCAN_T, 0, s, proj->tiles, proj->depth, P, vec, bsums, bmins);
   gs_launch(k_scan_bsums, 1, 1024, 0, s, bsums, nsb, bmins, d_min);
-  gs_launch(k_vis_compact, (unsigned)nsb, SCAN_T, 0, s, proj->tiles, proj->depth, P, bsums, nsb, d_min, dkA, dvA,
-      d_vis, (const float4*)proj->xy, (const float4*)proj->conic_op, proj->radius, TX, TY, key_masks, desc);
+  gs_launch(desc ? k_vis_compact<true> : k_vis_compact<false>, (unsigned)nsb, SCAN_T, 0, s, proj->tiles, proj->depth,
+      P, bsums, nsb, d_min, dkA, dvA, d_vis, (const float4*)proj->xy, (const float4*)proj->conic_op, proj->radius, TX,
+      TY, key_masks, desc);
   // (three 9-bit passes and a skipped top pass measured slower: a 9-bit scatter pass took 76 us against
   // 48 us for an 8-bit one at 10M records)
   constexpr int DEPTH_PASSES = 4;
@@ -994,9 +1103,14 @@ static int depth_first_sort(const UnitTable& U, int64_t P, const gs_proj* proj, 
   uint32_t* ivA = v1;
   uint32_t* ikB = (uint32_t*)k0;
   uint32_t* ivB = (uint32_t*)k1;
-  gs_launch(k_dup_emit, (unsigned)nsb, SCAN_T, 0, s, U, (const float4*)proj->xy, (const float4*)proj->conic_op,
-      proj->radius, desc, dvA, dvB, cur, DEPTH_PASSES, d_vis, bsums, nsb, width, height, tile_bits, cap, key_masks,
-      ikA, ivA, d_num_instances, d_status);
+  if (desc)
+    gs_launch(k_dup_emit_packed, (unsigned)nsb, SCAN_T, 0, s, U, (const float4*)proj->xy, (const float4*)proj->conic_op,
+        proj->radius, desc, dvA, dvB, cur, DEPTH_PASSES, d_vis, bsums, nsb, width, height, tile_bits, cap, key_masks,
+        ikA, ivA, d_num_instances, d_status);
+  else
+    gs_launch(k_dup_emit, (unsigned)nsb, SCAN_T, 0, s, U, (const float4*)proj->xy, (const float4*)proj->conic_op,
+        proj->radius, dvA, dvB, cur, DEPTH_PASSES, d_vis, bsums, nsb, width, height, tile_bits, cap, key_masks, ikA,
+        ivA, d_num_instances, d_status);
   if (cap == 0) return gs_check_launch();
   // the instance passes keep their own buffer parity and digit totals
   int32_t* cur_t = cur + MAX_PASSES + 1;
