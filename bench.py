@@ -266,6 +266,18 @@ def kernel_launch_count(frame, lam, fused_pre=False):
     return pre + sort + fwd + loss + bwd + adam
 
 
+def step_launch_count(frame, lam, fused_pre=False):
+    """kernel_launch_count, with the launches that depend on the frame's sizes: up to 8192 lists the schedule is one
+    launch instead of seven, and the scheduled forward is the empty lists and the front, and the chunk, combine and
+    stop passes where the capacity allows a list of more than 16 chunks."""
+    n = kernel_launch_count(frame, lam, fused_pre)
+    if frame.use_masks:
+        if frame.n_tiles * frame.units.n <= 8192:
+            n -= 6
+        n += (2 + (3 if frame.cap // frame.chunk + 1 > 16 and not frame.walk_whole_lists else 0)) - 3
+    return n
+
+
 def run_ours(args, wl, rank, world):
     import torch
     import paper_2509_12138_gb300 as gs
@@ -457,7 +469,7 @@ def run_ours(args, wl, rank, world):
                 render_mode=render_mode, visible=visible, zero_grad_frac=float(np.mean(zero_frac)),
                 sort_design=args.sort,
                 sparse_adam=bool(args.sparse_adam), fused_pre=fuse, h2d=(3 * H * W * 4 + H * W), d2h=4,
-                launches=kernel_launch_count(frame, LAMBDA_SSIM, fuse) * args.steps, N=N, W=W, H=H)
+                launches=step_launch_count(frame, LAMBDA_SSIM, fuse) * args.steps, N=N, W=W, H=H)
 
 
 # Blend kernels' algorithmic work: FP32 issue slots (one per lane-operation, FMA and MUFU included) per

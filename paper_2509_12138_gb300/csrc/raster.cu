@@ -1616,17 +1616,26 @@ __global__ void k_order_hist(const uint2* __restrict__ ranges, int n, uint32_t* 
 __global__ void k_order_scatter(const uint2* __restrict__ ranges, int n, const uint32_t* __restrict__ hist,
                                 uint32_t* __restrict__ cursor, uint32_t* __restrict__ order) {
   gs_wait_previous();
-  __shared__ uint32_t s_base[33];
+  __shared__ uint32_t s_base[33], s_cnt[33];
+  if (threadIdx.x < 33) { s_base[threadIdx.x] = hist[threadIdx.x]; s_cnt[threadIdx.x] = 0u; }
+  __syncthreads();
   if (threadIdx.x == 0) {
     uint32_t acc = 0;
-    for (int c = 32; c >= 0; --c) { s_base[c] = acc; acc += hist[c]; }  // heavy classes first
+    for (int c = 32; c >= 0; --c) { const uint32_t h = s_base[c]; s_base[c] = acc; acc += h; }  // heavy classes first
+  }
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  int c = 0;
+  uint32_t rank = 0u;
+  if (i < n) {
+    uint2 r = ranges[i];
+    c = 32 - __clz(r.y - r.x);
+    rank = atomicAdd(&s_cnt[c], 1u);
   }
   __syncthreads();
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  uint2 r = ranges[i];
-  int c = 32 - __clz(r.y - r.x);
-  order[s_base[c] + atomicAdd(&cursor[c], 1u)] = (uint32_t)i;
+  // one global atomic per block and class (most lists are empty: one per list queued up on that class's counter)
+  if (threadIdx.x < 33 && s_cnt[threadIdx.x]) s_base[threadIdx.x] += atomicAdd(&cursor[threadIdx.x], s_cnt[threadIdx.x]);
+  __syncthreads();
+  if (i < n) order[s_base[c] + rank] = (uint32_t)i;
 }
 
 // Work counters of one rendered view (diagnostic, outside any timed region):

@@ -964,6 +964,91 @@ __global__ void __launch_bounds__(256) k_ranges32(const uint32_t* __restrict__ k
   }
 }
 
+// The whole schedule of up to SCHED_ONE lists in one CTA: the tile order
+// (heaviest length classes first), the job base of every order position and
+// the chunk jobs.  It replaces a memset and seven launches of a few
+// microseconds each, 25 us of a 1080p view's sort; beyond the lists one CTA
+// holds, those pay.
+constexpr int SCHED_ONE = 8192, SCHED_T = 1024, SCHED_PER = SCHED_ONE / SCHED_T;
+__global__ void __launch_bounds__(SCHED_T) k_schedule(const uint2* __restrict__ ranges, int NT, int K,
+                                                      uint32_t* __restrict__ order, uint32_t* __restrict__ job_base,
+                                                      uint32_t* __restrict__ jobs, int64_t max_jobs) {
+  gs_wait_previous();
+  constexpr int NW = SCHED_T / 32, CLASSES = 34;  // class c: lengths of c bits; 33: past the last list
+  __shared__ uint32_t s_wc[NW][CLASSES + 1];  // per-warp class counts, then each warp's next place within the class
+  __shared__ uint32_t s_class[CLASSES];
+  __shared__ uint32_t s_base[SCHED_ONE + 1];  // chunks per order position, then the jobs in front of it
+  __shared__ uint32_t s_warp[33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint32_t len[SCHED_PER];
+  #pragma unroll
+  for (int e = 0; e < SCHED_PER; ++e) {
+    const int i = e * SCHED_T + (int)threadIdx.x;
+    const uint2 r = i < NT ? __ldg(ranges + i) : make_uint2(0u, 0u);
+    len[e] = r.y - r.x;
+  }
+  for (int c = lane; c <= CLASSES; c += 32) s_wc[w][c] = 0u;
+  __syncwarp();
+  // every warp counts its own lists (atomics on the classes' counters would queue up: most lists are empty)
+  #pragma unroll
+  for (int e = 0; e < SCHED_PER; ++e) {
+    const int c = e * SCHED_T + (int)threadIdx.x < NT ? 32 - __clz((int)len[e]) : 33;
+    const uint32_t peers = __match_any_sync(0xffffffffu, c);
+    if (lane == __ffs(peers) - 1) s_wc[w][c] += (uint32_t)__popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+  for (int c = w; c < 33; c += NW) {  // class c: exclusive scan over the warps
+    const uint32_t v = s_wc[lane][c], inc = warp_incl_scan(v);
+    s_wc[lane][c] = inc - v;
+    if (lane == 31) s_class[c] = inc;
+  }
+  __syncthreads();
+  if (w == 0) {  // exclusive scan from class 32 down; class 0 takes what is left
+    const uint32_t v = s_class[32 - lane], inc = warp_incl_scan(v);
+    s_class[32 - lane] = inc - v;
+    __syncwarp();
+    if (lane == 31) s_class[0] = inc;
+  }
+  __syncthreads();
+  #pragma unroll
+  for (int e = 0; e < SCHED_PER; ++e) {
+    const int i = e * SCHED_T + (int)threadIdx.x;
+    const int c = i < NT ? 32 - __clz((int)len[e]) : 33;
+    const uint32_t peers = __match_any_sync(0xffffffffu, c);
+    const uint32_t o = s_class[min(c, 32)] + s_wc[w][c] + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+    __syncwarp();
+    if (lane == __ffs(peers) - 1) s_wc[w][c] += (uint32_t)__popc(peers);
+    __syncwarp();
+    if (c < 33) {
+      order[o] = (uint32_t)i;
+      s_base[o] = (len[e] + (uint32_t)K - 1u) / (uint32_t)K;
+    }
+  }
+  __syncthreads();
+  const int p0 = (int)threadIdx.x * SCHED_PER;
+  uint32_t n[SCHED_PER], sum = 0u, total;
+  #pragma unroll
+  for (int e = 0; e < SCHED_PER; ++e) { n[e] = p0 + e < NT ? s_base[p0 + e] : 0u; sum += n[e]; }
+  uint32_t at = block_excl_scan(sum, s_warp, &total);  // (its barriers: every count is read before it is replaced)
+  #pragma unroll
+  for (int e = 0; e < SCHED_PER; ++e) {
+    if (p0 + e < NT) s_base[p0 + e] = at;
+    at += n[e];
+  }
+  if (threadIdx.x == 0) s_base[NT] = total;
+  __syncthreads();
+  for (int o = threadIdx.x; o <= NT; o += SCHED_T) job_base[o] = s_base[o];
+  for (int o = w; o < NT; o += SCHED_T / 32) {
+    const uint32_t b = s_base[o], end = s_base[o + 1];
+    if (b == end) break;  // the lists behind it are empty too
+    for (uint32_t j = b + (uint32_t)lane; j < end && (int64_t)j < max_jobs; j += 32) {
+      jobs[2 * (int64_t)j] = (uint32_t)o;
+      jobs[2 * (int64_t)j + 1] = j - b;
+    }
+  }
+}
+
 // number of chunks of each list, in tile order
 __global__ void k_chunk_count(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order, int NT, int K,
                               uint32_t* __restrict__ counts) {
@@ -1020,6 +1105,11 @@ int gs_tile_order_impl(const uint32_t* ranges, int n, uint32_t* ws, uint32_t* or
 // Tile order, then the chunk jobs in that order.
 int gs_schedule_jobs(const uint32_t* ranges, int NT, char* order_ws, char* scan_ws, const gs_schedule* sched,
                      cudaStream_t s) {
+  if (NT <= SCHED_ONE) {
+    gs_launch(k_schedule, 1, SCHED_T, 0, s, (const uint2*)ranges, NT, sched->chunk, sched->tile_order, sched->job_base,
+        sched->jobs, sched->max_jobs);
+    return gs_check_launch();
+  }
   int r = gs_tile_order_impl(ranges, NT, (uint32_t*)order_ws, sched->tile_order, s);
   if (r != GS_OK) return r;
   unsigned nb = (unsigned)((NT + 255) / 256);

@@ -160,7 +160,7 @@ def _lists_by_numpy(fr, cap):
 @pytest.mark.parametrize("n,views,W,H,cap", [
     (1, 1, 16, 16, 64), (33, 2, 40, 24, 1000), (1025, 3, 100, 60, 1 << 15), (1500, 2, 64, 64, 2000),
     (1500, 2, 64, 64, 1), (16384, 1, 48, 48, 1 << 17), (16385, 1, 48, 48, 1 << 17), (700, 1, 1024, 1024, 1 << 15),
-    (300, 1, 1040, 1024, 1 << 15)])
+    (300, 1, 1040, 1024, 1 << 15), (500, 1, 2048, 1024, 1 << 16), (500, 1, 2064, 1024, 1 << 16)])
 def test_sort_lists_at_design_limits(n, views, W, H, cap):
     """Both sides of the small sort's limits (records per unit, number of lists), partial warps and rounds, several
     units, and a capacity that runs out, inside a record too: lists, ranges, counts and the chunk jobs."""
