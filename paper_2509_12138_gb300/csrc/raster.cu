@@ -491,6 +491,8 @@ __device__ __forceinline__ int scan_hits(const uint16_t* __restrict__ masks, int
   return qn;
 }
 
+__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
 // Front-to-back walk of list entries [beg, end) (indices from the list's
 // start `off`) for one warp's pixel block (tile-local origin (ox, oy)):
 // composites into (T, c, last) of the lanes that are not done; a lane whose
@@ -508,9 +510,12 @@ __device__ __forceinline__ void walk_fwd(const uint32_t* __restrict__ vals, cons
   vals += off;
   masks += off;
   int scan = beg, qn = 0, qh = 0;  // next entry to scan; queued entries are q[qh .. qn)
-  for (;;) {
-    const uint32_t act = __ballot_sync(FULL, !done);
-    if (!act) break;
+  // Queues the next batch's entries and starts its records on their way to L1, one batch ahead of their use, and the
+  // masks and ids of the following scan (the next chunk's too: no gain).  The warps that fit (20 per SM at 96
+  // registers) do not cover the latency of masks, ids and records in turn: waiting for each, the forward stage took 4
+  // to 8% longer (10M at 1080p, two views, 1203, 1515 -> 1147, 1398 us; merged 100M at 4K 7462 -> 7092; 6M at 400x300
+  // 1249 -> 1151).
+  auto next_batch = [&]() -> uint32_t {
     if (qn - qh < 32 && scan < end) {
       // the left-over entries to the front, then whole scans until a batch is full
       const uint32_t keep = qh + lane < qn ? sc.q[qh + lane] : 0u;
@@ -523,13 +528,34 @@ __device__ __forceinline__ void walk_fwd(const uint32_t* __restrict__ vals, cons
         scan += SCAN;
       } while (qn < 32 && scan < end);
       __syncwarp();
+      // one lane per 128 bytes: 64 masks or 32 ids
+      const int ahead = scan + (lane < SCAN / 64 ? 64 * lane : 32 * (lane - SCAN / 64));
+      if (lane < SCAN / 64 + SCAN / 32 && ahead < end) {
+        if (lane < SCAN / 64) prefetch_l1(masks + ahead);
+        else prefetch_l1(vals + ahead);
+      }
     }
+    uint32_t p = 0u;
+    if (qh + lane < qn) {
+      p = vals[sc.q[qh + lane]];
+      prefetch_l1(xy + p);
+      prefetch_l1(conic_op + p);
+      prefetch_l1(rgb + p);
+    }
+    return p;
+  };
+  uint32_t pn = next_batch();
+  for (;;) {
+    const uint32_t act = __ballot_sync(FULL, !done);
+    if (!act) break;
     const int nb = min(32, qn - qh);
     if (nb == 0) break;
+    const uint32_t p = pn, entry = lane < nb ? sc.q[qh + lane] : 0u;
+    qh += nb;
+    pn = next_batch();
     // record-major: alpha of hit `lane` at the pixels its box reaches
     uint32_t valid = 0u;
     if (lane < nb) {
-      const uint32_t p = vals[sc.q[qh + lane]];
       const float4 m = xy[p], co = conic_op[p], c = rgb[p];
       const float rx = rel_pos(m.x, m.z, tox), ry = rel_pos(m.y, m.w, toy);
       sc.r[lane] = c.x; sc.g[lane] = c.y; sc.b[lane] = c.z;
@@ -573,8 +599,8 @@ __device__ __forceinline__ void walk_fwd(const uint32_t* __restrict__ vals, cons
         }
       }
     }
-    if (lj >= 0) last = (int)sc.q[qh + lj] + 1;
-    qh += nb;
+    const int at = (int)__shfl_sync(FULL, entry, max(lj, 0));
+    if (lj >= 0) last = at + 1;
     __syncwarp();
   }
   __syncwarp();
@@ -619,8 +645,9 @@ __device__ __forceinline__ void walk_fwd(const uint32_t* __restrict__ vals, cons
 // 1926, 1853 -> 1274, 1211; 1M there 396, 395 / 465, 494 / 542, 619 -> 390, 390.
 // Where the capacity bounds every list to FRONT_CHUNKS chunks, the passes behind
 // the front are not launched at all (5 us each with nothing to do).
-// 88 registers, 22 warps per SM; held to 80, 72 and 64 the 10M views took 1275,
-// 1265 and 1423 us.
+// (Figures before the records were fetched a batch ahead.  Held to 80, 72 and 64
+// of its then 88 registers the front took 1275, 1265 and 1423 us on the first 10M
+// view.)
 constexpr int FRONT_CHUNKS = 16;
 __device__ __forceinline__ int front_chunks(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
                                             uint32_t jobs, uint32_t lists, uint32_t warps, int K) {
