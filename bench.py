@@ -564,7 +564,7 @@ def rooflines(res, workload=None, issue=None, random_order=False):
         work.pop("preprocess")
     kernel = {"preprocess": "k_preprocess", "bin_sort": "sort chain",
               "project_bwd_adam": "k_project_bwd_adam1 (+ the next step's a1)" if fused else "k_project_bwd_adam1",
-              "loss": "loss kernels", "render_fwd": "k_render_fwd_m + k_render_fwd_combine + k_render_fwd_stop",
+              "loss": "loss kernels", "render_fwd": "k_render_fwd_front + _chunk + _combine + _stop",
               "blend_bwd": "k_render_bwd_m"}
     out = {}
     for name, ms in zip(res["stages"], res["stage_ms"]):

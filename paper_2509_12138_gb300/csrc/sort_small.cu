@@ -1,7 +1,7 @@
 // a2 for small problems: the lists, ranges and blend schedule of gs_bin_sort in
 // four launches.
 //
-// The general design takes 33 launches whatever the size; with a few thousand
+// The general design takes 27 launches whatever the size; with a few thousand
 // records each of them is a few microseconds of launch and one round of memory
 // latency.  Here one CTA per unit sorts the unit's records by depth in shared
 // memory, and every (unit, tile) list is then made by a warp of its own that
