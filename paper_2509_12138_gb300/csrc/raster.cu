@@ -454,7 +454,10 @@ __device__ __forceinline__ uint32_t eval_hit(float rx, float ry, float4 co, floa
 // and the order of a pixel's compositing are those of a sequential walk.  Bound
 // by instruction issue (47-70% of cycles on a 2M scene) and, on edge-on views,
 // by the longest block's serial walk.  Forward stage at one lane per pixel and
-// hit -> this: 200k at 960x540 134 -> 98 us, 1M at 1080p 319 -> 199 us.
+// hit -> this: 200k at 960x540 134 -> 88 us, 1M at 1080p 319 -> 181 us.  Three
+// or four pairs per step of the pixel-major loop, or four pixels per step of the
+// record-major one, cost registers and were slower (10M at 1080p 1157 us with
+// two, 1208, 1302 and 1264).
 constexpr int SCAN = 256;            // entries whose masks are read at a time (8 per lane)
 constexpr int QUEUE_CAP = SCAN + 32; // queued entries: a full scan behind at most 31 left over
 constexpr int MROW = 33;             // row stride of the (hit, pixel) matrices
