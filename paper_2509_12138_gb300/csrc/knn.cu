@@ -83,9 +83,12 @@ __device__ __forceinline__ float dist2(float4 a, float4 b) {
   return __fmaf_rn(ez, ez, __fmaf_rn(ey, ey, __fmul_rn(ex, ex)));
 }
 
-// distance along one axis from p to cells c + lo .. c + hi (0 inside)
-__device__ __forceinline__ float axis_gap(float p, float lo, const Grid& g, int c0, int c1) {
-  return fmaxf(0.f, fmaxf(lo + (float)c0 * g.h - p, p - (lo + (float)(c1 + 1) * g.h)) - g.slack);
+// distance along one axis from p to the points held by cells c0 .. c1 (0 inside).  Points from outside the grid are
+// held by its outermost cells, so those reach on without end.
+__device__ __forceinline__ float axis_gap(float p, float lo, const Grid& g, int c0, int c1, int dim) {
+  const float below = c0 > 0 ? lo + (float)c0 * g.h - p : 0.f;
+  const float above = c1 < dim - 1 ? p - (lo + (float)(c1 + 1) * g.h) : 0.f;
+  return fmaxf(0.f, fmaxf(below, above) - g.slack);
 }
 
 // Calls f(point) for the points of the cells that cube radius R adds to radius
@@ -99,7 +102,7 @@ __device__ __forceinline__ void visit(const Grid& g, const uint32_t* __restrict_
     xa = max(xa, 0);
     xb = min(xb, g.dim[0] - 1);
     if (xa > xb) return;
-    const float gx = axis_gap(p[0], g.lo[0], g, xa, xb);
+    const float gx = axis_gap(p[0], g.lo[0], g, xa, xb, g.dim[0]);
     if ((d2yz + gx * gx) * 0.999f > limit()) return;
     const uint32_t e = start[row + xb + 1];
     for (uint32_t q = start[row + xa]; q < e; ++q) f(sorted[q]);
@@ -107,11 +110,11 @@ __device__ __forceinline__ void visit(const Grid& g, const uint32_t* __restrict_
   for (int dz = -R; dz <= R; ++dz) {
     const int z = c[2] + dz;
     if (z < 0 || z >= g.dim[2]) continue;
-    const float gz = axis_gap(p[2], g.lo[2], g, z, z);
+    const float gz = axis_gap(p[2], g.lo[2], g, z, z, g.dim[2]);
     for (int dy = -R; dy <= R; ++dy) {
       const int y = c[1] + dy;
       if (y < 0 || y >= g.dim[1]) continue;
-      const float gy = axis_gap(p[1], g.lo[1], g, y, y);
+      const float gy = axis_gap(p[1], g.lo[1], g, y, y, g.dim[1]);
       const float d2 = gz * gz + gy * gy;
       const int64_t row = ((int64_t)z * g.dim[1] + y) * g.dim[0];
       if (whole || dz == -R || dz == R || dy == -R || dy == R) {

@@ -97,6 +97,44 @@ def test_knn_ties_exact(n, k):
         assert np.array_equal(idx[i], want) and np.array_equal(dist[i], wd)
 
 
+def _knn_on_grid(pts, k, lo, h, dims, aligned=True):
+    """gs_knn on a grid of the caller's choice; aligned False: results to arrays 4 bytes past a 16-byte boundary."""
+    L, n = gi._lib.load(), len(pts)
+    p = torch.from_numpy(pts).cuda()
+    lo, dims = np.asarray(lo, np.float32), np.asarray(dims, np.int32)
+    dp = dims.ctypes.data_as(gi._lib.c_i32p)
+    ws = torch.empty(L.gs_knn_workspace_size(n, dp), dtype=torch.uint8, device="cuda")
+    idx, dist = torch.empty((n, k), dtype=torch.int32, device="cuda"), torch.empty((n, k), device="cuda")
+    if not aligned:
+        idx, dist = _off_by_one(idx), _off_by_one(dist)
+    gi.check(L.gs_knn(gi._ptr(p), n, k, lo.ctypes.data_as(gi._lib.c_f32p), h, dp, gi._ptr(ws), ws.numel(),
+                      gi._ptr(idx), gi._ptr(dist), gi._stream()), "gs_knn")
+    return idx.cpu().numpy(), dist.cpu().numpy()
+
+
+def _nearest_on_lattice(pts, i, k):
+    """The k nearest others of point i by (distance, index), exact for points on a lattice of eighths."""
+    q = (pts * 8).astype(np.int64)
+    d2 = ((q - q[i]) ** 2).sum(1)
+    o = np.lexsort((np.arange(len(pts)), d2))
+    o = o[o != i][:k]
+    return o, np.sqrt((d2[o] / 64.0).astype(np.float32))
+
+
+@pytest.mark.parametrize("k", [3, 8, 16])
+@pytest.mark.parametrize("cells", [1, 2, 8])
+def test_knn_points_outside_the_grid(k, cells):
+    """Points from outside the grid are held by its outermost cells and have the neighbours that all points' distances
+    give, whichever side of it they and their neighbours lie on."""
+    g = np.random.default_rng(k + cells)
+    pts = (g.integers(-12, 21, (700, 3)) / 8.0).astype(np.float32)
+    pts[:20] += 40.0  # a group far away from the grid
+    idx, dist = _knn_on_grid(pts, k, (0.0, 0.0, 0.0), 1.0 / cells, (cells,) * 3)
+    for i in range(len(pts)):
+        want, wd = _nearest_on_lattice(pts, i, k)
+        assert np.array_equal(idx[i], want) and np.array_equal(dist[i], wd)
+
+
 @pytest.mark.parametrize("W,H,units", [(1, 1, 1), (31, 33, 2), (32, 32, 1), (65, 10, 3), (100, 71, 2)])
 def test_loss_partial_tiles(W, H, units):
     """Image edges inside the loss kernels' tiles, planes that are no multiple of 16 bytes, several units; bounds
