@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(KNN_T) k_knn_query(int64_t n, Grid g, const ui
   visit(g, start, sorted, c, p, R, true, kth, [&](float4 o) {
     const float d = dist2(o, me);
     const int j = __float_as_int(o.w);
-    if (!(d <= last) || j == i) return;
+    if (!(d <= last) || !(d < INFINITY) || j == i) return;  // (a distance past the float range is no neighbour's)
     const unsigned long long key = ((unsigned long long)__float_as_uint(d) << 32) | (uint32_t)j;
     if (d < last) {
       if (n1 < K) s_best[n1++][threadIdx.x] = key;

@@ -135,6 +135,21 @@ def test_knn_points_outside_the_grid(k, cells):
         assert np.array_equal(idx[i], want) and np.array_equal(dist[i], wd)
 
 
+@pytest.mark.parametrize("k", [3, 8, 16])
+def test_knn_distances_past_the_float_range(k):
+    """A point whose squared distance overflows float32 is no neighbour: its slot is -1 / inf, as when there are too few."""
+    x = np.array([0.0, 1.0, 2.0, 1e20, 1e20 + 1e13, 3e20, np.nan, np.inf], np.float32)
+    pts = np.zeros((len(x), 3), np.float32)
+    pts[:, 0] = x
+    idx, dist = _knn_on_grid(pts, k, (-1.0, -1.0, -1.0), 1e20, (4, 1, 1))
+    with np.errstate(over="ignore", invalid="ignore"):
+        d2 = (x[:, None] - x[None, :]) ** 2
+    for i in range(len(x)):
+        near = sorted((d2[i, j], j) for j in range(len(x)) if j != i and np.isfinite(d2[i, j]))[:k]
+        assert idx[i].tolist() == [j for _, j in near] + [-1] * (k - len(near))
+        assert dist[i].tolist() == [float(np.sqrt(d)) for d, _ in near] + [np.inf] * (k - len(near))
+
+
 @pytest.mark.parametrize("W,H,units", [(1, 1, 1), (31, 33, 2), (32, 32, 1), (65, 10, 3), (100, 71, 2)])
 def test_loss_partial_tiles(W, H, units):
     """Image edges inside the loss kernels' tiles, planes that are no multiple of 16 bytes, several units; bounds
