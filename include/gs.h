@@ -232,10 +232,10 @@ int gs_bin_sort(const gs_proj* proj, const gs_units* units, int width, int heigh
  * (depth, record index) order.  It needs unit | tile ids of at most 16 bits
  * (one 4K unit: 15 bits; eight 1080p units: 16); for more it runs
  * gs_bin_sort_global.  On capacity overflow the nearest instances are kept.
- * Small problems (at most 16,384 records per unit, 4,096 lists and 2^26 records
- * x tiles per unit grid) take four launches instead: each unit's records sorted
- * by depth in one CTA, each list gathered by a warp from its unit's tile
- * rectangles in that order.
+ * Small problems take four launches instead: each unit's records sorted by
+ * depth in one CTA, each list gathered by a warp from its unit's tile
+ * rectangles in that order.  They have at most 4,096 lists, and at most 2,048 +
+ * 640 max_instances / n_proj records per unit, 16,384 in any case.
  *
  * gs_bin_sort_global and gs_bin_sort_bucketed: the same lists, ranges,
  * instance count and schedule as gs_bin_sort (same arguments and workspace)

@@ -1224,7 +1224,7 @@ static int depth_first_sort(const UnitTable& U, int64_t P, const gs_proj* proj, 
   return gs_check_launch();
 }
 
-bool gs_small_sort_applies(const UnitTable& U, int64_t P, int n_tiles);
+bool gs_small_sort_applies(const UnitTable& U, int64_t P, int n_tiles, int64_t cap);
 size_t gs_small_sort_ctrl_words();
 int gs_small_sort(const UnitTable& U, const gs_proj* proj, int width, int height, int64_t cap, uint32_t* rec,
                   uint2* rect, uint32_t* count, void* ctrl_ws, uint32_t* sorted_vals, uint32_t* ranges,
@@ -1275,7 +1275,7 @@ int gs_bin_sort_impl(const gs_proj* proj, const gs_units* units, int width, int 
   // its buffers: rectangles and records in the key buffers (8 bytes per record each), list lengths in the digit
   // totals (4096 words), control words in the schedule's scan scratch (over 4000 words)
   static_assert(RS_BINS_MAX * MAX_PASSES >= 4096 && MAX_SCHED_TILES / SCAN_BLOCK > 1024, "small sort's scratch");
-  if (method == 2 && P > 0 && max_instances > 0 && gs_small_sort_applies(U, P, n_tiles))
+  if (method == 2 && P > 0 && max_instances > 0 && gs_small_sort_applies(U, P, n_tiles, max_instances))
     return gs_small_sort(U, proj, width, height, max_instances, (uint32_t*)k1, (uint2*)k0, totals, ws + L.jscan,
                          sorted_vals, ranges, d_num_instances, sched, d_status, s);
   if (cudaMemsetAsync(ranges, 0, sizeof(uint32_t) * 2 * (size_t)n_tiles * U.n, s) != cudaSuccess ||

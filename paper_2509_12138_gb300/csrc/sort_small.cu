@@ -1,7 +1,7 @@
 // a2 for small problems: the lists, ranges and blend schedule of gs_bin_sort in
 // four launches.
 //
-// The general design takes 27 launches whatever the size; with a few thousand
+// The general design takes 23 launches (26 with over 256 lists), schedule included; with a few thousand
 // records each of them is a few microseconds of launch and one round of memory
 // latency.  Here one CTA per unit sorts the unit's records by depth in shared
 // memory, and every (unit, tile) list is then made by a warp of its own that
@@ -13,6 +13,7 @@
 // of 2,000 records on 64 tiles: 204 -> 66 us (43 and 90 us with 32 records per
 // step of a list's warp instead of 128, and 8 lists per block instead of 4).
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -26,8 +27,7 @@ constexpr int ST = 1024;                 // threads of the unit sort
 constexpr int SW = ST / 32;
 constexpr int ROUNDS = 16;               // records per thread
 constexpr int UNIT_MAX = ST * ROUNDS;    // records per unit
-constexpr int LISTS_MAX = 4096;          // (unit, tile) lists
-constexpr int64_t TESTS_MAX = 1 << 26;   // records x tiles
+constexpr int LISTS_MAX = 4096;          // (unit, tile) lists; with UNIT_MAX records each, at most 2^26 tests and instances
 
 // device words shared by the launches
 struct Ctrl {
@@ -435,13 +435,22 @@ __global__ void __launch_bounds__(LW * 32) k_small_fill(UnitTable U, int W, int 
 
 }  // namespace
 
-// Whether the design applies: every unit's records fit one CTA's shared memory
-// and the tests of every list against its unit's records stay far below what
-// the general design's launches cost.
-bool gs_small_sort_applies(const UnitTable& U, int64_t P, int n_tiles) {
-  if ((int64_t)U.n * n_tiles > LISTS_MAX || P * n_tiles > TESTS_MAX) return false;
+// Whether the design applies: it is taken up to where its time crosses the general design's.  A list's warp reads all
+// records of its unit, twice, so this design takes 13 us + 20 ns per record of the largest unit, whatever they cover;
+// the general one hardly depends on the number of so few records but on their instances, since one thread emits all of
+// a record's: 85 us + 10 to 35 us per instance a record has.  The capacity stands for the instances (where it was
+// fitted, 1.25 times their number).  us per call, this design / general / the limit (splats of a sphere's surface;
+// the last one random sizes):
+//   48 x 48, 1 unit       2,000   57 / 80 / 3,850    4,000   93 / 88 / 3,640     8,000  172 / 90 / 3,500
+//   128 x 128, 8 units    3,000   78 / 122 / 4,620   5,000  116 / 107 / 4,210    8,000  174 / 103 / 3,940
+//   256 x 256, 8 units    3,000   83 / 175 / 7,150   5,000  124 / 144 / 5,870    8,000  177 / 130 / 5,070
+//   512 x 512, 4 units    4,000  107 / 369 / 12,480  8,000  176 / 226 / 8,540   16,384  313 / 142 / 6,300
+//   1024 x 1024, 1 unit   4,000   99 / 1549 / 16,384 8,000  158 / 728 / 16,384  16,384  412 / 27680 / 16,384
+bool gs_small_sort_applies(const UnitTable& U, int64_t P, int n_tiles, int64_t cap) {
+  if ((int64_t)U.n * n_tiles > LISTS_MAX) return false;
+  const double most = fmin((double)UNIT_MAX, 2048.0 + 640.0 * (double)cap / (double)P);
   for (int u = 0; u < U.n; ++u)
-    if (U.proj_base[u + 1] - U.proj_base[u] > UNIT_MAX) return false;
+    if ((double)(U.proj_base[u + 1] - U.proj_base[u]) > most) return false;
   return true;
 }
 

@@ -1,5 +1,6 @@
 """Helpers for the GPU parity tests: run the CUDA path through the C ABI and
 compare with the oracle under the exclusion rules for FP32-vs-FP64 near-ties."""
+import ctypes as C
 import math
 
 import numpy as np
@@ -105,3 +106,24 @@ def exclusion_mask(o_proj, g_xy4, g_radius, g_tiles, margin, W, H, margin_tol=1e
     pix = np.kron(bad_tile, np.ones((TILE, TILE), bool))[:H, :W]
     pix |= margin < margin_tol
     return pix, int(mism.sum()), flagged
+
+
+def captured_kernels(fn):
+    """Kernels that fn launches on the current stream (captured into a graph, not run)."""
+    rt = C.CDLL("libcudart.so." + torch.version.cuda.split(".")[0])
+    stream, graph, n = torch.cuda.Stream(), C.c_void_p(), C.c_size_t()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        assert rt.cudaStreamBeginCapture(C.c_void_p(stream.cuda_stream), 2) == 0  # relaxed
+        try:
+            fn()
+        finally:
+            assert rt.cudaStreamEndCapture(C.c_void_p(stream.cuda_stream), C.byref(graph)) == 0
+    assert rt.cudaGraphGetNodes(graph, None, C.byref(n)) == 0
+    nodes, kind, kernels = (C.c_void_p * n.value)(), C.c_int(), 0
+    assert rt.cudaGraphGetNodes(graph, nodes, C.byref(n)) == 0
+    for node in nodes:
+        assert rt.cudaGraphNodeGetType(C.c_void_p(node), C.byref(kind)) == 0
+        kernels += kind.value == 0
+    assert rt.cudaGraphDestroy(graph) == 0
+    return kernels

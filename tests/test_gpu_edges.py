@@ -7,6 +7,7 @@ import oracle
 import synth
 from paper_2509_12138_gb300 import Frame, Units
 from paper_2509_12138_gb300 import init as gi
+from tests.gpu_util import captured_kernels
 
 pytestmark = pytest.mark.gpu
 
@@ -238,6 +239,32 @@ def test_sort_lists_at_design_limits(n, views, W, H, cap):
     assert sorted(order.tolist()) == list(range(len(lens))) and np.array_equal(np.diff(base), chunks)
     assert np.array_equal(jobs[:, 0], np.repeat(np.arange(len(order)), chunks))
     assert np.array_equal(jobs[:, 1], np.concatenate([np.arange(c) for c in chunks]))
+
+
+@pytest.mark.parametrize("n,views,W,H,cap", [
+    (3328, 1, 48, 48, 6656), (3329, 1, 48, 48, 6658), (4096, 3, 80, 64, 1 << 17), (16384, 1, 48, 48, 1 << 19),
+    (5000, 2, 64, 64, 4097), (6000, 1, 200, 150, 9001), (9000, 2, 100, 60, 20000), (9000, 2, 100, 60, 1)])
+def test_sort_lists_at_record_limit(n, views, W, H, cap):
+    """Both sides of the small sort's limits of records per unit, and a capacity that runs out in the general design:
+    in its first window of 4,096 staged instances, behind it, and inside a record."""
+    test_sort_lists_at_design_limits(n, views, W, H, cap)
+
+
+@pytest.mark.parametrize("n,views,W,H,cap,small", [
+    (3328, 1, 48, 48, 2, True), (3329, 1, 48, 48, 2, False), (4608, 8, 128, 128, 4, True),
+    (4609, 8, 128, 128, 4, False), (16384, 1, 64, 64, 4, False), (16384, 1, 64, 64, 23, True),
+    (16384, 1, 64, 64, 22, False), (16385, 1, 64, 64, 40, False), (500, 1, 2048, 512, 4, True),
+    (500, 1, 2048, 1024, 4, False)])
+def test_sort_design_by_sizes(n, views, W, H, cap, small):
+    """The small sort's four launches up to 4,096 lists and 2,048 + 640 records per unit and instance that the capacity
+    leaves a record (16,384 at most), the general design's beyond: there it is the faster one."""
+    import paper_2509_12138_gb300 as gs
+    g = synth.random_gaussians(n, 0, n, extent=0.8, log_scale_range=(-4.0, -3.0))
+    cams = synth.orbital_cameras(8, 3.0, width=W, height=H).subset(list(range(views)))
+    fr = Frame(n, Units.single(n, views), W, H, 0, max_instances=cap * n * views, with_backward=False, with_loss=False)
+    fr.preprocess(gs.pack_params(g, 0), gs.pack_cameras(cams))
+    kernels = captured_kernels(fr.sort)
+    assert kernels == 4 if small else kernels >= 18
 
 
 @pytest.mark.parametrize("wide", [False, True])

@@ -198,3 +198,27 @@ def test_depth_first_sort_depth_range(z_far):
     d = fr.depth.cpu().numpy()[fr.radius.cpu().numpy() > 0].view(np.uint32).astype(np.int64)
     span = int(d.max() - d.min())
     assert (span >= 1 << 24) == (z_far > 2.0), span
+
+
+@pytest.mark.parametrize("z_far", [1.9, 1e6])
+def test_depth_first_sort_depth_range_of_many_records(z_far):
+    """Depths as above in more records than the small sort takes, a few pixels each: the depth-first design's own radix
+    passes, with the top one skipped (1.9) and run (1e6), and two instance passes."""
+    rng = np.random.default_rng(int(z_far) % 89)
+    W = H = 288
+    cams = scenes.identity_camera(W, H)
+    f, cx = float(cams.fx[0]), float(cams.cx[0])
+    n = 20000
+    z = np.exp(rng.uniform(np.log(0.5), np.log(z_far), n))
+    u, v = rng.uniform(0, W - 1, n), rng.uniform(0, H - 1, n)
+    means = np.stack([(u - cx) / f * z, (v - cx) / f * z, z], 1)
+    g = dict(means=means.astype(np.float32),
+             log_scales=np.log(rng.uniform(0.3, 4.0, n) * z / f)[:, None].repeat(3, 1).astype(np.float32),
+             quats=np.tile(np.array([1, 0, 0, 0], np.float32), (n, 1)),
+             logit_opacity=np.zeros(n, np.float32), sh=np.zeros((n, 1, 3), np.float32))
+    _same(*_all(g, cams, 0))
+    fr = gs.Frame(n, gs.Units.single(n), W, H, 0, with_backward=False, with_loss=False)
+    fr.preprocess(gs.pack_params(g, 0), gs.pack_cameras(cams))
+    torch.cuda.synchronize()
+    d = fr.depth.cpu().numpy()[fr.radius.cpu().numpy() > 0].view(np.uint32).astype(np.int64)
+    assert (int(d.max() - d.min()) >= 1 << 24) == (z_far > 2.0)
