@@ -631,35 +631,41 @@ __device__ __forceinline__ void walk_fwd(const uint32_t* __restrict__ vals, cons
 // Per pixel the blended entries and the stop decision are those of the
 // sequential walk; the combine changes only the rounding order of T and C.
 // gs_schedule.walk_whole_lists is M = infinity.
-// M depends on the lists alone (a split that followed the timing would change
-// the rounding of the checkpoints from run to run):
+// M depends on the lists and on how many warps the device holds, not on the
+// timing (a split that followed it would change the rounding of the checkpoints
+// from run to run).  With the blocks of lists with entries and the smaller of
+// the resident warps and the image's blocks:
 //   all lists of at most 8 chunks (by the heaviest's class): no split, the
 //     passes behind the front would cost more than its last blocks' walks;
-//   fewer blocks than resident warps: 1, a serial walk leaves warps idle;
-//   else the chunks or blocks a resident warp gets, the fewer, 4 to 16, so that
-//     a serial walk is no longer than the whole pass; the parallel passes walk
-//     chunks behind stops, so as much as that bound allows stays in front.
+//   fewer blocks than that (a small image with empty lists), or fewer than an
+//     eighth of the resident warps (any image of up to 47 tiles): 1, a serial
+//     walk leaves warps idle;
+//   else the chunks or blocks a warp gets, the fewer, 4 to 16, so that a serial
+//     walk is no longer than the whole pass; the parallel passes walk chunks
+//     behind stops, so as much as that bound allows stays in front.
 // Forward stage, two views each (us), M = 1 / 4 / 16 -> by this rule: 10M at
-// 1080p 1997, 1773 / 1822, 1755 / 1223, 1503 -> 1250, 1526; 1M at 1080p 292,
-// 329 / 195, 312 / 194, 249 -> 195, 254; 8 partitions of 2.8M at 1080p 771, 726
-// / 769, 728 / 879, 804 -> 859, 777; 4M at 1800x1300 731, 803 / 694, 754 / 551,
-// 772 -> 556, 764; 3M in 3 partitions at 400x300, two views, 1265, 1222 / 1398,
-// 1356 / 2075, 1841 -> 1248, 1241; 6M at 400x300 1260, 1206 / 1457, 1403 /
-// 1926, 1853 -> 1274, 1211; 1M there 396, 395 / 465, 494 / 542, 619 -> 390, 390.
+// 1080p 1846, 1626 / 1687, 1592 / 1144, 1351 -> 1142, 1342; 1M at 1080p 268, 309
+// / 179, 280 / 180, 218 -> 180, 220; 8 partitions of 2.8M at 1080p 726, 678 /
+// 703, 665 / 779, 704 -> 762, 696; 4M at 1800x1300 696, 768 / 668, 723 / 525,
+// 673 -> 522, 674; 3M in 3 partitions at 400x300, two views, 1119, 1089 / 1223,
+// 1197 / 1754, 1559 -> 1113, 1093; 6M at 400x300 1120, 1069 / 1299, 1240 / 1648,
+// 1643 -> 1124, 1079; 1M there 368, 369 / 429, 450 / 415, 542 -> 366, 370.
+// Images covered by lists of many chunks, M = 1 / 4 / 8: 32x32, 50,000 faint
+// splats, 116 / 178 / 266; 64x64, 1M, 226 / 353 / 497 (but 50,000 opaque ones
+// 98 / 89 / 66, so the line is not exact); 128x128, 300,000 of some pixels, 451 /
+// 375 / 270; 256x256, 50,000 of many, 368 / 126 / 126.
 // Where the capacity bounds every list to FRONT_CHUNKS chunks, the passes behind
 // the front are not launched at all (5 us each with nothing to do).
-// (Figures before the records were fetched a batch ahead.  Held to 80, 72 and 64
-// of its then 88 registers the front took 1275, 1265 and 1423 us on the first 10M
-// view.)
 constexpr int FRONT_CHUNKS = 16;
 __device__ __forceinline__ int front_chunks(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
-                                            uint32_t jobs, uint32_t lists, uint32_t warps, int K) {
+                                            uint32_t jobs, uint32_t lists, uint32_t NT, uint32_t resident, int K) {
   if (lists == 0u) return FRONT_CHUNKS;
   const uint32_t units = 8u * lists;
   const uint2 first = ranges[order[0]];  // of the heaviest lists' class: less than twice its length is the longest
   const uint32_t longest = 2u << (31 - __clz((int)max(first.y - first.x, 1u)));
   if (longest <= 8u * (uint32_t)K) return FRONT_CHUNKS;
-  if (units < warps) return 1;
+  const uint32_t warps = min(resident, 8u * NT);
+  if (units < warps || 8u * units <= resident) return 1;
   return (int)min((uint32_t)FRONT_CHUNKS, max(4u, 8u * min(jobs, units) / warps));
 }
 constexpr uint32_t STOP_BIT = 0x80000000u;  // partial or front state: the pixel has stopped
@@ -785,8 +791,8 @@ __device__ __forceinline__ float4 walk_chunk(const uint32_t* __restrict__ vals, 
 template <int BW>
 __global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict__ ranges,
                                                          const uint32_t* __restrict__ order,
-                                                         const uint32_t* __restrict__ job_base, int K, bool whole, bool later,
-                                                         int NT,
+                                                         const uint32_t* __restrict__ job_base, int K, bool whole,
+                                                         uint32_t resident, int NT,
                                                          float4* __restrict__ ckpt, uint32_t* __restrict__ chunk_last,
                                                          const uint32_t* __restrict__ vals,
                                                          const uint16_t* __restrict__ masks,
@@ -803,7 +809,7 @@ __global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict
   const int lane = threadIdx.x & 31;
   const int lists = lists_in_use(job_base, NT);
   const uint32_t total = (uint32_t)lists * 8u;
-  const int M = later ? front_chunks(ranges, order, job_base[NT], (uint32_t)lists, gridDim.x, K) : INT_MAX;
+  const int M = resident ? front_chunks(ranges, order, job_base[NT], (uint32_t)lists, (uint32_t)NT, resident, K) : INT_MAX;
   auto unit = [&](uint32_t vb) {
     const int o = (int)(vb >> 3), w = (int)(vb & 7u);
     PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
@@ -1782,10 +1788,11 @@ int gs_render_fwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const u
     const uint2* rg = (const uint2*)ranges;                                                                           \
     gs_launch(k_render_fwd_empty, grid, TILE_PIX, 0, s, rg, width, height, TX, TX * TY, bg[0], bg[1], bg[2],       \
         img, final_T, n_contrib, tk, q + qcap);                                                                    \
-    gs_launch(k_render_fwd_front<BW>, gs_resident_grid<k_render_fwd_front<BW>>(32, 0, (int64_t)grid.x * 8), 32,    \
-        0, s, rg, sched->tile_order, sched->job_base, sched->chunk, sched->walk_whole_lists != 0, later,           \
-        (int)grid.x, ck, sched->chunk_last, sorted_vals, sched->block_masks, pxy, pco, prgb, width, height, TX,    \
-        TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib, q, qcap, tk);                                       \
+    const unsigned resident = gs_resident_grid<k_render_fwd_front<BW>>(32, 0, INT_MAX);                               \
+    gs_launch(k_render_fwd_front<BW>, resident < 8 * grid.x ? resident : 8 * grid.x, 32, 0, s, rg, sched->tile_order, \
+        sched->job_base, sched->chunk, sched->walk_whole_lists != 0, later ? resident : 0u, (int)grid.x, ck,          \
+        sched->chunk_last, sorted_vals, sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], \
+        bg[2], img, final_T, n_contrib, q, qcap, tk);                                                                 \
     if (later) {                                                                                                      \
       gs_launch(k_render_fwd_chunk<BW>, gs_resident_grid<k_render_fwd_chunk<BW>>(32, 0, (int64_t)qcap), 32, 0,     \
           s, rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last,             \

@@ -325,3 +325,44 @@ def test_front_split_rules(n, W, H, log_scales):
     assert bool(((ta - tb).abs() <= eps * tb.clamp_min(1e-6))[same].all())
     assert bool(((ia - ib).abs() <= eps * colour)[:, same].all())
     assert bool(((ia - ib).abs() <= (2 * torch.maximum(ta, tb) + eps) * colour).all())
+
+
+def _chunks_in_front(fr, K):
+    """The M for which every list's 8x4-pixel blocks leave all chunks from M on to the parallel passes (no pixel stops;
+    blocks past the image's edge have nothing to do)."""
+    r = fr.ranges.cpu().numpy()
+    nch = (r[:, 1] - r[:, 0] + K - 1) // K
+    left = int(fr.stop_queue[-1])
+    cols = np.clip((fr.W - 16 * np.arange(fr.TX) + 7) // 8, 0, 2)
+    rows = np.clip((fr.H - 16 * np.arange(fr.TY) + 3) // 4, 0, 4)
+    blocks = (rows[:, None] * cols).reshape(-1)
+    fit = [m for m in range(1, 17) if int((blocks * np.maximum(nch - m, 0)).sum()) == left]
+    assert fit, (left, nch.max())
+    return nch, fit
+
+
+@pytest.mark.parametrize("n,W,H,extent,log_scales,m", [
+    (600, 64, 64, 3.0, (-3.5, -2.5), 16),      # lists of at most 8 chunks: all in front
+    (4000, 32, 32, 3.0, (-3.5, -2.5), 1),      # covered, far fewer blocks than warps
+    (12000, 64, 64, 3.0, (-3.5, -2.5), 1),
+    (100000, 256, 256, 3.0, (-4.0, -3.0), 8),  # covered, about as many blocks as warps
+    (30000, 200, 200, 0.5, (-3.8, -3.0), 1),   # fewer blocks than warps, empty lists
+    (100000, 500, 500, 3.0, (-3.5, -2.5), None),  # more blocks than warps: 4 to 16
+])
+def test_front_split_by_lists(n, W, H, extent, log_scales, m):
+    """How many chunks of 32 the front pass walks, read from the chunks it leaves to the passes behind it; splats so
+    faint that no pixel stops."""
+    import paper_2509_12138_gb300 as gs
+    K = 32
+    g = synth.random_gaussians(n, 0, 4, extent=extent, log_scale_range=log_scales)
+    g["logit_opacity"][:] = -5.0
+    cams = gs.pack_cameras(synth.orbital_cameras(8, 3.0, width=W, height=H).subset([0]))
+    params = gs.pack_params(g, 0)
+    fr = Frame(n, Units.single(n, 1), W, H, 0, with_backward=False, with_loss=False, chunk=K)
+    fr.fit_capacity(params, cams)
+    fr.forward(params, cams, (0.2, 0.4, 0.6))
+    assert fr.read_status() == 0 and float(fr.final_T.min()) > 1e-3
+    nch, fit = _chunks_in_front(fr, K)
+    assert (nch.min() > 0) == (extent > 1.0)
+    assert (nch.max() > 8) == (m != 16)
+    assert m in fit if m else all(4 <= x <= 16 for x in fit)
