@@ -1462,8 +1462,8 @@ __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict
   }
 }
 
-struct BwdScratch {
-  float w[32 * MROW];   // o G of an accepted (hit, pixel) pair, then its colour weight alpha T
+struct __align__(16) BwdScratch {
+  float w[32 * MROW];   // o G of an accepted (hit, pixel) pair, then its colour weight alpha T (few hits: their Rec)
   float dp[32 * MROW];  // dL/dpower of the pair (0 when alpha was clamped)
   float r[32], g[32], b[32];     // the batch's colours
   float g0[32], g1[32], g2[32];  // dL/dimg of the block's pixels
@@ -1478,6 +1478,14 @@ struct BwdScratch {
 // memory, and a third, record-major phase forms the pairs' gradients and sums
 // them in its lane's registers, in pixel order, so that nothing depends on
 // scheduling.  700k at 1011x757: 578 us with a warp reduction per hit, 240 us.
+// A record-major phase lasts as long as the widest hit has pixels (32 where it
+// covers the block), however few hits there are, so batches of up to FEW_HITS
+// take the warp reduction per hit.  Lists of 3 entries of some pixels each, at
+// 1080p: 74 us record-major, 42 this way (39 with a reduction for every hit); of
+// 6 entries 79, 50 (45); up to 4, 6, 8 and 12 hits the worst of 150 scenes took
+// 1.36, 1.19, 1.12 and 1.06 times what reductions throughout take, but with 12
+// some scenes more than record-major phases throughout (1.14; 1.05 with 8).
+constexpr int FEW_HITS = 8;
 template <int BW>
 __global__ void __launch_bounds__(32, 20) k_render_bwd_det(const uint2* __restrict__ ranges,
                                                            const uint32_t* __restrict__ order,
@@ -1557,6 +1565,61 @@ __global__ void __launch_bounds__(32, 20) k_render_bwd_det(const uint2* __restri
       }
       const int nb = min(32, qn - qh);
       if (nb == 0) break;
+      if (nb <= FEW_HITS) {
+        // each lane its own pixel's share of every hit, summed over the warp per hit
+        Rec* rec = reinterpret_cast<Rec*>(sc.w);
+        if (lane < nb) {
+          const uint32_t id = lv[sc.q[qh + lane]];
+          const float4 m = xy[id], k = conic_op[id];
+          rec[lane].a = make_float4(rel_pos(m.x, m.z, tox), rel_pos(m.y, m.w, toy), k.x, k.y);
+          rec[lane].b = make_float4(k.z, k.w, 0.f, __uint_as_float(id));
+          rec[lane].c = rgb[id];
+        }
+        __syncwarp();
+        for (int j = 0; j < nb; ++j) {
+          const float4 ra = rec[j].a, rb = rec[j].b;
+          const float dx = ra.x - (ox + (float)(lane & (BW - 1))), dy = ra.y - (oy + (float)(lane / BW));
+          const float power = splat_power(ra.z, ra.w, rb.x, dx, dy);
+          const float G = __expf(power), araw = rb.y * G;
+          const bool clamped = araw > ALPHA_MAX;  // a clamped alpha passes no gradient to opacity, conic or position
+          const float alpha = clamped ? ALPHA_MAX : araw;
+          const bool pair = !(power > 0.f) && !(alpha < ALPHA_MIN) && (int)sc.q[qh + j] < last;
+          const unsigned cm = __ballot_sync(FULL, pair);
+          if (!cm) continue;
+          float v[9];
+          #pragma unroll
+          for (int e = 0; e < 9; ++e) v[e] = 0.f;
+          if (pair) {
+            const float4 rc = rec[j].c;
+            const float om = 1.f - alpha;
+            T = __fdividef(T, om);  // transmittance in front of this entry
+            const float wgt = alpha * T;
+            v[6] = wgt * g0; v[7] = wgt * g1; v[8] = wgt * g2;
+            float dalpha = T * ((rc.x - S0) * g0 + (rc.y - S1) * g1 + (rc.z - S2) * g2);
+            if (qT != 0.f) dalpha -= __fdividef(qT, om);
+            S0 = alpha * rc.x + om * S0; S1 = alpha * rc.y + om * S1; S2 = alpha * rc.z + om * S2;
+            if (!clamped) {
+              v[5] = G * dalpha;
+              pos_conic_terms(dx, dy, araw * dalpha, ra.z, ra.w, rb.x, v);
+            }
+          }
+          const int64_t id = (int64_t)__float_as_uint(rb.w);
+          if ((cm & (cm - 1)) == 0) {
+            if (pair) add_lane(nullptr, nullptr, nullptr, fixed, id, v);
+          } else {
+            const float tot = reduce8(v, lane);
+            float e8 = v[8];
+            #pragma unroll
+            for (int d = 16; d > 0; d >>= 1) e8 += __shfl_xor_sync(FULL, e8, d);
+            const int slot = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+            if ((lane & 3) == 0) add_one(nullptr, nullptr, nullptr, fixed, id, slot, tot);
+            else if (lane == 1) add_one(nullptr, nullptr, nullptr, fixed, id, 8, e8);
+          }
+        }
+        qh += nb;
+        __syncwarp();
+        continue;
+      }
       // record-major: o G of hit `lane` at the pixels its box reaches
       uint32_t pr = 0u, valid = 0u;
       float rx = 0.f, ry = 0.f;

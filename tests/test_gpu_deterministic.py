@@ -115,3 +115,29 @@ def test_graph_captured_batched_training_is_bitwise_reproducible():
         assert tr.check() == 0
         runs.append((p.clone(), tr.opt.m.clone()))
     assert torch.equal(runs[0][0], runs[1][0]) and torch.equal(runs[0][1], runs[1][1])
+
+
+@pytest.mark.parametrize("n", [1, 2, 8, 9, 33, 70])
+@pytest.mark.parametrize("variant", [0, 1, 2])
+def test_deterministic_gradients_of_few_hits(n, variant):
+    """Lists of a few entries and just over: both ways of summing a hit over a block's pixels agree with the float
+    path (bounds as above), for every block shape, ragged image edges and a pixel that stops inside a batch."""
+    W, H = 43, 38
+    g, cams = scenes.random_scene(n, 1, 90 + n, W, H, log_scale_range=(-2.5, -1.0))
+    g["logit_opacity"][:] = np.where(np.arange(n) % 3 == 0, 6.0, 0.0)
+    params, camd = gs.pack_params(g, 1), gs.pack_cameras(cams)
+    gt, mask = scenes.random_gt(W, H, 9)
+    out = []
+    for deterministic in (True, True, False):
+        fr = gs.Frame(n, gs.Units.single(n), W, H, 1, deterministic=deterministic, variant=variant, chunk=32)
+        fr.fit_capacity(params, camd)
+        fr.forward(params, camd, BG)
+        fr.loss(torch.from_numpy(gt).cuda()[None], torch.from_numpy(mask).cuda()[None], 0.2)
+        fr.backward(params, camd, BG)
+        torch.cuda.synchronize()
+        assert fr.read_status() == 0
+        out.append([fr.dxy.clone(), fr.dco.clone(), fr.drgb.clone()])
+    assert all(torch.equal(a, b) for a, b in zip(out[0], out[1]))
+    assert all(float(f.abs().max()) > 0 for f in out[2])
+    for d, f in zip(out[0], out[2]):
+        assert torch.allclose(d, f, rtol=1e-4, atol=1e-5 * float(f.abs().max()))
