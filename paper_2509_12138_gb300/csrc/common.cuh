@@ -204,12 +204,12 @@ struct GsRange {
 };
 #define GS_RANGE(name) GsRange gs_range_guard_(name)
 
-// Blocks of `threads` threads and `smem` dynamic bytes of a kernel that stay resident on the current device,
-// at most `units`: the grid of a kernel whose blocks take units of work in turn (a grid sized for the capacity
-// would mostly hold blocks that find nothing to do).  The occupancy query costs a microsecond or two of host time
-// and its answer is a property of the kernel and the device, so it is asked once per device.
-template <auto Kernel>
-unsigned gs_resident_grid(int threads, size_t smem, int64_t units) {
+// Blocks of Threads threads and Smem dynamic bytes of a kernel that stay resident on the current device, at most
+// `units`: the grid of a kernel whose blocks take units of work in turn (a grid sized for the capacity would mostly
+// hold blocks that find nothing to do).  The occupancy query costs a microsecond or two of host time and its answer is
+// a property of the kernel, its launch shape and the device, so it is asked once per launch shape and device.
+template <auto Kernel, int Threads, size_t Smem = 0>
+unsigned gs_resident_grid(int64_t units) {
   constexpr int DEVICES = 64;
   static std::atomic<int> known[DEVICES];  // 0: not asked yet
   if (units < 1) return 1u;
@@ -219,7 +219,7 @@ unsigned gs_resident_grid(int threads, size_t smem, int64_t units) {
   if (g == 0) {
     int sms = 0, per = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, Kernel, threads, smem) != cudaSuccess || sms < 1 || per < 1)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, Kernel, Threads, Smem) != cudaSuccess || sms < 1 || per < 1)
       return (unsigned)units;
     g = sms * per;
     if (dev < DEVICES) known[dev].store(g, std::memory_order_relaxed);

@@ -1851,20 +1851,20 @@ int gs_render_fwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const u
     const uint2* rg = (const uint2*)ranges;                                                                           \
     gs_launch(k_render_fwd_empty, grid, TILE_PIX, 0, s, rg, width, height, TX, TX * TY, bg[0], bg[1], bg[2],       \
         img, final_T, n_contrib, tk, q + qcap);                                                                    \
-    const unsigned resident = gs_resident_grid<k_render_fwd_front<BW>>(32, 0, INT_MAX);                               \
+    const unsigned resident = gs_resident_grid<k_render_fwd_front<BW>, 32>(INT_MAX);                               \
     gs_launch(k_render_fwd_front<BW>, resident < 8 * grid.x ? resident : 8 * grid.x, 32, 0, s, rg, sched->tile_order, \
         sched->job_base, sched->chunk, sched->walk_whole_lists != 0, later ? resident : 0u, (int)grid.x, ck,          \
         sched->chunk_last, sorted_vals, sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], \
         bg[2], img, final_T, n_contrib, q, qcap, tk);                                                                 \
     if (later) {                                                                                                      \
-      gs_launch(k_render_fwd_chunk<BW>, gs_resident_grid<k_render_fwd_chunk<BW>>(32, 0, (int64_t)qcap), 32, 0,     \
+      gs_launch(k_render_fwd_chunk<BW>, gs_resident_grid<k_render_fwd_chunk<BW>, 32>((int64_t)qcap), 32, 0,        \
           s, rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last,             \
           sorted_vals, sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, n_contrib, q, qcap,         \
           tk + 1);                                                                                                 \
-      gs_launch(k_render_fwd_combine<BW>, gs_resident_grid<k_render_fwd_combine<BW>>(32, 0, (int64_t)qcap), 32,    \
+      gs_launch(k_render_fwd_combine<BW>, gs_resident_grid<k_render_fwd_combine<BW>, 32>((int64_t)qcap), 32,       \
           0, s, sched->tile_order, sched->job_base, sched->jobs, ck, sched->chunk_last, width, height, TX,         \
           TX * TY, bg[0], bg[1], bg[2], img, final_T, n_contrib, q, qcap, tk);                                     \
-      gs_launch(k_render_fwd_stop<BW>, gs_resident_grid<k_render_fwd_stop<BW>>(32, 0, (int64_t)qcap), 32, 0, s,    \
+      gs_launch(k_render_fwd_stop<BW>, gs_resident_grid<k_render_fwd_stop<BW>, 32>((int64_t)qcap), 32, 0, s,       \
           rg, sched->tile_order, sched->job_base, sched->jobs, sched->chunk, ck, sched->chunk_last,                \
           sorted_vals, sched->block_masks, pxy, pco, prgb, width, height, TX, TX * TY, bg[0], bg[1], bg[2],        \
           img, final_T, n_contrib, q, qcap, tk);                                                                   \
@@ -1910,14 +1910,14 @@ int gs_blend_bwd_impl(const gs_proj* proj, const uint32_t* sorted_vals, const ui
     {                                                                                                              \
       if (cudaMemsetAsync(sched_ticket(sched), 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;        \
       if (fixed) {                                                                                                   \
-        gs_launch(k_render_bwd_det<BW>, gs_resident_grid<k_render_bwd_det<BW>>(32, 0, sched->max_jobs * 8), 32,    \
+        gs_launch(k_render_bwd_det<BW>, gs_resident_grid<k_render_bwd_det<BW>, 32>(sched->max_jobs * 8), 32,       \
             0, s, (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,             \
             (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,           \
             (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY,                   \
             TX * TY * n_units, bg[0], bg[1], bg[2], img, final_T, n_contrib, dL_dimg, dL_dT, fixed,                \
             sched_ticket(sched));                                                                                  \
       } else {                                                                                                       \
-        gs_launch(k_render_bwd_m<BW>, gs_resident_grid<k_render_bwd_m<BW>>(32, 0, sched->max_jobs * 8), 32, 0,     \
+        gs_launch(k_render_bwd_m<BW>, gs_resident_grid<k_render_bwd_m<BW>, 32>(sched->max_jobs * 8), 32, 0,        \
             s, (const uint2*)ranges, sched->tile_order, sched->job_base, sched->jobs, sched->chunk,                \
             (const float4*)sched->checkpoints, sorted_vals, sched->block_masks, (const float4*)proj->xy,           \
             (const float4*)proj->conic_op, (const float4*)proj->rgb, width, height, TX, TX * TY,                   \

@@ -1161,9 +1161,9 @@ static int depth_first_sort(const UnitTable& U, int64_t P, const gs_proj* proj, 
       cudaFuncSetAttribute(k_radix_scatter<8, uint32_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)DYN32) != cudaSuccess)
     return GS_ERR_CUDA;
-  unsigned gh = gs_resident_grid<k_radix_hist<8, uint32_t>>(RS_T, 0, stride);
-  unsigned gsc = gs_resident_grid<k_radix_scatter<8, uint32_t>>(RS_T, DYN32, stride);
-  unsigned gscf = gs_resident_grid<k_radix_scatter<8, uint32_t, true>>(RS_T, DYN32, stride);
+  unsigned gh = gs_resident_grid<k_radix_hist<8, uint32_t>, RS_T>(stride);
+  unsigned gsc = gs_resident_grid<k_radix_scatter<8, uint32_t>, RS_T, DYN32>(stride);
+  unsigned gscf = gs_resident_grid<k_radix_scatter<8, uint32_t, true>, RS_T, DYN32>(stride);
   uint32_t* d_min = d_vis + 1;
   uint32_t* bmins = bmin_ws;  // nsb entries
   const int vec = (((uintptr_t)proj->tiles | (uintptr_t)proj->depth) & 15u) == 0;
@@ -1219,7 +1219,7 @@ static int depth_first_sort(const UnitTable& U, int64_t P, const gs_proj* proj, 
       gs_launch(k_radix_scatter<8, uint32_t>, gsc, RS_T, DYN32, s, ikA, ikB, ivA, ivB, cur_t, pass, d_num_instances,
           8 * pass, hist, stride, nullptr, nullptr);
   }
-  gs_launch(k_ranges32, gs_resident_grid<k_ranges32>(256, 0, (cap + 1023) / 1024), 256, 0, s, ikA, ikB, ivA, ivB,
+  gs_launch(k_ranges32, gs_resident_grid<k_ranges32, 256>((cap + 1023) / 1024), 256, 0, s, ikA, ikB, ivA, ivB,
       cur_t, tpasses, d_num_instances, tile_bits, n_tiles, ranges, sorted_vals, block_masks);
   return gs_check_launch();
 }
@@ -1319,10 +1319,10 @@ int gs_bin_sort_impl(const gs_proj* proj, const gs_units* units, int width, int 
         cudaFuncSetAttribute(k_radix_scatter<9, uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCATTER_DYN_SMEM) !=
             cudaSuccess)
       return GS_ERR_CUDA;
-    unsigned gh = digit == 9 ? gs_resident_grid<k_radix_hist<9, uint64_t>>(RS_T, 0, stride)
-                             : gs_resident_grid<k_radix_hist<8, uint64_t>>(RS_T, 0, stride);
-    unsigned gs = digit == 9 ? gs_resident_grid<k_radix_scatter<9, uint64_t>>(RS_T, SCATTER_DYN_SMEM, stride)
-                             : gs_resident_grid<k_radix_scatter<8, uint64_t>>(RS_T, SCATTER_DYN_SMEM, stride);
+    unsigned gh = digit == 9 ? gs_resident_grid<k_radix_hist<9, uint64_t>, RS_T>(stride)
+                             : gs_resident_grid<k_radix_hist<8, uint64_t>, RS_T>(stride);
+    unsigned gs = digit == 9 ? gs_resident_grid<k_radix_scatter<9, uint64_t>, RS_T, SCATTER_DYN_SMEM>(stride)
+                             : gs_resident_grid<k_radix_scatter<8, uint64_t>, RS_T, SCATTER_DYN_SMEM>(stride);
     for (int pass = 0; pass < passes; ++pass) {
       int shift = digit * pass;
       if (digit == 9) {
@@ -1339,7 +1339,7 @@ int gs_bin_sort_impl(const gs_proj* proj, const gs_units* units, int width, int 
             d_num_instances, shift, hist, stride, nullptr, nullptr);
       }
     }
-    gs_launch(k_ranges, gs_resident_grid<k_ranges>(256, 0, (max_instances + 255) / 256), 256, 0, s, k0, k1, v0, v1,
+    gs_launch(k_ranges, gs_resident_grid<k_ranges, 256>((max_instances + 255) / 256), 256, 0, s, k0, k1, v0, v1,
         cur, passes, d_num_instances, tile_bits, n_tiles, TX, ranges, sorted_vals, (const float4*)proj->xy,
         (const float4*)proj->conic_op, block_masks, key_masks);
   }
