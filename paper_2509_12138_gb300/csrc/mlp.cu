@@ -430,6 +430,8 @@ __global__ void __launch_bounds__(CONS_T + PROD_T, 1)
   const int steps = b0 < nb ? (int)((nb - b0 + gridDim.x - 1) / gridDim.x) : 0;
   auto base_of = [&](int k) { return (b0 + (int64_t)k * gridDim.x) * BATCH; };
   auto tile = [&](int k) { return (uint16_t*)(sm + ((k & 1) ? Smem::X2 : Smem::X)); };
+  // the barrier of both roles, which meet in it from different places of the code
+  auto both_roles = []() { bar_sync(0, CONS_T + PROD_T); };
   stage_weights(w, sm, true);
   __syncthreads();
   if (threadIdx.x >= CONS_T) {
@@ -442,9 +444,9 @@ __global__ void __launch_bounds__(CONS_T + PROD_T, 1)
       if (k + 1 < steps) load_row(row, knn_idx, knn_dist, n, base_of(k + 1) + tid, vec);
       bar_sync(2, PROD_T);
       build_features<PROD_T>(tid, pts, nrm, n, base_of(k), s_idx, s_dbar, tile(k));
-      __syncthreads();
+      both_roles();
     }
-    __syncthreads();  // the last batch is multiplied
+    both_roles();  // the last batch is multiplied
     return;
   }
   // ---- multipliers
@@ -474,7 +476,7 @@ __global__ void __launch_bounds__(CONS_T + PROD_T, 1)
   const uint32_t ONES[4] = {0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u};
   float lsum = 0.f;
   for (int k = 0; k < steps; ++k) {
-    __syncthreads();  // batch k's features are in its tile; every warp is done with batch k - 1
+    both_roles();  // batch k's features are in its tile; every warp is done with batch k - 1
     const uint16_t* X = tile(k);
     const int64_t r0 = base_of(k) + m0 + g, r1 = r0 + 8;
     float tg[4] = {0.f, 0.f, 0.f, 0.f};
@@ -624,7 +626,7 @@ __global__ void __launch_bounds__(CONS_T + PROD_T, 1)
       gb3[0] += s3[0]; gb3[1] += s3[1];
     }
   }
-  __syncthreads();  // (the builders' last barrier)
+  both_roles();  // (the builders' last barrier)
   // accumulator element e of a tile: row g (+ 8 for e >= 2), column 2 t + (e & 1)
   auto put = [&](int off, int ncols, int row, int col, const float* v) {
     #pragma unroll
