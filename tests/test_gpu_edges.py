@@ -292,6 +292,64 @@ def test_sort_of_many_records_equals_global(wide):
         assert all(torch.equal(a, b) for a, b in zip(other, got[2]))
 
 
+def _many_records(n, views, W, H, seed=5):
+    """n splats of about a pixel (every 200,003rd one of many tiles) as parameters on the device, and their cameras."""
+    import paper_2509_12138_gb300 as gs
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    params = torch.zeros((gs.param_planes(0), n, 4), device="cuda")
+    params[0, :, :3] = 1.8 * torch.rand((n, 3), generator=g, device="cuda") - 0.9
+    params[1, :, :3] = -6.5 + 0.5 * torch.randn((n, 3), generator=g, device="cuda")
+    params[1, ::200_003, :3] = -1.0
+    params[2] = torch.randn((n, 4), generator=g, device="cuda")
+    return params, gs.pack_cameras(synth.orbital_cameras(8, 3.0, width=W, height=H).subset(list(range(views))))
+
+
+@pytest.mark.parametrize("views,masks", [(1, True), (2, True), (1, False)])
+def test_sort_by_packed_rectangles_equals_global(views, masks):
+    """2^25 records on: with room for two instances a record the emission reads packed rectangles, with one less it
+    reads the records; one view and several, with block masks and without: the global sort's lists, bit for bit."""
+    n = (1 << 25) // views + 77
+    params, cams = _many_records(n, views, 333, 250)
+    got = []
+    for cap, design in ((2 * views * n, "depth_first"), (2 * views * n - 1, "depth_first"), (2 * views * n, "global")):
+        fr = Frame(n, Units.single(n, views), 333, 250, 0, max_instances=cap, with_backward=False, with_loss=False)
+        fr.use_masks = masks
+        fr.preprocess(params, cams)
+        fr.sort(design)
+        count = fr.instances()
+        assert fr.read_status() == 0 and n * views // 2 < count <= cap
+        got.append([fr.sorted_vals[:count].clone(), fr.ranges.clone()] + ([fr.block_masks[:count].clone()] if masks else []))
+        del fr
+    for other in got[:2]:
+        assert all(torch.equal(a, b) for a, b in zip(other, got[2]))
+
+
+def test_sort_by_packed_rectangles_keeps_the_nearest():
+    """More instances than the capacity behind packed rectangles: every list keeps its first entries, the capacity is
+    full, and nothing dropped is nearer than anything kept."""
+    n = (1 << 25) + 77
+    params, cams = _many_records(n, 1, 1200, 900)
+    params[1, :, :3] += 0.9  # some three instances a record
+    out = []
+    for cap in (4 * n, 2 * n):
+        fr = Frame(n, Units.single(n, 1), 1200, 900, 0, max_instances=cap, with_backward=False, with_loss=False)
+        fr.preprocess(params, cams)
+        fr.sort()
+        out.append((fr.read_status(), fr.instances(), fr.sorted_vals.clone(), fr.ranges.long().clone(), fr.depth.clone()))
+        del fr
+    (sa, na, va, ra, depth), (sb, nb, vb, rb, _) = out
+    assert sa == 0 and sb == 2 and nb == 2 * n < na <= 4 * n
+    la, lb = ra[:, 1] - ra[:, 0], rb[:, 1] - rb[:, 0]
+    assert bool((lb <= la).all()) and int(lb.sum()) == nb
+    list_of = torch.repeat_interleave(torch.arange(len(lb), device="cuda"), lb)
+    within = torch.arange(nb, device="cuda") - rb[list_of, 0]
+    assert torch.equal(vb[:nb], va[ra[list_of, 0] + within])
+    cut = torch.ones(na, dtype=torch.bool, device="cuda")
+    cut[ra[list_of, 0] + within] = False
+    assert float(depth[vb[:nb].long()].max()) <= float(depth[va[:na][cut].long()].min())
+
+
 @pytest.mark.parametrize("n,W,H,log_scales", [
     (3000, 100, 60, (-4.0, -2.5)),    # few short lists: no split
     (30000, 100, 60, (-3.5, -2.5)),   # fewer blocks than warps, long lists: everything behind the first chunk
