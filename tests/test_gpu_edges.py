@@ -151,6 +151,14 @@ def test_knn_distances_past_the_float_range(k):
         assert dist[i].tolist() == [float(np.sqrt(d)) for d, _ in near] + [np.inf] * (k - len(near))
 
 
+@pytest.mark.parametrize("n,k", [(5, 8), (17, 16), (600, 16), (600, 8)])
+def test_knn_unaligned_results(n, k):
+    """Rows of results that do not start on 16 bytes are stored one value at a time: the same indices and distances."""
+    pts = np.random.default_rng(n + k).uniform(0, 1, (n, 3)).astype(np.float32)
+    want, got = (_knn_on_grid(pts, k, (-0.1, -0.1, -0.1), 0.25, (5, 5, 5), aligned) for aligned in (True, False))
+    assert np.array_equal(want[0], got[0]) and np.array_equal(want[1], got[1])
+
+
 @pytest.mark.parametrize("W,H,units", [(1, 1, 1), (31, 33, 2), (32, 32, 1), (65, 10, 3), (100, 71, 2)])
 def test_loss_partial_tiles(W, H, units):
     """Image edges inside the loss kernels' tiles, planes that are no multiple of 16 bytes, several units; bounds
@@ -265,6 +273,26 @@ def test_sort_design_by_sizes(n, views, W, H, cap, small):
     fr.preprocess(gs.pack_params(g, 0), gs.pack_cameras(cams))
     kernels = captured_kernels(fr.sort)
     assert kernels == 4 if small else kernels >= 18
+
+
+@pytest.mark.parametrize("array", ["tiles", "depth"])
+def test_sort_unaligned_records(array):
+    """Records whose tile counts or depths do not start on 16 bytes are counted one at a time: the same lists."""
+    import paper_2509_12138_gb300 as gs
+    n = 3 * 2048 + 5
+    g = synth.random_gaussians(n, 0, 6, extent=0.8, log_scale_range=(-5.0, -3.0))
+    cams = gs.pack_cameras(synth.orbital_cameras(8, 3.0, width=1040, height=1040).subset([0]))
+    fr = Frame(n, Units.single(n, 1), 1040, 1040, 0, with_backward=False, with_loss=False)
+    fr.fit_capacity(gs.pack_params(g, 0), cams)
+    fr.sort()
+    want = fr.sorted_lists()
+    moved = _off_by_one(getattr(fr, array))
+    setattr(fr.proj, array, moved.data_ptr())
+    fr.sorted_vals.zero_()
+    fr.sort()
+    got = fr.sorted_lists()
+    assert fr.read_status() == 0 and len(want[0]) > n
+    assert np.array_equal(want[0], got[0]) and np.array_equal(want[1], got[1])
 
 
 @pytest.mark.parametrize("wide", [False, True])
