@@ -243,8 +243,9 @@ def cpu_baseline(scene, frac: int):
 
 # ---------------------------------------------------------------- our arm
 def kernel_launch_count(frame, lam, fused_pre=False):
-    """Kernels libgs launches for one training step (a1-a6) of this frame (the kernel launches ncu lists
-    for the timed steps; the 4-byte memsets of the ticket counters are not kernels)."""
+    """Kernels of one training step (a1-a6) with the general sort, a blend schedule of seven launches and a forward of
+    three; step_launch_count has what the frame's sizes make of these (the 4-byte memsets of the ticket counters are
+    not kernels)."""
     tile_bits = (frame.n_tiles - 1).bit_length()
     unit_bits = (frame.units.n - 1).bit_length()
     key_bits = 32 + tile_bits + unit_bits
@@ -266,14 +267,27 @@ def kernel_launch_count(frame, lam, fused_pre=False):
     return pre + sort + fwd + loss + bwd + adam
 
 
+def small_sort_applies(frame):
+    """Whether gs_bin_sort takes the four launches for few lists and few records per unit (sort_small.cu)."""
+    records = int(frame.units.proj_base[-1])
+    if getattr(frame, "sort_design", "depth_first") != "depth_first" or records < 1 or frame.cap < 1:
+        return False
+    most = min(16384, 2048 + 640 * frame.cap / records)
+    return frame.n_tiles * frame.units.n <= 4096 and int(np.diff(frame.units.proj_base).max()) <= most
+
+
 def step_launch_count(frame, lam, fused_pre=False):
-    """kernel_launch_count, with the launches that depend on the frame's sizes: up to 8192 lists the schedule is one
-    launch instead of seven, and the scheduled forward is the empty lists and the front, and the chunk, combine and
-    stop passes where the capacity allows a list of more than 16 chunks."""
+    """Kernels libgs launches for one training step (a1-a6) of this frame: kernel_launch_count with the sort and the
+    schedule of small problems in four launches; up to 8192 lists the schedule in one; and the scheduled forward as the
+    empty lists and the front, with the chunk, combine and stop passes where the capacity allows a list of more than 16
+    chunks."""
     n = kernel_launch_count(frame, lam, fused_pre)
+    if small_sort_applies(frame):
+        rest = (0 if fused_pre else 1) + (3 if frame.use_masks else 1) + (4 if lam > 0 else 3) + 1 + 2
+        n = rest + 4
+    elif frame.use_masks and frame.n_tiles * frame.units.n <= 8192:
+        n -= 6
     if frame.use_masks:
-        if frame.n_tiles * frame.units.n <= 8192:
-            n -= 6
         n += (2 + (3 if frame.cap // frame.chunk + 1 > 16 and not frame.walk_whole_lists else 0)) - 3
     return n
 

@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+import bench
 import oracle
 import synth
 from paper_2509_12138_gb300 import Frame, Units
@@ -452,3 +453,32 @@ def test_front_split_by_lists(n, W, H, extent, log_scales, m):
     assert (nch.min() > 0) == (extent > 1.0)
     assert (nch.max() > 8) == (m != 16)
     assert m in fit if m else all(4 <= x <= 16 for x in fit)
+
+
+@pytest.mark.parametrize("n,views,W,H,cap,lam,masks,whole", [
+    (500, 1, 64, 64, None, 0.2, True, False), (300, 2, 64, 48, 1 << 15, 0.0, False, False),
+    (20000, 1, 333, 250, None, 0.2, True, False), (20000, 1, 333, 250, None, 0.2, True, True),
+    (4000, 1, 160, 160, 8000, 0.0, True, False), (300, 2, 1920, 1080, 1 << 15, 0.2, True, False),
+    (300, 9, 1920, 1080, 1 << 15, 0.2, False, False)])
+def test_launch_count_of_a_step(n, views, W, H, cap, lam, masks, whole):
+    """The launches the benchmark reports for a step are those of a captured one, whatever its sizes make of it."""
+    import paper_2509_12138_gb300 as gs
+    g = synth.random_gaussians(n, 1, 8, extent=0.8, log_scale_range=(-4.0, -3.0))
+    cams = gs.pack_cameras(synth.orbital_cameras(9, 3.0, width=W, height=H).subset(list(range(views))))
+    params = gs.pack_params(g, 1)
+    fr = Frame(n, Units.single(n, views), W, H, 1, max_instances=cap)
+    if cap is None:
+        fr.fit_capacity(params, cams)
+    fr.use_masks, fr.walk_whole_lists = masks, whole
+    gt, mask = torch.rand_like(fr.img), torch.ones((views, H, W), dtype=torch.uint8, device="cuda")
+    opt = gs.Adam(params, 1)
+
+    def step():
+        fr.preprocess(params, cams)
+        fr.sort()
+        fr.render((1.0, 1.0, 1.0))
+        fr.loss(gt, mask, lam)
+        fr.blend_backward((1.0, 1.0, 1.0))
+        opt.fused_step(fr, cams)
+
+    assert captured_kernels(step) == bench.step_launch_count(fr, lam)
