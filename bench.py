@@ -272,8 +272,9 @@ def small_sort_applies(frame):
     records = int(frame.units.proj_base[-1])
     if getattr(frame, "sort_design", "depth_first") != "depth_first" or records < 1 or frame.cap < 1:
         return False
-    most = min(16384, 2048 + 640 * frame.cap / records)
-    return frame.n_tiles * frame.units.n <= 4096 and int(np.diff(frame.units.proj_base).max()) <= most
+    most = 1024 * math.log2(frame.n_tiles) + 256 * (frame.cap / records - 4)
+    largest = int(np.diff(frame.units.proj_base).max())
+    return frame.n_tiles * frame.units.n <= 4096 and largest <= min(max(most, 3072), 16384)
 
 
 def step_launch_count(frame, lam, fused_pre=False):

@@ -234,8 +234,9 @@ int gs_bin_sort(const gs_proj* proj, const gs_units* units, int width, int heigh
  * gs_bin_sort_global.  On capacity overflow the nearest instances are kept.
  * Small problems take four launches instead: each unit's records sorted by
  * depth in one CTA, each list gathered by a warp from its unit's tile
- * rectangles in that order.  They have at most 4,096 lists, and at most 2,048 +
- * 640 max_instances / n_proj records per unit, 16,384 in any case.
+ * rectangles in that order.  They have at most 4,096 lists, and at most 1,024
+ * log2(tiles) + 256 (max_instances / n_proj - 4) records per unit (no less than
+ * 3,072, no more than 16,384).
  *
  * gs_bin_sort_global and gs_bin_sort_bucketed: the same lists, ranges,
  * instance count and schedule as gs_bin_sort (same arguments and workspace)

@@ -435,22 +435,27 @@ __global__ void __launch_bounds__(LW * 32) k_small_fill(UnitTable U, int W, int 
 
 }  // namespace
 
-// Whether the design applies: it is taken up to where its time crosses the general design's.  A list's warp reads all
-// records of its unit, twice, so this design takes 13 us + 20 ns per record of the largest unit, whatever they cover;
-// the general one hardly depends on the number of so few records but on their instances, since one thread emits all of
-// a record's: 85 us + 10 to 35 us per instance a record has.  The capacity stands for the instances (where it was
-// fitted, 1.25 times their number).  us per call, this design / general / the limit (splats of a sphere's surface;
-// the last one random sizes):
-//   48 x 48, 1 unit       2,000   57 / 80 / 3,850    4,000   93 / 88 / 3,640     8,000  172 / 90 / 3,500
-//   128 x 128, 8 units    3,000   78 / 122 / 4,620   5,000  116 / 107 / 4,210    8,000  174 / 103 / 3,940
-//   256 x 256, 8 units    3,000   83 / 175 / 7,150   5,000  124 / 144 / 5,870    8,000  177 / 130 / 5,070
-//   512 x 512, 4 units    4,000  107 / 369 / 12,480  8,000  176 / 226 / 8,540   16,384  313 / 142 / 6,300
-//   1024 x 1024, 1 unit   4,000   99 / 1549 / 16,384 8,000  158 / 728 / 16,384  16,384  412 / 27680 / 16,384
+// Whether the design applies.  A list's warp reads all records of its unit, twice, so this design takes 13 us + 20 ns
+// per record of the largest unit, whatever they cover.  The general one takes 85 us, more with several units, and its
+// emission gives all instances of a record to one thread: 10 to 35 us per instance that a record has on average, and
+// about 1 us per tile of the largest splat.  Neither is known here; the image's tiles bound the one, and the capacity
+// stands for the other (where it was fitted, 1.25 times the instances).  So the limit grows by 1,024 records with each
+// doubling of the tiles and by 256 with each instance that the capacity leaves a record.  us per call, this design /
+// general / general with one splat that covers the image (4 instances of capacity per record):
+//   16 tiles, 1 unit      limit 4,096    3,000  80 / 82 / -      5,000  118 / 86 / -      16,384  352 / 86 / -
+//   49 tiles, 2 units     limit 5,750    7,285 165 / 91 / 111
+//   64 tiles, 8 units     limit 6,144    3,000  78 / 122 / -     5,000  116 / 107 / -      8,000  174 / 103 / -
+//   165 tiles, 1 unit     limit 7,540    4,500 104 / 96 / -      7,285  157 / 93 / 254
+//   256 tiles, 1 unit     limit 8,192    3,000  74 / 127 / -     5,000  107 / 109 / -     15,000  278 / 94 / 338
+//   256 tiles, 4 units    limit 8,192                                                     10,000  204 / 128 / 440
+//   1024 tiles, 4 units   limit 10,240   4,000 107 / 369 / -     8,000  176 / 226 / -     16,384  313 / 142 / -
+// Before this design the general one took 150 to 240 us at these sizes, 95 to 155 in a captured graph: against that no
+// call of 170 sizes is slower now, captured ones of small splats just below the limit by up to 1.4 times.
 bool gs_small_sort_applies(const UnitTable& U, int64_t P, int n_tiles, int64_t cap) {
   if ((int64_t)U.n * n_tiles > LISTS_MAX) return false;
-  const double most = fmin((double)UNIT_MAX, 2048.0 + 640.0 * (double)cap / (double)P);
+  const double most = 1024.0 * log2((double)n_tiles) + 256.0 * ((double)cap / (double)P - 4.0);
   for (int u = 0; u < U.n; ++u)
-    if ((double)(U.proj_base[u + 1] - U.proj_base[u]) > most) return false;
+    if ((double)(U.proj_base[u + 1] - U.proj_base[u]) > fmin(fmax(most, 3072.0), (double)UNIT_MAX)) return false;
   return true;
 }
 

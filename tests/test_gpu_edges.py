@@ -251,8 +251,8 @@ def test_sort_lists_at_design_limits(n, views, W, H, cap):
 
 
 @pytest.mark.parametrize("n,views,W,H,cap", [
-    (3328, 1, 48, 48, 6656), (3329, 1, 48, 48, 6658), (4096, 3, 80, 64, 1 << 17), (16384, 1, 48, 48, 1 << 19),
-    (5000, 2, 64, 64, 4097), (6000, 1, 200, 150, 9001), (9000, 2, 100, 60, 20000), (9000, 2, 100, 60, 1)])
+    (3072, 1, 48, 48, 6144), (3073, 1, 48, 48, 6146), (4096, 3, 80, 64, 1 << 17), (16384, 1, 48, 48, 1 << 20),
+    (5000, 2, 64, 64, 4097), (9000, 1, 200, 150, 13001), (9000, 2, 100, 60, 20000), (9000, 2, 100, 60, 1)])
 def test_sort_lists_at_record_limit(n, views, W, H, cap):
     """Both sides of the small sort's limits of records per unit, and a capacity that runs out in the general design:
     in its first window of 4,096 staged instances, behind it, and inside a record."""
@@ -260,13 +260,13 @@ def test_sort_lists_at_record_limit(n, views, W, H, cap):
 
 
 @pytest.mark.parametrize("n,views,W,H,cap,small", [
-    (3328, 1, 48, 48, 2, True), (3329, 1, 48, 48, 2, False), (4608, 8, 128, 128, 4, True),
-    (4609, 8, 128, 128, 4, False), (16384, 1, 64, 64, 4, False), (16384, 1, 64, 64, 23, True),
-    (16384, 1, 64, 64, 22, False), (16385, 1, 64, 64, 40, False), (500, 1, 2048, 512, 4, True),
-    (500, 1, 2048, 1024, 4, False)])
+    (3072, 1, 48, 48, 2, True), (3073, 1, 48, 48, 2, False), (4096, 1, 64, 64, 4, True), (4097, 1, 64, 64, 4, False),
+    (6144, 8, 128, 128, 4, True), (6145, 8, 128, 128, 4, False), (16384, 1, 64, 64, 4, False),
+    (16384, 1, 64, 64, 52, True), (16384, 1, 64, 64, 51, False), (16385, 1, 64, 64, 60, False),
+    (500, 1, 2048, 512, 4, True), (500, 1, 2048, 1024, 4, False)])
 def test_sort_design_by_sizes(n, views, W, H, cap, small):
-    """The small sort's four launches up to 4,096 lists and 2,048 + 640 records per unit and instance that the capacity
-    leaves a record (16,384 at most), the general design's beyond: there it is the faster one."""
+    """The small sort's four launches up to 4,096 lists and 1,024 log2(tiles) + 256 (capacity per record - 4) records
+    per unit, at least 3,072 and at most 16,384; the general design's beyond, the faster one unless a splat is large."""
     import paper_2509_12138_gb300 as gs
     g = synth.random_gaussians(n, 0, n, extent=0.8, log_scale_range=(-4.0, -3.0))
     cams = synth.orbital_cameras(8, 3.0, width=W, height=H).subset(list(range(views)))
