@@ -172,9 +172,10 @@ __host__ __device__ __forceinline__ int param_planes(int deg) {
 // chains of 4 to 45 short kernels, and launching them back to back left 1 to 3
 // us between each two: a training step of 200k Gaussians 747 -> 647 us, of 1M
 // 1461 -> 1357, deterministic gradients of 700k 1022 -> 916, 8 views of 2,000
-// 397 -> 365.  Kernels of a captured graph gain nothing.  Letting the next kernel's blocks start before this one's end
-// (griddepcontrol.launch_dependents behind the wait) measured 682, 1379, 948
-// and 364: they take the slots of blocks that still have work.
+// 397 -> 365.  Kernels of a captured graph gain nothing.  Letting the next
+// kernel's blocks start before this one's end (griddepcontrol.launch_dependents
+// behind the wait) measured 682, 1379, 948 and 364: they take the slots of
+// blocks that still have work.
 __device__ __forceinline__ void gs_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 }  // namespace gs

@@ -127,9 +127,10 @@ __device__ __forceinline__ void visit(const Grid& g, const uint32_t* __restrict_
   }
 }
 
-// Bound by the latency of the rows of cells.  1M points of an interface, k = 16:
-// 1721 us with sorted (distance, index) insertions, cells visited one by one and
-// points in input order, 673 us.
+// Bound by instruction issue (59% of cycles) with 12 of 32 lanes active, the
+// warp's points' rows ending at different lengths.  1M points of an interface, k
+// = 16: 1721 us with sorted (distance, index) insertions, cells visited one by
+// one and points in input order, 673 us.
 constexpr int KNN_T = 128;
 template <int K>
 __global__ void __launch_bounds__(KNN_T) k_knn_query(int64_t n, Grid g, const uint32_t* __restrict__ start,

@@ -984,7 +984,9 @@ __global__ void __launch_bounds__(PBA_T) k_project_bwd_adam1(float4* __restrict_
 }
 
 __global__ void k_step_advance(int32_t* s) {
-  gs_wait_previous(); *s += 1; }
+  gs_wait_previous();
+  *s += 1;
+}
 
 }  // namespace
 

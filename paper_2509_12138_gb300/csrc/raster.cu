@@ -454,7 +454,12 @@ __device__ __forceinline__ uint32_t eval_hit(float rx, float ry, float4 co, floa
 // and the order of a pixel's compositing are those of a sequential walk.  Bound
 // by instruction issue (47-70% of cycles on a 2M scene) and, on edge-on views,
 // by the longest block's serial walk.  Forward stage at one lane per pixel and
-// hit -> this: 200k at 960x540 134 -> 88 us, 1M at 1080p 319 -> 181 us.  Three
+// hit -> this: 200k at 960x540 134 -> 72 us, 1M at 1080p 319 -> 181 us.  Where a
+// splat covers whole blocks, one lane per pixel and hit evaluates as few pairs
+// and is the faster one by 5 to 20% (whole lists of 1M splats of 6 pixels at
+// 1080p 730 us, this 854; of a few dozen entries at 800x600 18, this 30), but a
+// choice per batch or per list within the kernel cost the small splats 3 to 10%
+// in registers, and a second kernel more than that.  Three
 // or four pairs per step of the pixel-major loop, or four pixels per step of the
 // record-major one, cost registers and were slower (10M at 1080p 1157 us with
 // two, 1208, 1302 and 1264).
@@ -809,7 +814,8 @@ __global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict
   const int lane = threadIdx.x & 31;
   const int lists = lists_in_use(job_base, NT);
   const uint32_t total = (uint32_t)lists * 8u;
-  const int M = resident ? front_chunks(ranges, order, job_base[NT], (uint32_t)lists, (uint32_t)NT, resident, K) : INT_MAX;
+  const int M = resident ? front_chunks(ranges, order, job_base[NT], (uint32_t)lists, (uint32_t)NT, resident, K)
+                         : INT_MAX;
   auto unit = [&](uint32_t vb) {
     const int o = (int)(vb >> 3), w = (int)(vb & 7u);
     PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
@@ -828,11 +834,13 @@ __global__ void __launch_bounds__(32) k_render_fwd_front(const uint2* __restrict
       if (__all_sync(0xffffffffu, done)) break;
       const float Tin = T, i0 = c0, i1 = c1, i2 = c2;
       const bool was = done;
-      const float4 loc = walk_chunk<BW>(vals, masks, xy, conic_op, rgb, rg.x, c * K, min(c * K + K, L), P.wbits, (float)(P.tx * TILE),
-                     (float)(P.ty * TILE), (float)P.ox, (float)P.oy, s_walk, T, c0, c1, c2, last, done,
-                     c > 0 && P.inside, cpp + (int64_t)(c - 1) * TILE_PIX, clp + (int64_t)(c - 1) * TILE_PIX);
-      // a chunk without a stop enters by its partial, as the combine's do, so that images do not depend on M;
-      // from a stop chunk on (and in whole-list walks) the walked state counts
+      const float4 loc = walk_chunk<BW>(vals, masks, xy, conic_op, rgb, rg.x, c * K, min(c * K + K, L), P.wbits,
+                                        (float)(P.tx * TILE), (float)(P.ty * TILE), (float)P.ox, (float)P.oy, s_walk,
+                                        T, c0, c1, c2, last, done, c > 0 && P.inside,
+                                        cpp + (int64_t)(c - 1) * TILE_PIX, clp + (int64_t)(c - 1) * TILE_PIX);
+      // a chunk without a stop enters by its partial, as the combine's do, so that images do not depend on M (but for
+      // a pixel whose stop falls on the two sides of one rounding); from a stop chunk on (and in whole-list walks) the
+      // walked state counts
       in_order = in_order || !(Tin * loc.x >= T_MIN);
       if (!in_order && !done && !was) {
         T = Tin * loc.x;
@@ -1062,74 +1070,77 @@ __global__ void __launch_bounds__(32) k_render_fwd_stop(const uint2* __restrict_
   __shared__ FwdScratch s_walk;
   const uint32_t total = queue[qcap];
   auto job = [&](uint32_t ent) {
-  uint32_t jid = ent >> 3;
-  int o = (int)jobs[2 * (int64_t)jid], ch = (int)jobs[2 * (int64_t)jid + 1];
-  if (ch == 0) return;
-  int nch = (int)(job_base[o + 1] - job_base[o]);
-  int w = (int)(ent & 7u);
-  PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
-  uint2 rg = ranges[(int64_t)P.u * n_tiles + P.tile];
-  int L = (int)(rg.y - rg.x);
-  int64_t plane = (int64_t)W * H;
-  int64_t pix = (int64_t)P.py * W + P.px;
-  float* im = img + (int64_t)P.u * 3 * plane;
-  float* fT = final_T + (int64_t)P.u * plane;
-  uint32_t* nc = n_contrib + (int64_t)P.u * plane;
-  bool mine = false;
-  float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-  int last = 0;
-  int64_t cp0 = (int64_t)job_base[o] - o;
-  if (P.inside) {
-    uint32_t lw = nc[pix];
-    mine = (lw & REWALK_BIT) != 0u && (int)(lw & ~REWALK_BIT) == ch;
-    if (mine) {
-      last = (int)chunk_last[(cp0 + ch - 1) * TILE_PIX + P.pix_local];  // left there by the combine
-      c0 = im[pix]; c1 = im[plane + pix]; c2 = im[2 * plane + pix];
-      T = fT[pix];
+    uint32_t jid = ent >> 3;
+    int o = (int)jobs[2 * (int64_t)jid], ch = (int)jobs[2 * (int64_t)jid + 1];
+    if (ch == 0) return;
+    int nch = (int)(job_base[o + 1] - job_base[o]);
+    int w = (int)(ent & 7u);
+    PixelOf<BW> P(order, o, w, n_tiles, TX, W, H);
+    uint2 rg = ranges[(int64_t)P.u * n_tiles + P.tile];
+    int L = (int)(rg.y - rg.x);
+    int64_t plane = (int64_t)W * H;
+    int64_t pix = (int64_t)P.py * W + P.px;
+    float* im = img + (int64_t)P.u * 3 * plane;
+    float* fT = final_T + (int64_t)P.u * plane;
+    uint32_t* nc = n_contrib + (int64_t)P.u * plane;
+    bool mine = false;
+    float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
+    int last = 0;
+    int64_t cp0 = (int64_t)job_base[o] - o;
+    if (P.inside) {
+      uint32_t lw = nc[pix];
+      mine = (lw & REWALK_BIT) != 0u && (int)(lw & ~REWALK_BIT) == ch;
+      if (mine) {
+        last = (int)chunk_last[(cp0 + ch - 1) * TILE_PIX + P.pix_local];  // left there by the combine
+        c0 = im[pix]; c1 = im[plane + pix]; c2 = im[2 * plane + pix];
+        T = fT[pix];
+      }
     }
-  }
-  // only the 4x4 pixel blocks of this warp's walking pixels: records whose block mask misses them
-  // cannot reach those pixels
-  uint32_t my_block = mine ? 1u << (4 * ((P.py - P.ty * TILE) >> 2) + ((P.px - P.tx * TILE) >> 2)) : 0u;
-  uint32_t wbits = __reduce_or_sync(0xffffffffu, my_block);
-  if (!wbits) return;
-  bool done = !mine;
-  // walk chunk c* (and, should the pixel not stop there after all, the chunks after it), keeping each
-  // walked chunk's partial and the T in front of it; chunks behind the stop get the identity partial
-  int c = ch;
-  for (; c < nch; ++c) {
-    walk_chunk<BW>(vals, masks, xy, conic_op, rgb, rg.x, c * K, min(c * K + K, L), wbits, (float)(P.tx * TILE),
-                   (float)(P.ty * TILE), (float)P.ox, (float)P.oy, s_walk, T, c0, c1, c2, last, done, mine,
-                   ckpt + (cp0 + c - 1) * TILE_PIX + P.pix_local, chunk_last + (cp0 + c - 1) * TILE_PIX + P.pix_local);
-    if (__all_sync(0xffffffffu, done)) break;
-  }
-  if (!mine) return;
-  // checkpoints: (T in front of boundary b, colour behind it per unit T), composited back to front
-  float4* cpp = ckpt + cp0 * TILE_PIX + P.pix_local;  // slot of boundary b: cpp[(b - 1) * TILE_PIX]
-  const uint32_t* clp = chunk_last + cp0 * TILE_PIX + P.pix_local;
-  for (int b = nch - 1; b > c; --b)
-    cpp[(int64_t)(b - 1) * TILE_PIX] = make_float4(T, bg0, bg1, bg2);  // behind the stop: final state
-  float S0 = bg0, S1 = bg1, S2 = bg2;
-  close_checkpoints(cpp, clp, ch, min(c, nch - 1), S0, S1, S2);  // walked chunks
-  for (int bb = 1; bb < ch; bb += CB) {  // in front of c*: S_b = A_b + B_b S_c* as left by the combine
-    float4 abv[CB];
-    uint32_t tv[CB];
-    #pragma unroll
-    for (int q = 0; q < CB; ++q)
-      if (bb + q < ch) { abv[q] = cpp[(int64_t)(bb + q - 1) * TILE_PIX]; tv[q] = clp[(int64_t)(bb + q - 1) * TILE_PIX]; }
-    #pragma unroll
-    for (int q = 0; q < CB; ++q) {
-      if (bb + q >= ch) break;
-      float4 ab = abv[q];
-      cpp[(int64_t)(bb + q - 1) * TILE_PIX] = make_float4(__uint_as_float(tv[q]), ab.y + ab.x * S0,
-                                                          ab.z + ab.x * S1, ab.w + ab.x * S2);
+    // only the 4x4 pixel blocks of this warp's walking pixels: records whose block mask misses them
+    // cannot reach those pixels
+    uint32_t my_block = mine ? 1u << (4 * ((P.py - P.ty * TILE) >> 2) + ((P.px - P.tx * TILE) >> 2)) : 0u;
+    uint32_t wbits = __reduce_or_sync(0xffffffffu, my_block);
+    if (!wbits) return;
+    bool done = !mine;
+    // walk chunk c* (and, should the pixel not stop there after all, the chunks after it), keeping each
+    // walked chunk's partial and the T in front of it; chunks behind the stop get the identity partial
+    int c = ch;
+    for (; c < nch; ++c) {
+      walk_chunk<BW>(vals, masks, xy, conic_op, rgb, rg.x, c * K, min(c * K + K, L), wbits, (float)(P.tx * TILE),
+                     (float)(P.ty * TILE), (float)P.ox, (float)P.oy, s_walk, T, c0, c1, c2, last, done, mine,
+                     ckpt + (cp0 + c - 1) * TILE_PIX + P.pix_local, chunk_last + (cp0 + c - 1) * TILE_PIX + P.pix_local);
+      if (__all_sync(0xffffffffu, done)) break;
     }
-  }
-  im[pix] = c0 + T * bg0;
-  im[plane + pix] = c1 + T * bg1;
-  im[2 * plane + pix] = c2 + T * bg2;
-  fT[pix] = T;
-  nc[pix] = (uint32_t)last;
+    if (!mine) return;
+    // checkpoints: (T in front of boundary b, colour behind it per unit T), composited back to front
+    float4* cpp = ckpt + cp0 * TILE_PIX + P.pix_local;  // slot of boundary b: cpp[(b - 1) * TILE_PIX]
+    const uint32_t* clp = chunk_last + cp0 * TILE_PIX + P.pix_local;
+    for (int b = nch - 1; b > c; --b)
+      cpp[(int64_t)(b - 1) * TILE_PIX] = make_float4(T, bg0, bg1, bg2);  // behind the stop: final state
+    float S0 = bg0, S1 = bg1, S2 = bg2;
+    close_checkpoints(cpp, clp, ch, min(c, nch - 1), S0, S1, S2);  // walked chunks
+    for (int bb = 1; bb < ch; bb += CB) {  // in front of c*: S_b = A_b + B_b S_c* as left by the combine
+      float4 abv[CB];
+      uint32_t tv[CB];
+      #pragma unroll
+      for (int q = 0; q < CB; ++q)
+        if (bb + q < ch) {
+          abv[q] = cpp[(int64_t)(bb + q - 1) * TILE_PIX];
+          tv[q] = clp[(int64_t)(bb + q - 1) * TILE_PIX];
+        }
+      #pragma unroll
+      for (int q = 0; q < CB; ++q) {
+        if (bb + q >= ch) break;
+        float4 ab = abv[q];
+        cpp[(int64_t)(bb + q - 1) * TILE_PIX] = make_float4(__uint_as_float(tv[q]), ab.y + ab.x * S0,
+                                                            ab.z + ab.x * S1, ab.w + ab.x * S2);
+      }
+    }
+    im[pix] = c0 + T * bg0;
+    im[plane + pix] = c1 + T * bg1;
+    im[2 * plane + pix] = c2 + T * bg2;
+    fT[pix] = T;
+    nc[pix] = (uint32_t)last;
   };
   const bool lead = (threadIdx.x & 31) == 0;
   uint32_t e = __shfl_sync(0xffffffffu, lead ? atomicAdd(ticket, 1u) : 0u, 0);
@@ -1209,9 +1220,9 @@ __device__ __forceinline__ void bwd_queue_flush(const float4* s_q, int head, int
 // [c K, min((c + 1) K, L)) of the list back to front.  It starts from the
 // forward's checkpoint at the chunk's end (T in front of it and the colour
 // behind it per unit T), or from final_T and the background for the last
-// chunk.  Headers two rounds ahead, hit records one round ahead, as in the
-// forward.  The gradient terms of sparse hits go through a per-warp ring (float
-// accumulation; k_render_bwd_det has the deterministic one).
+// chunk.  Masks and ids are read two rounds of 32 entries ahead, hit records one
+// round ahead.  The gradient terms of sparse hits go through a per-warp ring
+// (float accumulation; k_render_bwd_det has the deterministic one).
 template <int BW>
 __global__ void __launch_bounds__(32, 32) k_render_bwd_m(const uint2* __restrict__ ranges,
                                                            const uint32_t* __restrict__ order,

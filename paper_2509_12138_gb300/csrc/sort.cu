@@ -11,8 +11,9 @@
 //   scan    : one CTA per digit scans that digit's per-block counts in block
 //             order and adds the digit's global base; a pass whose keys all
 //             share one digit is detected here and skipped (no data moves);
-//   scatter : each block ranks its keys stably (warp match + per-warp digit
-//             counts, in key order) and writes them to the other buffer.
+//   scatter : each block ranks its keys stably (votes on the digit bits, or the
+//             match instruction, and per-warp digit counts, in key order) and
+//             writes them to the other buffer.
 // Which buffer holds the current keys is tracked on the device (cur[pass]),
 // so skipped passes need no host decision.
 #include <cuda_runtime.h>
@@ -580,19 +581,19 @@ __global__ void __launch_bounds__(SCAN_T) k_vis_reduce(const uint32_t* __restric
       add(t4[j].x, d4[j].x); add(t4[j].y, d4[j].y); add(t4[j].z, d4[j].z); add(t4[j].w, d4[j].w);
     }
   } else {
-  #pragma unroll
-  for (int j = 0; j < SCAN_ITEMS; ++j) {
-    int64_t k = base + (int64_t)j * SCAN_T + threadIdx.x;
-    if (k < P) {
-      // both loads issued before either is tested (a depth load behind the visibility test doubled the
-      // kernel's time)
-      uint32_t tk = tiles[k], dk = __float_as_uint(depth[k]);
-      if (tk > 0u) {
-        ++s;
-        mn = min(mn, dk);
+    #pragma unroll
+    for (int j = 0; j < SCAN_ITEMS; ++j) {
+      int64_t k = base + (int64_t)j * SCAN_T + threadIdx.x;
+      if (k < P) {
+        // both loads issued before either is tested (a depth load behind the visibility test doubled the
+        // kernel's time)
+        uint32_t tk = tiles[k], dk = __float_as_uint(depth[k]);
+        if (tk > 0u) {
+          ++s;
+          mn = min(mn, dk);
+        }
       }
     }
-  }
   }
   mn = __reduce_min_sync(0xffffffffu, mn);
   __syncthreads();  // s_min initialised
@@ -670,8 +671,8 @@ __device__ __forceinline__ uint32_t tile_blocks(int b, int e, int t) {
 // view's depths stay within a factor of ~4 (then the device skips the top radix pass).
 // Round j of a block covers its records [256 j, 256 j + 256) (coalesced loads); a record's slot is the
 // block's base, the visible records of earlier (round, warp) pairs and those of lower lanes.  Every load of a
-// thread's records is issued first, wanted or not: bound by the loads in flight (10M records 123 us with the
-// depth read behind the visibility test, the tests one after the other).
+// thread's records is issued first, wanted or not: bound by the loads in flight (10M records 23 us; 24 to 26
+// with the depth read behind the visibility test).
 // DESC: also the visible records' packed rectangles, by record.
 template <bool DESC>
 __global__ void __launch_bounds__(SCAN_T) k_vis_compact(const uint32_t* __restrict__ tiles,
@@ -967,8 +968,8 @@ __global__ void __launch_bounds__(256) k_ranges32(const uint32_t* __restrict__ k
 // The whole schedule of up to SCHED_ONE lists in one CTA: the tile order
 // (heaviest length classes first), the job base of every order position and
 // the chunk jobs.  It replaces a memset and seven launches of a few
-// microseconds each, 25 us of a 1080p view's sort; beyond the lists one CTA
-// holds, those pay.
+// microseconds each, 25 us of a 1080p view's sort.  8192 lists are 8 per thread
+// and 37 KB of shared memory (a 1080p view has 8160); more were not measured.
 constexpr int SCHED_ONE = 8192, SCHED_T = 1024, SCHED_PER = SCHED_ONE / SCHED_T;
 __global__ void __launch_bounds__(SCHED_T) k_schedule(const uint2* __restrict__ ranges, int NT, int K,
                                                       uint32_t* __restrict__ order, uint32_t* __restrict__ job_base,

@@ -139,7 +139,7 @@ def test_knn_points_outside_the_grid(k, cells):
 
 @pytest.mark.parametrize("k", [3, 8, 16])
 def test_knn_distances_past_the_float_range(k):
-    """A point whose squared distance overflows float32 is no neighbour: its slot is -1 / inf, as when there are too few."""
+    """A point whose squared distance overflows float32 is no neighbour: its slot is -1 / inf, as with too few points."""
     x = np.array([0.0, 1.0, 2.0, 1e20, 1e20 + 1e13, 3e20, np.nan, np.inf], np.float32)
     pts = np.zeros((len(x), 3), np.float32)
     pts[:, 0] = x
@@ -348,7 +348,9 @@ def test_sort_by_packed_rectangles_equals_global(views, masks):
         fr.sort(design)
         count = fr.instances()
         assert fr.read_status() == 0 and n * views // 2 < count <= cap
-        got.append([fr.sorted_vals[:count].clone(), fr.ranges.clone()] + ([fr.block_masks[:count].clone()] if masks else []))
+        got.append([fr.sorted_vals[:count].clone(), fr.ranges.clone()])
+        if masks:
+            got[-1].append(fr.block_masks[:count].clone())
         del fr
     for other in got[:2]:
         assert all(torch.equal(a, b) for a, b in zip(other, got[2]))
