@@ -607,7 +607,8 @@ int gs_opacity_reset(float* params, float* m, float* v, int64_t n_gauss, float m
  *
  * gs_knn: exact k nearest neighbours (self excluded) of n points [n][3] on a
  * uniform grid of grid_dims[0..2] cells of edge cell_size starting at
- * grid_lo (host float[3]; the grid must cover the points' bounding box),
+ * grid_lo (host float[3]; the grid should cover the points' bounding box:
+ * points outside it are held by its outermost cells, which costs time),
  * k in {3, 8, 16}.  idx [n][k] int32, dist [n][k] fp32 (Euclidean),
  * ordered by (distance, index); -1 / inf when fewer than k other points
  * exist.  Workspace: gs_knn_workspace_size(n, grid_dims (host int32[3])). */
